@@ -1,123 +1,60 @@
 // A*X products of SNMPBB: the only O(n^2 r) (dense) / O(nnz r) (sparse) step of an
 // iteration (Sec. 4.1 complexity list; the V H^T product of Eqs. (2.1)-(2.2)).
 //
-//   k_gemm_dense : CUDA-core tiled GEMM for FP64 / FP32 A (64x64 CTA tile, 4x4 register
-//                  micro-tile, smem staged, register prefetch).  Split-K writes each split
-//                  to its own workspace slice; the finish pass sums the slices in a fixed
-//                  order, so results are deterministic.
+//   k_gemm_dense : CUDA-core tiled product for FP64 / FP32 A, and for the final evaluation of
+//                  BF16 and E4M3 A (gemm_dev.cuh).  Split-K writes each split to its own
+//                  workspace slice; the finish pass sums the slices in a fixed order, so
+//                  results are deterministic.
 //   k_spmm_csr   : one warp per row, lanes across the factor columns (coalesced rows of X).
 //   k_ax_finish  : fused epilogue: sum of split slices, Y += c X2, and per-restart FP64
 //                  partials of <P1, A X> and <P2, A X> (e.g. tr(W^T A W)).
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <mutex>
 
 #include "common.cuh"
+#include "gemm_dev.cuh"
 
 namespace snmf {
 
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16, TM = 4, TN = 4;
-
-__device__ __forceinline__ float ld_a(const __nv_bfloat16* p) { return __bfloat162float(*p); }
 __device__ __forceinline__ float ld_a(const float* p) { return *p; }
 __device__ __forceinline__ double ld_a(const double* p) { return *p; }
 
-// TA: stored type of A (T, or BF16 read into FP32 registers: the FP32-accumulated product
-// of the stored BF16 operator, used where the tensor-core accumulation is not accurate
-// enough, i.e. the closed-form objective of the final evaluation)
-// SYM: A holds the upper 128 x 128 tiles of the symmetric matrix (sym_tile, lda = tiles a side);
-// entry (r, k) below the diagonal tiles is entry (k, r) of the stored mirror tile.
-template <typename T, typename TA = T, bool SYM = false>
-__global__ void __launch_bounds__(256)
-k_gemm_dense(const TA* __restrict__ A, int64_t lda, const T* __restrict__ X, int64_t ld,
-             T* __restrict__ Y, int64_t n, int cols, int64_t kchunk, const int* run) {
+template <typename C, typename TA, int PER_SM>
+__global__ void __launch_bounds__(C::NT, PER_SM)
+k_gemm_dense(const TA* __restrict__ A, int64_t lda, const typename C::T* __restrict__ X, int64_t ld,
+             typename C::T* __restrict__ Y, int64_t n, int cols, int64_t kchunk, bool avec, bool xvec, GemmA8 a8,
+             const int* run) {
+  using T = typename C::T;
+  extern __shared__ __align__(16) unsigned char gemm_sm[];
   if (run && *run == 0) return;
-  __shared__ T As[2][BK][BM + 4];
-  __shared__ T Xs[2][BK][BN + 4];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int64_t row0 = (int64_t)blockIdx.y * BM;
-  const int col0 = blockIdx.x * BN;
-  const int64_t k_begin = (int64_t)blockIdx.z * kchunk;
-  const int64_t k_end = min(n, k_begin + kchunk);
+  const int64_t row0 = (int64_t)blockIdx.y * C::BM, k0 = (int64_t)blockIdx.z * kchunk;
+  const int col0 = blockIdx.x * C::BN;
+  T acc[C::TM][C::TN];
+  gemm_tile<C>(A, lda, X, ld, n, cols, row0, col0, k0, min(n, k0 + kchunk), avec, xvec, a8,
+               reinterpret_cast<T*>(gemm_sm), acc);
   T* Yout = Y + (int64_t)blockIdx.z * n * ld;
-
-  // loader mapping: A tile BM x BK (row-major A: consecutive k contiguous)
-  // each thread loads 4 elements: rows la_r + 16*m, column la_c
-  const int la_c = threadIdx.x & 15;      // k offset
-  const int la_r = threadIdx.x >> 4;      // 0..15
-  // X tile BK x BN: thread loads 4 elements: row lx_r, cols lx_c + 16*m
-  const int lx_c = threadIdx.x & 15;
-  const int lx_r = threadIdx.x >> 4;
-
-  T acc[TM][TN];
+  const int tx = threadIdx.x % C::TX, ty = threadIdx.x / C::TX;
 #pragma unroll
-  for (int i = 0; i < TM; ++i)
-#pragma unroll
-    for (int j = 0; j < TN; ++j) acc[i][j] = T(0);
-
-  T ra[4], rx[4];
-  auto load_regs = [&](int64_t k0) {
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      int64_t r = row0 + la_r + 16 * m;
-      int64_t k = k0 + la_c;
-      const TA* pa;
-      if constexpr (SYM) {
-        const int64_t ta = r >> 7, tb = k >> 7;
-        pa = ta <= tb ? A + (sym_tile(ta, tb, lda) << 14) + ((r & 127) << 7) + (k & 127)
-                      : A + (sym_tile(tb, ta, lda) << 14) + ((k & 127) << 7) + (r & 127);
-      } else {
-        pa = A + r * lda + k;
-      }
-      ra[m] = (r < n && k < k_end) ? (T)ld_a(pa) : T(0);
-      int c = col0 + lx_c + 16 * m;
-      int64_t kr = k0 + lx_r;
-      rx[m] = (kr < k_end && c < cols) ? X[kr * ld + c] : T(0);
-    }
-  };
-  auto store_smem = [&](int buf) {
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      As[buf][la_c][la_r + 16 * m] = ra[m];
-      Xs[buf][lx_r][lx_c + 16 * m] = rx[m];
-    }
-  };
-
-  int buf = 0;
-  if (k_begin < k_end) {
-    load_regs(k_begin);
-    store_smem(0);
-  }
-  __syncthreads();
-  for (int64_t k0 = k_begin; k0 < k_end; k0 += BK) {
-    const bool more = (k0 + BK) < k_end;
-    if (more) load_regs(k0 + BK);
-#pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      T a[TM], x[TN];
-#pragma unroll
-      for (int i = 0; i < TM; ++i) a[i] = As[buf][kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < TN; ++j) x[j] = Xs[buf][kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], x[j], acc[i][j]);
-    }
-    if (more) store_smem(buf ^ 1);
-    __syncthreads();
-    buf ^= 1;
-  }
-#pragma unroll
-  for (int i = 0; i < TM; ++i) {
-    int64_t r = row0 + ty + 16 * i;
+  for (int i = 0; i < C::TM; ++i) {
+    const int64_t r = row0 + ty + C::TY * i;
     if (r >= n) continue;
 #pragma unroll
-    for (int j = 0; j < TN; ++j) {
-      int c = col0 + tx + 16 * j;
-      if (c < cols) Yout[r * ld + c] = acc[i][j];
+    for (int j = 0; j < C::TN; j += C::VW) {
+      const int c = col0 + C::col(tx, j);
+      T* p = Yout + r * ld + c;
+      if (C::VW == 4 && xvec) {  // the pitch and the columns of Y are X's
+        if (c < cols) *reinterpret_cast<float4*>(p) = make_float4(acc[i][j], acc[i][j + 1 < C::TN ? j + 1 : j],
+                                                                  acc[i][j + 2 < C::TN ? j + 2 : j],
+                                                                  acc[i][j + 3 < C::TN ? j + 3 : j]);
+      } else {
+#pragma unroll
+        for (int u = 0; u < C::VW; ++u)
+          if (c + u < cols) p[u] = acc[i][j + u];
+      }
     }
   }
 }
@@ -154,40 +91,80 @@ k_spmm_csr(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colid
   }
 }
 
-// Epilogue over a row tile x one restart.  splits > 1: Y = sum_s ws[s] (fixed order).
-template <typename T>
+// Epilogue over a row tile x one restart.  splits > 1: Y = sum_s ws[s] (fixed order).  V values of
+// a row per access (16 bytes where r and the pitch allow it), four accesses of a thread and up to
+// eight of their slices in flight.  8192 x 64 in FP32, 8 slices: 24 us with single values, one after
+// the other.
+template <typename T, int V>
 __global__ void __launch_bounds__(256)
 k_ax_finish(int64_t n, int r, int64_t ld, T* __restrict__ Y, const T* __restrict__ ws,
             int splits, double c, const T* __restrict__ X2, const T* __restrict__ P1,
             const T* __restrict__ P2, double* __restrict__ part, int q0, int b,
             const int* run, int dots_after) {
+  struct alignas(V * sizeof(T)) Vec {
+    T v[V];
+  };
   __shared__ T sh[32];
   const int j = blockIdx.y;
   const int64_t i0 = (int64_t)blockIdx.x * kRowTile;
   T d1 = T(0), d2 = T(0);  // per-CTA partials in the working type (FP64 across CTAs)
   if (!(run && *run == 0)) {
-    const int tile = kRowTile * r;
-    for (int e = threadIdx.x; e < tile; e += blockDim.x) {
-      const int64_t i = i0 + e / r;
-      if (i >= n) break;
-      const int64_t idx = i * ld + (int64_t)j * r + (e % r);
-      T y;
-      if (splits > 1) {
-        y = ws[idx];
-        for (int s = 1; s < splits; ++s) y += ws[(int64_t)s * n * ld + idx];
-      } else {
-        y = Y[idx];
+    const int rv = r / V, rows = (int)min((int64_t)kRowTile, n - i0);
+    const int tile = rows * rv;
+    const int64_t slice = n * ld;
+    constexpr int U = 4;
+    for (int e0 = threadIdx.x; e0 < tile; e0 += 256 * U) {
+      Vec y[U], x2[U], p1[U], p2[U];
+      int64_t idx[U];
+      bool ok[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int e = e0 + 256 * u;
+        ok[u] = e < tile;
+        const int i = ok[u] ? e / rv : 0;
+        idx[u] = (i0 + i) * ld + (int64_t)j * r + (ok[u] ? e - i * rv : 0) * V;
+        auto get = [&](const T* p) {
+          Vec v;
+          if (p && ok[u]) return *reinterpret_cast<const Vec*>(p + idx[u]);
+#pragma unroll
+          for (int k = 0; k < V; ++k) v.v[k] = T(0);
+          return v;
+        };
+        y[u] = get(splits > 1 ? ws : Y);
+        x2[u] = get(X2);
+        p1[u] = get(P1);
+        p2[u] = get(P2);
       }
-      if (!dots_after) {
-        if (P1) d1 += P1[idx] * y;
-        if (P2) d2 += P2[idx] * y;
+#pragma unroll 2
+      for (int s = 1; s < splits; ++s) {
+        Vec w[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (ok[u]) w[u] = *reinterpret_cast<const Vec*>(ws + s * slice + idx[u]);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (ok[u]) {
+#pragma unroll
+            for (int k = 0; k < V; ++k) y[u].v[k] += w[u].v[k];
+          }
       }
-      if (X2) y = y + (T)c * X2[idx];
-      if (dots_after) {
-        if (P1) d1 += P1[idx] * y;
-        if (P2) d2 += P2[idx] * y;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (!ok[u]) continue;
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+          if (!dots_after) {
+            d1 += p1[u].v[k] * y[u].v[k];
+            d2 += p2[u].v[k] * y[u].v[k];
+          }
+          if (X2) y[u].v[k] = y[u].v[k] + (T)c * x2[u].v[k];
+          if (dots_after) {
+            d1 += p1[u].v[k] * y[u].v[k];
+            d2 += p2[u].v[k] * y[u].v[k];
+          }
+        }
+        *reinterpret_cast<Vec*>(Y + idx[u]) = y[u];
       }
-      Y[idx] = y;
     }
   }
   d1 = block_sum_t(d1, sh);
@@ -229,34 +206,80 @@ void launch_csr_check(const int32_t* rowptr, const int32_t* colidx, int64_t n, i
   k_csr_check<<<blocks, 256, 0, s>>>(rowptr, colidx, n, nnz, bad);
 }
 
+namespace {
+
+template <typename C, typename TA, int PER_SM>
+int launch_gemm_cfg(const AxArgs& a, int64_t n, int cols, int64_t ld, const void* X, void* Y, void* ws, size_t ws_elems,
+                    const int* run, cudaStream_t s, const ProdTune* tune) {
+  using T = typename C::T;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    cudaFuncSetAttribute(k_gemm_dense<C, TA, PER_SM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+  });
+  const int gx = cdiv64(cols, C::BN), gy = cdiv64(n, C::BM);
+  // split-K: the number of K chunks (of 64 columns and more, 32 in FP64, where a CTA is long) that
+  // fills whole waves of CTAs best; each further slice has to gain a per cent, for the finish
+  // pass (n = 8192, 64 columns: 8 slices leave a sixth of the SMs a CTA short)
+  constexpr int64_t kMin = sizeof(T) == 8 ? 32 : 64;
+  const int64_t tiles = (int64_t)gx * gy, slots = (int64_t)152 * PER_SM;
+  const int64_t most = std::min<int64_t>({(n + kMin - 1) / kMin, 32, (int64_t)(ws_elems / ((size_t)n * (size_t)ld))});
+  int64_t splits = 1;
+  double best = 0.0;
+  for (int64_t sp = 1; sp <= std::max<int64_t>(1, most); ++sp) {
+    const int64_t ctas = tiles * sp, waves = (ctas + slots - 1) / slots;
+    const double gain = (double)ctas / (double)(waves * slots) * (1.0 - 0.01 * (double)sp);
+    if (gain > best) { best = gain; splits = sp; }
+  }
+  if (tune && tune->splits > 0) splits = tune->splits;  // autotuned
+  splits = std::max<int64_t>(1, std::min<int64_t>(splits, ws_elems / ((size_t)n * (size_t)ld)));
+  const int64_t kchunk = (cdiv64(n, (int)splits) + 31) / 32 * 32;
+  splits = cdiv64(n, kchunk);
+  constexpr int64_t KV = C::KV;
+  const bool avec = C::KIND == GA_SAME && a.lda % KV == 0 && n % KV == 0 && !((uintptr_t)a.A & 15);
+  const bool xvec = ld % KV == 0 && cols % KV == 0 && !((uintptr_t)X & 15) && !((uintptr_t)Y & 15);
+  dim3 grid(gx, gy, (unsigned)splits);
+  k_gemm_dense<C, TA, PER_SM><<<grid, C::NT, C::SMEM, s>>>((const TA*)a.A, a.lda, (const T*)X, ld,
+                                                           (T*)(splits > 1 ? ws : Y), n, cols, kchunk, avec, xvec,
+                                                           GemmA8{a.a_scale, (int)((n + 127) / 128)}, run);
+  return (int)splits;
+}
+
+}  // namespace
+
 int launch_ax(const AxArgs& a, int tdtype, int64_t n, int cols, int64_t ld, const void* X,
               void* Y, void* ws, size_t ws_elems, const int* run, cudaStream_t s, const ProdTune* tune) {
   if (a.kind == AX_DENSE) {
-    const int gx = cdiv64(cols, BN), gy = cdiv64(n, BM);
-    // split-K: aim for >= 2 CTAs per SM (152 SMs) with chunks of >= 256
-    int splits = 1;
-    const int target = 2 * 152;
-    while (gx * gy * splits < target && n / (splits * 2) >= 256) splits *= 2;
-    if (tune && tune->splits > 0) splits = tune->splits;  // autotuned
-    if ((size_t)splits * (size_t)n * (size_t)ld > ws_elems) splits = 1;
-    int64_t kchunk = (n + splits - 1) / splits;
-    kchunk = (kchunk + BK - 1) / BK * BK;
-    dim3 grid(gx, gy, splits);
-    void* out = splits > 1 ? ws : Y;
-    if (a.a_dtype == 2 && a.sym)
-      k_gemm_dense<float, __nv_bfloat16, true><<<grid, 256, 0, s>>>((const __nv_bfloat16*)a.A, a.lda,
-                                                                    (const float*)X, ld, (float*)out, n, cols,
-                                                                    kchunk, run);
-    else if (a.a_dtype == 2)
-      k_gemm_dense<float, __nv_bfloat16><<<grid, 256, 0, s>>>((const __nv_bfloat16*)a.A, a.lda, (const float*)X,
-                                                              ld, (float*)out, n, cols, kchunk, run);
-    else if (tdtype == 0)
-      k_gemm_dense<double><<<grid, 256, 0, s>>>((const double*)a.A, a.lda, (const double*)X, ld,
-                                                (double*)out, n, cols, kchunk, run);
-    else
-      k_gemm_dense<float><<<grid, 256, 0, s>>>((const float*)a.A, a.lda, (const float*)X, ld,
-                                               (float*)out, n, cols, kchunk, run);
-    return splits;
+    // The tile is as narrow as the columns allow: 128 columns where a tile of 64 would not save a
+    // padded half, else 64, 32, 16; FP64, whose pipes bound every size, down to 8 in steps that
+    // waste at most a third (n = 2500, 10 columns: 910 us in a 64-wide tile).  Fewer than two CTAs
+    // per SM at the most splits: half the rows per tile.
+#define GEMM(T, TA, KIND, BM, BN, TM, TN, BK, OCC) \
+  return launch_gemm_cfg<GemmCfg<T, KIND, BM, BN, TM, TN, BK>, TA, OCC>(a, n, cols, ld, X, Y, ws, ws_elems, run, s, tune)
+    if (a.a_dtype == 0) {
+      if (cols <= 8) GEMM(double, double, GA_SAME, 64, 8, 4, 2, 16, 6);
+      if (cols <= 12) GEMM(double, double, GA_SAME, 64, 12, 4, 3, 16, 6);
+      if (cols <= 16) GEMM(double, double, GA_SAME, 64, 16, 4, 4, 16, 6);
+      if (cols <= 24) GEMM(double, double, GA_SAME, 64, 24, 4, 3, 16, 4);
+      if (cols <= 32) GEMM(double, double, GA_SAME, 64, 32, 4, 4, 16, 4);
+      GEMM(double, double, GA_SAME, 64, 64, 4, 4, 16, 2);
+    }
+    const bool wide = cols > 64 && (cols + 127) / 128 * 2 <= (cols + 63) / 64;
+#define GEMM_WIDTHS(TA, KIND)                                     \
+  if (wide) GEMM(float, TA, KIND, 128, 128, 8, 8, 16, 2);         \
+  if (cols > 32) GEMM(float, TA, KIND, 128, 64, 8, 8, 16, 4);     \
+  if (cols > 16) GEMM(float, TA, KIND, 128, 32, 8, 4, 32, 3);     \
+  GEMM(float, TA, KIND, 128, 16, 4, 4, 32, 3)
+    if (a.a_dtype == 3) { GEMM_WIDTHS(__nv_fp8_storage_t, GA_FP8); }
+    if (a.a_dtype == 2 && a.sym) { GEMM_WIDTHS(__nv_bfloat16, GA_BF16_SYM); }
+    if (a.a_dtype == 2) { GEMM_WIDTHS(__nv_bfloat16, GA_BF16); }
+    if ((int64_t)cdiv64(n, 128) * cdiv64(cols, 64) * std::min<int64_t>(n / 64, 32) < 2 * 152) {
+      if (cols > 32) GEMM(float, float, GA_SAME, 64, 64, 4, 8, 16, 4);
+      if (cols > 16) GEMM(float, float, GA_SAME, 64, 32, 4, 4, 32, 4);
+      GEMM(float, float, GA_SAME, 64, 16, 4, 4, 32, 6);
+    }
+    GEMM_WIDTHS(float, GA_SAME);
+#undef GEMM_WIDTHS
+#undef GEMM
   }
   // CSR
   const int cpl = cols > 128 ? 8 : (cols > 64 ? 4 : (cols > 32 ? 2 : 1));
@@ -285,14 +308,18 @@ int launch_ax_finish_impl(int tdtype, const Dims& d, void* Y, const void* ws, in
                           double c, const void* X2, const void* P1, const void* P2,
                           double* part, int q0, const int* run, cudaStream_t s, int dots_after) {
   dim3 grid(cdiv64(d.n, kRowTile), d.b);
-  if (tdtype == 0)
-    k_ax_finish<double><<<grid, 256, 0, s>>>(d.n, d.r, d.ld, (double*)Y, (const double*)ws, splits,
-                                             c, (const double*)X2, (const double*)P1,
-                                             (const double*)P2, part, q0, d.b, run, dots_after);
-  else
-    k_ax_finish<float><<<grid, 256, 0, s>>>(d.n, d.r, d.ld, (float*)Y, (const float*)ws, splits, c,
-                                            (const float*)X2, (const float*)P1, (const float*)P2,
-                                            part, q0, d.b, run, dots_after);
+  const int v = tdtype == 0 ? 2 : 4;
+  const uintptr_t all = (uintptr_t)Y | (uintptr_t)ws | (uintptr_t)X2 | (uintptr_t)P1 | (uintptr_t)P2;
+  const bool vec = d.r % v == 0 && d.ld % v == 0 && !(all & 15);
+#define FIN(T, V)                                                                                                    \
+  k_ax_finish<T, V><<<grid, 256, 0, s>>>(d.n, d.r, d.ld, (T*)Y, (const T*)ws, splits, c, (const T*)X2, (const T*)P1, \
+                                         (const T*)P2, part, q0, d.b, run, dots_after)
+  if (tdtype == 0) {
+    if (vec) FIN(double, 2); else FIN(double, 1);
+  } else {
+    if (vec) FIN(float, 4); else FIN(float, 1);
+  }
+#undef FIN
   return grid.x;
 }
 

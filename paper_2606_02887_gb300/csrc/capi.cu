@@ -227,8 +227,7 @@ int product_kernel(snmf_ctx* h, const AxArgs& op, const void* X, void* Y, const 
       }
       // no tensor map for these codes: the CUDA-core product below
     }
-    return launch_ax_fp8(op.A, op.a_scale, h->n, (const float*)X, h->N, h->N, (float*)Y, (float*)h->ws,
-                         h->ws_elems, run, h->s, tn);
+    return launch_ax(op, h->tdtype, h->n, h->N, h->N, X, Y, h->ws, h->ws_elems, run, h->s, tn);
   }
   if (op.kind == AX_DENSE && op.a_dtype == 2 && !op.accurate) {
     if (epi && epi->fused) {
@@ -801,7 +800,8 @@ snmf_status alloc_buffers(snmf_ctx* h) {
     CK(cudaMalloc(&h->buf[i], fe * h->esz));
     CK(cudaMemsetAsync(h->buf[i], 0, fe * h->esz, h->s));
   }
-  h->ws_elems = (h->kind == AX_DENSE) ? 8 * fe : 0;
+  // split-K slices: ten, and more of a small factor, whose K has to be split further to fill the GPU
+  h->ws_elems = (h->kind == AX_DENSE) ? std::max<size_t>(10 * fe, std::min<size_t>(32 * fe, 2 << 20)) : 0;
   if (h->ws_elems) CK(cudaMalloc(&h->ws, h->ws_elems * h->esz));
   const Dims d = dims(h);
   h->nrow = rowgemm_slots(d, h->tdtype);

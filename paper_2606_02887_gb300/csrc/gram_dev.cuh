@@ -1,0 +1,355 @@
+// Gram X^T Y of a row-major factor and the power method on it, as CTA bodies: one launch per
+// Gram in rowops.cu (a restart = a column range), work items of the uneven batch in batch.cu.
+#pragma once
+
+#include <math.h>
+
+#include "common.cuh"
+
+namespace snmf {
+
+namespace {
+
+// The Gram tile is as wide as the rank needs (16, 32 or 64 columns; tiles of 64 above), so a
+// rank of 10 or 20 does not pay for a 64 x 64 tile.
+__host__ __device__ inline int gram_tw(int r) { return r <= 16 ? 16 : (r <= 32 ? 32 : 64); }
+
+constexpr int kGramGroup = 16;         // chunk partials summed by one CTA at each level
+constexpr int kGramStageBytes = 8192;  // one staged operand block
+constexpr int kGramStages = 3;
+
+template <typename T>
+constexpr size_t gram_smem(bool same) {
+  // the staging ring; after the row loop the same memory holds the 4096 tile partials
+  return kGramStages * kGramStageBytes * (same ? 1 : 2) > 4096 * sizeof(T)
+             ? (size_t)kGramStages * kGramStageBytes * (same ? 1 : 2)
+             : 4096 * sizeof(T);
+}
+
+template <typename T>
+struct alignas(16) Quad {
+  T v[4];
+};
+
+__device__ __forceinline__ Quad<float> ldcg_quad(const float* p) {
+  const float4 t = __ldcg(reinterpret_cast<const float4*>(p));
+  return {{t.x, t.y, t.z, t.w}};
+}
+__device__ __forceinline__ Quad<double> ldcg_quad(const double* p) {
+  const double2 a = __ldcg(reinterpret_cast<const double2*>(p)), b = __ldcg(reinterpret_cast<const double2*>(p) + 1);
+  return {{a.x, a.y, b.x, b.y}};
+}
+
+// 16-, 8- or 4-byte asynchronous copy to shared memory; bytes beyond `valid` are zero
+template <int BYTES>
+__device__ __forceinline__ void cp_async(void* dst, const void* src, bool valid) {
+  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+  const int n = valid ? BYTES : 0;
+  if constexpr (BYTES == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(d), "l"(src), "n"(BYTES), "r"(n) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// ------------------------------------------------------------------------------
+// Power method (Alg. 1 line 2, Eq. (2.11)): ||G||_2 by `iters` iterations from the ones vector
+// and the Rayleigh quotient.  The block holds G; row p of G v is summed by TPR adjacent lanes,
+// W = P2 / TPR columns each (P2: r rounded up to a power of two), through `dot(v)`.  A fixed
+// count of serial products bounds it, so an iteration is one shared read of v, the FMAs, the
+// lane butterfly and one barrier: v is double buffered and G scaled by a power of two to a
+// trace below one (exact; ||G|| <= trace for a Gram), so v only has to be rescaled every eighth
+// iteration (it shrinks by at most r each).  n = 64: 13 us with the norm taken in every
+// iteration, 4 us so.
+// Threads t < nact = P2 TPR take part (a multiple of 32), on barrier 1.  vs: 2 (P2 + 4 TPR)
+// values, red: 2 nact / 32 values.  0 for a zero G.
+// ------------------------------------------------------------------------------
+__device__ __forceinline__ void bar_sync(int id, int count) {
+  asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+
+template <typename T>
+__device__ __forceinline__ T lanes_sum(T v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+template <typename T, int TPR, typename Dot>
+__device__ __forceinline__ T power_norm(int r, int W, int nact, int iters, Dot dot, T* vs, T* red) {
+  const int t = threadIdx.x, p = t / TPR, part = t % TPR;
+  const int lane = t & 31, wid = t >> 5, nw = nact >> 5;
+  const int len = (W + 4) * TPR;                        // columns of a part, 16 bytes apart in banks
+  auto at = [&](int q) { return q + (q / W) * 4; };
+  T* cur = vs;
+  T* nxt = vs + len;
+  if (part == 0) cur[at(p)] = p < r ? T(1) : T(0);
+  bar_sync(1, nact);
+  auto total = [&](T x) {  // fixed-order sum over the rows (x counts in part 0 only)
+    x = lanes_sum(part == 0 ? x : T(0));
+    if (lane == 0) red[wid] = x;
+    bar_sync(1, nact);
+    T s = T(0);
+    for (int w = 0; w < nw; ++w) s += red[w];
+    return s;
+  };
+  auto row = [&]() {
+    T s = dot(cur + part * (W + 4));
+#pragma unroll
+    for (int o = 1; o < TPR; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+  };
+  for (int it = 0; it < iters; ++it) {
+    T s = row();
+    if ((it & 7) == 7 || it == iters - 1) {
+      const T tot = total(fabs(s));
+      if (tot == T(0)) return T(0);
+      s /= tot;
+    }
+    if (part == 0) nxt[at(p)] = s;
+    bar_sync(1, nact);
+    T* x = cur;
+    cur = nxt;
+    nxt = x;
+  }
+  const T s = row(), v = cur[at(p)];
+  const T num = total(v * s);
+  bar_sync(1, nact);  // red read by every thread before it is written again
+  const T den = total(v * v);
+  return num / den;
+}
+
+// power-of-two scale that brings a positive trace below one
+__device__ __forceinline__ int trace_exponent(float tr) { return tr > 0.f && tr < INFINITY ? ilogbf(tr) + 1 : 0; }
+__device__ __forceinline__ int trace_exponent(double tr) { return tr > 0.0 && tr < INFINITY ? ilogb(tr) + 1 : 0; }
+
+__device__ __forceinline__ void set_rho(Ctl& c, double norm, double rho_scale, double rho_shift) {
+  double rr = rho_scale * norm + rho_shift;  // shift: gamma ||L||_2 of a graph block
+  if (!(rr > 0.0)) rr = 1.0;                 // zero Gram: unit scaling
+  c.rho = rr;
+}
+
+// rho of the r x r Gram in shared memory (row stride TW, zero beyond r), r <= TW
+template <typename T, int TW>
+__device__ __forceinline__ void rho_in_smem(const T* Gs, int r, int iters, double rho_scale, double rho_shift, Ctl& c) {
+  constexpr int W = TW / 4, NACT = 4 * TW;
+  __shared__ __align__(16) T vs[2 * (TW + 16)];
+  __shared__ T red[2 * NACT / 32];
+  const int t = threadIdx.x;
+  if (t >= NACT) return;
+  const int lane = t & 31;
+  T tr = T(0);
+  for (int q = lane; q < r; q += 32) tr += Gs[q * TW + q];
+  tr = lanes_sum(tr);
+  const int e = trace_exponent(tr);
+  T g[W];
+#pragma unroll
+  for (int u = 0; u < W; ++u) g[u] = (T)ldexp(Gs[(t >> 2) * TW + (t & 3) * W + u], -e);
+  const T norm = power_norm<T, 4>(r, W, NACT, iters,
+                                  [&](const T* v) {
+                                    T s[4] = {T(0), T(0), T(0), T(0)};
+#pragma unroll
+                                    for (int u = 0; u < W; u += 4) {
+                                      const Quad<T> x = *reinterpret_cast<const Quad<T>*>(v + u);
+#pragma unroll
+                                      for (int k = 0; k < 4; ++k) s[k] = fma(g[u + k], x.v[k], s[k]);
+                                    }
+                                    return (s[0] + s[1]) + (s[2] + s[3]);
+                                  },
+                                  vs, red);
+  if (t == 0) set_rho(c, ldexp((double)norm, e), rho_scale, rho_shift);
+}
+
+// ------------------------------------------------------------------------------
+// One chunk of rows [i_begin, i_end) of a TW x TW Gram tile: X, Y at the tile's first columns
+// (wx, wy of them exist), row pitch ld, VEC elements per copy (16 bytes when the columns and
+// the pitch allow it, else single elements).  256 threads: NG = 4096 / TW^2 row groups, each a
+// (TW / 4)^2 grid of 4 x 4 micro tiles read as two 16-byte shared loads per row.  The groups'
+// sums leave the row loop in shared memory; the thread returns its entries e = 4 (t + 256 u).
+// Bound by HBM for long factors (n = 2e6, r = 32: 797 us with 152 chunks of two staged rounds
+// and scalar shared reads) and by latency for short ones.
+// ------------------------------------------------------------------------------
+template <typename T, int TW, int VEC>
+__device__ __forceinline__ void gram_chunk(const T* __restrict__ X, const T* __restrict__ Y, int wx, int wy, int64_t ld,
+                                           int64_t i_begin, int64_t i_end, bool same, T* sm, Quad<T>* out) {
+  constexpr int RS = kGramStageBytes / (TW * (int)sizeof(T));  // rows per stage
+  constexpr int NG = 4096 / (TW * TW), GT = 256 / NG, TX = TW / 4;
+  constexpr int CPR = TW / VEC;             // copies per row
+  constexpr int NC = RS * CPR / 256;        // copies per thread and operand
+  constexpr int STAGE = RS * TW;
+  const int t = threadIdx.x;
+  T* Xs = sm;
+  T* Ys = same ? sm : sm + kGramStages * STAGE;
+  auto fetch = [&](int64_t i0, int st) {
+#pragma unroll
+    for (int m = 0; m < NC; ++m) {
+      const int e = t + 256 * m, rr = e / CPR, cc = (e % CPR) * VEC;
+      const int64_t i = i0 + rr;
+      const bool vx = i < i_end && cc < wx;
+      cp_async<VEC * (int)sizeof(T)>(Xs + st * STAGE + rr * TW + cc, vx ? X + i * ld + cc : X, vx);
+      if (!same) {
+        const bool vy = i < i_end && cc < wy;
+        cp_async<VEC * (int)sizeof(T)>(Ys + st * STAGE + rr * TW + cc, vy ? Y + i * ld + cc : Y, vy);
+      }
+    }
+  };
+  const int rounds = (int)((i_end - i_begin + RS - 1) / RS);
+#pragma unroll
+  for (int s = 0; s < kGramStages - 1; ++s) {
+    if (s < rounds) fetch(i_begin + (int64_t)s * RS, s);
+    cp_async_commit();
+  }
+  T acc[4][4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[a][c] = T(0);
+  const int grp = t / GT, tx = (t % GT) % TX, ty = (t % GT) / TX;
+  for (int k = 0; k < rounds; ++k) {
+    cp_async_wait<kGramStages - 2>();
+    __syncthreads();  // stage k is in; every thread is done with the stage refilled below
+    if (k + kGramStages - 1 < rounds)
+      fetch(i_begin + (int64_t)(k + kGramStages - 1) * RS, (k + kGramStages - 1) % kGramStages);
+    cp_async_commit();
+    const T* xs = Xs + (k % kGramStages) * STAGE + 4 * ty;
+    const T* ys = Ys + (k % kGramStages) * STAGE + 4 * tx;
+#pragma unroll 4
+    for (int rr = grp; rr < RS; rr += NG) {
+      const Quad<T> xa = *reinterpret_cast<const Quad<T>*>(xs + rr * TW);
+      const Quad<T> yb = *reinterpret_cast<const Quad<T>*>(ys + rr * TW);
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[a][c] = fma(xa.v[a], yb.v[c], acc[a][c]);
+    }
+  }
+  cp_async_wait<0>();
+  __syncthreads();  // the ring is free: it takes the groups' tiles
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+    *reinterpret_cast<Quad<T>*>(sm + grp * TW * TW + (4 * ty + a) * TW + 4 * tx) =
+        Quad<T>{{acc[a][0], acc[a][1], acc[a][2], acc[a][3]}};
+  __syncthreads();
+  constexpr int NE = TW * TW / 4 >= 256 ? TW * TW / 1024 : 1;
+#pragma unroll
+  for (int u = 0; u < NE; ++u) {
+    const int e = 4 * (t + 256 * u);
+    if (e < TW * TW) {
+      Quad<T> s = *reinterpret_cast<const Quad<T>*>(sm + e);
+#pragma unroll
+      for (int g = 1; g < NG; ++g) {
+        const Quad<T> v = *reinterpret_cast<const Quad<T>*>(sm + g * TW * TW + e);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s.v[k] += v.v[k];
+      }
+      out[u] = s;
+    }
+  }
+}
+
+// Where a Gram tile goes: entry (p, q) of the tile is (p0 + p, q0 + q) of the r x r matrix.
+template <typename T>
+struct GramOut {
+  double* G64;
+  T* GT;  // factor-type copy with lam on the diagonal (NULL: none)
+  T lam;
+  int r, p0, q0;
+  Ctl* rho_ctl;  // the tile is the whole Gram: rho = rho_scale ||G||_2 + rho_shift (NULL: no)
+  int rho_iters;
+  double rho_scale, rho_shift;
+};
+
+// CTA `c` of the nch chunks of one tile.  Partials go to gp (nch + ng tiles of TW^2 values) and
+// are summed in chunk order by the last CTA of each of the ng groups of 16 chunks and then, in group
+// order, by the last group's (arrival counters cnt[0 .. ng], zero between launches): a fixed
+// order, and no CTA reads many partials in a row, which had kept the number of chunks, and with it
+// the CTAs, low.  ng = 0: one level, every chunk in order.
+__host__ __device__ inline int gram_groups(int nch) { return nch > kGramGroup ? (nch + kGramGroup - 1) / kGramGroup : 0; }
+
+template <typename T, int TW, int VEC>
+__device__ __forceinline__ void gram_body(const T* X, const T* Y, int wx, int wy, int64_t ld, int64_t n, int64_t chunk,
+                                          int c, int nch, int ng, bool same, T* gp, unsigned* cnt, const GramOut<T>& o,
+                                          T* sm) {
+  constexpr int NE = TW * TW / 4 >= 256 ? TW * TW / 1024 : 1;
+  constexpr int TW2 = TW * TW;
+  __shared__ unsigned s_ticket;
+  const int t = threadIdx.x;
+  const bool owns = 4 * t < TW2;
+  Quad<T> s[NE];
+  const int64_t i0 = (int64_t)c * chunk;
+  gram_chunk<T, TW, VEC>(X, Y, wx, wy, ld, i0, min(n, i0 + chunk), same, sm, s);
+  auto publish = [&](T* dst) {
+#pragma unroll
+    for (int u = 0; u < NE; ++u)
+      if (owns) *reinterpret_cast<Quad<T>*>(dst + 4 * (t + 256 * u)) = s[u];
+    __threadfence();
+    __syncthreads();
+  };
+  auto arrive = [&](unsigned* counter, int of) {  // CTA-uniform: the last of `of` arrivals
+    if (t == 0) {
+      s_ticket = atomicAdd(counter, 1u);
+      if (s_ticket == (unsigned)(of - 1)) *counter = 0u;  // ready for the next launch
+    }
+    __syncthreads();
+    const bool last = s_ticket == (unsigned)(of - 1);
+    __syncthreads();
+    return last;
+  };
+  auto sum = [&](const T* src, int m) {  // s = the m tiles at src in order, 16 loads in flight
+#pragma unroll
+    for (int u = 0; u < NE; ++u) {
+      s[u] = Quad<T>{{T(0), T(0), T(0), T(0)}};
+      if (!owns) continue;
+      const T* q = src + 4 * (t + 256 * u);
+      for (int k0 = 0; k0 < m; k0 += 8) {
+        Quad<T> v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = k0 + k < m ? ldcg_quad(q + (int64_t)(k0 + k) * TW2) : Quad<T>{{T(0), T(0), T(0), T(0)}};
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+#pragma unroll
+          for (int w = 0; w < 4; ++w) s[u].v[w] += v[k].v[w];
+      }
+    }
+  };
+  if (nch > 1) {
+    publish(gp + (int64_t)c * TW2);
+    const int g = c / kGramGroup, gs = min(kGramGroup, nch - g * kGramGroup);
+    if (!arrive(cnt + (ng ? 1 + g : 0), ng ? gs : nch)) return;
+    __threadfence();
+    sum(gp + (int64_t)(ng ? g * kGramGroup : 0) * TW2, ng ? gs : nch);
+    if (ng) {
+      publish(gp + (int64_t)(nch + g) * TW2);
+      if (!arrive(cnt, ng)) return;
+      __threadfence();
+      sum(gp + (int64_t)nch * TW2, ng);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < NE; ++u) {
+    const int e = 4 * (t + 256 * u);
+    if (!owns) continue;
+    if (o.rho_ctl) *reinterpret_cast<Quad<T>*>(sm + e) = s[u];
+    const int p = o.p0 + e / TW;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int q = o.q0 + e % TW + k;
+      if (p < o.r && q < o.r) {
+        o.G64[(int64_t)p * o.r + q] = (double)s[u].v[k];
+        if (o.GT) o.GT[(int64_t)p * o.r + q] = s[u].v[k] + (p == q ? o.lam : T(0));
+      }
+    }
+  }
+  if (o.rho_ctl) {
+    __syncthreads();
+    rho_in_smem<T, TW>(sm, o.r, o.rho_iters, o.rho_scale, o.rho_shift, *o.rho_ctl);
+  }
+}
+
+}  // namespace
+
+}  // namespace snmf
