@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstddef>
+#include <mutex>
 #include <numeric>
 #include <string>
 #include <vector>
@@ -32,15 +33,18 @@
 #include "ax_tc.cuh"
 #include "batch.cuh"
 #include "common.cuh"
+#include "gemm_dev.cuh"
 #include "rowops.cuh"
 #include "rowops_dev.cuh"
+#include "rowstep_dev.cuh"
 
 namespace snmf {
 
 namespace {
 
-constexpr int kPBM = 64;      // product rows per work item
-constexpr int kGChunk = 256;  // Gram rows per work item
+constexpr int kPBM = 128;     // product rows per work item
+constexpr int kRowThreads = 128;  // threads of a row item
+constexpr int kGChunk = 256;  // Gram rows per work item (two staged rounds of the widest tile at least)
 
 // Per-problem sizes and offsets (device-resident table).
 struct BProb {
@@ -57,7 +61,8 @@ struct BProb {
   int64_t xoff; // element offset of the problem's factor blocks
   int64_t goff; // offset of its r x r factor-type matrix
   int64_t g3off;// offset of its three FP64 r x r Grams
-  int64_t gpoff;// offset (doubles) of its Gram chunk partials
+  int64_t gpoff;// offset (elements) of its Gram chunk partials
+  int gcnt;     // its first Gram arrival counter
   double lam;   // penalty weight lambda_p
   double normA2;// ||A_p||_F^2 of the stored values
 };
@@ -124,105 +129,82 @@ __global__ void k_bsums_reduce(const BProb* __restrict__ probs, const double* __
   }
 }
 
-// Grouped product (CUDA cores): item (p, t) computes rows t*64 .. of Y_p = A_p X_p over the
-// full K = n_p (A_p rows streamed once, X_p from L2), epilogue Y += lambda_p X and, when
-// P1 is given, the per-item partial <P1, A_p X_p> in the item's partial slot.  CTAs beyond
-// the *cnt items of the (compacted) list return at once.
-template <typename T, typename TA>
-__global__ void __launch_bounds__(256)
+// Grouped product (CUDA cores): item (p, t) computes rows t*128 .. of Y_p = A_p X_p over the
+// full K = n_p (A_p rows streamed once, X_p from L2) in a tile as wide as r_p needs, epilogue
+// Y += lambda_p X and, when P1 is given, the per-item partial <P1, A_p X_p> in the item's partial
+// slot.  CTAs beyond the *cnt items of the (compacted) list return at once.  Bound by the FMA
+// pipes; 256 problems of n <= 2048, r <= 32 with BF16 A: 2045 us with 64-wide tiles for every r.
+template <typename C, typename TA>
+__device__ __forceinline__ typename C::T bgemm_item(const TA* A, int64_t lda, const BProb& pb, int tile,
+                                                    const typename C::T* X, typename C::T* Y, int add_lam,
+                                                    const typename C::T* P1, typename C::T* sm) {
+  using T = typename C::T;
+  const int64_t n = pb.n, row0 = (int64_t)tile * kPBM;
+  const int r = pb.r;
+  const bool xvec = r % C::KV == 0 && pb.xoff % C::KV == 0;
+  T acc[C::TM][C::TN];
+  // A_all is zero beyond column n_p, so its 16-byte copies may run over the end of a row
+  gemm_tile<C>(A + pb.arow * lda, lda, X + pb.xoff, r, n, r, row0, 0, 0, n, true, xvec, GemmA8{}, sm, acc);
+  const T lam = (T)pb.lam;
+  const int tx = threadIdx.x % C::TX, ty = threadIdx.x / C::TX;
+  T d1 = T(0);
+#pragma unroll
+  for (int i = 0; i < C::TM; ++i) {
+    const int64_t row = row0 + ty + C::TY * i;
+    if (row >= n) continue;
+#pragma unroll
+    for (int j = 0; j < C::TN; ++j) {
+      const int c = C::col(tx, j);
+      if (c >= r) continue;
+      const int64_t idx = pb.xoff + row * r + c;
+      T y = acc[i][j];
+      if (P1) d1 += P1[idx] * y;
+      if (add_lam) y += lam * X[idx];
+      Y[idx] = y;
+    }
+  }
+  return d1;
+}
+
+// the tiles of one working type: 16, 32 and 64 columns, the same threads for all
+template <typename T, int KIND>
+struct BGemm {
+  static constexpr int NT = 128, PER_SM = 3;
+  using C16 = GemmCfg<T, KIND, kPBM, 16, 4, 4, 32>;
+  using C32 = GemmCfg<T, KIND, kPBM, 32, 8, 4, 32>;
+  using C64 = GemmCfg<T, KIND, kPBM, 64, 8, 8, 16>;
+};
+template <int KIND>
+struct BGemm<double, KIND> {
+  static constexpr int NT = 256, PER_SM = 2;
+  using C16 = GemmCfg<double, KIND, kPBM, 16, 4, 2, 16>;
+  using C32 = GemmCfg<double, KIND, kPBM, 32, 4, 4, 16>;
+  using C64 = GemmCfg<double, KIND, kPBM, 64, 8, 4, 16>;
+};
+template <typename B>
+constexpr size_t bgemm_smem() {
+  const size_t a = B::C16::SMEM, b = B::C32::SMEM, c = B::C64::SMEM;
+  return a > b ? (a > c ? a : c) : (b > c ? b : c);
+}
+
+template <typename T, typename TA, int KIND>
+__global__ void __launch_bounds__(BGemm<T, KIND>::NT, BGemm<T, KIND>::PER_SM)
 k_bgemm(const TA* __restrict__ A, int64_t lda, const BProb* __restrict__ probs, const int2* __restrict__ items,
         const int* __restrict__ cnt, const T* __restrict__ X, T* __restrict__ Y, int add_lam,
         const T* __restrict__ P1, double* __restrict__ part, const Ctl* __restrict__ ctl, const int* __restrict__ run) {
-  constexpr int BK = sizeof(T) == 8 ? 16 : 32;
-  if ((int)blockIdx.x >= *cnt) return;
-  constexpr int NA = kPBM * BK / 256;
-  constexpr int NX = BK * 64 / 256;
-  __shared__ T As[2][BK][kPBM + 4];
-  __shared__ T Xs[2][BK][64 + 4];
+  using B = BGemm<T, KIND>;
+  static_assert(B::C16::NT == B::NT && B::C32::NT == B::NT && B::C64::NT == B::NT, "one block size");
+  extern __shared__ __align__(16) unsigned char bsm[];
   __shared__ T sh[32];
+  if ((int)blockIdx.x >= *cnt) return;
   const int2 it = items[blockIdx.x];
-  const int p = it.x;
-  const BProb& pb = probs[p];
-  const int64_t n = pb.n;
-  const int r = pb.r;
-  const int64_t row0 = (int64_t)it.y * kPBM;
-  const T* Xp = X + pb.xoff;
-  const TA* Ap = A + (pb.arow + row0) * lda;
-  const bool live = !(run && *run == 0) && !(ctl && !ctl[p].active);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const BProb& pb = probs[it.x];
   T d1 = T(0);
-  if (live) {
-    T acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
-    T ra[NA], rx[NX];
-    auto load = [&](int64_t k0) {
-#pragma unroll
-      for (int m = 0; m < NA; ++m) {
-        const int e = threadIdx.x + 256 * m;
-        const int rr = e / BK, kk = e % BK;
-        ra[m] = (row0 + rr < n && k0 + kk < n) ? (T)to_f(Ap[(int64_t)rr * lda + k0 + kk]) : T(0);
-      }
-#pragma unroll
-      for (int m = 0; m < NX; ++m) {
-        const int e = threadIdx.x + 256 * m;
-        const int kr = e >> 6, c = e & 63;
-        rx[m] = (k0 + kr < n && c < r) ? Xp[(k0 + kr) * r + c] : T(0);
-      }
-    };
-    auto store = [&](int buf) {
-#pragma unroll
-      for (int m = 0; m < NA; ++m) {
-        const int e = threadIdx.x + 256 * m;
-        As[buf][e % BK][e / BK] = ra[m];
-      }
-#pragma unroll
-      for (int m = 0; m < NX; ++m) {
-        const int e = threadIdx.x + 256 * m;
-        Xs[buf][e >> 6][e & 63] = rx[m];
-      }
-    };
-    int buf = 0;
-    load(0);
-    store(0);
-    __syncthreads();
-    for (int64_t k0 = 0; k0 < n; k0 += BK) {
-      const bool more = k0 + BK < n;
-      if (more) load(k0 + BK);
-#pragma unroll
-      for (int kk = 0; kk < BK; ++kk) {
-        T a[4], x[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = As[buf][kk][ty + 16 * i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) x[j] = Xs[buf][kk][tx + 16 * j];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], x[j], acc[i][j]);
-      }
-      if (more) store(buf ^ 1);
-      __syncthreads();
-      buf ^= 1;
-    }
-    const T lam = (T)pb.lam;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int64_t row = row0 + ty + 16 * i;
-      if (row >= n) continue;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int c = tx + 16 * j;
-        if (c >= r) continue;
-        const int64_t idx = pb.xoff + row * r + c;
-        T y = acc[i][j];
-        if (P1) d1 += P1[idx] * y;
-        if (add_lam) y += lam * X[idx];
-        Y[idx] = y;
-      }
-    }
+  if (!(run && *run == 0) && !(ctl && !ctl[it.x].active)) {
+    T* sm = reinterpret_cast<T*>(bsm);
+    if (pb.r <= 16) d1 = bgemm_item<typename B::C16>(A, lda, pb, it.y, X, Y, add_lam, P1, sm);
+    else if (pb.r <= 32) d1 = bgemm_item<typename B::C32>(A, lda, pb, it.y, X, Y, add_lam, P1, sm);
+    else d1 = bgemm_item<typename B::C64>(A, lda, pb, it.y, X, Y, add_lam, P1, sm);
   }
   if (part) {
     d1 = block_sum_t(d1, sh);
@@ -230,40 +212,50 @@ k_bgemm(const TA* __restrict__ A, int64_t lda, const BProb* __restrict__ probs, 
   }
 }
 
-// Grouped Gram X_p^T Y_p (pair `pair` of `npairs`), chunk items; lambda_p on the diagonal
-// of the factor-type copy when use_lam; rho_p fused in the last CTA (FP32 working type).
+// Grouped Gram X_p^T Y_p (the problem's Gram `pair` of three in G64), chunk items; lambda_p on
+// the diagonal of the factor-type copy GT (NULL: none); rho_p in the last CTA of the problem.  The
+// tile is as wide as r_p needs, and 16-byte copies are used where the problem's block allows them.
 template <typename T>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 3)
 k_bgram(const BProb* __restrict__ probs, const int2* __restrict__ items, const int* __restrict__ cnt,
-        const T* __restrict__ X, const T* __restrict__ Y, double* __restrict__ gpart, int pair, int npairs,
-        const Ctl* __restrict__ ctl, const int* run, double* __restrict__ G64, T* __restrict__ GT, int tpair,
-        int use_lam, unsigned* __restrict__ counters, Ctl* __restrict__ rho_ctl, int rho_iters) {
+        const T* __restrict__ X, const T* __restrict__ Y, T* __restrict__ gpart, int pair,
+        const Ctl* __restrict__ ctl, const int* run, double* __restrict__ G64, T* __restrict__ GT,
+        unsigned* __restrict__ counters, Ctl* __restrict__ rho_ctl, int rho_iters) {
+  extern __shared__ __align__(16) unsigned char gsm[];
   if ((int)blockIdx.x >= *cnt) return;  // beyond the (compacted) list
   const int2 it = items[blockIdx.x];
   const BProb& pb = probs[it.x];
-  gram_body<T>(X + pb.xoff, Y + pb.xoff, pb.n, pb.r, 1, pb.r, kGChunk, 1, gpart + pb.gpoff, pair, npairs,
-               ctl ? ctl + it.x : nullptr, run, G64 + pb.g3off, GT ? GT + pb.goff : nullptr, tpair,
-               use_lam ? pb.lam : 0.0, counters + 3 * it.x, rho_ctl ? rho_ctl + it.x : nullptr, rho_iters,
-               1.0, 0.0, it.y, pb.gch, 0);
+  if ((run && *run == 0) || (ctl && !ctl[it.x].active)) return;
+  const int r = pb.r;
+  GramOut<T> o;
+  o.r = r;
+  o.p0 = o.q0 = 0;
+  o.G64 = G64 + pb.g3off + (int64_t)pair * r * r;
+  o.GT = GT ? GT + pb.goff : nullptr;
+  o.lam = (T)pb.lam;
+  o.rho_ctl = rho_ctl ? rho_ctl + it.x : nullptr;
+  o.rho_iters = rho_iters;
+  o.rho_scale = 1.0;
+  o.rho_shift = 0.0;
+  constexpr int V = 16 / (int)sizeof(T);
+  const bool vec = r % V == 0 && pb.xoff % V == 0;
+#define BG(TW, VEC)                                                                                              \
+  gram_body<T, TW, VEC>(X + pb.xoff, Y + pb.xoff, r, r, r, pb.n, kGChunk, it.y, pb.gch, gram_groups(pb.gch), X == Y, gpart + pb.gpoff, \
+                        counters + pb.gcnt, o, reinterpret_cast<T*>(gsm))
+#define BG_V(TW) \
+  if (vec) BG(TW, V); else BG(TW, 1)
+  if (r <= 16) { BG_V(16); }
+  else if (r <= 32) { BG_V(32); }
+  else { BG_V(64); }
+#undef BG_V
+#undef BG
 }
 
-// rho_p = ||G_p||_2 (FP64 working type), one block per problem
-template <typename PT>
-__global__ void __launch_bounds__(256)
-k_brho(const BProb* __restrict__ probs, const double* __restrict__ G64, int iters, Ctl* __restrict__ ctl) {
-  __shared__ double sh[32];
-  __shared__ PT v[64], w[64];
-  __shared__ PT Gs[64 * 64];
-  const BProb& pb = probs[blockIdx.x];
-  Ctl& c = ctl[blockIdx.x];
-  if (!c.active) return;
-  rho_body<PT>(G64 + pb.g3off, pb.r, iters, 1.0, 0.0, c, v, w, Gs, sh);
-}
-
-// Grouped row GEMM with the fused Algorithm-1 epilogues and the per-problem control step.
-template <typename T, int OP, int EPI, int BM, int NC>
-__global__ void __launch_bounds__(256, 2)
+// Grouped row kernels of a step (rowstep_dev.cuh) with the per-problem control step.
+template <typename T, int STEP, int NC>
+__global__ void __launch_bounds__(kRowThreads, 4)
 k_brow(RowArgs base, const BProb* __restrict__ probs, const int2* __restrict__ items, const int* __restrict__ cnt) {
+  extern __shared__ __align__(16) unsigned char rsm[];
   if ((int)blockIdx.x >= *cnt) return;  // beyond the (compacted) list
   const int2 it = items[blockIdx.x];
   const BProb& pb = probs[it.x];
@@ -276,116 +268,90 @@ k_brow(RowArgs base, const BProb* __restrict__ probs, const int2* __restrict__ i
   a.b = 1;
   a.ld = pb.r;
   a.G = (const T*)base.G + pb.goff;
-  a.X = cs(base.X); a.g_in = cs(base.g_in); a.Zin = cs(base.Zin); a.Din = cs(base.Din);
+  a.X = cs(base.X); a.g_in = cs(base.g_in);
   a.B = cs(base.B); a.LX = nullptr;
-  a.Xout = ms(base.Xout); a.gout = ms(base.gout); a.Dout = ms(base.Dout); a.D2out = ms(base.D2out);
-  a.Din2 = cs(base.Din2); a.gZout = ms(base.gZout);
-  a.Xold = cs(base.Xold); a.gold = cs(base.gold); a.Zold = cs(base.Zold); a.gZold = cs(base.gZold);
-  a.Wcur = cs(base.Wcur); a.gWcur = cs(base.gWcur);
+  a.Xout = ms(base.Xout); a.gout = ms(base.gout);
+  a.gZout = ms(base.gZout);
+  a.gZold = cs(base.gZold);
   a.ctl = base.ctl + it.x;
   a.part = base.part + (int64_t)pb.slot0 * kNQ;
   a.counters = base.counters + it.x;
-  a.G64fix = base.G64fix ? base.G64fix + pb.g3off : nullptr;
   a.P.nr = pb.n * (int64_t)pb.r;
-  rowgemm_body<T, OP, EPI, BM, NC>(a, 0, it.y, 0, 1, (unsigned)pb.nrt);
-}
-
-// The same for problems with r <= 32 through the shared-memory tile body (TileCfg rows per
-// item); dynamic shared memory of rowtile_smem bytes.
-template <typename T, int OP, int EPI, int NC>
-__global__ void __launch_bounds__(256, EPI == EPI_GRAD ? 2 : 3)
-k_browt(RowArgs base, const BProb* __restrict__ probs, const int2* __restrict__ items, const int* __restrict__ cnt) {
-  extern __shared__ __align__(16) unsigned char tsm[];
-  if ((int)blockIdx.x >= *cnt) return;  // beyond the (compacted) list
-  const int2 it = items[blockIdx.x];
-  const BProb& pb = probs[it.x];
-  RowArgs a = base;
-  const size_t o = (size_t)pb.xoff * sizeof(T);
-  auto cs = [&](const void* q) -> const void* { return q ? (const void*)((const char*)q + o) : nullptr; };
-  auto ms = [&](void* q) -> void* { return q ? (void*)((char*)q + o) : nullptr; };
-  a.n = pb.n;
-  a.r = pb.r;
-  a.b = 1;
-  a.ld = pb.r;
-  a.G = (const T*)base.G + pb.goff;
-  a.X = cs(base.X); a.g_in = cs(base.g_in); a.Zin = cs(base.Zin); a.Din = cs(base.Din);
-  a.B = cs(base.B); a.LX = nullptr;
-  a.Xout = ms(base.Xout); a.gout = ms(base.gout); a.Dout = ms(base.Dout); a.D2out = ms(base.D2out);
-  a.Din2 = cs(base.Din2); a.gZout = ms(base.gZout);
-  a.Xold = cs(base.Xold); a.gold = cs(base.gold); a.Zold = cs(base.Zold); a.gZold = cs(base.gZold);
-  a.Wcur = cs(base.Wcur); a.gWcur = cs(base.gWcur);
-  a.ctl = base.ctl + it.x;
-  a.part = base.part + (int64_t)pb.slot0 * kNQ;
-  a.counters = base.counters + it.x;
-  a.G64fix = base.G64fix ? base.G64fix + pb.g3off : nullptr;
-  a.P.nr = pb.n * (int64_t)pb.r;
-  rowtile_body<T, OP, EPI, NC>(a, 0, it.y, (unsigned)pb.nrt, reinterpret_cast<T*>(tsm));
+  rowstep_body<T, STEP, NC, rowstep_mr<T>()>(a, 0, it.y, (unsigned)pb.nrt, pb.r % 4 == 0 && pb.xoff % 4 == 0,
+                                    reinterpret_cast<T*>(rsm));
 }
 
 // Work-list compaction: the items of the problems that are still active, in the original
-// order, for the five lists (row items of the tile body, row items of the generic body,
-// Gram chunks, CUDA-core product tiles, tensor-core product tiles); counts to cnt[0..4];
-// *run = any problem active.  One block; problems in list order `order`.
+// order, for the four lists (row items, Gram chunks, CUDA-core product tiles, tensor-core product
+// tiles); counts to cnt[0..3]; *run = any problem active.  Block L = one list (and block 0 the run
+// flag); the offsets of the problems in list order `order` by a scan of the warps' sums, then one
+// warp per problem copies its items (one block for all lists, a thread per problem: 30 us for 256
+// problems).
 struct CompactArgs {
   const int* order;
   int nprob;
   const Ctl* ctl;
-  const int2* full[4];
-  int2* comp[4];
+  const int2* full[3];
+  int2* comp[3];
   const TcItem* tfull;
   TcItem* tcomp;
-  const int* pst;   // [5][nprob]: first item of problem p in each full list
-  const int* psz;   // [5][nprob]: items of problem p in each list
+  const int* pst;   // [4][nprob]: first item of problem p in each full list
+  const int* psz;   // [4][nprob]: items of problem p in each list
   int* cnt;
   int* run;
 };
 
 __global__ void __launch_bounds__(1024) k_bcompact(CompactArgs ca) {
-  __shared__ int sc[5][1024];
-  const int tid = threadIdx.x;
-  const int per = (ca.nprob + 1023) / 1024;
-  const int i0 = min(ca.nprob, tid * per), i1 = min(ca.nprob, i0 + per);
-  int loc[5] = {0, 0, 0, 0, 0};
-  int any = 0;
-  for (int i = i0; i < i1; ++i) {
-    const int p = ca.order[i];
-    if (!ca.ctl[p].active) continue;
-    any = 1;
-    for (int L = 0; L < 5; ++L) loc[L] += ca.psz[L * ca.nprob + p];
-  }
-  for (int L = 0; L < 5; ++L) sc[L][tid] = loc[L];
-  __syncthreads();
-  for (int off = 1; off < 1024; off <<= 1) {  // inclusive scan
-    int v[5];
-    for (int L = 0; L < 5; ++L) v[L] = tid >= off ? sc[L][tid - off] : 0;
-    __syncthreads();
-    for (int L = 0; L < 5; ++L) sc[L][tid] += v[L];
-    __syncthreads();
-  }
-  int pos[5];
-  for (int L = 0; L < 5; ++L) pos[L] = sc[L][tid] - loc[L];
-  for (int i = i0; i < i1; ++i) {
-    const int p = ca.order[i];
-    if (!ca.ctl[p].active) continue;
-    for (int L = 0; L < 5; ++L) {
-      const int st = ca.pst[L * ca.nprob + p], sz = ca.psz[L * ca.nprob + p];
-      for (int t = 0; t < sz; ++t) {
-        if (L < 4) ca.comp[L][pos[L] + t] = ca.full[L][st + t];
-        else ca.tcomp[pos[L] + t] = ca.tfull[st + t];
-      }
-      pos[L] += sz;
+  __shared__ int wsum[32];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, L = blockIdx.x;
+  int base = 0, any = 0;
+  for (int i0 = 0; i0 < ca.nprob; i0 += 1024) {  // 1024 problems at a time
+    const int i = i0 + tid;
+    const int p = i < ca.nprob ? ca.order[i] : 0;
+    const bool act = i < ca.nprob && ca.ctl[p].active;
+    const int st = act ? ca.pst[L * ca.nprob + p] : 0, sz = act ? ca.psz[L * ca.nprob + p] : 0;
+    any |= act;
+    int inc = sz;  // inclusive scan over the warp, then over the warps
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += v;
     }
+    if (lane == 31) wsum[wid] = inc;
+    __syncthreads();
+    if (wid == 0) {
+      int v = wsum[lane];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+      }
+      wsum[lane] = v;
+    }
+    __syncthreads();
+    const int pos = base + (wid ? wsum[wid - 1] : 0) + inc - sz;
+    base += wsum[31];
+    for (int q = 0; q < 32; ++q) {  // the warp's problems, their items over the lanes
+      const int qst = __shfl_sync(0xffffffffu, st, q), qsz = __shfl_sync(0xffffffffu, sz, q);
+      const int qpos = __shfl_sync(0xffffffffu, pos, q);
+      for (int t = lane; t < qsz; t += 32) {
+        if (L < 3) ca.comp[L][qpos + t] = ca.full[L][qst + t];
+        else ca.tcomp[qpos + t] = ca.tfull[qst + t];
+      }
+    }
+    __syncthreads();  // wsum is written again
   }
   any = __syncthreads_or(any);
-  if (tid == 1023)
-    for (int L = 0; L < 5; ++L) ca.cnt[L] = sc[L][1023];
-  if (tid == 0) *ca.run = any;
+  if (tid == 0) {
+    ca.cnt[L] = base;
+    if (L == 0) *ca.run = any;
+  }
 }
 
 
-// final per-problem statistics (one warp per problem); tc: the product partials are per
+// final per-problem statistics (one block per problem); tc: the product partials are per
 // tensor-core item
-__global__ void k_bfinal(Ctl* __restrict__ ctl, const double* __restrict__ pax, const double* __restrict__ prow,
+__global__ void __launch_bounds__(256) k_bfinal(Ctl* __restrict__ ctl, const double* __restrict__ pax, const double* __restrict__ prow,
                          const double* __restrict__ G64p, const BProb* __restrict__ probs, int tc) {
   __shared__ double sh[32];
   const BProb& pb = probs[blockIdx.x];
@@ -396,7 +362,7 @@ __global__ void k_bfinal(Ctl* __restrict__ ctl, const double* __restrict__ pax, 
                  pb.nrt, G, G + rr, G + 2 * rr, 1, 0, pb.r, pb.normA2, sh);
 }
 
-enum { XB_W = 0, XB_HT, XB_B, XB_G, XB_Z, XB_D, XB_GZ, XB_D2, XB_N };
+enum { XB_W = 0, XB_HT, XB_B, XB_G, XB_Z, XB_GZ, XB_N };
 
 }  // namespace
 
@@ -407,8 +373,8 @@ struct BatchCtx {
   size_t esz = 4;
   std::vector<BProb> hp;
   BProb* dp = nullptr;
-  std::vector<int2> h_row, h_rowg, h_prod, h_gram;  // row items: tile body (r <= 32) / generic
-  int2* it_rowg = nullptr;
+  std::vector<int2> h_row, h_prod, h_gram;
+  size_t row_smem = 0;  // dynamic shared memory of the row kernels: the most over the problems' ranks
   int nslot = 0;
   std::vector<TcItem> h_tc;        // BF16: tensor-core product items
   TcItem* it_tc = nullptr;
@@ -420,7 +386,7 @@ struct BatchCtx {
   int2 *it_row = nullptr, *it_prod = nullptr, *it_gram = nullptr;
   // compacted lists of the active problems (rebuilt by k_bcompact), per-problem ranges in the
   // full lists, counts (cnt_full: constant full sizes; cnt_act: compacted)
-  int2 *c_row = nullptr, *c_rowg = nullptr, *c_gram = nullptr, *c_prod = nullptr;
+  int2 *c_row = nullptr, *c_gram = nullptr, *c_prod = nullptr;
   TcItem* c_tc = nullptr;
   int *pst = nullptr, *psz = nullptr, *d_order = nullptr, *cnt_full = nullptr, *cnt_act = nullptr;
   std::vector<int> order;
@@ -429,11 +395,11 @@ struct BatchCtx {
   int64_t lda = 0, rows_total = 0, xtot = 0;
   void* A = nullptr;
   void* buf[XB_N] = {};
-  double *prow = nullptr, *pax = nullptr, *gpart = nullptr, *G64fix = nullptr, *G64p = nullptr, *dsc = nullptr;
-  void* GT = nullptr;
+  double *prow = nullptr, *pax = nullptr, *G64fix = nullptr, *G64p = nullptr, *dsc = nullptr;
+  void *GT = nullptr, *gpart = nullptr;
   Ctl* ctl = nullptr;
   int* run = nullptr;
-  unsigned* counters = nullptr;
+  unsigned *counters = nullptr, *gcounters = nullptr;
   __nv_bfloat16* mlp_w = nullptr;
   float *rec_feat = nullptr, *rec_targ = nullptr;
   int* rec_count = nullptr;
@@ -487,16 +453,14 @@ Params bparams(const BatchCtx* b) {
   return P;
 }
 
-int row_bm(const BatchCtx* b) { return b->tdtype == 0 ? 32 : 64; }
-
 // ---- grouped launches -------------------------------------------------------------------
-// list L (0 row tile body, 1 row generic body, 2 Gram, 3 CUDA-core product, 4 tensor-core
-// product) and its device count for the launches being recorded
+// list L (0 row kernels, 1 Gram, 2 CUDA-core product, 3 tensor-core product) and its device
+// count for the launches being recorded
+constexpr int kLists = 4;
 const int* bcnt(const BatchCtx* b, int L) { return (b->use_full ? b->cnt_full : b->cnt_act) + L; }
 const int2* blist(const BatchCtx* b, int L) {
   if (L == 0) return b->use_full ? b->it_row : b->c_row;
-  if (L == 1) return b->use_full ? b->it_rowg : b->c_rowg;
-  if (L == 2) return b->use_full ? b->it_gram : b->c_gram;
+  if (L == 1) return b->use_full ? b->it_gram : b->c_gram;
   return b->use_full ? b->it_prod : b->c_prod;
 }
 
@@ -506,43 +470,45 @@ void bprod(BatchCtx* b, const void* X, void* Y, const void* P1, double* part, co
     // tcgen05: X_p split into BF16 hi / lo parts (transposed), then one CTA per 128-row tile
     const int nt = (int)b->h_tc.size();
     const TcItem* tl = b->use_full ? b->it_tc : b->c_tc;
-    launch_bsplit_x(tl, nt, bcnt(b, 4), (const float*)X, b->xh, b->xl, b->lda, ctl, sizeof(Ctl),
+    launch_bsplit_x(tl, nt, bcnt(b, 3), (const float*)X, b->xh, b->xl, b->lda, ctl, sizeof(Ctl),
                     offsetof(Ctl, active), run, b->s);
-    if (launch_bgemm_tc(b->A, b->lda, b->rows_total, b->xh, b->xl, b->xt_rows, tl, nt, bcnt(b, 4), (const float*)X,
+    if (launch_bgemm_tc(b->A, b->lda, b->rows_total, b->xh, b->xl, b->xt_rows, tl, nt, bcnt(b, 3), (const float*)X,
                         (float*)Y, 1, (const float*)P1, part, kNQ, ctl, sizeof(Ctl), offsetof(Ctl, active), run,
                         b->dev_err, b->budget, b->s) < 0)
       b->tc_fail = tc_last_status() ? tc_last_status() : -1;
     return;
   }
-  const int2* il = blist(b, 3);
-  const int* c = bcnt(b, 3);
-  if (b->tdtype == 0)
-    k_bgemm<double, double><<<g, 256, 0, b->s>>>((const double*)b->A, b->lda, b->dp, il, c, (const double*)X,
-                                                 (double*)Y, 1, (const double*)P1, part, ctl, run);
-  else if (b->a_dtype == 2)
-    k_bgemm<float, __nv_bfloat16><<<g, 256, 0, b->s>>>((const __nv_bfloat16*)b->A, b->lda, b->dp, il, c,
-                                                       (const float*)X, (float*)Y, 1, (const float*)P1, part,
-                                                       ctl, run);
-  else
-    k_bgemm<float, float><<<g, 256, 0, b->s>>>((const float*)b->A, b->lda, b->dp, il, c, (const float*)X,
-                                               (float*)Y, 1, (const float*)P1, part, ctl, run);
+  const int2* il = blist(b, 2);
+  const int* c = bcnt(b, 2);
+#define BGEMM(T, TA, KIND)                                                                                            \
+  do {                                                                                                                \
+    constexpr size_t smem = bgemm_smem<BGemm<T, KIND>>();                                                             \
+    static std::once_flag once;                                                                                       \
+    std::call_once(once, [] {                                                                                         \
+      cudaFuncSetAttribute(k_bgemm<T, TA, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);             \
+    });                                                                                                               \
+    k_bgemm<T, TA, KIND><<<g, BGemm<T, KIND>::NT, smem, b->s>>>((const TA*)b->A, b->lda, b->dp, il, c, (const T*)X,   \
+                                                                (T*)Y, 1, (const T*)P1, part, ctl, run);              \
+  } while (0)
+  if (b->tdtype == 0) BGEMM(double, double, GA_SAME);
+  else if (b->a_dtype == 2) BGEMM(float, __nv_bfloat16, GA_BF16);
+  else BGEMM(float, float, GA_SAME);
+#undef BGEMM
 }
 
-void bgram(BatchCtx* b, const void* X, const void* Y, int pair, int npairs, const Ctl* ctl, const int* run,
-           double* G64, void* GT, int tpair, int use_lam, Ctl* rho_ctl, cudaStream_t st = nullptr) {
+void bgram(BatchCtx* b, const void* X, const void* Y, int pair, const Ctl* ctl, const int* run, double* G64, void* GT,
+           Ctl* rho_ctl, cudaStream_t st = nullptr) {
   const unsigned g = (unsigned)b->h_gram.size();
   const int it = b->opt.power_iters;
   if (!st) st = b->s;
   if (b->tdtype == 0)
-    k_bgram<double><<<g, 256, 0, st>>>(b->dp, blist(b, 2), bcnt(b, 2), (const double*)X, (const double*)Y,
-                                       b->gpart, pair, npairs, ctl, run, G64, (double*)GT, tpair, use_lam,
-                                       b->counters, nullptr, it);
+    k_bgram<double><<<g, 256, gram_smem<double>(X == Y), st>>>(b->dp, blist(b, 1), bcnt(b, 1), (const double*)X,
+                                                               (const double*)Y, (double*)b->gpart, pair, ctl, run, G64,
+                                                               (double*)GT, b->gcounters, rho_ctl, it);
   else
-    k_bgram<float><<<g, 256, 0, st>>>(b->dp, blist(b, 2), bcnt(b, 2), (const float*)X, (const float*)Y,
-                                      b->gpart, pair, npairs, ctl, run, G64, (float*)GT, tpair, use_lam,
-                                      b->counters, rho_ctl, it);
-  if (b->tdtype == 0 && rho_ctl)
-    k_brho<double><<<b->nprob, 256, 0, st>>>(b->dp, G64, it, rho_ctl);
+    k_bgram<float><<<g, 256, gram_smem<float>(X == Y), st>>>(b->dp, blist(b, 1), bcnt(b, 1), (const float*)X,
+                                                             (const float*)Y, (float*)b->gpart, pair, ctl, run, G64,
+                                                             (float*)GT, b->gcounters, rho_ctl, it);
 }
 
 RowArgs brow_base(BatchCtx* b, const Params& P) {
@@ -551,45 +517,32 @@ RowArgs brow_base(BatchCtx* b, const Params& P) {
   a.ctl = b->ctl;
   a.run = b->run;
   a.part = b->prow;
-  a.counters = b->counters + 3 * b->nprob;
+  a.counters = b->counters;
   a.G64fix = b->G64fix;
   a.P = P;
   return a;
 }
 
-template <typename T, int OP, int EPI, int NC>
-void launch_browt(BatchCtx* b, const RowArgs& a) {
-  static bool attr = false;
-  const size_t smem = rowtile_smem<T>(EPI == EPI_DIR ? 2 + NC : 2);
-  if (!attr) {
-    cudaFuncSetAttribute(k_browt<T, OP, EPI, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr = true;
-  }
-  k_browt<T, OP, EPI, NC><<<(unsigned)b->h_row.size(), 256, smem, b->s>>>(a, b->dp, blist(b, 0), bcnt(b, 0));
+template <typename T, int STEP, int NC>
+void launch_brow(BatchCtx* b, const RowArgs& a) {
+  static std::once_flag once;
+  std::call_once(once, [] {
+    cudaFuncSetAttribute(k_brow<T, STEP, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+  });
+  k_brow<T, STEP, NC><<<(unsigned)b->h_row.size(), kRowThreads, b->row_smem, b->s>>>(a, b->dp, blist(b, 0), bcnt(b, 0));
 }
 
-void brow(BatchCtx* b, int op, int epi, const RowArgs& a, int nc = 1) {
-  if (!b->h_row.empty()) {
-#define BT(T)                                                                    \
-    if (epi == EPI_GRAD) {                                                       \
-      if (op == OP_LOAD) launch_browt<T, OP_LOAD, EPI_GRAD, 1>(b, a);            \
-      else launch_browt<T, OP_UPD, EPI_GRAD, 1>(b, a);                           \
-    } else if (nc == 1) launch_browt<T, OP_ZSTEP, EPI_DIR, 1>(b, a);             \
-    else launch_browt<T, OP_ZSTEP, EPI_DIR, 2>(b, a);
-    if (b->tdtype == 0) { BT(double) } else { BT(float) }
-#undef BT
+void brow(BatchCtx* b, int step, const RowArgs& a, int nc = 1) {
+#define BR(T)                                        \
+  if (step == RS_GRAD) launch_brow<T, RS_GRAD, 1>(b, a); \
+  else if (step == RS_D) {                           \
+    if (nc == 2) launch_brow<T, RS_D, 2>(b, a);      \
+    else launch_brow<T, RS_D, 1>(b, a);              \
+  } else {                                           \
+    if (nc == 2) launch_brow<T, RS_U, 2>(b, a);      \
+    else launch_brow<T, RS_U, 1>(b, a);              \
   }
-  if (b->h_rowg.empty()) return;
-  const unsigned g = (unsigned)b->h_rowg.size();
-#define BR(T, O, E, M, C) k_brow<T, O, E, M, C><<<g, 256, 0, b->s>>>(a, b->dp, blist(b, 1), bcnt(b, 1))
-#define BR_T(T, M)                                                       \
-  if (epi == EPI_GRAD) {                                                 \
-    if (op == OP_LOAD) BR(T, OP_LOAD, EPI_GRAD, M, 1);                   \
-    else BR(T, OP_UPD, EPI_GRAD, M, 1);                                  \
-  } else if (nc == 1) BR(T, OP_ZSTEP, EPI_DIR, M, 1);                    \
-  else BR(T, OP_ZSTEP, EPI_DIR, M, 2);  /* record mode is not offered on batch handles */
-  if (b->tdtype == 0) { BR_T(double, 32) } else { BR_T(float, 64) }
-#undef BR_T
+  if (b->tdtype == 0) { BR(double) } else { BR(float) }
 #undef BR
 }
 
@@ -599,15 +552,15 @@ void bany(BatchCtx* b) {
   ca.order = b->d_order;
   ca.nprob = b->nprob;
   ca.ctl = b->ctl;
-  ca.full[0] = b->it_row; ca.full[1] = b->it_rowg; ca.full[2] = b->it_gram; ca.full[3] = b->it_prod;
-  ca.comp[0] = b->c_row; ca.comp[1] = b->c_rowg; ca.comp[2] = b->c_gram; ca.comp[3] = b->c_prod;
+  ca.full[0] = b->it_row; ca.full[1] = b->it_gram; ca.full[2] = b->it_prod;
+  ca.comp[0] = b->c_row; ca.comp[1] = b->c_gram; ca.comp[2] = b->c_prod;
   ca.tfull = b->it_tc;
   ca.tcomp = b->c_tc;
   ca.pst = b->pst;
   ca.psz = b->psz;
   ca.cnt = b->cnt_act;
   ca.run = b->run;
-  k_bcompact<<<1, 1024, 0, b->s>>>(ca);
+  k_bcompact<<<kLists, 1024, 0, b->s>>>(ca);
 }
 
 // one block of Algorithm 1 for all problems (penalty form; mirrors the single-problem path)
@@ -618,7 +571,7 @@ void bpen_block(BatchCtx* b, int xv, int xf, bool is_w, const Params& P) {
   // product (a fork and a join of the captured graph) and share no buffer with it
   cudaEventRecord(b->evfork, b->s);
   cudaStreamWaitEvent(b->s2, b->evfork, 0);
-  bgram(b, Xf, Xf, 0, 1, b->ctl, b->run, b->G64fix, b->GT, 0, 1, b->ctl, b->s2);
+  bgram(b, Xf, Xf, 0, b->ctl, b->run, b->G64fix, b->GT, b->ctl, b->s2);
   cudaEventRecord(b->evjoin, b->s2);
   bprod(b, Xf, b->buf[XB_B], nullptr, nullptr, b->ctl, b->run);             // B = A Xf + lam Xf
   cudaStreamWaitEvent(b->s, b->evjoin, 0);
@@ -626,46 +579,31 @@ void bpen_block(BatchCtx* b, int xv, int xf, bool is_w, const Params& P) {
     RowArgs a = brow_base(b, P);
     a.X = X; a.B = b->buf[XB_B]; a.gout = b->buf[XB_G];
     a.ctl_mode = is_w ? CTL_START_W : CTL_START_H;
-    brow(b, OP_LOAD, EPI_GRAD, a);
+    brow(b, RS_GRAD, a);
   }
   bany(b);
   const int K = b->opt.inner_iters;
-  const int nc = b->opt.step_controller == 1 ? 2 : (b->opt.step_controller == 2 ? kNCand : 1);
+  const int nc = b->opt.step_controller == 1 ? 2 : 1;  // record mode is not offered on batch handles
   for (int k = 0; k < K; ++k) {
-    {
-      RowArgs a = brow_base(b, P);
-      a.B = b->buf[XB_B];
-      a.Dout = b->buf[XB_D]; a.gZout = b->buf[XB_GZ];
-      a.Wcur = X; a.gWcur = b->buf[XB_G];
-      a.X = X; a.g_in = b->buf[XB_G]; a.Xout = b->buf[XB_Z];
-      a.want_q = 1;
-      a.ctl_mode = CTL_LS;
-      a.dstore = nc == kNCand ? 4 : 0;
-      a.D2out = b->buf[XB_D2];
-      brow(b, OP_ZSTEP, EPI_DIR, a, nc);
-    }
-    {
-      RowArgs a = brow_base(b, P);
-      a.B = b->buf[XB_B];
-      a.gout = b->buf[XB_G];
-      a.Xold = X; a.gold = b->buf[XB_G];
-      a.Zold = b->buf[XB_Z]; a.gZold = b->buf[XB_GZ];
-      a.Xout = X;
-      a.ctl_mode = is_w ? CTL_UPD_W : (k == K - 1 ? CTL_UPD_H_LAST : CTL_UPD_H);
-      a.Zin = b->buf[XB_Z]; a.Din = b->buf[XB_D]; a.Din2 = b->buf[XB_D2];
-      brow(b, OP_UPD, EPI_GRAD, a);
-    }
+    RowArgs a = brow_base(b, P);
+    a.X = X; a.g_in = b->buf[XB_G]; a.B = b->buf[XB_B]; a.gZout = b->buf[XB_GZ];
+    a.ctl_mode = CTL_LS;
+    brow(b, RS_D, a, nc);
+    RowArgs u = brow_base(b, P);
+    u.Xout = X; u.gout = b->buf[XB_G]; u.gZold = b->buf[XB_GZ]; u.B = b->buf[XB_B];
+    u.ctl_mode = is_w ? CTL_UPD_W : (k == K - 1 ? CTL_UPD_H_LAST : CTL_UPD_H);
+    brow(b, RS_U, u, nc);
   }
 }
 
 void bpen_init(BatchCtx* b, const Params& P) {
   bany(b);
   bprod(b, b->buf[XB_W], b->buf[XB_B], nullptr, nullptr, b->ctl, b->run);
-  bgram(b, b->buf[XB_W], b->buf[XB_W], 0, 1, b->ctl, b->run, b->G64fix, b->GT, 0, 1, nullptr);
+  bgram(b, b->buf[XB_W], b->buf[XB_W], 0, b->ctl, b->run, b->G64fix, b->GT, nullptr);
   RowArgs a = brow_base(b, P);
   a.X = b->buf[XB_HT]; a.B = b->buf[XB_B]; a.gout = b->buf[XB_G];
   a.ctl_mode = CTL_START_INIT;
-  brow(b, OP_LOAD, EPI_GRAD, a);
+  brow(b, RS_GRAD, a);
 }
 
 void bpen_iteration(BatchCtx* b, const Params& P) {
@@ -681,16 +619,16 @@ void bpen_final(BatchCtx* b, const Params& P) {
   b->use_full = true;
   b->accurate = true;
   bprod(b, b->buf[XB_HT], b->buf[XB_B], b->buf[XB_W], b->pax, nullptr, nullptr);
-  bgram(b, b->buf[XB_W], b->buf[XB_W], 0, 3, nullptr, nullptr, b->G64p, b->GT, 1, 1, nullptr);
-  bgram(b, b->buf[XB_HT], b->buf[XB_HT], 1, 3, nullptr, nullptr, b->G64p, b->GT, 1, 1, nullptr);
-  bgram(b, b->buf[XB_W], b->buf[XB_HT], 2, 3, nullptr, nullptr, b->G64p, b->GT, 1, 1, nullptr);
+  bgram(b, b->buf[XB_W], b->buf[XB_W], 0, nullptr, nullptr, b->G64p, nullptr, nullptr);
+  bgram(b, b->buf[XB_HT], b->buf[XB_HT], 1, nullptr, nullptr, b->G64p, b->GT, nullptr);
+  bgram(b, b->buf[XB_W], b->buf[XB_HT], 2, nullptr, nullptr, b->G64p, nullptr, nullptr);
   RowArgs a = brow_base(b, P);
   a.X = b->buf[XB_W]; a.B = b->buf[XB_B]; a.gout = b->buf[XB_G];
   a.run = nullptr;
   a.ctl = b->ctl + b->nprob;  // second Ctl array: all live
   a.ctl_mode = CTL_NONE;
-  brow(b, OP_LOAD, EPI_GRAD, a);
-  k_bfinal<<<b->nprob, 32, 0, b->s>>>(b->ctl, b->pax, b->prow, b->G64p, b->dp, 0);
+  brow(b, RS_GRAD, a);
+  k_bfinal<<<b->nprob, 256, 0, b->s>>>(b->ctl, b->pax, b->prow, b->G64p, b->dp, 0);
   b->use_full = false;
   b->accurate = false;
 }
@@ -786,13 +724,16 @@ snmf_status batch_create(BatchCtx** out, const snmf_matrix* Am, const snmf_optio
   b->lda = (nmax + 63) / 64 * 64;
   b->hp.resize(np);
   int64_t arow = 0, xoff = 0, goff = 0, g3off = 0, gpoff = 0;
-  const int bm = row_bm(b);
+  int gcnt = 0;
   for (int p = 0; p < np; ++p) {
     BProb& q = b->hp[p];
     q.n = ns[p];
     q.r = (int)rs[p];
-    const int rows = rs[p] <= 32 ? (b->tdtype == 0 ? TileCfg<double>::TR : TileCfg<float>::TR) : bm;
+    const int mr = b->tdtype == 0 ? rowstep_mr<double>() : rowstep_mr<float>();
+    const int rows = rowstep_rows(q.r, kRowThreads, mr);
     q.nrt = (int)((ns[p] + rows - 1) / rows);
+    b->row_smem = std::max(b->row_smem, b->tdtype == 0 ? rowstep_smem<double>(q.r, kRowThreads, mr)
+                                                       : rowstep_smem<float>(q.r, kRowThreads, mr));
     q.npt = (int)((ns[p] + kPBM - 1) / kPBM);
     q.gch = (int)((ns[p] + kGChunk - 1) / kGChunk);
     q.arow = arow;
@@ -804,7 +745,10 @@ snmf_status batch_create(BatchCtx** out, const snmf_matrix* Am, const snmf_optio
     xoff += ns[p] * rs[p];
     goff += rs[p] * rs[p];
     g3off += 3 * rs[p] * rs[p];
-    gpoff += (int64_t)q.gch * 3 * rs[p] * rs[p];
+    q.gcnt = gcnt;
+    const int tw = gram_tw(q.r), ng = gram_groups(q.gch);
+    gpoff += (int64_t)(q.gch + ng) * tw * tw;
+    gcnt += 1 + ng;
   }
   b->rows_total = arow;
   b->xtot = xoff;
@@ -816,8 +760,7 @@ snmf_status batch_create(BatchCtx** out, const snmf_matrix* Am, const snmf_optio
     BProb& q = b->hp[p];
     q.slot0 = nslot;
     nslot += q.nrt;
-    std::vector<int2>& lst = q.r <= 32 ? b->h_row : b->h_rowg;
-    for (int t = 0; t < q.nrt; ++t) lst.push_back(make_int2(p, t));
+    for (int t = 0; t < q.nrt; ++t) b->h_row.push_back(make_int2(p, t));
     q.pslot0 = (int)b->h_prod.size();
     for (int t = 0; t < q.npt; ++t) b->h_prod.push_back(make_int2(p, t));
     for (int c = 0; c < q.gch; ++c) b->h_gram.push_back(make_int2(p, c));
@@ -855,14 +798,10 @@ snmf_status batch_create(BatchCtx** out, const snmf_matrix* Am, const snmf_optio
   // ---- device tables and workspaces ----
   CKB(cudaMalloc(&b->dp, np * sizeof(BProb)));
   b->nslot = nslot;
-  CKB(cudaMalloc(&b->it_row, std::max<size_t>(b->h_row.size(), 1) * sizeof(int2)));
-  CKB(cudaMalloc(&b->it_rowg, std::max<size_t>(b->h_rowg.size(), 1) * sizeof(int2)));
-  if (!b->h_rowg.empty())
-    CKB(cudaMemcpyAsync(b->it_rowg, b->h_rowg.data(), b->h_rowg.size() * sizeof(int2), cudaMemcpyHostToDevice, b->s));
+  CKB(cudaMalloc(&b->it_row, b->h_row.size() * sizeof(int2)));
   CKB(cudaMalloc(&b->it_prod, b->h_prod.size() * sizeof(int2)));
   CKB(cudaMalloc(&b->it_gram, b->h_gram.size() * sizeof(int2)));
-  if (!b->h_row.empty())
-    CKB(cudaMemcpyAsync(b->it_row, b->h_row.data(), b->h_row.size() * sizeof(int2), cudaMemcpyHostToDevice, b->s));
+  CKB(cudaMemcpyAsync(b->it_row, b->h_row.data(), b->h_row.size() * sizeof(int2), cudaMemcpyHostToDevice, b->s));
   CKB(cudaMemcpyAsync(b->it_prod, b->h_prod.data(), b->h_prod.size() * sizeof(int2), cudaMemcpyHostToDevice, b->s));
   CKB(cudaMemcpyAsync(b->it_gram, b->h_gram.data(), b->h_gram.size() * sizeof(int2), cudaMemcpyHostToDevice, b->s));
   CKB(cudaMemcpyAsync(b->dp, b->hp.data(), np * sizeof(BProb), cudaMemcpyHostToDevice, b->s));
@@ -875,14 +814,18 @@ snmf_status batch_create(BatchCtx** out, const snmf_matrix* Am, const snmf_optio
   CKB(cudaMalloc(&b->dev_err, sizeof(int)));
   CKB(cudaMemsetAsync(b->dev_err, 0, sizeof(int), b->s));
   if (o.timeout_cycles > 0) b->budget = o.timeout_cycles;
-  CKB(cudaMalloc(&b->gpart, std::max<int64_t>(gpoff, 1) * sizeof(double)));
+  CKB(cudaMalloc(&b->gpart, gpoff * b->esz));
+  CKB(cudaMalloc(&b->gcounters, gcnt * sizeof(unsigned)));
+  CKB(cudaMemsetAsync(b->gcounters, 0, gcnt * sizeof(unsigned), b->s));
+  CKB(cudaFuncSetAttribute(k_bgram<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gram_smem<double>(false)));
+  CKB(cudaFuncSetAttribute(k_bgram<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gram_smem<float>(false)));
   CKB(cudaMalloc(&b->G64fix, g3off * sizeof(double)));
   CKB(cudaMalloc(&b->G64p, g3off * sizeof(double)));
   CKB(cudaMalloc(&b->GT, goff * b->esz));
   CKB(cudaMalloc(&b->ctl, 2 * np * sizeof(Ctl)));
   CKB(cudaMalloc(&b->run, sizeof(int)));
-  CKB(cudaMalloc(&b->counters, 4 * np * sizeof(unsigned)));
-  CKB(cudaMemsetAsync(b->counters, 0, 4 * np * sizeof(unsigned), b->s));
+  CKB(cudaMalloc(&b->counters, np * sizeof(unsigned)));
+  CKB(cudaMemsetAsync(b->counters, 0, np * sizeof(unsigned), b->s));
   CKB(cudaMalloc(&b->dsc, (2 * b->h_prod.size() + 2 * np) * sizeof(double)));
   CKB(cudaMallocHost(&b->h_flag, sizeof(int)));
   if (o.step_controller == 1 || o.step_controller == 3) {
@@ -964,36 +907,34 @@ snmf_status batch_create(BatchCtx** out, const snmf_matrix* Am, const snmf_optio
   // full counts, and the compacted copies (start as the full lists)
   {
     b->order = order;
-    std::vector<int> pst(5 * np, 0), psz(5 * np, 0);
+    std::vector<int> pst(kLists * np, 0), psz(kLists * np, 0);
     auto fill = [&](int L, int i, int p) {
       if (psz[L * np + p] == 0) pst[L * np + p] = i;
       psz[L * np + p]++;
     };
     for (size_t i = 0; i < b->h_row.size(); ++i) fill(0, (int)i, b->h_row[i].x);
-    for (size_t i = 0; i < b->h_rowg.size(); ++i) fill(1, (int)i, b->h_rowg[i].x);
-    for (size_t i = 0; i < b->h_gram.size(); ++i) fill(2, (int)i, b->h_gram[i].x);
-    for (size_t i = 0; i < b->h_prod.size(); ++i) fill(3, (int)i, b->h_prod[i].x);
-    for (size_t i = 0; i < b->h_tc.size(); ++i) fill(4, (int)i, b->h_tc[i].prob);
-    const int cf[5] = {(int)b->h_row.size(), (int)b->h_rowg.size(), (int)b->h_gram.size(), (int)b->h_prod.size(),
-                       (int)b->h_tc.size()};
-    CKB(cudaMalloc(&b->pst, 5 * np * sizeof(int)));
-    CKB(cudaMalloc(&b->psz, 5 * np * sizeof(int)));
+    for (size_t i = 0; i < b->h_gram.size(); ++i) fill(1, (int)i, b->h_gram[i].x);
+    for (size_t i = 0; i < b->h_prod.size(); ++i) fill(2, (int)i, b->h_prod[i].x);
+    for (size_t i = 0; i < b->h_tc.size(); ++i) fill(3, (int)i, b->h_tc[i].prob);
+    const int cf[kLists] = {(int)b->h_row.size(), (int)b->h_gram.size(), (int)b->h_prod.size(), (int)b->h_tc.size()};
+    CKB(cudaMalloc(&b->pst, kLists * np * sizeof(int)));
+    CKB(cudaMalloc(&b->psz, kLists * np * sizeof(int)));
     CKB(cudaMalloc(&b->d_order, np * sizeof(int)));
-    CKB(cudaMalloc(&b->cnt_full, 5 * sizeof(int)));
-    CKB(cudaMalloc(&b->cnt_act, 5 * sizeof(int)));
-    CKB(cudaMemcpyAsync(b->pst, pst.data(), 5 * np * sizeof(int), cudaMemcpyHostToDevice, b->s));
-    CKB(cudaMemcpyAsync(b->psz, psz.data(), 5 * np * sizeof(int), cudaMemcpyHostToDevice, b->s));
+    CKB(cudaMalloc(&b->cnt_full, kLists * sizeof(int)));
+    CKB(cudaMalloc(&b->cnt_act, kLists * sizeof(int)));
+    CKB(cudaMemcpyAsync(b->pst, pst.data(), kLists * np * sizeof(int), cudaMemcpyHostToDevice, b->s));
+    CKB(cudaMemcpyAsync(b->psz, psz.data(), kLists * np * sizeof(int), cudaMemcpyHostToDevice, b->s));
     CKB(cudaMemcpyAsync(b->d_order, order.data(), np * sizeof(int), cudaMemcpyHostToDevice, b->s));
-    CKB(cudaMemcpyAsync(b->cnt_full, cf, 5 * sizeof(int), cudaMemcpyHostToDevice, b->s));
-    CKB(cudaMemcpyAsync(b->cnt_act, cf, 5 * sizeof(int), cudaMemcpyHostToDevice, b->s));
-    int2** comp[4] = {&b->c_row, &b->c_rowg, &b->c_gram, &b->c_prod};
-    const int2* full[4] = {b->it_row, b->it_rowg, b->it_gram, b->it_prod};
-    for (int L = 0; L < 4; ++L) {
-      CKB(cudaMalloc(comp[L], std::max(cf[L], 1) * sizeof(int2)));
-      if (cf[L]) CKB(cudaMemcpyAsync(*comp[L], full[L], cf[L] * sizeof(int2), cudaMemcpyDeviceToDevice, b->s));
+    CKB(cudaMemcpyAsync(b->cnt_full, cf, kLists * sizeof(int), cudaMemcpyHostToDevice, b->s));
+    CKB(cudaMemcpyAsync(b->cnt_act, cf, kLists * sizeof(int), cudaMemcpyHostToDevice, b->s));
+    int2** comp[3] = {&b->c_row, &b->c_gram, &b->c_prod};
+    const int2* full[3] = {b->it_row, b->it_gram, b->it_prod};
+    for (int L = 0; L < 3; ++L) {
+      CKB(cudaMalloc(comp[L], cf[L] * sizeof(int2)));
+      CKB(cudaMemcpyAsync(*comp[L], full[L], cf[L] * sizeof(int2), cudaMemcpyDeviceToDevice, b->s));
     }
-    CKB(cudaMalloc(&b->c_tc, std::max(cf[4], 1) * sizeof(TcItem)));
-    if (cf[4]) CKB(cudaMemcpyAsync(b->c_tc, b->it_tc, cf[4] * sizeof(TcItem), cudaMemcpyDeviceToDevice, b->s));
+    CKB(cudaMalloc(&b->c_tc, std::max(cf[3], 1) * sizeof(TcItem)));
+    if (cf[3]) CKB(cudaMemcpyAsync(b->c_tc, b->it_tc, cf[3] * sizeof(TcItem), cudaMemcpyDeviceToDevice, b->s));
     CKB(cudaStreamSynchronize(b->s));
   }
 #undef CKB
@@ -1179,8 +1120,7 @@ void batch_destroy(BatchCtx* b) {
   cudaFree(b->it_row);
   cudaFree(b->it_prod);
   cudaFree(b->it_gram);
-  cudaFree(b->it_rowg);
-  for (void* q : {(void*)b->c_row, (void*)b->c_rowg, (void*)b->c_gram, (void*)b->c_prod, (void*)b->c_tc,
+  for (void* q : {(void*)b->c_row, (void*)b->c_gram, (void*)b->c_prod, (void*)b->c_tc,
                   (void*)b->pst, (void*)b->psz, (void*)b->d_order, (void*)b->cnt_full, (void*)b->cnt_act})
     cudaFree(q);
   cudaFree(b->it_tc);
@@ -1188,9 +1128,11 @@ void batch_destroy(BatchCtx* b) {
   cudaFree(b->xl);
   cudaFree(b->dev_err);
   for (void* p : b->buf) cudaFree(p);
-  double* d[] = {b->prow, b->pax, b->gpart, b->G64fix, b->G64p, b->dsc};
+  double* d[] = {b->prow, b->pax, b->G64fix, b->G64p, b->dsc};
   for (double* p : d) cudaFree(p);
   cudaFree(b->GT);
+  cudaFree(b->gpart);
+  cudaFree(b->gcounters);
   cudaFree(b->ctl);
   cudaFree(b->run);
   cudaFree(b->counters);

@@ -59,9 +59,9 @@ struct snmf_ctx {
   bool graph = false;
   double gamma = 0.0;
   double normL = 0.0;  // ||L||_2 (power method), enters rho of graph-regularised blocks
-  int use_tile = 0;    // row kernels through the shared-memory tile body (r <= 32)
-  int use_fuse = 0;    // D step and update through rowfuse.cu (FP32, r in {16, 32, 64}, no Z / D stored)
-  int row_tc = 0;      // with use_fuse: row products on the tensor cores, 1 rowtc.cu, 2 rowtma.cu (r = 64; tuned)
+  int use_row = 0;     // row kernels through rowstep.cu (penalty form, r <= 64, no record mode)
+  RowStepPlan rplan{};
+  int row_tc = 0;      // with use_row: row products on the tensor cores, 1 rowtc.cu, 2 rowtma.cu (r = 64; tuned)
   int row_bm = 0;      // general row kernel, FP32: rows per CTA (0: built-in choice; autotuned)
   AxArgs L{};
   int32_t* L_rowptr = nullptr;
@@ -79,14 +79,15 @@ struct snmf_ctx {
   double *prow = nullptr, *pax = nullptr, *pax2 = nullptr, *pax3 = nullptr, *pax4 = nullptr,
          *pclip = nullptr;
   int nrow = 0, nax = 0;
-  double* gpart = nullptr;
-  int nchunks = 1;
+  void* gpart = nullptr;      // Gram chunk partials
+  GramPlan gplan{};
+  unsigned* gcounters = nullptr;
   double *G64fix = nullptr, *G64p = nullptr;  // G64p: 3 pairs [pair][b][r*r]
   void* GT = nullptr;
   Ctl* ctl = nullptr;
   int* run = nullptr;
   int* recompute = nullptr;
-  unsigned* counters = nullptr;  // arrival counters of the fused Gram reduction
+  unsigned* counters = nullptr;  // per-restart arrival counters of the row kernels
   int* dev_err = nullptr;        // device error code of bounded waits (tensor-core product)
   void* xh = nullptr;            // BF16 hi / lo parts of the product operand (transposed)
   void* xl = nullptr;
@@ -283,22 +284,13 @@ int ax_L(snmf_ctx* h, const void* X, void* Y, const void* P1, const void* P2, do
   return ax_apply(h, h->L, false, X, Y, 0.0, nullptr, P1, P2, part, run);
 }
 
-int choose_chunks(int64_t n, int b, int r) {
-  // about one CTA per SM, at least 512 rows per chunk (fewer partials to reduce)
-  const int ntile = (r + 63) / 64;
-  const int64_t per = (int64_t)b * ntile * ntile;
-  int64_t c = (152 + per - 1) / per;
-  c = std::max<int64_t>(1, std::min<int64_t>(c, n / 512));
-  return (int)c;
-}
-
 // Gram X^T Y per restart into G64 (+ factor-type copy GT with lam I when pair == tpair);
 // inside the iteration it follows ctl[j].active and the run flag, in the initial and
 // final evaluations (ctl == NULL) every restart is computed.
-void gram1(snmf_ctx* h, const void* X, const void* Y, int pair, int npairs, const Ctl* ctl,
-           double* G64, void* GT, int tpair, double lam) {
-  launch_gram(h->tdtype, X, Y, dims(h), pair, npairs, h->gpart, h->nchunks, ctl,
-              ctl ? h->run : nullptr, G64, GT, tpair, lam, h->counters, h->s);
+void gram1(snmf_ctx* h, const void* X, const void* Y, int pair, const Ctl* ctl, double* G64, void* GT, int tpair,
+           double lam) {
+  launch_gram(h->tdtype, X, Y, dims(h), h->gplan, pair, h->gpart, ctl, ctl ? h->run : nullptr, G64, GT, tpair, lam,
+              h->gcounters, h->s);
 }
 
 RowArgs row_base(snmf_ctx* h, const Params* P = nullptr) {
@@ -309,12 +301,33 @@ RowArgs row_base(snmf_ctx* h, const Params* P = nullptr) {
   a.run = h->run;
   a.gamma = h->graph ? h->gamma : 0.0;
   a.part = h->prow;
-  a.counters = h->counters + 16384;
+  a.counters = h->counters;
+  a.gcounters = h->rplan.groups ? h->counters + h->b : nullptr;
   a.G64fix = h->G64fix;
-  a.tile = h->use_tile;
   a.bm = h->row_bm;
   if (P) a.P = *P;
   return a;
+}
+
+// The D step and the update of a block without graph term: on the tensor cores where the autotuner
+// chose them, else rowstep.cu.
+void row_dstep(snmf_ctx* h, const RowArgs& a, int nc) {
+  if (h->row_tc == 2 && launch_rowtma_dstep(a, h->dev_err, h->s)) return;
+  if (h->row_tc) launch_rowtc_dstep(a, h->dev_err, h->s);
+  else launch_rowstep_d(h->tdtype, a, h->rplan, nc, h->s);
+}
+
+void row_update(snmf_ctx* h, const RowArgs& a, int nc) {
+  if (h->row_tc == 2 && launch_rowtma_update(a, h->dev_err, h->s)) return;
+  if (h->row_tc) launch_rowtc_update(a, h->dev_err, h->s);
+  else launch_rowstep_update(h->tdtype, a, h->rplan, nc, h->s);
+}
+
+// Gradient of a given X (block start; an update of a graph-regularised block; the final point).
+void row_grad(snmf_ctx* h, const RowArgs& a) {
+  if (h->use_row && h->row_tc && !a.LX && !a.Xold && a.ctl_mode) launch_rowtc_grad(a, h->dev_err, h->s);
+  else if (h->use_row) launch_rowstep_grad(h->tdtype, a, h->rplan, h->s);
+  else launch_rowgemm(h->tdtype, OP_LOAD, EPI_GRAD, a, h->s);
 }
 
 // Mean time of one D-step launch and one update launch of a W block (the row kernels of
@@ -353,15 +366,11 @@ snmf_status time_steps(snmf_ctx* h, int iters, double* ms_dstep, double* ms_upda
   au.ctl_mode = CTL_UPD_W;
   au.Zin = h->buf[B_Z]; au.Din = h->buf[B_D]; au.Din2 = h->buf[B_AD];
   auto dstep = [&] {
-    if (h->use_fuse && h->row_tc == 2 && launch_rowtma_dstep(ad, h->dev_err, h->s)) {
-    } else if (h->use_fuse && h->row_tc) launch_rowtc_dstep(ad, h->dev_err, h->s);
-    else if (h->use_fuse) launch_rowfuse_dstep(ad, h->row_bm, nc, h->s);
+    if (h->use_row) row_dstep(h, ad, nc);
     else launch_rowgemm(td, OP_ZSTEP, EPI_DIR, ad, h->s, nc);
   };
   auto update = [&] {
-    if (h->use_fuse && h->row_tc == 2 && launch_rowtma_update(au, h->dev_err, h->s)) {
-    } else if (h->use_fuse && h->row_tc) launch_rowtc_update(au, h->dev_err, h->s);
-    else if (h->use_fuse) launch_rowfuse_update(au, h->row_bm, nc, h->s);
+    if (h->use_row) row_update(h, au, nc);
     else launch_rowgemm(td, OP_UPD, EPI_GRAD, au, h->s);
   };
   cudaEvent_t e[4];
@@ -396,23 +405,22 @@ snmf_status autotune_product(snmf_ctx* h) {
                           "/n" + std::to_string(h->n) + "/r" + std::to_string(h->r) + "/N" + std::to_string(h->N);
   const std::string dev = tune_device_key();
   TuneEntry e;
-  const bool tune_rows =
-      (!h->use_tile || h->use_fuse) && h->tdtype == 1 && h->opt.formulation != SNMF_DIRECT && h->r <= 64;
-  // rows per CTA offered to the search: the fused kernels' heights, else the general kernel's
+  // the general row kernel's heights (FP32, the forms that rowstep.cu does not take), and the
+  // tensor-core bodies beside rowstep.cu
+  const bool tune_rows = h->tdtype == 1 && h->opt.formulation != SNMF_DIRECT && h->r <= 64;
   std::vector<int> bms;
-  if (h->use_fuse) bms = h->r == 16 ? std::vector<int>{128, 256} : std::vector<int>{128, 64};
-  else bms = {64, 32};
+  if (!h->use_row) bms = {64, 32};
   if (tune_lookup(h->opt.tune_cache, dev, key, &e)) {
     h->tune = e;
     h->tuned = 2;
     if (tune_rows && std::find(bms.begin(), bms.end(), e.cfg.row_bm) != bms.end()) {
       h->row_bm = e.cfg.row_bm;
-      if (!h->use_tile) h->nrow = rowgemm_slots(dims(h), h->tdtype, 0, h->row_bm);
+      h->nrow = rowgemm_slots(dims(h), h->tdtype, h->row_bm);
     }
     const int tnc = h->opt.step_controller == 1 ? 2 : 1;
     h->row_tc = 0;
-    if (tune_rows && h->use_fuse && e.cfg.row_tc == 1 && rowtc_supported(h->tdtype, h->r, tnc)) h->row_tc = 1;
-    if (tune_rows && h->use_fuse && e.cfg.row_tc == 2 && rowtma_supported(h->tdtype, h->r, tnc, h->N)) h->row_tc = 2;
+    if (tune_rows && h->use_row && e.cfg.row_tc == 1 && rowtc_supported(h->tdtype, h->r, tnc)) h->row_tc = 1;
+    if (tune_rows && h->use_row && e.cfg.row_tc == 2 && rowtma_supported(h->tdtype, h->r, tnc, h->N)) h->row_tc = 2;
     return SNMF_OK;
   }
   std::vector<ProdTune> cand;
@@ -484,26 +492,34 @@ snmf_status autotune_product(snmf_ctx* h) {
     return SNMF_OK;
   }
   h->tune = best;
-  // the general row kernel's tile height (FP32 penalty form): D step + update per inner step
   if (tune_rows) {
     double bt = 1e30;
+    if (h->use_row) {
+      double md = 0.0, mu = 0.0;
+      const snmf_status st = time_steps(h, 5, &md, &mu);
+      if (st != SNMF_OK) return st;
+      bt = md + mu;
+    }
+    // the general row kernel's tile height: D step + update per inner step
     int bbm = 0;
     for (int bm : bms) {
       h->row_bm = bm;
-      if (!h->use_tile) h->nrow = rowgemm_slots(dims(h), h->tdtype, 0, bm);
+      h->nrow = rowgemm_slots(dims(h), h->tdtype, bm);
       double md = 0.0, mu = 0.0;
       const snmf_status st = time_steps(h, 5, &md, &mu);
       if (st != SNMF_OK) return st;
       if (md + mu < bt) { bt = md + mu; bbm = bm; }
     }
-    h->row_bm = bbm;
-    if (!h->use_tile) h->nrow = rowgemm_slots(dims(h), h->tdtype, 0, bbm);
+    if (!h->use_row) {
+      h->row_bm = bbm;
+      h->nrow = rowgemm_slots(dims(h), h->tdtype, bbm);
+    }
     h->tune.cfg.row_bm = bbm;
     // the tensor-core row products (r = 64): per-CTA tiles (1) and the persistent TMA
     // pipeline (2), each kept when faster than the best so far and free of device errors
     const int tnc = h->opt.step_controller == 1 ? 2 : 1;
     h->row_tc = 0;
-    for (int kind = 1; kind <= 2 && h->use_fuse; ++kind) {
+    for (int kind = 1; kind <= 2 && h->use_row; ++kind) {
       if (kind == 1 && !rowtc_supported(h->tdtype, h->r, tnc)) continue;
       if (kind == 2 && !rowtma_supported(h->tdtype, h->r, tnc, h->N)) continue;
       const int prev = h->row_tc;
@@ -540,15 +556,15 @@ void pen_block(snmf_ctx* h, int xv, int xf, bool is_w, const Params& P, bool nai
   // The Gram and rho_0 depend on Xfix alone, so they run on the side stream beside the
   // product (a fork and a join of the captured graph); they share no buffer with it.
   // G = Xfix^T Xfix (+ lambda I in the factor-type copy); rho_0 = ||Xfix^T Xfix||_2, computed
-  // by the Gram's last CTA when the restart is one tile (FP32 path), else by k_rho
+  // by the Gram's last CTA when the restart is one tile (r <= 64), else by k_rho_wide
   cudaEventRecord(h->evfork, h->s);
   cudaStreamWaitEvent(h->s2, h->evfork, 0);
-  const bool rho_fused = td == 1 && h->r <= 64;
+  const bool rho_fused = h->gplan.ntile == 1;
   // graph-regularised H block: rho_0 = ||W^T W||_2 + gamma ||L||_2 (Lipschitz constant of its gradient)
   const double shift = gr ? h->gamma * h->normL : 0.0;
-  launch_gram(td, Xf, Xf, d, 0, 1, h->gpart, h->nchunks, h->ctl, h->run, h->G64fix, h->GT, 0, h->lam,
-              h->counters, h->s2, rho_fused ? h->ctl : nullptr, h->opt.power_iters, 1.0, shift);
-  if (!rho_fused) launch_rho(td, h->G64fix, d, h->opt.power_iters, 1.0, h->ctl, 0, h->s2, shift);
+  launch_gram(td, Xf, Xf, d, h->gplan, 0, h->gpart, h->ctl, h->run, h->G64fix, h->GT, 0, h->lam, h->gcounters, h->s2,
+              h->ctl, h->opt.power_iters, 1.0, shift);
+  if (!rho_fused) launch_rho(td, h->G64fix, d, h->opt.power_iters, 1.0, h->ctl, h->s2, shift);
   cudaEventRecord(h->evjoin, h->s2);
   // B = A Xfix + lambda Xfix (Eq. (2.1)/(2.2))
   ax_A(h, Xf, h->buf[B_B], h->lam, Xf, nullptr, nullptr, h->pax, h->run);
@@ -560,30 +576,53 @@ void pen_block(snmf_ctx* h, int xv, int xf, bool is_w, const Params& P, bool nai
     a.X = X; a.B = h->buf[B_B]; a.LX = gr ? h->buf[B_LX] : nullptr;
     a.gout = h->buf[B_G];
     a.ctl_mode = is_w ? CTL_START_W : CTL_START_H;
-    if (h->use_fuse && h->row_tc && !gr) launch_rowtc_grad(a, h->dev_err, h->s);  // X G on tcgen05
-    else launch_rowgemm(td, OP_LOAD, EPI_GRAD, a, h->s);
+    if (gr && h->use_row) a.Znext = h->buf[B_Z];
+    row_grad(h, a);
   }
   launch_any_active(h->ctl, h->b, h->run, nullptr, h->s);
   const int K = h->opt.inner_iters;
   const bool fused_q = h->r <= 64 && !gr;
-  if (h->use_fuse && !gr) {
-    // D step (g(Z) and the line search) and the update recomputing Z and D (rowfuse.cu);
-    // the learned step with fallback (controller 1) carries the plain BB direction as well
+  auto upd_mode = [&](int k) {
+    return is_w ? (naive && k == K - 1 ? CTL_UPD_W_LAST_NAIVE : CTL_UPD_W) : (k == K - 1 ? CTL_UPD_H_LAST : CTL_UPD_H);
+  };
+  if (h->use_row && !gr) {
+    // D step (g(Z) and the line search) and the update recomputing Z and D; the learned step with
+    // fallback (controller 1) carries the plain BB direction as well
     const int nc = h->opt.step_controller == 1 ? 2 : 1;
     for (int k = 0; k < K; ++k) {
       RowArgs a = row_base(h, &P);
       a.X = X; a.g_in = h->buf[B_G]; a.B = h->buf[B_B]; a.gZout = h->buf[B_GZ];
       a.ctl_mode = CTL_LS;
-      if (h->row_tc == 2 && launch_rowtma_dstep(a, h->dev_err, h->s)) {
-      } else if (h->row_tc) launch_rowtc_dstep(a, h->dev_err, h->s);
-      else launch_rowfuse_dstep(a, h->row_bm, nc, h->s);
+      row_dstep(h, a, nc);
       RowArgs u = row_base(h, &P);
       u.Xout = X; u.gout = h->buf[B_G]; u.gZold = h->buf[B_GZ]; u.B = h->buf[B_B];
-      u.ctl_mode = is_w ? (naive && k == K - 1 ? CTL_UPD_W_LAST_NAIVE : CTL_UPD_W)
-                        : (k == K - 1 ? CTL_UPD_H_LAST : CTL_UPD_H);
-      if (h->row_tc == 2 && launch_rowtma_update(u, h->dev_err, h->s)) {
-      } else if (h->row_tc) launch_rowtc_update(u, h->dev_err, h->s);
-      else launch_rowfuse_update(u, h->row_bm, nc, h->s);
+      u.ctl_mode = upd_mode(k);
+      row_update(h, u, nc);
+    }
+    return;
+  }
+  if (h->use_row) {
+    // graph-regularised block: L Z, L D and L X' are products of their own, so Z (written by the
+    // gradient kernel before it), D and X' are stored
+    for (int k = 0; k < K; ++k) {
+      ax_L(h, h->buf[B_Z], h->buf[B_LZ], nullptr, nullptr, h->pax2, h->run);
+      RowArgs a = row_base(h, &P);
+      a.X = h->buf[B_Z]; a.LX = h->buf[B_LZ]; a.B = h->buf[B_B];
+      a.Dout = h->buf[B_D]; a.gZout = h->buf[B_GZ];
+      a.Wcur = X; a.gWcur = h->buf[B_G];
+      launch_rowstep_dz(td, a, h->rplan, h->s);
+      const int nl = ax_L(h, h->buf[B_D], h->buf[B_LD], h->buf[B_D], nullptr, h->pax3, h->run);
+      launch_ctl_pen_ls(h->ctl, h->prow, h->nrow, h->pax3, nl, h->b, h->r, h->G64fix, nullptr, P, 1, h->s);
+      launch_xupd(td, d, h->buf[B_Z], h->buf[B_D], h->buf[B_XN], nullptr, nullptr, nullptr, h->ctl, h->pclip, h->s);
+      ax_L(h, h->buf[B_XN], h->buf[B_LX], nullptr, nullptr, h->pax2, h->run);
+      RowArgs u = row_base(h, &P);
+      u.X = h->buf[B_XN]; u.LX = h->buf[B_LX]; u.B = h->buf[B_B];
+      u.gout = h->buf[B_G]; u.Xout = X;
+      u.Xold = X; u.gold = h->buf[B_G];
+      u.Zold = h->buf[B_Z]; u.gZold = h->buf[B_GZ];
+      if (k + 1 < K) u.Znext = h->buf[B_Z];
+      u.ctl_mode = upd_mode(k);
+      row_grad(h, u);
     }
     return;
   }
@@ -603,8 +642,7 @@ void pen_block(snmf_ctx* h, int xv, int xf, bool is_w, const Params& P, bool nai
         a.X = X; a.g_in = h->buf[B_G]; a.Xout = h->buf[B_Z];
         a.want_q = fused_q ? 1 : 0;
         a.ctl_mode = fused_q ? CTL_LS : CTL_NONE;  // line search in the last CTA of each restart
-        // learned controller: proposal + plain BB direction; record mode: 9 candidates
-        const int nc = h->opt.step_controller == 1 ? 2 : (h->opt.step_controller == 2 ? kNCand : 1);
+        const int nc = h->opt.step_controller == 2 ? kNCand : 1;  // record mode: 9 candidates
         a.dstore = nc == kNCand ? 4 : 0;
         a.D2out = h->buf[B_AD];
         launch_rowgemm(td, OP_ZSTEP, EPI_DIR, a, h->s, nc);
@@ -612,7 +650,7 @@ void pen_block(snmf_ctx* h, int xv, int xf, bool is_w, const Params& P, bool nai
     }
     if (!fused_q) {
       // curvature of the line-search quadratic from the Gram D^T D; graph term <D, L D>
-      gram1(h, h->buf[B_D], h->buf[B_D], 0, 1, h->ctl, h->G64p, nullptr, -1, 0.0);
+      gram1(h, h->buf[B_D], h->buf[B_D], 0, h->ctl, h->G64p, nullptr, -1, 0.0);
       int nl = 0;
       if (gr) nl = ax_L(h, h->buf[B_D], h->buf[B_LD], h->buf[B_D], nullptr, h->pax3, h->run);
       launch_ctl_pen_ls(h->ctl, h->prow, h->nrow, h->pax3, gr ? nl : 0, h->b, h->r, h->G64fix, h->G64p, P,
@@ -626,8 +664,7 @@ void pen_block(snmf_ctx* h, int xv, int xf, bool is_w, const Params& P, bool nai
       a.Xold = X; a.gold = h->buf[B_G];
       a.Zold = h->buf[B_Z]; a.gZold = h->buf[B_GZ];
       a.Xout = X;
-      a.ctl_mode = is_w ? (naive && k == K - 1 ? CTL_UPD_W_LAST_NAIVE : CTL_UPD_W)
-                        : (k == K - 1 ? CTL_UPD_H_LAST : CTL_UPD_H);
+      a.ctl_mode = upd_mode(k);
       if (gr) {
         launch_xupd(td, d, h->buf[B_Z], h->buf[B_D], h->buf[B_XN], nullptr, nullptr, nullptr,
                     h->ctl, h->pclip, h->s);
@@ -644,17 +681,15 @@ void pen_block(snmf_ctx* h, int xv, int xf, bool is_w, const Params& P, bool nai
 
 // H gradient at the start point (enters the first joint projected gradient).
 void pen_init(snmf_ctx* h, const Params& P) {
-  const Dims d = dims(h);
-  const int td = h->tdtype;
   launch_any_active(h->ctl, h->b, h->run, nullptr, h->s);
   ax_A(h, h->buf[B_W], h->buf[B_B], h->lam, h->buf[B_W], nullptr, nullptr, h->pax, h->run);
-  gram1(h, h->buf[B_W], h->buf[B_W], 0, 1, h->ctl, h->G64fix, h->GT, 0, h->lam);
+  gram1(h, h->buf[B_W], h->buf[B_W], 0, h->ctl, h->G64fix, h->GT, 0, h->lam);
   if (h->graph) ax_L(h, h->buf[B_HT], h->buf[B_LX], nullptr, nullptr, h->pax2, h->run);
   RowArgs a = row_base(h, &P);
   a.X = h->buf[B_HT]; a.B = h->buf[B_B]; a.LX = h->graph ? h->buf[B_LX] : nullptr;
   a.gout = h->buf[B_G];
   a.ctl_mode = CTL_START_INIT;  // records the H gradient of the start
-  launch_rowgemm(td, OP_LOAD, EPI_GRAD, a, h->s);
+  row_grad(h, a);
 }
 
 void pen_iteration(snmf_ctx* h, const Params& P) {
@@ -675,8 +710,6 @@ void naive_iteration(snmf_ctx* h, const Params& P) {
 }
 
 void pen_final(snmf_ctx* h, const Params& P) {
-  const Dims d = dims(h);
-  const int td = h->tdtype;
   // every restart contributes to the final evaluation.  The closed-form objective
   // ||A||^2 - 2 <W, A Ht> + ... cancels to a small residual, so <W, A Ht> is taken from an
   // FP32 CUDA-core product of the stored BF16 A: the tensor-core FP32 accumulation carries
@@ -685,9 +718,9 @@ void pen_final(snmf_ctx* h, const Params& P) {
   fin.accurate = 1;
   int nax = ax_apply(h, fin, h->lai, h->buf[B_HT], h->buf[B_B], h->lam, h->buf[B_HT],
                      h->buf[B_W], nullptr, h->pax, nullptr);
-  gram1(h, h->buf[B_W], h->buf[B_W], 0, 3, nullptr, h->G64p, h->GT, 1, h->lam);
-  gram1(h, h->buf[B_HT], h->buf[B_HT], 1, 3, nullptr, h->G64p, h->GT, 1, h->lam);
-  gram1(h, h->buf[B_W], h->buf[B_HT], 2, 3, nullptr, h->G64p, h->GT, 1, h->lam);
+  gram1(h, h->buf[B_W], h->buf[B_W], 0, nullptr, h->G64p, h->GT, 1, h->lam);
+  gram1(h, h->buf[B_HT], h->buf[B_HT], 1, nullptr, h->G64p, h->GT, 1, h->lam);
+  gram1(h, h->buf[B_W], h->buf[B_HT], 2, nullptr, h->G64p, h->GT, 1, h->lam);
   // W gradient at the final point (projected-gradient statistic); uses a temporary
   // "all active" view: the row kernel is run with ctl entries forced live by the host.
   RowArgs a = row_base(h);
@@ -695,7 +728,7 @@ void pen_final(snmf_ctx* h, const Params& P) {
   a.gout = h->buf[B_G];
   a.run = nullptr;
   a.ctl = h->ctl + h->b;  // second Ctl array: all active (set by the host)
-  launch_rowgemm(td, OP_LOAD, EPI_GRAD, a, h->s);
+  row_grad(h, a);
   const int64_t rr = (int64_t)h->r * h->r * h->b;
   launch_ctl_final_pen(h->ctl, h->pax, nax, h->prow, h->nrow, h->G64p, h->G64p + rr,
                        h->G64p + 2 * rr, h->b, h->r, P, h->s);
@@ -712,7 +745,7 @@ void dir_init(snmf_ctx* h, const Params& P) {
   int nlx = 0;
   if (h->graph)
     nlx = ax_L(h, h->buf[B_W], h->buf[B_LX], h->buf[B_W], nullptr, h->pax2, nullptr);
-  gram1(h, h->buf[B_W], h->buf[B_W], 0, 1, nullptr, h->G64fix, h->GT, 0, 0.0);
+  gram1(h, h->buf[B_W], h->buf[B_W], 0, nullptr, h->G64fix, h->GT, 0, 0.0);
   RowArgs a = row_base(h);
   a.X = h->buf[B_W]; a.B = h->buf[B_B]; a.LX = h->graph ? h->buf[B_LX] : nullptr;
   a.gout = h->buf[B_G];
@@ -732,13 +765,13 @@ void dir_iteration(snmf_ctx* h, const Params& P) {
   void *Z = h->buf[B_Z], *AZ = h->buf[B_AZ], *D = h->buf[B_D], *AD = h->buf[B_AD];
   void *Wn = h->buf[B_XN], *AWn = h->buf[B_AWN], *gn = h->buf[B_GN];
   // rho_k = factor ||W^T W||_2 and alpha_k
-  launch_rho(td, h->G64fix, d, h->opt.power_iters, h->opt.direct_rho_factor, h->ctl, 0, h->s,
+  launch_rho(td, h->G64fix, d, h->opt.power_iters, h->opt.direct_rho_factor, h->ctl, h->s,
              h->graph ? h->gamma * h->normL : 0.0);
   launch_ctl_dir_alpha(h->ctl, h->b, P, h->s);
   launch_zstep(td, d, W, g, Z, h->ctl, h->s);
   int nz = ax_A(h, Z, AZ, 0.0, nullptr, Z, nullptr, h->pax, h->run);
   if (h->graph) ax_L(h, Z, h->buf[B_LZ], Z, nullptr, h->pax3, h->run);
-  gram1(h, Z, Z, 0, 1, h->ctl, h->G64p, h->GT, 0, 0.0);
+  gram1(h, Z, Z, 0, h->ctl, h->G64p, h->GT, 0, 0.0);
   {
     RowArgs a = row_base(h);
     a.X = Z; a.B = AZ; a.LX = h->graph ? h->buf[B_LZ] : nullptr;
@@ -747,8 +780,8 @@ void dir_iteration(snmf_ctx* h, const Params& P) {
   }
   int nd = ax_A(h, D, AD, 0.0, nullptr, Z, D, h->pax2, h->run);
   if (h->graph) ax_L(h, D, h->buf[B_LD], D, nullptr, h->pax4, h->run);
-  gram1(h, Z, D, 0, 2, h->ctl, h->G64p + rr, nullptr, -1, 0.0);
-  gram1(h, D, D, 1, 2, h->ctl, h->G64p + rr, nullptr, -1, 0.0);
+  gram1(h, Z, D, 0, h->ctl, h->G64p + rr, nullptr, -1, 0.0);
+  gram1(h, D, D, 1, h->ctl, h->G64p + rr, nullptr, -1, 0.0);
   launch_ctl_dir_ls(h->ctl, h->pax, nz, h->prow, h->nrow, h->pax2, nd, h->G64p, h->G64p + rr,
                     h->G64p + 2 * rr, h->graph ? h->pax3 : nullptr, h->graph ? h->pax4 : nullptr,
                     h->b, h->r, P, h->s);
@@ -757,7 +790,7 @@ void dir_iteration(snmf_ctx* h, const Params& P) {
   int nre = ax_A(h, Wn, AWn, 0.0, nullptr, Wn, nullptr, h->pax, h->recompute);
   int nlx = 0;
   if (h->graph) nlx = ax_L(h, Wn, h->buf[B_LX], Wn, nullptr, h->pax3, h->run);
-  gram1(h, Wn, Wn, 0, 1, h->ctl, h->G64fix, h->GT, 0, 0.0);
+  gram1(h, Wn, Wn, 0, h->ctl, h->G64fix, h->GT, 0, 0.0);
   {
     RowArgs a = row_base(h);
     a.X = Wn; a.B = AWn; a.LX = h->graph ? h->buf[B_LX] : nullptr;
@@ -776,22 +809,10 @@ void dir_final(snmf_ctx* h, const Params& P) {
   launch_ctl_final_dir(h->ctl, h->G64fix, h->b, h->r, P, h->s);
 }
 
-// Row kernels through the shared-memory tile body: r <= 32, penalty form, at most two step
-// candidates, no graph term, and enough row tiles to fill the GPU (a tile holds 128 FP32 /
-// 64 FP64 rows; small problems keep the general kernel's finer grid).
-int tile_rule(const snmf_ctx* h) {
-  const int64_t tr = h->tdtype == 0 ? 64 : 128;
-  const int64_t tiles = (h->n + tr - 1) / tr * h->b;
-  return (h->r <= 32 && h->opt.formulation != SNMF_DIRECT && h->opt.step_controller != 2 && !h->graph &&
-          tiles >= 2 * 152) ? 1 : 0;
-}
-
-// D step and update through rowfuse.cu: FP32 factors, r in {16, 32, 64}, penalty form, the
-// plain step or a learned step (with or without the fallback direction; not record mode), no
-// graph term.
-int fuse_rule(const snmf_ctx* h) {
-  return (rowfuse_supported(h->tdtype, h->r) && h->opt.formulation != SNMF_DIRECT &&
-          h->opt.step_controller != 2 && !h->graph) ? 1 : 0;
+// Row kernels through rowstep.cu: penalty (or naive) form, r <= 64, with or without a graph term;
+// record mode's nine candidates, the direct form and larger ranks keep the general kernel.
+int row_rule(const snmf_ctx* h) {
+  return h->r <= 64 && h->opt.formulation != SNMF_DIRECT && h->opt.step_controller != 2;
 }
 
 snmf_status alloc_buffers(snmf_ctx* h) {
@@ -806,21 +827,22 @@ snmf_status alloc_buffers(snmf_ctx* h) {
   const Dims d = dims(h);
   h->nrow = rowgemm_slots(d, h->tdtype);
   h->nax = (int)((h->n + kRowTile - 1) / kRowTile);
-  // room for every row-kernel layout (BM = 32 has the most slots; the tile body fewer)
-  const int nrow_max = std::max(h->nrow, rowgemm_slots(d, h->tdtype, 0, 32));
+  // room for every row-kernel layout
+  h->use_row = row_rule(h);
+  h->rplan = rowstep_plan(h->tdtype, h->n, std::min(h->r, 64), h->b);
+  const int nrow_max = std::max({h->nrow, rowgemm_slots(d, h->tdtype, 32), h->rplan.slots + h->rplan.groups});
   const size_t prec_n = (size_t)std::max(nrow_max, h->nax) * h->b * kNQ;
-  // the shared-memory tile body where tile_rule allows it
-  h->use_tile = tile_rule(h);
-  if (h->use_tile) h->nrow = rowgemm_slots(d, h->tdtype, 1);
-  h->use_fuse = fuse_rule(h);
+  if (h->use_row) h->nrow = h->rplan.slots;
   double** parts[] = {&h->prow, &h->pax, &h->pax2, &h->pax3, &h->pax4, &h->pclip};
   for (double** p : parts) {
     CK(cudaMalloc(p, prec_n * sizeof(double)));
     CK(cudaMemsetAsync(*p, 0, prec_n * sizeof(double), h->s));
   }
-  h->nchunks = choose_chunks(h->n, h->b, h->r);
+  h->gplan = gram_plan(h->n, h->r, h->b);
   const size_t rr = (size_t)h->r * h->r * h->b;
-  CK(cudaMalloc(&h->gpart, (size_t)h->nchunks * 3 * rr * sizeof(double)));
+  CK(cudaMalloc(&h->gpart, h->gplan.part_elems * h->esz));
+  CK(cudaMalloc(&h->gcounters, h->gplan.counters * sizeof(unsigned)));
+  CK(cudaMemsetAsync(h->gcounters, 0, h->gplan.counters * sizeof(unsigned), h->s));
   CK(cudaMalloc(&h->G64fix, rr * sizeof(double)));
   CK(cudaMalloc(&h->G64p, 3 * rr * sizeof(double)));
   CK(cudaMalloc(&h->GT, rr * h->esz));
@@ -839,8 +861,9 @@ snmf_status alloc_buffers(snmf_ctx* h) {
     CK(cudaMemsetAsync(h->tcount, 0, nt * sizeof(unsigned), h->s));
   }
   if (h->opt.timeout_cycles > 0) h->budget = h->opt.timeout_cycles;
-  CK(cudaMalloc(&h->counters, (16384 + 4096) * sizeof(unsigned)));  // Gram tiles, then restarts
-  CK(cudaMemsetAsync(h->counters, 0, (16384 + 4096) * sizeof(unsigned), h->s));
+  const size_t ncount = (size_t)h->b * (1 + h->rplan.groups);
+  CK(cudaMalloc(&h->counters, ncount * sizeof(unsigned)));
+  CK(cudaMemsetAsync(h->counters, 0, ncount * sizeof(unsigned), h->s));
   CK(cudaMalloc(&h->dsc, 4096 * sizeof(double)));
   CK(cudaMalloc(&h->ring, (size_t)h->b * h->ring_cap * kRingVals * sizeof(double)));
   CK(cudaMemsetAsync(h->ring, 0, (size_t)h->b * h->ring_cap * kRingVals * sizeof(double), h->s));
@@ -1198,9 +1221,6 @@ snmf_status snmf_set_graph_reg(snmf_handle h, const snmf_matrix* L, double gamma
     h->graph = false;
     h->gamma = 0.0;
     h->exec_form = -1;
-    h->use_tile = tile_rule(h);
-    h->use_fuse = fuse_rule(h);
-    h->nrow = rowgemm_slots(dims(h), h->tdtype, h->use_tile, h->row_bm);
     return SNMF_OK;
   }
   if (!L) {
@@ -1276,9 +1296,6 @@ snmf_status snmf_set_graph_reg(snmf_handle h, const snmf_matrix* L, double gamma
   h->graph = true;
   h->gamma = gamma;
   h->exec_form = -1;
-  h->use_tile = 0;  // the graph term runs through the general row kernel
-  h->use_fuse = 0;
-  h->nrow = rowgemm_slots(dims(h), h->tdtype, 0, h->row_bm);
   // ||L||_2 by power_iters power iterations from s_i = 1 + (i mod 2) (L 1 = 0 for a
   // Laplacian, so the start must not be constant) and the Rayleigh quotient; the device
   // applies L (CSR product), the host normalises in FP64.
@@ -1673,16 +1690,13 @@ snmf_status snmf_step_config(snmf_handle h, int32_t* body, int32_t* rows_per_cta
   const int nc = h->opt.step_controller == 1 ? 2 : (h->opt.step_controller == 2 ? kNCand : 1);
   int kind = 0, rows = 0;
   int64_t bd = 0, bu = 0;
-  if (h->use_fuse) {
+  if (h->use_row && !h->graph) {
     kind = h->row_tc == 2 ? 4 : (h->row_tc ? 3 : 2);
-    rows = h->row_tc ? 128 : rowfuse_bm(h->r, h->row_bm);
+    rows = h->row_tc ? 128 : h->rplan.rows;
     bd = 4 * fb;  // X, g, B in; g(Z) out
     bu = 6 * fb;  // X, g, g(Z), B in; X', g(X') out
   } else {
-    kind = h->use_tile ? 1 : 0;
-    const Dims d = dims(h);
-    rows = h->use_tile ? (int)((h->n + rowgemm_slots(d, h->tdtype, 1) - 1) / rowgemm_slots(d, h->tdtype, 1))
-                       : (int)((h->n + h->nrow / ((h->r + 63) / 64) - 1) / (h->nrow / ((h->r + 63) / 64)));
+    rows = (int)((h->n + h->nrow / ((h->r + 63) / 64) - 1) / (h->nrow / ((h->r + 63) / 64)));
     bd = (6 + (nc == 2 ? 1 : 0)) * fb;  // X, g, B in; Z, g(Z), D (+ the second direction) out
     bu = 8 * fb;                        // Z, D, B, X, g, g(Z) in; X', g(X') out
   }
@@ -1829,9 +1843,11 @@ snmf_status snmf_destroy(snmf_handle h) {
   if (h->evdone) cudaEventDestroy(h->evdone);
   for (void* p : h->buf) cudaFree(p);
   cudaFree(h->ws);
-  double* parts[] = {h->prow, h->pax, h->pax2, h->pax3, h->pax4, h->pclip, h->gpart, h->G64fix,
+  double* parts[] = {h->prow, h->pax, h->pax2, h->pax3, h->pax4, h->pclip, h->G64fix,
                      h->G64p, h->dsc, h->ring};
   for (double* p : parts) cudaFree(p);
+  cudaFree(h->gpart);
+  cudaFree(h->gcounters);
   cudaFree(h->GT);
   cudaFree(h->ctl);
   cudaFree(h->run);

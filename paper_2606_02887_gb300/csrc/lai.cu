@@ -436,7 +436,8 @@ int lai_build(LaiOp& op, const AxArgs& A, int td, int64_t n, int k, int ell, int
   const size_t esz = td == 0 ? 8 : 4;
   const size_t blk = (size_t)n * ell;
   void *Y = nullptr, *Q = nullptr, *ws = nullptr, *xh = nullptr, *xl = nullptr, *RinvT = nullptr, *Pk = nullptr;
-  double *G = nullptr, *Rinv = nullptr, *V = nullptr, *gpart = nullptr, *part = nullptr, *sums = nullptr;
+  double *G = nullptr, *Rinv = nullptr, *V = nullptr, *part = nullptr, *sums = nullptr;
+  void* gpart = nullptr;
   unsigned* counters = nullptr;
   int *fail = nullptr, *err = nullptr;
   int rc = 0;
@@ -458,17 +459,17 @@ int lai_build(LaiOp& op, const AxArgs& A, int td, int64_t n, int k, int ell, int
     LCK(cudaMalloc(&xh, (size_t)ell * tc_ld(n) * 2));
     LCK(cudaMalloc(&xl, (size_t)ell * tc_ld(n) * 2));
   }
-  const int nch = (int)std::max<int64_t>(1, std::min<int64_t>(152 / ((ell + 63) / 64 * ((ell + 63) / 64)), n / 512));
+  const GramPlan gp = gram_plan_sketch(n, ell);
   LCK(cudaMalloc(&G, (size_t)ell * ell * sizeof(double)));
   LCK(cudaMalloc(&Rinv, (size_t)ell * ell * sizeof(double)));
   LCK(cudaMalloc(&V, (size_t)ell * ell * sizeof(double)));
   LCK(cudaMalloc(&RinvT, (size_t)ell * ell * esz));
   LCK(cudaMalloc(&Pk, (size_t)ell * k * esz));
-  LCK(cudaMalloc(&gpart, (size_t)nch * ell * ell * sizeof(double)));
+  LCK(cudaMalloc(&gpart, gp.part_elems * esz));
   LCK(cudaMalloc(&part, (size_t)1024 * sizeof(double)));
   LCK(cudaMalloc(&sums, 4 * sizeof(double)));
-  LCK(cudaMalloc(&counters, 64 * sizeof(unsigned)));
-  LCK(cudaMemsetAsync(counters, 0, 64 * sizeof(unsigned), s));
+  LCK(cudaMalloc(&counters, gp.counters * sizeof(unsigned)));
+  LCK(cudaMemsetAsync(counters, 0, gp.counters * sizeof(unsigned), s));
   LCK(cudaMalloc(&fail, sizeof(int)));
   LCK(cudaMemsetAsync(fail, 0, sizeof(int), s));
   LCK(cudaMalloc(&err, sizeof(int)));
@@ -488,7 +489,7 @@ int lai_build(LaiOp& op, const AxArgs& A, int td, int64_t n, int k, int ell, int
   auto cholqr = [&](void* Yb, void* Qb) -> int {
     for (int pass = 0; pass < 2; ++pass) {
       const void* src = pass == 0 ? Yb : Qb;
-      launch_gram(td, src, src, dl, 0, 1, gpart, nch, nullptr, nullptr, G, nullptr, -1, 0.0, counters, s);
+      launch_gram(td, src, src, dl, gp, 0, gpart, nullptr, nullptr, G, nullptr, -1, 0.0, counters, s);
       if (td == 0)
         k_chol<double><<<1, 256, 0, s>>>(G, ell, pass == 0 ? 1e-14 : 0.0, Rinv, (double*)RinvT, fail);
       else
@@ -510,7 +511,7 @@ int lai_build(LaiOp& op, const AxArgs& A, int td, int64_t n, int k, int ell, int
   }
   // T = Q^T (A Q), symmetrised; eigendecomposition; U = Q P_k
   if ((rc = product(Q, Y))) { cleanup(); return rc; }
-  launch_gram(td, Q, Y, dl, 0, 1, gpart, nch, nullptr, nullptr, G, nullptr, -1, 0.0, counters, s);
+  launch_gram(td, Q, Y, dl, gp, 0, gpart, nullptr, nullptr, G, nullptr, -1, 0.0, counters, s);
   k_sym<double><<<1, 256, 0, s>>>(G, ell);
   const int h = (ell + 1) / 2;
   k_jacobi<<<1, 256, 4 * h * sizeof(double), s>>>(G, V, ell, 40, 1e-13);

@@ -1,8 +1,5 @@
 // O(n r^2) kernels of an SNMPBB step and the per-restart FP64 control logic.
 //
-//   k_gram       r x r Gram X_j^T Y_j of each restart j (Eq. (2.1): H H^T, and the
-//                Z^T D, D^T D products of the line-search polynomial); FP64 partials per
-//                row chunk, reduced in a fixed order by the last CTA of each tile.
 //   k_rowgemm    X G - B (+ gamma L X): the gradients of Eqs. (2.1)-(2.2) with the
 //                r x r factor G in shared memory, fused with the elementwise steps of
 //                Algorithm 1 (Z step, D direction, relaxed update) and the FP64
@@ -20,40 +17,9 @@ namespace snmf {
 
 namespace {
 
-template <typename T, int TW, int RS>
-__global__ void __launch_bounds__(256)
-k_gram(const T* __restrict__ X, const T* __restrict__ Y, int64_t n, int r, int b, int64_t ld,
-       int64_t chunk, int ntile, double* __restrict__ gpart, int pair, int npairs,
-       const Ctl* __restrict__ ctl, const int* run, double* __restrict__ G64, T* __restrict__ GT,
-       int tpair, double lam_shift, unsigned* __restrict__ counters, Ctl* __restrict__ rho_ctl,
-       int rho_iters, double rho_scale, double rho_shift) {
-  gram_body<T, TW, RS>(X, Y, n, r, b, ld, chunk, ntile, gpart, pair, npairs, ctl, run, G64, GT, tpair,
-                       lam_shift, counters, rho_ctl, rho_iters, rho_scale, rho_shift, blockIdx.x, gridDim.x,
-                       blockIdx.y);
-}
-
 template <typename T, int OP, int EPI, int BM, int NC>
 __global__ void __launch_bounds__(256, BM == 32 ? 4 : 3) k_rowgemm(RowArgs a) {
   rowgemm_body<T, OP, EPI, BM, NC>(a, blockIdx.z, blockIdx.x, blockIdx.y, gridDim.y, gridDim.x * gridDim.y);
-}
-
-// r <= 32: the shared-memory tile body, CTA = TileCfg<T>::TR rows of restart blockIdx.z
-template <typename T, int OP, int EPI, int NC>
-__global__ void __launch_bounds__(256, EPI == EPI_GRAD ? 2 : 3) k_rowtile(RowArgs a) {
-  extern __shared__ __align__(16) unsigned char tsm[];
-  rowtile_body<T, OP, EPI, NC>(a, blockIdx.z, blockIdx.x, gridDim.x, reinterpret_cast<T*>(tsm));
-}
-
-template <typename T, int OP, int EPI, int NC>
-void launch_rowtile(const RowArgs& a, cudaStream_t s) {
-  static bool attr = false;
-  const size_t smem = rowtile_smem<T>(EPI == EPI_DIR ? 2 + NC : 2);
-  if (!attr) {
-    cudaFuncSetAttribute(k_rowtile<T, OP, EPI, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr = true;
-  }
-  dim3 grid((unsigned)((a.n + TileCfg<T>::TR - 1) / TileCfg<T>::TR), 1, a.b);
-  k_rowtile<T, OP, EPI, NC><<<grid, 256, smem, s>>>(a);
 }
 
 // Elementwise: Z = Proj[X - g / rho] (Alg. 1 line 2) for restarts that are live.
@@ -117,38 +83,26 @@ __global__ void k_copy_live(int64_t n, int r, int b, int64_t ld, const T* __rest
 }  // namespace
 
 // ---------------------------------------------------------------------------
-// rho = ||G||_2 by the power method from the ones vector (fixed count) and the
-// Rayleigh quotient; rho_scale multiplies the result (direct form).  PT is the
-// arithmetic type (double in FP64 precision, float otherwise).
-// ---------------------------------------------------------------------------
-template <typename PT>
-__global__ void k_rho(const double* __restrict__ G64, int r, int iters, double rho_scale, double rho_shift,
-                      Ctl* __restrict__ ctl, int set_alpha) {
-  extern __shared__ unsigned char smem_raw[];
-  __shared__ double sh[32];
-  __shared__ PT v[kMaxR], w[kMaxR];
-  const int j = blockIdx.x;
-  Ctl& c = ctl[j];
-  if (!c.active) return;
-  PT* Gs = ((size_t)r * r * sizeof(PT) <= 96 * 1024) ? reinterpret_cast<PT*>(smem_raw) : nullptr;
-  rho_body<PT>(G64 + (int64_t)j * r * r, r, iters, rho_scale, rho_shift, c, v, w, Gs, sh);
-  (void)set_alpha;
-}
-
-// ---------------------------------------------------------------------------
 // Penalty form control (Sec. 2.1) as a separate launch: the line search.  The block start and
 // the update run fused into the producing row kernels (fused_control).
 // prow: row-kernel partials (q layout of EPI_GRAD / EPI_DIR), nrow slots.
 // ---------------------------------------------------------------------------
-// After DIR (q: 0 gd, 1 dd, 2 f(Z)-f(X_k)) and the Gram of D (pair `dpair`):
-// line search on f(Z + beta D) - f(Z) = beta gd + beta^2/2 q with
-// q = <D^T D, H H^T> + lambda ||D||^2 + gamma <D, L D>.
-__global__ void k_ctl_pen_ls(Ctl* __restrict__ ctl, const double* __restrict__ prow, int nrow,
+// After DIR (q: 0 gd, 1 dd, 2 f(Z)-f(X_k), 4 <D G, D> without DtD): line search on
+// f(Z + beta D) - f(Z) = beta gd + beta^2/2 q with q = <D^T D, H H^T> + lambda ||D||^2 (from the
+// Gram DtD of D, or the row products) + gamma <D, L D>.
+__global__ void __launch_bounds__(256) k_ctl_pen_ls(Ctl* __restrict__ ctl, const double* __restrict__ prow, int nrow,
                              const double* __restrict__ pax, int nax, int b, int r,
                              const double* __restrict__ G64fix, const double* __restrict__ DtD,
                              Params P, int graph) {
-  __shared__ double sh[32];
-  pen_ls_body(ctl[blockIdx.x], prow, nrow, pax, nax, b, r, blockIdx.x, G64fix, DtD, P, graph, sh);
+  __shared__ double sh[32], rec[8][8], qs[8];
+  const int j = blockIdx.x;
+  Ctl& c = ctl[j];
+  if (!c.active) return;
+  slot_sums<8>(prow, nrow, b, j, rec, qs);
+  double q = qs[4];
+  if (DtD) q = dot_rr(DtD + (int64_t)j * r * r, G64fix + (int64_t)j * r * r, r, sh) + c.lam * qs[1];
+  if (graph) q += P.gamma * reduce_slots(pax, nax, b, j, 0, sh);
+  if (threadIdx.x == 0) pen_ls_body(c, qs, q, P);
 }
 
 // ---------------------------------------------------------------------------
@@ -160,7 +114,7 @@ __device__ double direct_f(double normA2, double xax, double gg, double gam, dou
 }
 
 // init: pax q0 = <W, AW>; prow (EPI_GRAD) q0 = pg2; GW = W^T W; graph: plx q0 = <W,LW>
-__global__ void k_ctl_dir_init(Ctl* __restrict__ ctl, const double* __restrict__ pax, int nax,
+__global__ void __launch_bounds__(256) k_ctl_dir_init(Ctl* __restrict__ ctl, const double* __restrict__ pax, int nax,
                                const double* __restrict__ prow, int nrow,
                                const double* __restrict__ plx, int nlx, const double* __restrict__ GW,
                                int b, int r, Params P) {
@@ -199,7 +153,7 @@ __global__ void k_ctl_dir_alpha(Ctl* __restrict__ ctl, Params P) {
 // Quartic line search.  pz: q0 <Z,AZ>; prow (EPI_DIR): q0 gd, q1 dd; pd: q0 <Z,AD>, q1 <D,AD>;
 // Grams: P0 = Z^T Z (GZ), M = Z^T D (ZD), P2 = D^T D (DD).  Graph: pgl q0 <Z,LZ>, q1 <D,LZ>
 // (from the LZ finish) and pgd q0 <D,LD>.
-__global__ void k_ctl_dir_ls(Ctl* __restrict__ ctl, const double* __restrict__ pz, int nz,
+__global__ void __launch_bounds__(256) k_ctl_dir_ls(Ctl* __restrict__ ctl, const double* __restrict__ pz, int nz,
                              const double* __restrict__ prow, int nrow,
                              const double* __restrict__ pd, int nd, const double* __restrict__ GZ,
                              const double* __restrict__ ZD, const double* __restrict__ DDm,
@@ -254,7 +208,7 @@ __global__ void k_ctl_dir_ls(Ctl* __restrict__ ctl, const double* __restrict__ p
 }
 
 // clip counts from k_xupd (q0); sets *recompute when any live restart clipped
-__global__ void k_ctl_dir_clip(Ctl* __restrict__ ctl, const double* __restrict__ pclip, int nslots,
+__global__ void __launch_bounds__(256) k_ctl_dir_clip(Ctl* __restrict__ ctl, const double* __restrict__ pclip, int nslots,
                                int b, int* __restrict__ recompute) {
   __shared__ double sh[32];
   const int j = blockIdx.x;
@@ -268,7 +222,7 @@ __global__ void k_ctl_dir_clip(Ctl* __restrict__ ctl, const double* __restrict__
 
 // after the gradient at W' (prow EPI_GRAD: q0 pg2, q2 ss, q3 sy, q4 yy), Gram GW of W',
 // optional recomputed <W', AW'> (pax q0), graph <W', LW'> (plx q0).
-__global__ void k_ctl_dir_upd(Ctl* __restrict__ ctl, const double* __restrict__ prow, int nrow,
+__global__ void __launch_bounds__(256) k_ctl_dir_upd(Ctl* __restrict__ ctl, const double* __restrict__ prow, int nrow,
                               const double* __restrict__ pax, int nax,
                               const double* __restrict__ plx, int nlx,
                               const double* __restrict__ GW, const int* __restrict__ recompute,
@@ -411,7 +365,7 @@ __global__ void k_convert(const TS* __restrict__ src, int64_t rows, int64_t cols
 
 // final per-restart stats (penalty): pax q0 = <W, A Ht>; GW = W^T W, GH = Ht^T Ht,
 // WH = W^T Ht; prow q0 = pg2 of the W gradient at the final point.
-__global__ void k_ctl_final_pen(Ctl* __restrict__ ctl, const double* __restrict__ pax, int nax,
+__global__ void __launch_bounds__(256) k_ctl_final_pen(Ctl* __restrict__ ctl, const double* __restrict__ pax, int nax,
                                 const double* __restrict__ prow, int nrow,
                                 const double* __restrict__ GW, const double* __restrict__ GH,
                                 const double* __restrict__ WH, int b, int r, Params P) {
@@ -436,7 +390,7 @@ __global__ void k_ctl_final_pen(Ctl* __restrict__ ctl, const double* __restrict_
 }
 
 // final per-restart stats (direct)
-__global__ void k_ctl_final_dir(Ctl* __restrict__ ctl, const double* __restrict__ GW, int b, int r,
+__global__ void __launch_bounds__(256) k_ctl_final_dir(Ctl* __restrict__ ctl, const double* __restrict__ GW, int b, int r,
                                 Params P) {
   __shared__ double sh[32];
   const int j = blockIdx.x;
@@ -453,54 +407,20 @@ __global__ void k_ctl_final_dir(Ctl* __restrict__ ctl, const double* __restrict_
 // ---------------------------------------------------------------------------
 // host launchers
 // ---------------------------------------------------------------------------
-void launch_gram(int tdtype, const void* X, const void* Y, const Dims& d, int pair, int npairs,
-                 double* gpart, int nchunks, const Ctl* ctl, const int* run, double* G64, void* GT,
-                 int tpair, double lam_shift, unsigned* counters, cudaStream_t s, Ctl* rho_ctl,
-                 int rho_iters, double rho_scale, double rho_shift) {
-  // r <= 32: one 32 x 32 tile per restart (a 64-wide tile would compute 4x the entries)
-  const bool narrow = d.r <= 32;
-  const int ntile = narrow ? 1 : (d.r + 63) / 64;
-  const int64_t chunk = (d.n + nchunks - 1) / nchunks;
-  dim3 grid(nchunks, d.b * ntile * ntile);
-#define GRAM_ARGS(T) (const T*)X, (const T*)Y, d.n, d.r, d.b, d.ld, chunk, ntile, gpart, pair, npairs, ctl, run, \
-                     G64, (T*)GT, tpair, lam_shift, counters
-  if (tdtype == 0) {
-    if (narrow) k_gram<double, 32, 32><<<grid, 256, 0, s>>>(GRAM_ARGS(double), nullptr, 0, 1.0, 0.0);
-    else k_gram<double, 64, 32><<<grid, 256, 0, s>>>(GRAM_ARGS(double), nullptr, 0, 1.0, 0.0);
-  } else {
-    if (narrow)
-      k_gram<float, 32, 64><<<grid, 256, 0, s>>>(GRAM_ARGS(float), rho_ctl, rho_iters, rho_scale, rho_shift);
-    else
-      k_gram<float, 64, 32><<<grid, 256, 0, s>>>(GRAM_ARGS(float), rho_ctl, rho_iters, rho_scale, rho_shift);
-  }
-#undef GRAM_ARGS
-}
-
+// ---------------------------------------------------------------------------
+// host launchers
+// ---------------------------------------------------------------------------
 static int rowgemm_bm(const Dims& d, int tdtype) {
   if (tdtype == 0) return 32;  // FP64: keeps the operand/D tile and the G tile within 48 KB
   return (d.n + 63) / 64 * ((d.r + 63) / 64) * d.b >= 2 * 152 ? 64 : 32;
 }
 
-int rowgemm_slots(const Dims& d, int tdtype, int tile, int bm_req) {
-  if (tile) return cdiv(d.n, tdtype == 0 ? TileCfg<double>::TR : TileCfg<float>::TR);
+int rowgemm_slots(const Dims& d, int tdtype, int bm_req) {
   const int bm = (tdtype == 1 && (bm_req == 32 || bm_req == 64)) ? bm_req : rowgemm_bm(d, tdtype);
   return cdiv(d.n, bm) * cdiv(d.r, 64);
 }
 
 void launch_rowgemm(int tdtype, int op, int epi, const RowArgs& a, cudaStream_t s, int ncand) {
-  if (a.tile && a.r <= 32 && !a.LX && ncand <= 2) {
-#define TB(T)                                                                   \
-    if (epi == EPI_GRAD) {                                                      \
-      if (op == OP_LOAD) launch_rowtile<T, OP_LOAD, EPI_GRAD, 1>(a, s);         \
-      else if (op == OP_ZSTEP) launch_rowtile<T, OP_ZSTEP, EPI_GRAD, 1>(a, s);  \
-      else launch_rowtile<T, OP_UPD, EPI_GRAD, 1>(a, s);                        \
-    } else if (op == OP_LOAD) launch_rowtile<T, OP_LOAD, EPI_DIR, 1>(a, s);     \
-    else if (ncand == 1) launch_rowtile<T, OP_ZSTEP, EPI_DIR, 1>(a, s);         \
-    else launch_rowtile<T, OP_ZSTEP, EPI_DIR, 2>(a, s);
-    if (tdtype == 0) { TB(double) } else { TB(float) }
-#undef TB
-    return;
-  }
   Dims d;
   d.n = a.n; d.r = a.r; d.b = a.b; d.N = a.r * a.b; d.ld = a.ld;
   const int bm = (tdtype == 1 && (a.bm == 32 || a.bm == 64)) ? a.bm : rowgemm_bm(d, tdtype);
@@ -511,13 +431,10 @@ void launch_rowgemm(int tdtype, int op, int epi, const RowArgs& a, cudaStream_t 
 #define RG_T(T)                                                             \
   if (epi == EPI_GRAD) {                                                    \
     if (op == OP_LOAD) { RG_M(T, OP_LOAD, EPI_GRAD, 1) }                    \
-    else if (op == OP_ZSTEP) { RG_M(T, OP_ZSTEP, EPI_GRAD, 1) }             \
     else { RG_M(T, OP_UPD, EPI_GRAD, 1) }                                   \
   } else if (ncand == 1) {                                                  \
     if (op == OP_LOAD) { RG_M(T, OP_LOAD, EPI_DIR, 1) }                     \
     else { RG_M(T, OP_ZSTEP, EPI_DIR, 1) }                                  \
-  } else if (ncand == 2) {                                                  \
-    RG_M(T, OP_ZSTEP, EPI_DIR, 2)                                           \
   } else {                                                                  \
     RG_M(T, OP_ZSTEP, EPI_DIR, kNCand)                                      \
   }
@@ -561,27 +478,6 @@ void launch_copy_live(int tdtype, const Dims& d, const void* src, void* dst, con
     k_copy_live<double><<<blocks, 256, 0, s>>>(d.n, d.r, d.b, d.ld, (const double*)src, (double*)dst, ctl);
   else
     k_copy_live<float><<<blocks, 256, 0, s>>>(d.n, d.r, d.b, d.ld, (const float*)src, (float*)dst, ctl);
-}
-
-void init_kernel_attributes() {
-  static bool done = false;
-  if (done) return;
-  cudaFuncSetAttribute(k_rho<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-  cudaFuncSetAttribute(k_rho<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-  done = true;
-}
-
-void launch_rho(int tdtype, const double* G64, const Dims& d, int iters, double scale, Ctl* ctl,
-                int set_alpha, cudaStream_t s, double shift) {
-  if (tdtype == 0) {
-    size_t sm = (size_t)d.r * d.r * sizeof(double);
-    if (sm > 96 * 1024) sm = 0;
-    k_rho<double><<<d.b, 256, sm, s>>>(G64, d.r, iters, scale, shift, ctl, set_alpha);
-  } else {
-    size_t sm = (size_t)d.r * d.r * sizeof(float);
-    if (sm > 96 * 1024) sm = 0;
-    k_rho<float><<<d.b, 256, sm, s>>>(G64, d.r, iters, scale, shift, ctl, set_alpha);
-  }
 }
 
 void launch_philox_uniform(int tdtype, void* out, int64_t rows, int cols, int64_t ld, uint64_t seed,
@@ -634,12 +530,12 @@ void launch_convert(int sdtype, int ddtype, const void* src, int64_t rows, int64
 void launch_ctl_pen_ls(Ctl* ctl, const double* prow, int nrow, const double* pax, int nax, int b,
                        int r, const double* G64fix, const double* DtD, const Params& P, int graph,
                        cudaStream_t s) {
-  k_ctl_pen_ls<<<b, 32, 0, s>>>(ctl, prow, nrow, pax, nax, b, r, G64fix, DtD, P, graph);
+  k_ctl_pen_ls<<<b, 256, 0, s>>>(ctl, prow, nrow, pax, nax, b, r, G64fix, DtD, P, graph);
 }
 void launch_ctl_dir_init(Ctl* ctl, const double* pax, int nax, const double* prow, int nrow,
                          const double* plx, int nlx, const double* GW, int b, int r, const Params& P,
                          cudaStream_t s) {
-  k_ctl_dir_init<<<b, 32, 0, s>>>(ctl, pax, nax, prow, nrow, plx, nlx, GW, b, r, P);
+  k_ctl_dir_init<<<b, 256, 0, s>>>(ctl, pax, nax, prow, nrow, plx, nlx, GW, b, r, P);
 }
 void launch_ctl_dir_alpha(Ctl* ctl, int b, const Params& P, cudaStream_t s) {
   k_ctl_dir_alpha<<<b, 32, 0, s>>>(ctl, P);
@@ -648,16 +544,16 @@ void launch_ctl_dir_ls(Ctl* ctl, const double* pz, int nz, const double* prow, i
                        const double* pd, int nd, const double* GZ, const double* ZD,
                        const double* DDm, const double* pgl, const double* pgd, int b, int r,
                        const Params& P, cudaStream_t s) {
-  k_ctl_dir_ls<<<b, 32, 0, s>>>(ctl, pz, nz, prow, nrow, pd, nd, GZ, ZD, DDm, pgl, pgd, b, r, P);
+  k_ctl_dir_ls<<<b, 256, 0, s>>>(ctl, pz, nz, prow, nrow, pd, nd, GZ, ZD, DDm, pgl, pgd, b, r, P);
 }
 void launch_ctl_dir_clip(Ctl* ctl, const double* pclip, int nslots, int b, int* recompute,
                          cudaStream_t s) {
-  k_ctl_dir_clip<<<b, 32, 0, s>>>(ctl, pclip, nslots, b, recompute);
+  k_ctl_dir_clip<<<b, 256, 0, s>>>(ctl, pclip, nslots, b, recompute);
 }
 void launch_ctl_dir_upd(Ctl* ctl, const double* prow, int nrow, const double* pax, int nax,
                         const double* plx, int nlx, const double* GW, const int* recompute, int b,
                         int r, const Params& P, cudaStream_t s) {
-  k_ctl_dir_upd<<<b, 32, 0, s>>>(ctl, prow, nrow, pax, nax, plx, nlx, GW, recompute, b, r, P);
+  k_ctl_dir_upd<<<b, 256, 0, s>>>(ctl, prow, nrow, pax, nax, plx, nlx, GW, recompute, b, r, P);
 }
 void launch_any_active(const Ctl* ctl, int b, int* flag, int* recompute, cudaStream_t s) {
   k_any_active<<<1, 32, 0, s>>>(ctl, b, flag, recompute);
@@ -665,10 +561,10 @@ void launch_any_active(const Ctl* ctl, int b, int* flag, int* recompute, cudaStr
 void launch_ctl_final_pen(Ctl* ctl, const double* pax, int nax, const double* prow, int nrow,
                           const double* GW, const double* GH, const double* WH, int b, int r,
                           const Params& P, cudaStream_t s) {
-  k_ctl_final_pen<<<b, 32, 0, s>>>(ctl, pax, nax, prow, nrow, GW, GH, WH, b, r, P);
+  k_ctl_final_pen<<<b, 256, 0, s>>>(ctl, pax, nax, prow, nrow, GW, GH, WH, b, r, P);
 }
 void launch_ctl_final_dir(Ctl* ctl, const double* GW, int b, int r, const Params& P, cudaStream_t s) {
-  k_ctl_final_dir<<<b, 32, 0, s>>>(ctl, GW, b, r, P);
+  k_ctl_final_dir<<<b, 256, 0, s>>>(ctl, GW, b, r, P);
 }
 
 }  // namespace snmf

@@ -42,25 +42,30 @@ struct RowArgs {
   const void* Xold; const void* gold;    // EPI_GRAD: S = X - Xold, Y = g - gold
   const void* Zold; const void* gZold;   // EPI_GRAD: increment f(X) - f(Zold)
   const void* Wcur; const void* gWcur;   // EPI_DIR: increment f(Z) - f(Wcur)
+  void* Znext;         // rowstep gradient: Z = Proj[X - g / rho] of the next step (NULL: none)
   int want_q;          // EPI_DIR, one column tile: also <D G, D> -> q4
   double* part;
   int ctl_mode;        // CTL_*: control step run by the last CTA of each restart
   unsigned* counters;  // per-restart arrival counters (zero between launches)
+  unsigned* gcounters; // rowstep: arrival counters of a restart's groups of CTAs (NULL: no groups)
   const double* G64fix;
   Params P;
-  int tile;            // 1: the shared-memory tile body (r <= 32, no graph term, <= 2 candidates)
   int bm;              // general body, FP32: rows per CTA (32 or 64; 0 = built-in choice)
 };
 
-// Row kernels of a step for FP32 penalty blocks with r in {16, 32, 64} (rowfuse.cu): the D step
-// writes g(Z) only (RowArgs X, g_in, B -> gZout; fused line search, ctl_mode CTL_LS) and the
-// update recomputes Z and D from X, g, g(Z) (RowArgs Xout = X and gout = g, updated in place,
-// gZold, B; ctl_mode CTL_UPD_*).  bm: rows per CTA (64 or 128; r = 16: 128 or 256).  nc = 2:
-// the learned step with fallback (the proposal and the plain BB direction, Ctl::cand_alpha).
-bool rowfuse_supported(int tdtype, int r);
-int rowfuse_bm(int r, int bm_req);
-void launch_rowfuse_dstep(const RowArgs& a, int bm, int nc, cudaStream_t s);
-void launch_rowfuse_update(const RowArgs& a, int bm, int nc, cudaStream_t s);
+// Row kernels of a step of the penalty form for r <= 64 (rowstep_dev.cuh): the block-start (or
+// given-X') gradient, the D step from X and g (nc = 2: the learned step with fallback) or from a
+// given Z (graph term), and the relaxed update that recomputes Z and D.
+struct RowStepPlan {
+  int threads, mr;  // threads per CTA, rows per thread
+  int rows, slots;  // rows per CTA, CTAs (partial slots) per restart
+  int groups;       // groups of CTAs per restart: their records follow the slots (0: none)
+};
+RowStepPlan rowstep_plan(int tdtype, int64_t n, int r, int b);
+void launch_rowstep_grad(int tdtype, const RowArgs& a, const RowStepPlan& pl, cudaStream_t s);
+void launch_rowstep_d(int tdtype, const RowArgs& a, const RowStepPlan& pl, int nc, cudaStream_t s);
+void launch_rowstep_dz(int tdtype, const RowArgs& a, const RowStepPlan& pl, cudaStream_t s);
+void launch_rowstep_update(int tdtype, const RowArgs& a, const RowStepPlan& pl, int nc, cudaStream_t s);
 // The same pair with the row products on the tensor cores (rowtc.cu: tcgen05 kind::tf32 with
 // hi / lo operand parts; FP32 factors, r = 64, one direction per step).  err: device error
 // code, set when a bounded wait for the tensor cores runs out.
@@ -79,12 +84,26 @@ bool rowtma_supported(int tdtype, int r, int nc, int64_t ld);
 bool launch_rowtma_dstep(const RowArgs& a, int* err, cudaStream_t s);
 bool launch_rowtma_update(const RowArgs& a, int* err, cudaStream_t s);
 
-void launch_gram(int tdtype, const void* X, const void* Y, const Dims& d, int pair, int npairs,
-                 double* gpart, int nchunks, const Ctl* ctl, const int* run, double* G64, void* GT,
-                 int tpair, double lam_shift, unsigned* counters, cudaStream_t s,
-                 Ctl* rho_ctl = nullptr, int rho_iters = 0, double rho_scale = 1.0, double rho_shift = 0.0);
-// partial slots per restart written by launch_rowgemm (tile: the tile body's row tiles)
-int rowgemm_slots(const Dims& d, int tdtype, int tile = 0, int bm = 0);
+// How a Gram is split over CTAs: tiles of tw columns, nch chunks of `chunk` rows per tile;
+// part_elems factor-type elements of partials and `counters` zeroed arrival counters.
+struct GramPlan {
+  int tw, ntile, nch, ng;
+  int64_t chunk;
+  size_t part_elems, counters;
+};
+GramPlan gram_plan(int64_t n, int r, int b);
+// The split of the eigen-sketch's Grams (n x ell, one level of at most 152 chunks over the tiles).
+// Which eigenpairs a sketch keeps near its cut, where they are close, depends on the last bits
+// of these sums: their order is part of what a seed reproduces.
+GramPlan gram_plan_sketch(int64_t n, int ell);
+// G64[pair][b][r x r] = X_j^T Y_j per restart, GT the factor-type copy with lam_shift I when pair ==
+// tpair; rho_ctl: also rho = rho_scale ||G||_2 + rho_shift where the Gram is one tile (r <= 64).
+void launch_gram(int tdtype, const void* X, const void* Y, const Dims& d, const GramPlan& pl, int pair, void* gpart,
+                 const Ctl* ctl, const int* run, double* G64, void* GT, int tpair, double lam_shift, unsigned* counters,
+                 cudaStream_t s, Ctl* rho_ctl = nullptr, int rho_iters = 0, double rho_scale = 1.0,
+                 double rho_shift = 0.0);
+// partial slots per restart written by launch_rowgemm
+int rowgemm_slots(const Dims& d, int tdtype, int bm = 0);
 void launch_rowgemm(int tdtype, int op, int epi, const RowArgs& a, cudaStream_t s, int ncand = 1);
 void launch_zstep(int tdtype, const Dims& d, const void* X, const void* g, void* Z, const Ctl* ctl,
                   cudaStream_t s);
@@ -93,8 +112,8 @@ int launch_xupd(int tdtype, const Dims& d, const void* Z, const void* D, void* X
 void launch_copy_live(int tdtype, const Dims& d, const void* src, void* dst, const Ctl* ctl,
                       cudaStream_t s);
 // rho = scale ||G||_2 + shift per restart (shift: gamma ||L||_2 of a graph-regularised block)
-void launch_rho(int tdtype, const double* G64, const Dims& d, int iters, double scale, Ctl* ctl,
-                int set_alpha, cudaStream_t s, double shift = 0.0);
+void launch_rho(int tdtype, const double* G64, const Dims& d, int iters, double scale, Ctl* ctl, cudaStream_t s,
+                double shift = 0.0);
 void launch_philox_uniform(int tdtype, void* out, int64_t rows, int cols, int64_t ld, uint64_t seed,
                            double scale, cudaStream_t s);
 void launch_philox_gaussian(int tdtype, void* out, int64_t rows, int cols, uint64_t seed,

@@ -1,0 +1,85 @@
+// Launchers of the row kernels of rowstep_dev.cuh over the restarts of a handle.
+#include <algorithm>
+#include <mutex>
+
+#include "common.cuh"
+#include "rowops.cuh"
+#include "rowstep_dev.cuh"
+
+namespace snmf {
+
+namespace {
+
+template <typename T, int STEP, int NC, int MR>
+__global__ void __launch_bounds__(256, 2) k_rowstep(RowArgs a, bool vec) {
+  extern __shared__ __align__(16) unsigned char rsm[];
+  rowstep_body<T, STEP, NC, MR>(a, blockIdx.y, blockIdx.x, gridDim.x, vec, reinterpret_cast<T*>(rsm));
+}
+
+template <typename T, int STEP, int NC, int MR>
+void launch_t(const RowArgs& a, const RowStepPlan& pl, cudaStream_t s) {
+  static std::once_flag once;
+  std::call_once(once, [] {  // the most over the ranks: r = 64 with 256 threads
+    cudaFuncSetAttribute(k_rowstep<T, STEP, NC, MR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)rowstep_smem<T>(64, 256, MR) + 32 * 1024);
+  });
+  uintptr_t all = 0;
+  for (const void* p : {a.X, a.g_in, a.B, a.LX, (const void*)a.Xout, (const void*)a.gout, (const void*)a.Dout,
+                        (const void*)a.gZout, a.Xold, a.gold, a.Zold, a.gZold, a.Wcur, a.gWcur, (const void*)a.Znext})
+    all |= (uintptr_t)p;
+  const bool vec = a.r % 4 == 0 && a.ld % 4 == 0 && !(all & 15);
+  dim3 grid((unsigned)pl.slots, (unsigned)a.b);
+  k_rowstep<T, STEP, NC, MR><<<grid, pl.threads, rowstep_smem<T>(a.r, pl.threads, MR), s>>>(a, vec);
+}
+
+}  // namespace
+
+RowStepPlan rowstep_plan(int tdtype, int64_t n, int r, int b) {
+  // 4 (FP64: 2) rows per thread of 128 or (r > 32) 256 threads; one row, and half the threads, while that
+  // still makes no more than two CTAs per SM (n = 1000, r = 20: 84 CTAs of 12 rows; the general
+  // kernel had 32 of 32)
+  const int big = (r + 3) / 4 > 8 ? 256 : 128;
+  RowStepPlan pl{big, tdtype == 0 ? rowstep_mr<double>() : rowstep_mr<float>(), 0, 0, 0};
+  for (const auto& o : {std::pair<int, int>{big / 2, 1}, std::pair<int, int>{big, 1}}) {
+    const int64_t rows = rowstep_rows(r, o.first, o.second);
+    if ((n + rows - 1) / rows * b <= 2 * 152) {
+      pl.threads = o.first;
+      pl.mr = o.second;
+      break;
+    }
+  }
+  pl.rows = rowstep_rows(r, pl.threads, pl.mr);
+  pl.slots = (int)((n + pl.rows - 1) / pl.rows);
+  pl.groups = rowstep_groups(pl.slots);
+  return pl;
+}
+
+#define ROWSTEP(T, STEP, NC)                                    \
+  do {                                                          \
+    if (pl.mr == 1) launch_t<T, STEP, NC, 1>(a, pl, s);         \
+    else launch_t<T, STEP, NC, rowstep_mr<T>()>(a, pl, s);      \
+  } while (0)
+#define ROWSTEP_T(STEP, NC)                                     \
+  do {                                                          \
+    if (tdtype == 0) ROWSTEP(double, STEP, NC);                 \
+    else ROWSTEP(float, STEP, NC);                              \
+  } while (0)
+
+void launch_rowstep_grad(int tdtype, const RowArgs& a, const RowStepPlan& pl, cudaStream_t s) { ROWSTEP_T(RS_GRAD, 1); }
+
+void launch_rowstep_d(int tdtype, const RowArgs& a, const RowStepPlan& pl, int nc, cudaStream_t s) {
+  if (nc == 2) ROWSTEP_T(RS_D, 2);
+  else ROWSTEP_T(RS_D, 1);
+}
+
+void launch_rowstep_dz(int tdtype, const RowArgs& a, const RowStepPlan& pl, cudaStream_t s) { ROWSTEP_T(RS_DZ, 1); }
+
+void launch_rowstep_update(int tdtype, const RowArgs& a, const RowStepPlan& pl, int nc, cudaStream_t s) {
+  if (nc == 2) ROWSTEP_T(RS_U, 2);
+  else ROWSTEP_T(RS_U, 1);
+}
+
+#undef ROWSTEP_T
+#undef ROWSTEP
+
+}  // namespace snmf

@@ -1,5 +1,5 @@
 // Row kernels of an Algorithm-1 step on the tensor cores (tcgen05, kind::tf32), FP32 penalty
-// blocks with r = 64: the same data flow as rowfuse.cu (the D step writes g(Z) only, the update
+// blocks with r = 64: the same data flow as rowstep_dev.cuh (the D step writes g(Z) only, the update
 // recomputes Z and D from X, g, g(Z)), with the two r x r row products Z G and D G (D step) and
 // X' G (update) as UMMA M = 128, N = 64, K = 64 contractions into TMEM.
 //
@@ -224,8 +224,7 @@ __device__ __forceinline__ void block_partials(const RowArgs& a, const float (&d
   __syncthreads();
   if (*ticket == per - 1) {
     if (threadIdx.x == 0) a.counters[j] = 0u;
-    if (threadIdx.x < 32)
-      fused_control(a.ctl_mode, const_cast<Ctl&>(a.ctl[j]), a.part, (int)per, a.b, a.r, j, a.P, a.G64fix, nullptr, 1);
+    control_tail<8>(a, j, 0, (int)per, 1);
   }
 }
 

@@ -569,7 +569,9 @@ __global__ void __launch_bounds__(NTHR, 1) k_rowtma(const __grid_constant__ RowM
     for (int u = 0; u < S.ntodo; ++u) {
       const int jj = S.todo[u];
       if (lane == 0) a.counters[jj] = 0u;  // ready for the next launch
-      fused_control(a.ctl_mode, const_cast<Ctl&>(a.ctl[jj]), a.part, RT, a.b, a.r, jj, a.P, a.G64fix, nullptr, 1);
+      double qs[8];
+      slot_sums_warp(a.part, RT, a.b, jj, qs);
+      fused_control(a.ctl_mode, const_cast<Ctl&>(a.ctl[jj]), qs, jj, a.P, 1);
     }
   }
   // drain after an abort: products committed but not seen complete, loads not consumed
