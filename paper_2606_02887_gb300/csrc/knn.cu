@@ -16,6 +16,7 @@
 #include <climits>
 #include <cmath>
 #include <limits>
+#include <mutex>
 #include <vector>
 
 #include "../../include/snmf.h"
@@ -24,82 +25,204 @@
 namespace snmf {
 namespace {
 
-constexpr int QB = 64;  // queries per CTA (one per thread)
-constexpr int CB = 64;  // candidates staged per round
+constexpr int QB = 64;    // queries per CTA
+constexpr int CB = 128;   // candidates per tile
+constexpr int DT = 32;    // coordinates staged per round
 constexpr int KMAX = 32;
+// the dimensions that the library takes (rows of QB + 64 points in 200 KB)
+constexpr size_t kKnnMaxBytes = 200 * 1024;
 
-// Top-K (K = compile-time bound, k <= K at run time) by squared distance, candidates in
-// increasing index order; a candidate replaces an entry only when strictly closer (or the entry
-// is still empty), so equal distances keep the lower index first and every slot ends up holding
-// a valid index (k < n).  A non-finite distance counts as +inf and raises *bad.
-template <int K>
-__global__ void __launch_bounds__(QB) k_knn(const float* __restrict__ X, int64_t n, int d, int k,
-                                            int32_t* __restrict__ nbr, float* __restrict__ nd2,
-                                            int* __restrict__ bad) {
-  extern __shared__ float ksm[];
-  const int ds = d + 1;  // odd row stride: conflict-free per-thread rows
-  float* Qs = ksm;
-  float* Cs = ksm + QB * ds;
-  const int64_t q = (int64_t)blockIdx.x * QB + threadIdx.x;
-  for (int e = threadIdx.x; e < QB * d; e += QB) {
-    const int r = e / d, t = e % d;
-    const int64_t i = (int64_t)blockIdx.x * QB + r;
-    Qs[r * ds + t] = i < n ? X[i * d + t] : 0.f;
+// A list of the 32 best (distance, index) pairs, sorted, lane t holding rank t: insertion of (v, vi)
+// by one warp.
+__device__ __forceinline__ void knn_insert(float& kd, int32_t& ki, float v, int32_t vi) {
+  const int pos = __popc(__ballot_sync(0xffffffffu, kd < v || (kd == v && ki < vi)));
+  const float ud = __shfl_up_sync(0xffffffffu, kd, 1);
+  const int32_t ui = __shfl_up_sync(0xffffffffu, ki, 1);
+  const int lane = threadIdx.x & 31;
+  if (lane > pos) {
+    kd = ud;
+    ki = ui;
+  } else if (lane == pos) {
+    kd = v;
+    ki = vi;
   }
-  float kd[K];
-  int32_t ki[K];
+}
+
+// The k nearest of the candidates [z per, (z + 1) per) for the 64 queries of CTA (x, z): partial
+// lists at [z][n][k], sorted by distance and then index (empty slots are (inf, INT_MAX)).  Distances of a 128 x 64 tile, 8 candidates x 4 queries per thread, two
+// candidates per instruction: sum over t ascending of (q_t - c_t)^2 with one FMA each, candidates
+// staged negated.  A distance not above the query's k-th so far goes to the query's buffer in shared
+// memory; after the tile its warp (eight queries each) inserts the buffer, in any order with the
+// same result.  A non-finite distance counts as +inf and raises *bad.  Bound by the FP32 pipes (2 n^2 d
+// lane operations): n = 20000, d = 64, k = 10 took 23.1 ms with one thread per query and the list
+// updated for every candidate.
+struct KnnSmem {
+  float q[2][DT][QB];
+  float c[2][DT][CB];
+  float bd[QB][CB + 1];
+  uint8_t bi[QB][CB];
+  float thr[QB];
+  int cnt[QB];
+};
+
+__global__ void __launch_bounds__(256, 2)
+k_knn(const float* __restrict__ X, int64_t n, int d, int k, int64_t per, bool vec, int32_t* __restrict__ nbr,
+      float* __restrict__ nd2, int* __restrict__ bad) {
+  extern __shared__ __align__(16) unsigned char knn_raw[];
+  KnnSmem& S = *reinterpret_cast<KnnSmem*>(knn_raw);
+  const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
+  const int64_t q0 = (int64_t)blockIdx.x * QB;
+  const int64_t cb = (int64_t)blockIdx.y * per, ce = min(n, cb + per);
+  const int lane = t & 31, w8 = (t >> 5) * 8;  // the warp's queries w8 .. w8 + 7
+  float kd[8];
+  int32_t ki[8];
 #pragma unroll
-  for (int t = 0; t < K; ++t) {
-    kd[t] = INFINITY;
-    ki[t] = INT_MAX;
+  for (int u = 0; u < 8; ++u) {
+    kd[u] = INFINITY;
+    ki[u] = INT_MAX;
   }
-  for (int64_t c0 = 0; c0 < n; c0 += CB) {
-    __syncthreads();
-    for (int e = threadIdx.x; e < CB * d; e += QB) {
-      const int r = e / d, t = e % d;
-      const int64_t j = c0 + r;
-      Cs[r * ds + t] = j < n ? X[j * d + t] : 0.f;
+  if (t < QB) {
+    S.thr[t] = INFINITY;
+    S.cnt[t] = 0;
+  }
+  const int nd = (d + DT - 1) / DT;
+  const int rounds = ce > cb ? (int)((ce - cb + CB - 1) / CB) * nd : 0;
+  // staging: thread t loads 8 coordinates of query t % 64 and 16 of candidate t % 128
+  float rq[8], rc[16];
+  auto load = [&](int s) {
+    const int t0 = s % nd * DT;
+    const int64_t qi = q0 + (t & 63), ci = cb + (int64_t)(s / nd) * CB + (t & 127);
+    const int tq = t0 + (t >> 6) * 8, tc = t0 + (t >> 7) * 16;
+    auto get = [&](float* r, int m, int64_t i, bool on, int tt) {
+#pragma unroll
+      for (int u = 0; u < m; u += 4) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float* p = X + i * d + tt + u;
+        if (on && vec) {
+          if (tt + u < d) v = *reinterpret_cast<const float4*>(p);
+        } else if (on) {
+          if (tt + u < d) v.x = p[0];
+          if (tt + u + 1 < d) v.y = p[1];
+          if (tt + u + 2 < d) v.z = p[2];
+          if (tt + u + 3 < d) v.w = p[3];
+        }
+        r[u] = v.x; r[u + 1] = v.y; r[u + 2] = v.z; r[u + 3] = v.w;
+      }
+    };
+    get(rq, 8, qi, qi < n, tq);
+    get(rc, 16, ci, ci < ce, tc);
+  };
+  auto put = [&](int s) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) S.q[s & 1][(t >> 6) * 8 + u][t & 63] = rq[u];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) S.c[s & 1][(t >> 7) * 16 + u][t & 127] = -rc[u];
+  };
+  float2 acc[4][4];  // [query][candidate pair]
+  if (rounds > 0) {
+    load(0);
+    put(0);
+  }
+  __syncthreads();
+  for (int s = 0; s < rounds; ++s) {
+    if (s + 1 < rounds) load(s + 1);
+    const int ch = s % nd;
+    if (ch == 0) {
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[a][c] = make_float2(0.f, 0.f);
     }
-    __syncthreads();
-    if (q < n) {
-      const int cn = (int)(n - c0 < CB ? n - c0 : CB);
-      const float* qr = Qs + threadIdx.x * ds;
-      for (int c = 0; c < cn; ++c) {
-        const int64_t j = c0 + c;
-        if (j == q) continue;
-        const float* cr = Cs + c * ds;
-        float acc = 0.f;
-        for (int t = 0; t < d; ++t) {
-          const float df = qr[t] - cr[t];
-          acc = fmaf(df, df, acc);
-        }
-        float v = acc;
-        if (!isfinite(v)) {
-          v = INFINITY;
-          atomicOr(bad, 1);
-        }
-        int32_t vi = (int32_t)j;
+    const int dt = min(DT, d - ch * DT);
+    const float* qp = &S.q[s & 1][0][4 * tx];
+    const float* cp = &S.c[s & 1][0][4 * ty];
+#pragma unroll 4
+    for (int u = 0; u < dt; ++u) {
+      const float4 q4 = *reinterpret_cast<const float4*>(qp + u * QB);
+      const float4 ca = *reinterpret_cast<const float4*>(cp + u * CB);
+      const float4 cc = *reinterpret_cast<const float4*>(cp + u * CB + 64);
+      const float qs[4] = {q4.x, q4.y, q4.z, q4.w};
+      const float2 c2[4] = {make_float2(ca.x, ca.y), make_float2(ca.z, ca.w), make_float2(cc.x, cc.y),
+                            make_float2(cc.z, cc.w)};
 #pragma unroll
-        for (int t = 0; t < K; ++t) {
-          if (t < k && (v < kd[t] || (v == kd[t] && vi < ki[t]))) {
-            const float tv = kd[t];
-            const int32_t ti = ki[t];
-            kd[t] = v;
-            ki[t] = vi;
-            v = tv;
-            vi = ti;
+      for (int a = 0; a < 4; ++a) {
+        const float2 qq = make_float2(qs[a], qs[a]);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const float2 df = __fadd2_rn(qq, c2[c]);
+          acc[a][c] = __ffma2_rn(df, df, acc[a][c]);
+        }
+      }
+    }
+    if (ch == nd - 1) {
+      const int64_t c0 = cb + (int64_t)(s / nd) * CB;
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        const int ql = 4 * tx + a;
+        const int64_t q = q0 + ql;
+        const float thr = S.thr[ql];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const int cl = (c >> 2) * 64 + 4 * ty + (c & 3);
+          const int64_t j = c0 + cl;
+          float v = c & 1 ? acc[a][c >> 1].y : acc[a][c >> 1].x;
+          if (q >= n || j >= ce || j == q) continue;
+          if (!isfinite(v)) {
+            v = INFINITY;
+            atomicOr(bad, 1);
+          }
+          if (v <= thr) {
+            const int pos = atomicAdd(&S.cnt[ql], 1);  // at most one entry per candidate of the tile
+            S.bd[ql][pos] = v;
+            S.bi[ql][pos] = (uint8_t)cl;
           }
         }
       }
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int m = S.cnt[w8 + u];
+        if (!m) continue;
+        for (int e = 0; e < m; ++e) knn_insert(kd[u], ki[u], S.bd[w8 + u][e], (int32_t)(c0 + S.bi[w8 + u][e]));
+        __syncwarp();
+        if (lane == k - 1) {
+          S.thr[w8 + u] = kd[u];
+          S.cnt[w8 + u] = 0;
+        }
+      }
+    }
+    if (s + 1 < rounds) put(s + 1);  // the other buffer: its readers passed the last barrier
+    __syncthreads();
+  }
+  if (lane < k) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int64_t q = q0 + w8 + u;
+      if (q >= n) continue;
+      const int64_t o = ((int64_t)blockIdx.y * n + q) * k + lane;
+      nbr[o] = ki[u];
+      nd2[o] = kd[u];
     }
   }
-  if (q < n) {
-#pragma unroll
-    for (int t = 0; t < K; ++t)
-      if (t < k) {
-        nbr[q * k + t] = ki[t];
-        nd2[q * k + t] = kd[t];
-      }
+}
+
+// one warp per query: the k best of its `parts` partial lists
+__global__ void __launch_bounds__(256) k_knn_merge(const int32_t* __restrict__ pi, const float* __restrict__ pd, int64_t n,
+                                                   int k, int parts, int32_t* __restrict__ nbr, float* __restrict__ nd2) {
+  const int lane = threadIdx.x & 31;
+  const int64_t q = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (q >= n) return;
+  float kd = INFINITY;
+  int32_t ki = INT_MAX;
+  for (int z = 0; z < parts; ++z) {
+    const int64_t o = ((int64_t)z * n + q) * k + lane;
+    const float v = lane < k ? pd[o] : INFINITY;
+    const int32_t vi = lane < k ? pi[o] : INT_MAX;
+    for (int u = 0; u < k; ++u) knn_insert(kd, ki, __shfl_sync(0xffffffffu, v, u), __shfl_sync(0xffffffffu, vi, u));
+  }
+  if (lane < k) {
+    nbr[q * k + lane] = ki;
+    nd2[q * k + lane] = kd;
   }
 }
 
@@ -149,56 +272,52 @@ __global__ void __launch_bounds__(1024) k_scan(const int32_t* __restrict__ v, in
 
 // both directions of every kNN pair into the rows' slots (order within a row arbitrary)
 __global__ void k_knn_fill(const int32_t* __restrict__ nbr, const float* __restrict__ sval, int64_t n, int k,
-                           const int32_t* __restrict__ off, int32_t* __restrict__ fill, int32_t* __restrict__ ecol,
-                           float* __restrict__ eval) {
+                           const int32_t* __restrict__ off, int32_t* __restrict__ fill, int32_t* __restrict__ erow,
+                           int32_t* __restrict__ ecol, float* __restrict__ eval) {
   const int64_t total = n * k;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     const int32_t i = (int32_t)(e / k), j = nbr[e];
     const float s = sval[e];
     const int32_t a = off[i] + atomicAdd(&fill[i], 1);
+    erow[a] = i;
     ecol[a] = j;
     eval[a] = s;
     const int32_t bslot = off[j] + atomicAdd(&fill[j], 1);
+    erow[bslot] = j;
     ecol[bslot] = i;
     eval[bslot] = s;
   }
 }
 
-// One warp per row.  A row holds each column at most twice (the forward kNN entry and the
-// reverse one).  pass 0: element x represents its column when no other element of the column
-// has a larger value (or the same value at a lower position); flags and counts.  pass 1: the
-// representative's rank among the row's representatives by column is its CSR position.
-__global__ void k_knn_dedupe(const int32_t* __restrict__ off, const int32_t* __restrict__ ecol,
-                             const float* __restrict__ eval, int64_t n, int pass, uint8_t* __restrict__ erep,
-                             int32_t* __restrict__ cntu, const int32_t* __restrict__ rowptr,
+// One thread per entry; a row holds each column at most twice (the forward kNN entry and the reverse
+// one).  pass 0: an entry represents its column when no other entry of the column has a larger
+// value (or the same value at a lower position); flags and counts.  pass 1: the representative's
+// rank among the row's representatives by column is its CSR position.  (A warp per row left the few
+// long rows of a graph's hubs to one warp each: 189 us at n = 20000, k = 10.)
+__global__ void k_knn_dedupe(const int32_t* __restrict__ off, const int32_t* __restrict__ erow,
+                             const int32_t* __restrict__ ecol, const float* __restrict__ eval, int64_t entries, int pass,
+                             uint8_t* __restrict__ erep, int32_t* __restrict__ cntu, const int32_t* __restrict__ rowptr,
                              int32_t* __restrict__ colidx, float* __restrict__ sout) {
-  const int lane = threadIdx.x & 31;
-  const int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (i >= n) return;
-  const int32_t b = off[i], L = off[i + 1] - off[i];
-  int reps = 0;
-  for (int x = lane; x < L; x += 32) {
-    const int32_t cx = ecol[b + x];
-    const float vx = eval[b + x];
-    if (pass == 0) {
-      bool rep = true;
-      for (int y = 0; y < L; ++y) {
-        const int32_t cy = ecol[b + y];
-        const float vy = eval[b + y];
-        if (cy == cx && y != x && (vy > vx || (vy == vx && y < x))) rep = false;
-      }
-      erep[b + x] = rep ? 1 : 0;
-      reps += rep ? 1 : 0;
-    } else if (erep[b + x]) {
-      int rank = 0;
-      for (int y = 0; y < L; ++y) rank += (erep[b + y] && ecol[b + y] < cx) ? 1 : 0;
-      colidx[rowptr[i] + rank] = cx;
-      sout[rowptr[i] + rank] = vx;
-    }
-  }
+  const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (x >= entries) return;
+  const int32_t i = erow[x], cx = ecol[x], b = off[i], e = off[i + 1];
+  const float vx = eval[x];
   if (pass == 0) {
-    for (int o = 16; o > 0; o >>= 1) reps += __shfl_xor_sync(0xffffffffu, reps, o);
-    if (lane == 0) cntu[i] = reps;
+    bool rep = true;
+#pragma unroll 4
+    for (int32_t y = b; y < e; ++y) {
+      const int32_t cy = ecol[y];
+      const float vy = eval[y];
+      if (cy == cx && y != x && (vy > vx || (vy == vx && y < x))) rep = false;
+    }
+    erep[x] = rep ? 1 : 0;
+    if (rep) atomicAdd(&cntu[i], 1);
+  } else if (erep[x]) {
+    int rank = 0;
+#pragma unroll 4
+    for (int32_t y = b; y < e; ++y) rank += (erep[y] && ecol[y] < cx) ? 1 : 0;
+    colidx[rowptr[i] + rank] = cx;
+    sout[rowptr[i] + rank] = vx;
   }
 }
 
@@ -251,11 +370,31 @@ __global__ void k_assign(const T* __restrict__ F, int64_t n, int64_t ld, int64_t
   }
 }
 
-template <int K>
-void launch_knn(const float* X, int64_t n, int d, int k, int32_t* nbr, float* nd2, int* bad, cudaStream_t s) {
-  const size_t smem = (size_t)(QB + CB) * (d + 1) * sizeof(float);
-  cudaFuncSetAttribute(k_knn<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_knn<K><<<(unsigned)((n + QB - 1) / QB), QB, smem, s>>>(X, n, d, k, nbr, nd2, bad);
+// Candidate ranges (partial lists per query): the number that fills whole waves of CTAs (two per
+// SM) best, each further list worth two per cent of merging, none shorter than 512 candidates.
+int knn_parts(int64_t n) {
+  const int64_t qb = (n + QB - 1) / QB, most = std::min<int64_t>(16, std::max<int64_t>(1, n / 512));
+  int parts = 1;
+  double best = 0.0;
+  for (int64_t p = 1; p <= most; ++p) {
+    const int64_t waves = (qb * p + 2 * 152 - 1) / (2 * 152);
+    const double gain = (double)(qb * p) / (double)(waves * 2 * 152) * (1.0 - 0.02 * (double)p);
+    if (gain > best) { best = gain; parts = (int)p; }
+  }
+  return parts;
+}
+
+void launch_knn(const float* X, int64_t n, int d, int k, int parts, int32_t* pi, float* pd, int32_t* nbr, float* nd2,
+                int* bad, cudaStream_t s) {
+  static std::once_flag once;
+  std::call_once(once, [] {
+    cudaFuncSetAttribute(k_knn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(KnnSmem));
+  });
+  const int64_t per = ((n + parts - 1) / parts + CB - 1) / CB * CB;
+  const bool vec = d % 4 == 0 && !((uintptr_t)X & 15);
+  dim3 grid((unsigned)((n + QB - 1) / QB), parts);
+  k_knn<<<grid, 256, sizeof(KnnSmem), s>>>(X, n, d, k, per, vec, parts > 1 ? pi : nbr, parts > 1 ? pd : nd2, bad);
+  if (parts > 1) k_knn_merge<<<(unsigned)((n + 7) / 8), 256, 0, s>>>(pi, pd, n, k, parts, nbr, nd2);
 }
 
 // Best one-to-one matching maximising the matched count: the Hungarian method with potentials
@@ -312,48 +451,51 @@ extern "C" snmf_status snmf_knn_graph(const float* X, int64_t n, int d, int k, i
   if (!X || !rowptr || !colidx || !a_hat || !nnz || n < 2 || d < 1 || d > 1024 || k < 1 || k > KMAX || k >= n ||
       sigma_rank < 1 || sigma_rank > k || 2 * n * (int64_t)k > INT_MAX)
     return SNMF_ERR_ARG;
-  if ((size_t)(QB + CB) * (d + 1) * sizeof(float) > 200 * 1024) return SNMF_ERR_ARG;
+  if ((size_t)(QB + 64) * (d + 1) * sizeof(float) > kKnnMaxBytes) return SNMF_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t nk = n * k;
-  int32_t *nbr = nullptr, *cnt = nullptr, *off = nullptr, *fill = nullptr, *ecol = nullptr, *cntu = nullptr;
-  float *nd2 = nullptr, *sval = nullptr, *eval = nullptr, *sv = nullptr, *dg = nullptr;
-  uint8_t* erep = nullptr;
-  int* bad = nullptr;
-  auto cleanup = [&] {
-    cudaFree(bad);
-    cudaFree(nbr); cudaFree(cnt); cudaFree(off); cudaFree(fill); cudaFree(ecol); cudaFree(cntu); cudaFree(erep);
-    cudaFree(nd2); cudaFree(sval); cudaFree(eval); cudaFree(sv); cudaFree(dg);
+  // the call's workspace in one piece
+  const int parts = knn_parts(n);
+  unsigned char* ws = nullptr;
+  size_t bytes = 0;
+  auto take = [&](size_t b) {
+    const size_t at = bytes;
+    bytes += (b + 255) / 256 * 256;
+    return at;
   };
+  const size_t o_nbr = take(nk * 4), o_nd2 = take(nk * 4), o_sval = take(nk * 4), o_cnt = take(n * 4), o_fill = take(n * 4),
+               o_off = take((n + 1) * 4), o_cntu = take(n * 4), o_erow = take(2 * nk * 4), o_ecol = take(2 * nk * 4), o_eval = take(2 * nk * 4),
+               o_sv = take(s_values ? 0 : 2 * nk * 4), o_dg = take(degree ? 0 : n * 4), o_erep = take(2 * nk),
+               o_bad = take(4), o_pi = take(parts > 1 ? parts * nk * 4 : 0), o_pd = take(parts > 1 ? parts * nk * 4 : 0);
+  auto cleanup = [&] { cudaFree(ws); };
   snmf_status st = SNMF_OK;
 #define KCK(call)                                                                                        \
   do {                                                                                                   \
     const cudaError_t e_ = (call);                                                                       \
     if (e_ != cudaSuccess) { st = e_ == cudaErrorMemoryAllocation ? SNMF_ERR_OOM : SNMF_ERR_CUDA; cleanup(); return st; } \
   } while (0)
-  KCK(cudaMalloc(&nbr, nk * sizeof(int32_t)));
-  KCK(cudaMalloc(&nd2, nk * sizeof(float)));
-  KCK(cudaMalloc(&sval, nk * sizeof(float)));
-  KCK(cudaMalloc(&cnt, n * sizeof(int32_t)));
-  KCK(cudaMalloc(&fill, n * sizeof(int32_t)));
-  KCK(cudaMalloc(&off, (n + 1) * sizeof(int32_t)));
-  KCK(cudaMalloc(&cntu, n * sizeof(int32_t)));
-  KCK(cudaMalloc(&ecol, 2 * nk * sizeof(int32_t)));
-  KCK(cudaMalloc(&eval, 2 * nk * sizeof(float)));
-  KCK(cudaMalloc(&sv, 2 * nk * sizeof(float)));
-  KCK(cudaMalloc(&dg, n * sizeof(float)));
-  KCK(cudaMalloc(&erep, 2 * nk));
-  KCK(cudaMalloc(&bad, sizeof(int)));
+  KCK(cudaMalloc(&ws, bytes));
+  auto i32 = [&](size_t o) { return reinterpret_cast<int32_t*>(ws + o); };
+  auto f32 = [&](size_t o) { return reinterpret_cast<float*>(ws + o); };
+  int32_t *nbr = i32(o_nbr), *cnt = i32(o_cnt), *off = i32(o_off), *fill = i32(o_fill), *erow = i32(o_erow), *ecol = i32(o_ecol),
+          *cntu = i32(o_cntu), *pi = i32(o_pi);
+  float *nd2 = f32(o_nd2), *sval = f32(o_sval), *eval = f32(o_eval), *pd = f32(o_pd);
+  float* sv = s_values ? s_values : f32(o_sv);
+  float* dg = degree ? degree : f32(o_dg);
+  uint8_t* erep = ws + o_erep;
+  int* bad = i32(o_bad);
   KCK(cudaMemsetAsync(bad, 0, sizeof(int), s));
   KCK(cudaMemsetAsync(cnt, 0, n * sizeof(int32_t), s));
+  KCK(cudaMemsetAsync(cntu, 0, n * sizeof(int32_t), s));
   KCK(cudaMemsetAsync(fill, 0, n * sizeof(int32_t), s));
-  if (k <= 16) launch_knn<16>(X, n, d, k, nbr, nd2, bad, s);
-  else launch_knn<32>(X, n, d, k, nbr, nd2, bad, s);
+  launch_knn(X, n, d, k, parts, pi, pd, nbr, nd2, bad, s);
   const int g = (int)std::min<int64_t>((nk + 255) / 256, 152 * 16);
   k_knn_sim<<<g, 256, 0, s>>>(nbr, nd2, n, k, sigma_rank, sval, cnt, bad);
   k_scan<<<1, 1024, 0, s>>>(cnt, n, k, off);  // row slots: k own + in-degree
-  k_knn_fill<<<g, 256, 0, s>>>(nbr, sval, n, k, off, fill, ecol, eval);
+  k_knn_fill<<<g, 256, 0, s>>>(nbr, sval, n, k, off, fill, erow, ecol, eval);
   const int rb = (int)((n + 7) / 8);
-  k_knn_dedupe<<<rb, 256, 0, s>>>(off, ecol, eval, n, 0, erep, cntu, nullptr, nullptr, nullptr);
+  const int eb = (int)((2 * nk + 255) / 256);
+  k_knn_dedupe<<<eb, 256, 0, s>>>(off, erow, ecol, eval, 2 * nk, 0, erep, cntu, nullptr, nullptr, nullptr);
   k_scan<<<1, 1024, 0, s>>>(cntu, n, 0, rowptr);
   int32_t total = 0;
   int hbad = 0;
@@ -363,11 +505,9 @@ extern "C" snmf_status snmf_knn_graph(const float* X, int64_t n, int d, int k, i
   *nnz = total;
   if (hbad) { cleanup(); return SNMF_ERR_NUMERIC; }
   if (total > capacity) { cleanup(); return SNMF_ERR_ARG; }
-  k_knn_dedupe<<<rb, 256, 0, s>>>(off, ecol, eval, n, 1, erep, cntu, rowptr, colidx, sv);
+  k_knn_dedupe<<<eb, 256, 0, s>>>(off, erow, ecol, eval, 2 * nk, 1, erep, cntu, rowptr, colidx, sv);
   k_knn_degree<<<rb, 256, 0, s>>>(rowptr, sv, n, dg);
   k_knn_normalize<<<rb, 256, 0, s>>>(rowptr, colidx, sv, dg, n, a_hat);
-  if (s_values) KCK(cudaMemcpyAsync(s_values, sv, (size_t)total * sizeof(float), cudaMemcpyDeviceToDevice, s));
-  if (degree) KCK(cudaMemcpyAsync(degree, dg, (size_t)n * sizeof(float), cudaMemcpyDeviceToDevice, s));
   KCK(cudaGetLastError());
   KCK(cudaStreamSynchronize(s));
 #undef KCK
