@@ -5,7 +5,7 @@
 //                  BF16 and E4M3 A (gemm_dev.cuh).  Split-K writes each split to its own
 //                  workspace slice; the finish pass sums the slices in a fixed order, so
 //                  results are deterministic.
-//   k_spmm_csr   : one warp per row, lanes across the factor columns (coalesced rows of X).
+//   k_spmm_csr   : lanes across the factor columns (coalesced rows of X), with Y += c X2.
 //   k_ax_finish  : fused epilogue: sum of split slices, Y += c X2, and per-restart FP64
 //                  partials of <P1, A X> and <P2, A X> (e.g. tr(W^T A W)).
 #include <cuda_bf16.h>
@@ -59,44 +59,99 @@ k_gemm_dense(const TA* __restrict__ A, int64_t lda, const typename C::T* __restr
   }
 }
 
-// CSR SpMM: warp per row, lane owns columns lane + 32 m (m < CPL) of a column window.
-template <typename TV, typename T, int CPL>
+// CSR SpMM, Y = A X (+ c X2): LPR lanes per row, V consecutive columns (16 bytes where the columns
+// allow it) per lane; blockIdx.y = window of LPR V columns, the slowest index of the grid, so the
+// windows of X pass through L2 one after the other.  The entries of a row are taken U at a time with
+// the next indices already in flight, and added in their order.  Bound by the gather from L2 (n =
+// 20000, 15 entries per row, 640 columns: 353 us with single columns and one entry at a time, and a
+// finish pass of its own).
+template <typename TV, typename T, int V, int LPR>
 __global__ void __launch_bounds__(256)
 k_spmm_csr(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colidx,
            const TV* __restrict__ vals, const T* __restrict__ X, int64_t ld,
-           T* __restrict__ Y, int64_t n, int cols, const int* run) {
+           T* __restrict__ Y, int64_t n, int cols, T c, const T* __restrict__ X2, const int* run) {
+  struct alignas(V * sizeof(T)) Vec {
+    T v[V];
+  };
+  constexpr int U = V * sizeof(T) == 16 ? 4 : 8;
   if (run && *run == 0) return;
   const int lane = threadIdx.x & 31;
-  const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int c0 = blockIdx.y * (32 * CPL);
-  if (row >= n) return;
-  T acc[CPL];
+  const int64_t row = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * (32 / LPR) + lane / LPR;
+  const int col = (blockIdx.y * LPR + lane % LPR) * V;
+  if (row >= n || col >= cols) return;
+  Vec acc;
 #pragma unroll
-  for (int m = 0; m < CPL; ++m) acc[m] = T(0);
+  for (int k = 0; k < V; ++k) acc.v[k] = T(0);
   const int beg = rowptr[row], end = rowptr[row + 1];
-  for (int e = beg; e < end; ++e) {
-    const int64_t col = colidx[e];
-    const T v = (T)vals[e];
-    const T* xr = X + col * ld;
+  int32_t ci[U];
+  T va[U];
+  auto load = [&](int e) {
 #pragma unroll
-    for (int m = 0; m < CPL; ++m) {
-      int c = c0 + lane + 32 * m;
-      if (c < cols) acc[m] = fma(v, xr[c], acc[m]);
+    for (int u = 0; u < U; ++u) {
+      ci[u] = e + u < end ? __ldg(colidx + e + u) : -1;
+      va[u] = e + u < end ? (T)__ldg(vals + e + u) : T(0);
     }
-  }
+  };
+  load(beg);
+  for (int e = beg; e < end; e += U) {
+    Vec x[U];
+    T w[U];
+    bool on[U];
 #pragma unroll
-  for (int m = 0; m < CPL; ++m) {
-    int c = c0 + lane + 32 * m;
-    if (c < cols) Y[row * ld + c] = acc[m];
+    for (int u = 0; u < U; ++u) {
+      on[u] = ci[u] >= 0;
+      w[u] = va[u];
+      if (on[u]) x[u] = *reinterpret_cast<const Vec*>(X + (int64_t)ci[u] * ld + col);
+    }
+    load(e + U);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (on[u]) {
+#pragma unroll
+        for (int k = 0; k < V; ++k) acc.v[k] = fma(w[u], x[u].v[k], acc.v[k]);
+      }
   }
+  const int64_t idx = row * ld + col;
+  if (X2) {
+    const Vec x2 = *reinterpret_cast<const Vec*>(X2 + idx);
+#pragma unroll
+    for (int k = 0; k < V; ++k) acc.v[k] = acc.v[k] + c * x2.v[k];
+  }
+  *reinterpret_cast<Vec*>(Y + idx) = acc;
 }
 
-// Epilogue over a row tile x one restart.  splits > 1: Y = sum_s ws[s] (fixed order).  V values of
-// a row per access (16 bytes where r and the pitch allow it), four accesses of a thread and up to
-// eight of their slices in flight.  8192 x 64 in FP32, 8 slices: 24 us with single values, one after
-// the other.
+// Y = sum_s ws[s] (splits > 1, in slice order) or Y (+ c X2) over `total` contiguous values, V per
+// thread (16 bytes), eight slices in flight.
 template <typename T, int V>
 __global__ void __launch_bounds__(256)
+k_ax_sum(int64_t total, T* __restrict__ Y, const T* __restrict__ ws, int splits, T c, const T* __restrict__ X2,
+         const int* run) {
+  struct alignas(V * sizeof(T)) Vec {
+    T v[V];
+  };
+  if (run && *run == 0) return;
+  const int64_t idx = ((int64_t)blockIdx.x * 256 + threadIdx.x) * V;
+  if (idx >= total) return;
+  Vec x2, y = *reinterpret_cast<const Vec*>((splits > 1 ? ws : Y) + idx);
+  if (X2) x2 = *reinterpret_cast<const Vec*>(X2 + idx);
+#pragma unroll 8
+  for (int s = 1; s < splits; ++s) {
+    const Vec w = *reinterpret_cast<const Vec*>(ws + s * total + idx);
+#pragma unroll
+    for (int k = 0; k < V; ++k) y.v[k] += w.v[k];
+  }
+  if (X2) {
+#pragma unroll
+    for (int k = 0; k < V; ++k) y.v[k] = y.v[k] + c * x2.v[k];
+  }
+  *reinterpret_cast<Vec*>(Y + idx) = y;
+}
+
+// Epilogue with inner products over a row tile x one restart.  splits > 1: Y = sum_s ws[s] (fixed
+// order).  V values of a row per access (16 bytes where r and the pitch allow it), two accesses of a
+// thread and their slices in flight.
+template <typename T, int V>
+__global__ void __launch_bounds__(128, 8)
 k_ax_finish(int64_t n, int r, int64_t ld, T* __restrict__ Y, const T* __restrict__ ws,
             int splits, double c, const T* __restrict__ X2, const T* __restrict__ P1,
             const T* __restrict__ P2, double* __restrict__ part, int q0, int b,
@@ -104,7 +159,7 @@ k_ax_finish(int64_t n, int r, int64_t ld, T* __restrict__ Y, const T* __restrict
   struct alignas(V * sizeof(T)) Vec {
     T v[V];
   };
-  __shared__ T sh[32];
+  __shared__ T sh[2][4];
   const int j = blockIdx.y;
   const int64_t i0 = (int64_t)blockIdx.x * kRowTile;
   T d1 = T(0), d2 = T(0);  // per-CTA partials in the working type (FP64 across CTAs)
@@ -112,30 +167,20 @@ k_ax_finish(int64_t n, int r, int64_t ld, T* __restrict__ Y, const T* __restrict
     const int rv = r / V, rows = (int)min((int64_t)kRowTile, n - i0);
     const int tile = rows * rv;
     const int64_t slice = n * ld;
-    constexpr int U = 4;
-    for (int e0 = threadIdx.x; e0 < tile; e0 += 256 * U) {
-      Vec y[U], x2[U], p1[U], p2[U];
+    constexpr int U = 2;
+    for (int e0 = threadIdx.x; e0 < tile; e0 += 128 * U) {
+      Vec y[U];
       int64_t idx[U];
       bool ok[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int e = e0 + 256 * u;
+        const int e = e0 + 128 * u;
         ok[u] = e < tile;
         const int i = ok[u] ? e / rv : 0;
         idx[u] = (i0 + i) * ld + (int64_t)j * r + (ok[u] ? e - i * rv : 0) * V;
-        auto get = [&](const T* p) {
-          Vec v;
-          if (p && ok[u]) return *reinterpret_cast<const Vec*>(p + idx[u]);
-#pragma unroll
-          for (int k = 0; k < V; ++k) v.v[k] = T(0);
-          return v;
-        };
-        y[u] = get(splits > 1 ? ws : Y);
-        x2[u] = get(X2);
-        p1[u] = get(P1);
-        p2[u] = get(P2);
+        if (ok[u]) y[u] = *reinterpret_cast<const Vec*>((splits > 1 ? ws : Y) + idx[u]);
       }
-#pragma unroll 2
+#pragma unroll 4
       for (int s = 1; s < splits; ++s) {
         Vec w[U];
 #pragma unroll
@@ -151,28 +196,39 @@ k_ax_finish(int64_t n, int r, int64_t ld, T* __restrict__ Y, const T* __restrict
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         if (!ok[u]) continue;
+        auto dots = [&] {
+          if (P1) {
+            const Vec p = *reinterpret_cast<const Vec*>(P1 + idx[u]);
 #pragma unroll
-        for (int k = 0; k < V; ++k) {
-          if (!dots_after) {
-            d1 += p1[u].v[k] * y[u].v[k];
-            d2 += p2[u].v[k] * y[u].v[k];
+            for (int k = 0; k < V; ++k) d1 += p.v[k] * y[u].v[k];
           }
-          if (X2) y[u].v[k] = y[u].v[k] + (T)c * x2[u].v[k];
-          if (dots_after) {
-            d1 += p1[u].v[k] * y[u].v[k];
-            d2 += p2[u].v[k] * y[u].v[k];
+          if (P2) {
+            const Vec p = *reinterpret_cast<const Vec*>(P2 + idx[u]);
+#pragma unroll
+            for (int k = 0; k < V; ++k) d2 += p.v[k] * y[u].v[k];
           }
+        };
+        if (!dots_after) dots();
+        if (X2) {
+          const Vec x2 = *reinterpret_cast<const Vec*>(X2 + idx[u]);
+#pragma unroll
+          for (int k = 0; k < V; ++k) y[u].v[k] = y[u].v[k] + (T)c * x2.v[k];
         }
-        *reinterpret_cast<Vec*>(Y + idx[u]) = y[u];
+        if (dots_after) dots();
+        if (splits > 1 || X2) *reinterpret_cast<Vec*>(Y + idx[u]) = y[u];
       }
     }
   }
-  d1 = block_sum_t(d1, sh);
-  d2 = block_sum_t(d2, sh);
-  if (threadIdx.x == 0) {
-    double* p = part + ((int64_t)blockIdx.x * b + j) * kNQ;
-    p[q0] = (double)d1;
-    p[q0 + 1] = (double)d2;
+  d1 = warp_sum(d1);
+  d2 = warp_sum(d2);
+  if ((threadIdx.x & 31) == 0) {
+    sh[0][threadIdx.x >> 5] = d1;
+    sh[1][threadIdx.x >> 5] = d2;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    const T* v = sh[threadIdx.x];
+    part[((int64_t)blockIdx.x * b + j) * kNQ + q0 + threadIdx.x] = (double)(((v[0] + v[1]) + v[2]) + v[3]);
   }
 }
 
@@ -246,8 +302,8 @@ int launch_gemm_cfg(const AxArgs& a, int64_t n, int cols, int64_t ld, const void
 
 }  // namespace
 
-int launch_ax(const AxArgs& a, int tdtype, int64_t n, int cols, int64_t ld, const void* X,
-              void* Y, void* ws, size_t ws_elems, const int* run, cudaStream_t s, const ProdTune* tune) {
+int launch_ax(const AxArgs& a, int tdtype, int64_t n, int cols, int64_t ld, const void* X, void* Y, void* ws,
+              size_t ws_elems, const int* run, cudaStream_t s, const ProdTune* tune, double c, const void* X2) {
   if (a.kind == AX_DENSE) {
     // The tile is as narrow as the columns allow: 128 columns where a tile of 64 would not save a
     // padded half, else 64, 32, 16; FP64, whose pipes bound every size, down to 8 in steps that
@@ -282,25 +338,27 @@ int launch_ax(const AxArgs& a, int tdtype, int64_t n, int cols, int64_t ld, cons
 #undef GEMM
   }
   // CSR
-  const int cpl = cols > 128 ? 8 : (cols > 64 ? 4 : (cols > 32 ? 2 : 1));
-  dim3 grid(cdiv64(n, 8), cdiv64(cols, 32 * cpl));
-#define SPMM_CASE(TV, T, C)                                                              \
-  k_spmm_csr<TV, T, C><<<grid, 256, 0, s>>>(a.rowptr, a.colidx, (const TV*)a.vals,       \
-                                            (const T*)X, ld, (T*)Y, n, cols, run)
-#define SPMM_CPL(TV, T)                \
-  switch (cpl) {                       \
-    case 1: SPMM_CASE(TV, T, 1); break; \
-    case 2: SPMM_CASE(TV, T, 2); break; \
-    case 4: SPMM_CASE(TV, T, 4); break; \
-    default: SPMM_CASE(TV, T, 8); break; \
-  }
+  const uintptr_t all = (uintptr_t)X | (uintptr_t)Y | (uintptr_t)X2;
+#define SPMM(TV, T, V, L)                                                                                            \
+  k_spmm_csr<TV, T, V, L><<<dim3(cdiv64(n, 8 * (32 / L)), cdiv64(cols, V * L)), 256, 0, s>>>(                        \
+      a.rowptr, a.colidx, (const TV*)a.vals, (const T*)X, ld, (T*)Y, n, cols, (T)c, (const T*)X2, run)
+#define SPMM_L(TV, T, V)                    \
+  if (cols <= 4 * V) SPMM(TV, T, V, 4);     \
+  else if (cols <= 8 * V) SPMM(TV, T, V, 8); \
+  else if (cols <= 16 * V) SPMM(TV, T, V, 16); \
+  else SPMM(TV, T, V, 32)
+#define SPMM_V(TV, T)                                                                                   \
+  if (sizeof(T) == 4 && cols % 4 == 0 && ld % 4 == 0 && !(all & 15)) { SPMM_L(TV, T, (16 / (int)sizeof(T))); } \
+  else if (cols % 2 == 0 && ld % 2 == 0 && !(all & (2 * sizeof(T) - 1))) { SPMM_L(TV, T, 2); }          \
+  else { SPMM_L(TV, T, 1); }
   if (tdtype == 0) {
-    if (a.v_dtype == 0) { SPMM_CPL(double, double) } else { SPMM_CPL(float, double) }
+    if (a.v_dtype == 0) { SPMM_V(double, double) } else { SPMM_V(float, double) }
   } else {
-    if (a.v_dtype == 0) { SPMM_CPL(double, float) } else { SPMM_CPL(float, float) }
+    if (a.v_dtype == 0) { SPMM_V(double, float) } else { SPMM_V(float, float) }
   }
-#undef SPMM_CPL
-#undef SPMM_CASE
+#undef SPMM_V
+#undef SPMM_L
+#undef SPMM
   return 1;
 }
 
@@ -310,9 +368,22 @@ int launch_ax_finish_impl(int tdtype, const Dims& d, void* Y, const void* ws, in
   dim3 grid(cdiv64(d.n, kRowTile), d.b);
   const int v = tdtype == 0 ? 2 : 4;
   const uintptr_t all = (uintptr_t)Y | (uintptr_t)ws | (uintptr_t)X2 | (uintptr_t)P1 | (uintptr_t)P2;
+  if (!P1 && !P2 && d.ld == d.N) {  // no inner products: one flat array
+    const int64_t total = d.n * d.N;
+    const bool flat = total % v == 0 && !(all & 15);  // the slices start on 16 bytes as well
+#define SUM(T, V)                                                                                            \
+  k_ax_sum<T, V><<<cdiv64(total, 256 * V), 256, 0, s>>>(total, (T*)Y, (const T*)ws, splits, (T)c, (const T*)X2, run)
+    if (tdtype == 0) {
+      if (flat) SUM(double, 2); else SUM(double, 1);
+    } else {
+      if (flat) SUM(float, 4); else SUM(float, 1);
+    }
+#undef SUM
+    return grid.x;
+  }
   const bool vec = d.r % v == 0 && d.ld % v == 0 && !(all & 15);
 #define FIN(T, V)                                                                                                    \
-  k_ax_finish<T, V><<<grid, 256, 0, s>>>(d.n, d.r, d.ld, (T*)Y, (const T*)ws, splits, c, (const T*)X2, (const T*)P1, \
+  k_ax_finish<T, V><<<grid, 128, 0, s>>>(d.n, d.r, d.ld, (T*)Y, (const T*)ws, splits, c, (const T*)X2, (const T*)P1, \
                                          (const T*)P2, part, q0, d.b, run, dots_after)
   if (tdtype == 0) {
     if (vec) FIN(double, 2); else FIN(double, 1);

@@ -277,7 +277,7 @@ k_brow(RowArgs base, const BProb* __restrict__ probs, const int2* __restrict__ i
   a.part = base.part + (int64_t)pb.slot0 * kNQ;
   a.counters = base.counters + it.x;
   a.P.nr = pb.n * (int64_t)pb.r;
-  rowstep_body<T, STEP, NC, rowstep_mr<T>()>(a, 0, it.y, (unsigned)pb.nrt, pb.r % 4 == 0 && pb.xoff % 4 == 0,
+  rowstep_body<T, STEP, NC, rowstep_mr<T>()>(a, 0, it.y, pb.nrt, pb.nrt, pb.r % 4 == 0 && pb.xoff % 4 == 0,
                                     reinterpret_cast<T*>(rsm));
 }
 
@@ -527,7 +527,8 @@ template <typename T, int STEP, int NC>
 void launch_brow(BatchCtx* b, const RowArgs& a) {
   static std::once_flag once;
   std::call_once(once, [] {
-    cudaFuncSetAttribute(k_brow<T, STEP, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+    cudaFuncSetAttribute(k_brow<T, STEP, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)rowstep_smem<T>(64, kRowThreads, rowstep_mr<T>(), 4));
   });
   k_brow<T, STEP, NC><<<(unsigned)b->h_row.size(), kRowThreads, b->row_smem, b->s>>>(a, b->dp, blist(b, 0), bcnt(b, 0));
 }
@@ -732,8 +733,8 @@ snmf_status batch_create(BatchCtx** out, const snmf_matrix* Am, const snmf_optio
     const int mr = b->tdtype == 0 ? rowstep_mr<double>() : rowstep_mr<float>();
     const int rows = rowstep_rows(q.r, kRowThreads, mr);
     q.nrt = (int)((ns[p] + rows - 1) / rows);
-    b->row_smem = std::max(b->row_smem, b->tdtype == 0 ? rowstep_smem<double>(q.r, kRowThreads, mr)
-                                                       : rowstep_smem<float>(q.r, kRowThreads, mr));
+    b->row_smem = std::max(b->row_smem, b->tdtype == 0 ? rowstep_smem<double>(q.r, kRowThreads, mr, 4)
+                                                       : rowstep_smem<float>(q.r, kRowThreads, mr, 4));
     q.npt = (int)((ns[p] + kPBM - 1) / kPBM);
     q.gch = (int)((ns[p] + kGChunk - 1) / kGChunk);
     q.arow = arow;

@@ -211,9 +211,9 @@ TcEpilogue tc_epilogue(snmf_ctx* h, void* Y, double c, const void* X2, const voi
 // The product kernel: CUDA cores (FP64/FP32 dense, CSR, the FP8 final evaluation) or tcgen05
 // (BF16 dense; E4M3 dense, decoded to BF16 in shared memory).  Returns the number of split-K
 // slices written to h->ws (1 = result in Y), or 0 when the epilogue `epi` was fused into the
-// product (the result, c X2 and the partials are complete).
+// product (the result, c X2 and the partials are complete).  A CSR product takes c X2 along.
 int product_kernel(snmf_ctx* h, const AxArgs& op, const void* X, void* Y, const int* run,
-                   const TcEpilogue* epi = nullptr) {
+                   const TcEpilogue* epi = nullptr, double c = 0.0, const void* X2 = nullptr) {
   const ProdTune* tn = (h->tuned && &op == &h->A) ? &h->tune.cfg : nullptr;  // the tuned shape only
   if (op.kind == AX_DENSE && op.a_dtype == 3) {
     if (!op.accurate && h->xh) {
@@ -249,7 +249,7 @@ int product_kernel(snmf_ctx* h, const AxArgs& op, const void* X, void* Y, const 
     }
     return sp;
   }
-  return launch_ax(op, h->tdtype, h->n, h->N, h->N, X, Y, h->ws, h->ws_elems, run, h->s, tn);
+  return launch_ax(op, h->tdtype, h->n, h->N, h->N, X, Y, h->ws, h->ws_elems, run, h->s, tn, c, X2);
 }
 
 
@@ -266,8 +266,12 @@ int ax_apply(snmf_ctx* h, const AxArgs& op, bool use_lai, const void* X, void* Y
   TcEpilogue epi;
   if (op.kind == AX_DENSE && (op.a_dtype == 2 || op.a_dtype == 3) && !op.accurate)
     epi = tc_epilogue(h, Y, c, X2, P1, P2, part);
-  const int splits = product_kernel(h, op, X, Y, run, &epi);
-  if (splits == 0) return (int)((h->n + kRowTile - 1) / kRowTile);  // epilogue done in the product
+  // a CSR product adds c X2 itself, unless the dots are of the product before it
+  const bool dots = P1 || P2, with = op.kind == AX_CSR && (!dots || dots_after);
+  const int splits = product_kernel(h, op, X, Y, run, &epi, c, with ? X2 : nullptr);
+  if (with) X2 = nullptr;
+  // complete already: the epilogue in the product, or nothing left to add or sum
+  if (splits == 0 || (splits == 1 && !X2 && !dots)) return (int)((h->n + kRowTile - 1) / kRowTile);
   return launch_ax_finish_impl(h->tdtype, d, Y, h->ws, splits, c, X2, P1, P2, part, 0, run, h->s, dots_after);
 }
 
@@ -302,7 +306,6 @@ RowArgs row_base(snmf_ctx* h, const Params* P = nullptr) {
   a.gamma = h->graph ? h->gamma : 0.0;
   a.part = h->prow;
   a.counters = h->counters;
-  a.gcounters = h->rplan.groups ? h->counters + h->b : nullptr;
   a.G64fix = h->G64fix;
   a.bm = h->row_bm;
   if (P) a.P = *P;
@@ -613,7 +616,7 @@ void pen_block(snmf_ctx* h, int xv, int xf, bool is_w, const Params& P, bool nai
       launch_rowstep_dz(td, a, h->rplan, h->s);
       const int nl = ax_L(h, h->buf[B_D], h->buf[B_LD], h->buf[B_D], nullptr, h->pax3, h->run);
       launch_ctl_pen_ls(h->ctl, h->prow, h->nrow, h->pax3, nl, h->b, h->r, h->G64fix, nullptr, P, 1, h->s);
-      launch_xupd(td, d, h->buf[B_Z], h->buf[B_D], h->buf[B_XN], nullptr, nullptr, nullptr, h->ctl, h->pclip, h->s);
+      launch_xnext(td, d, h->buf[B_Z], h->buf[B_D], h->buf[B_XN], h->ctl, h->s);
       ax_L(h, h->buf[B_XN], h->buf[B_LX], nullptr, nullptr, h->pax2, h->run);
       RowArgs u = row_base(h, &P);
       u.X = h->buf[B_XN]; u.LX = h->buf[B_LX]; u.B = h->buf[B_B];
@@ -830,7 +833,7 @@ snmf_status alloc_buffers(snmf_ctx* h) {
   // room for every row-kernel layout
   h->use_row = row_rule(h);
   h->rplan = rowstep_plan(h->tdtype, h->n, std::min(h->r, 64), h->b);
-  const int nrow_max = std::max({h->nrow, rowgemm_slots(d, h->tdtype, 32), h->rplan.slots + h->rplan.groups});
+  const int nrow_max = std::max({h->nrow, rowgemm_slots(d, h->tdtype, 32), h->rplan.slots});
   const size_t prec_n = (size_t)std::max(nrow_max, h->nax) * h->b * kNQ;
   if (h->use_row) h->nrow = h->rplan.slots;
   double** parts[] = {&h->prow, &h->pax, &h->pax2, &h->pax3, &h->pax4, &h->pclip};
@@ -838,7 +841,7 @@ snmf_status alloc_buffers(snmf_ctx* h) {
     CK(cudaMalloc(p, prec_n * sizeof(double)));
     CK(cudaMemsetAsync(*p, 0, prec_n * sizeof(double), h->s));
   }
-  h->gplan = gram_plan(h->n, h->r, h->b);
+  h->gplan = gram_plan(h->tdtype, h->n, h->r, h->b);
   const size_t rr = (size_t)h->r * h->r * h->b;
   CK(cudaMalloc(&h->gpart, h->gplan.part_elems * h->esz));
   CK(cudaMalloc(&h->gcounters, h->gplan.counters * sizeof(unsigned)));
@@ -861,9 +864,8 @@ snmf_status alloc_buffers(snmf_ctx* h) {
     CK(cudaMemsetAsync(h->tcount, 0, nt * sizeof(unsigned), h->s));
   }
   if (h->opt.timeout_cycles > 0) h->budget = h->opt.timeout_cycles;
-  const size_t ncount = (size_t)h->b * (1 + h->rplan.groups);
-  CK(cudaMalloc(&h->counters, ncount * sizeof(unsigned)));
-  CK(cudaMemsetAsync(h->counters, 0, ncount * sizeof(unsigned), h->s));
+  CK(cudaMalloc(&h->counters, h->b * sizeof(unsigned)));
+  CK(cudaMemsetAsync(h->counters, 0, h->b * sizeof(unsigned), h->s));
   CK(cudaMalloc(&h->dsc, 4096 * sizeof(double)));
   CK(cudaMalloc(&h->ring, (size_t)h->b * h->ring_cap * kRingVals * sizeof(double)));
   CK(cudaMemsetAsync(h->ring, 0, (size_t)h->b * h->ring_cap * kRingVals * sizeof(double), h->s));

@@ -180,10 +180,11 @@ struct AxArgs {
 
 // Y = A X (raw product, T = double/float), n x cols, ld = leading dimension of X and Y.
 // Dense products may split K: the splits write ws[s] (n x ld each) and the finish pass
-// sums them.  Returns the number of splits used (1 = result already in Y).
-int launch_ax(const AxArgs& a, int tdtype, int64_t n, int cols, int64_t ld,
-              const void* X, void* Y, void* ws, size_t ws_elems, const int* run_flag,
-              cudaStream_t s, const ProdTune* tune = nullptr);
+// sums them.  Returns the number of splits used (1 = result already in Y).  A CSR product adds
+// c X2 itself when X2 is given (a dense one ignores it).
+int launch_ax(const AxArgs& a, int tdtype, int64_t n, int cols, int64_t ld, const void* X, void* Y, void* ws,
+              size_t ws_elems, const int* run_flag, cudaStream_t s, const ProdTune* tune = nullptr, double c = 0.0,
+              const void* X2 = nullptr);
 
 // Structure check of a device CSR matrix: *bad |= 1 for a bad rowptr (rowptr[0] != 0,
 // rowptr[n] != nnz or decreasing), |= 2 for a column index outside [0, n).  *bad must be

@@ -104,14 +104,16 @@ __global__ void __launch_bounds__(1024) k_rho_wide(const double* __restrict__ G6
 
 }  // namespace
 
-GramPlan gram_plan(int64_t n, int r, int b) {
+GramPlan gram_plan(int tdtype, int64_t n, int r, int b) {
   GramPlan pl;
   pl.tw = gram_tw(r);
   pl.ntile = r <= 64 ? 1 : (r + 63) / 64;
   const int64_t tiles = (int64_t)b * pl.ntile * pl.ntile;
-  // four CTAs per SM over the tiles, chunks of at least 64 rows; up to 32 chunks fit one level
-  // of 16 partials (n = 1000, r = 20: 16 chunks 10 us, one chunk 50 us)
-  int64_t nch = std::min<int64_t>((n + 63) / 64, (4 * 152 + tiles - 1) / tiles);
+  // one wave of three CTAs per SM over the tiles, chunks of at least 64 rows (32 in FP64, whose pipes
+  // are slow); up to 32 chunks fit one level of 16 partials (n = 1000, r = 20: 16 chunks 10 us,
+  // one chunk 50 us)
+  const int64_t least = tdtype == 0 ? 32 : 64;
+  int64_t nch = std::min<int64_t>((n + least - 1) / least, 3 * 152 / tiles);
   if (nch > kGramGroup && nch <= 2 * kGramGroup) nch = kGramGroup;
   if (nch < 1) nch = 1;
   pl.chunk = ((n + nch - 1) / nch + 31) / 32 * 32;

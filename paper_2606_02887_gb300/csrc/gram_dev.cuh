@@ -4,6 +4,8 @@
 
 #include <math.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace snmf {
@@ -165,37 +167,42 @@ __device__ __forceinline__ void rho_in_smem(const T* Gs, int r, int iters, doubl
 }
 
 // ------------------------------------------------------------------------------
-// One chunk of rows [i_begin, i_end) of a TW x TW Gram tile: X, Y at the tile's first columns
-// (wx, wy of them exist), row pitch ld, VEC elements per copy (16 bytes when the columns and
-// the pitch allow it, else single elements).  256 threads: NG = 4096 / TW^2 row groups, each a
-// (TW / 4)^2 grid of 4 x 4 micro tiles read as two 16-byte shared loads per row.  The groups'
-// sums leave the row loop in shared memory; the thread returns its entries e = 4 (t + 256 u).
+// One chunk of rows [i_begin, i_end) of a TP x TQ tile of X^T Y: X, Y at the tile's first columns
+// (wx, wy of them exist), row pitches ldx, ldy, VEC elements per copy (16 bytes when the columns and
+// the pitches allow it, else single elements).  256 threads: NG = 4096 / (TP TQ) row groups, each a
+// (TP / 4) x (TQ / 4) grid of 4 x 4 micro tiles read as two 16-byte shared loads per row.  The
+// groups' sums leave the row loop in shared memory; the thread returns its entries e = 4 (t + 256 u).
 // Bound by HBM for long factors (n = 2e6, r = 32: 797 us with 152 chunks of two staged rounds
-// and scalar shared reads) and by latency for short ones.
+// and scalar shared reads, 177 us so) and by latency for short ones.
 // ------------------------------------------------------------------------------
-template <typename T, int TW, int VEC>
-__device__ __forceinline__ void gram_chunk(const T* __restrict__ X, const T* __restrict__ Y, int wx, int wy, int64_t ld,
-                                           int64_t i_begin, int64_t i_end, bool same, T* sm, Quad<T>* out) {
-  constexpr int RS = kGramStageBytes / (TW * (int)sizeof(T));  // rows per stage
-  constexpr int NG = 4096 / (TW * TW), GT = 256 / NG, TX = TW / 4;
-  constexpr int CPR = TW / VEC;             // copies per row
-  constexpr int NC = RS * CPR / 256;        // copies per thread and operand
-  constexpr int STAGE = RS * TW;
+template <int TP, int TQ>
+__host__ __device__ constexpr int tile_quads() { return TP * TQ >= 1024 ? TP * TQ / 1024 : 1; }  // 16-byte entries per thread
+
+template <typename T, int TP, int TQ, int VEC>
+__device__ __forceinline__ void gram_chunk(const T* __restrict__ X, const T* __restrict__ Y, int wx, int wy, int64_t ldx,
+                                           int64_t ldy, int64_t i_begin, int64_t i_end, bool same, T* sm,
+                                           Quad<T> (&out)[tile_quads<TP, TQ>()]) {
+  constexpr int TM = TP > TQ ? TP : TQ;
+  constexpr int RS = kGramStageBytes / (TM * (int)sizeof(T));  // rows per stage
+  constexpr int NG = 4096 / (TP * TQ), GT = 256 / NG, TX = TQ / 4;
+  constexpr int SX = RS * TP, SY = RS * TQ;
   const int t = threadIdx.x;
   T* Xs = sm;
-  T* Ys = same ? sm : sm + kGramStages * STAGE;
-  auto fetch = [&](int64_t i0, int st) {
+  T* Ys = same ? sm : sm + kGramStages * SX;
+  auto copy = [&](auto width, const T* P, int w, int64_t ld, T* dst, int64_t i0) {
+    constexpr int TW = decltype(width)::value, CPR = TW / VEC, NC = (RS * CPR + 255) / 256;
 #pragma unroll
     for (int m = 0; m < NC; ++m) {
       const int e = t + 256 * m, rr = e / CPR, cc = (e % CPR) * VEC;
+      if (RS * CPR % 256 && e >= RS * CPR) break;
       const int64_t i = i0 + rr;
-      const bool vx = i < i_end && cc < wx;
-      cp_async<VEC * (int)sizeof(T)>(Xs + st * STAGE + rr * TW + cc, vx ? X + i * ld + cc : X, vx);
-      if (!same) {
-        const bool vy = i < i_end && cc < wy;
-        cp_async<VEC * (int)sizeof(T)>(Ys + st * STAGE + rr * TW + cc, vy ? Y + i * ld + cc : Y, vy);
-      }
+      const bool v = i < i_end && cc < w;
+      cp_async<VEC * (int)sizeof(T)>(dst + rr * TW + cc, v ? P + i * ld + cc : P, v);
     }
+  };
+  auto fetch = [&](int64_t i0, int st) {
+    copy(std::integral_constant<int, TP>{}, X, wx, ldx, Xs + st * SX, i0);
+    if (!same) copy(std::integral_constant<int, TQ>{}, Y, wy, ldy, Ys + st * SY, i0);
   };
   const int rounds = (int)((i_end - i_begin + RS - 1) / RS);
 #pragma unroll
@@ -215,12 +222,12 @@ __device__ __forceinline__ void gram_chunk(const T* __restrict__ X, const T* __r
     if (k + kGramStages - 1 < rounds)
       fetch(i_begin + (int64_t)(k + kGramStages - 1) * RS, (k + kGramStages - 1) % kGramStages);
     cp_async_commit();
-    const T* xs = Xs + (k % kGramStages) * STAGE + 4 * ty;
-    const T* ys = Ys + (k % kGramStages) * STAGE + 4 * tx;
+    const T* xs = Xs + (k % kGramStages) * SX + 4 * ty;
+    const T* ys = Ys + (k % kGramStages) * SY + 4 * tx;
 #pragma unroll 4
     for (int rr = grp; rr < RS; rr += NG) {
-      const Quad<T> xa = *reinterpret_cast<const Quad<T>*>(xs + rr * TW);
-      const Quad<T> yb = *reinterpret_cast<const Quad<T>*>(ys + rr * TW);
+      const Quad<T> xa = *reinterpret_cast<const Quad<T>*>(xs + rr * TP);
+      const Quad<T> yb = *reinterpret_cast<const Quad<T>*>(ys + rr * TQ);
 #pragma unroll
       for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -231,18 +238,17 @@ __device__ __forceinline__ void gram_chunk(const T* __restrict__ X, const T* __r
   __syncthreads();  // the ring is free: it takes the groups' tiles
 #pragma unroll
   for (int a = 0; a < 4; ++a)
-    *reinterpret_cast<Quad<T>*>(sm + grp * TW * TW + (4 * ty + a) * TW + 4 * tx) =
+    *reinterpret_cast<Quad<T>*>(sm + grp * TP * TQ + (4 * ty + a) * TQ + 4 * tx) =
         Quad<T>{{acc[a][0], acc[a][1], acc[a][2], acc[a][3]}};
   __syncthreads();
-  constexpr int NE = TW * TW / 4 >= 256 ? TW * TW / 1024 : 1;
 #pragma unroll
-  for (int u = 0; u < NE; ++u) {
+  for (int u = 0; u < tile_quads<TP, TQ>(); ++u) {
     const int e = 4 * (t + 256 * u);
-    if (e < TW * TW) {
+    if (e < TP * TQ) {
       Quad<T> s = *reinterpret_cast<const Quad<T>*>(sm + e);
 #pragma unroll
       for (int g = 1; g < NG; ++g) {
-        const Quad<T> v = *reinterpret_cast<const Quad<T>*>(sm + g * TW * TW + e);
+        const Quad<T> v = *reinterpret_cast<const Quad<T>*>(sm + g * TP * TQ + e);
 #pragma unroll
         for (int k = 0; k < 4; ++k) s.v[k] += v.v[k];
       }
@@ -251,37 +257,20 @@ __device__ __forceinline__ void gram_chunk(const T* __restrict__ X, const T* __r
   }
 }
 
-// Where a Gram tile goes: entry (p, q) of the tile is (p0 + p, q0 + q) of the r x r matrix.
-template <typename T>
-struct GramOut {
-  double* G64;
-  T* GT;  // factor-type copy with lam on the diagonal (NULL: none)
-  T lam;
-  int r, p0, q0;
-  Ctl* rho_ctl;  // the tile is the whole Gram: rho = rho_scale ||G||_2 + rho_shift (NULL: no)
-  int rho_iters;
-  double rho_scale, rho_shift;
-};
-
-// CTA `c` of the nch chunks of one tile.  Partials go to gp (nch + ng tiles of TW^2 values) and
-// are summed in chunk order by the last CTA of each of the ng groups of 16 chunks and then, in group
-// order, by the last group's (arrival counters cnt[0 .. ng], zero between launches): a fixed
-// order, and no CTA reads many partials in a row, which had kept the number of chunks, and with it
-// the CTAs, low.  ng = 0: one level, every chunk in order.
+// Sum of the tiles of CTAs c = 0 .. nch - 1, each with its entries in s: true in one CTA, which holds
+// the sum.  Partials go to gp (nch + ng tiles of TT values) and are summed in chunk order by the
+// last CTA of each of the ng groups of 16 chunks and then, in group order, by the last group's
+// (arrival counters cnt[0 .. ng], zero between launches): a fixed order, and no CTA reads many
+// partials in a row, which had kept the number of chunks, and with it the CTAs, low.  ng = 0: one
+// level, every chunk in order.
 __host__ __device__ inline int gram_groups(int nch) { return nch > kGramGroup ? (nch + kGramGroup - 1) / kGramGroup : 0; }
 
-template <typename T, int TW, int VEC>
-__device__ __forceinline__ void gram_body(const T* X, const T* Y, int wx, int wy, int64_t ld, int64_t n, int64_t chunk,
-                                          int c, int nch, int ng, bool same, T* gp, unsigned* cnt, const GramOut<T>& o,
-                                          T* sm) {
-  constexpr int NE = TW * TW / 4 >= 256 ? TW * TW / 1024 : 1;
-  constexpr int TW2 = TW * TW;
+template <typename T, int TT, int NE>
+__device__ __forceinline__ bool sum_chunks(Quad<T> (&s)[NE], int c, int nch, int ng, T* gp, unsigned* cnt) {
   __shared__ unsigned s_ticket;
   const int t = threadIdx.x;
-  const bool owns = 4 * t < TW2;
-  Quad<T> s[NE];
-  const int64_t i0 = (int64_t)c * chunk;
-  gram_chunk<T, TW, VEC>(X, Y, wx, wy, ld, i0, min(n, i0 + chunk), same, sm, s);
+  const bool owns = 4 * t < TT;
+  if (nch == 1) return true;
   auto publish = [&](T* dst) {
 #pragma unroll
     for (int u = 0; u < NE; ++u)
@@ -299,7 +288,7 @@ __device__ __forceinline__ void gram_body(const T* X, const T* Y, int wx, int wy
     __syncthreads();
     return last;
   };
-  auto sum = [&](const T* src, int m) {  // s = the m tiles at src in order, 16 loads in flight
+  auto sum = [&](const T* src, int m) {  // s = the m tiles at src in order, 8 loads in flight
 #pragma unroll
     for (int u = 0; u < NE; ++u) {
       s[u] = Quad<T>{{T(0), T(0), T(0), T(0)}};
@@ -308,7 +297,8 @@ __device__ __forceinline__ void gram_body(const T* X, const T* Y, int wx, int wy
       for (int k0 = 0; k0 < m; k0 += 8) {
         Quad<T> v[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) v[k] = k0 + k < m ? ldcg_quad(q + (int64_t)(k0 + k) * TW2) : Quad<T>{{T(0), T(0), T(0), T(0)}};
+        for (int k = 0; k < 8; ++k)
+          v[k] = k0 + k < m ? ldcg_quad(q + (int64_t)(k0 + k) * TT) : Quad<T>{{T(0), T(0), T(0), T(0)}};
 #pragma unroll
         for (int k = 0; k < 8; ++k)
 #pragma unroll
@@ -316,19 +306,44 @@ __device__ __forceinline__ void gram_body(const T* X, const T* Y, int wx, int wy
       }
     }
   };
-  if (nch > 1) {
-    publish(gp + (int64_t)c * TW2);
-    const int g = c / kGramGroup, gs = min(kGramGroup, nch - g * kGramGroup);
-    if (!arrive(cnt + (ng ? 1 + g : 0), ng ? gs : nch)) return;
+  publish(gp + (int64_t)c * TT);
+  const int g = c / kGramGroup, gs = min(kGramGroup, nch - g * kGramGroup);
+  if (!arrive(cnt + (ng ? 1 + g : 0), ng ? gs : nch)) return false;
+  __threadfence();
+  sum(gp + (int64_t)(ng ? g * kGramGroup : 0) * TT, ng ? gs : nch);
+  if (ng) {
+    publish(gp + (int64_t)(nch + g) * TT);
+    if (!arrive(cnt, ng)) return false;
     __threadfence();
-    sum(gp + (int64_t)(ng ? g * kGramGroup : 0) * TW2, ng ? gs : nch);
-    if (ng) {
-      publish(gp + (int64_t)(nch + g) * TW2);
-      if (!arrive(cnt, ng)) return;
-      __threadfence();
-      sum(gp + (int64_t)nch * TW2, ng);
-    }
+    sum(gp + (int64_t)nch * TT, ng);
   }
+  return true;
+}
+
+// Where a Gram tile goes: entry (p, q) of the tile is (p0 + p, q0 + q) of the r x r matrix.
+template <typename T>
+struct GramOut {
+  double* G64;
+  T* GT;  // factor-type copy with lam on the diagonal (NULL: none)
+  T lam;
+  int r, p0, q0;
+  Ctl* rho_ctl;  // the tile is the whole Gram: rho = rho_scale ||G||_2 + rho_shift (NULL: no)
+  int rho_iters;
+  double rho_scale, rho_shift;
+};
+
+// CTA `c` of the nch chunks of one Gram tile (see sum_chunks).
+template <typename T, int TW, int VEC>
+__device__ __forceinline__ void gram_body(const T* X, const T* Y, int wx, int wy, int64_t ld, int64_t n, int64_t chunk,
+                                          int c, int nch, int ng, bool same, T* gp, unsigned* cnt, const GramOut<T>& o,
+                                          T* sm) {
+  constexpr int NE = tile_quads<TW, TW>();
+  const int t = threadIdx.x;
+  const bool owns = 4 * t < TW * TW;
+  Quad<T> s[NE];
+  const int64_t i0 = (int64_t)c * chunk;
+  gram_chunk<T, TW, TW, VEC>(X, Y, wx, wy, ld, ld, i0, min(n, i0 + chunk), same, sm, s);
+  if (!sum_chunks<T, TW * TW>(s, c, nch, ng, gp, cnt)) return;
 #pragma unroll
   for (int u = 0; u < NE; ++u) {
     const int e = 4 * (t + 256 * u);

@@ -1,11 +1,10 @@
 // LAI-SNMPBB (Sec. 2.3, Eq. (8)): randomized eigen-sketch A ~ U E U^T and the product
 // A X ~ U (E (U^T X)), U^T X formed first.
 //
-//   k_utx      M = E (U^T X) (k x N): CTA (row chunk, 64x64 output tile), partial per chunk
-//              in the working type, last CTA of each tile sums the chunks in order and scales
-//              row l by lambda_l.
-//   k_rowmul   Out = In M (n x K times K x m), K <= 128: 32-row x 64-column tiles, K staged
-//              in chunks of 32.  Serves U M, Y R^-1 (CholeskyQR) and Q P (Ritz vectors).
+//   k_utx      M = E (U^T X) (k x N): CTA (row chunk, 64 x 16, 32 or 64 output tile), partials summed
+//              as the Gram's (gram_dev.cuh), row l scaled by lambda_l.
+//   k_rowmul   Out = In M (n x K times K x m) (+ c X2), K <= 128, in the product tiles of
+//              gemm_dev.cuh.  Serves U M, Y R^-1 (CholeskyQR) and Q P (Ritz vectors).
 //   k_chol     Cholesky R^T R = G (+ shift) of an l x l FP64 Gram and R^-1, one block.
 //   k_jacobi   parallel cyclic Jacobi eigensolver of a symmetric l x l FP64 matrix, one block,
 //              round-robin pairing (l/2 disjoint rotations per round).
@@ -13,9 +12,11 @@
 #include <math.h>
 
 #include <algorithm>
+#include <mutex>
 #include <string>
 
 #include "ax_tc.cuh"
+#include "gemm_dev.cuh"
 #include "lai.cuh"
 #include "rowops.cuh"
 
@@ -25,185 +26,79 @@ namespace {
 
 inline int cdivi(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 
-// NT: output columns per tile (32 for N <= 32, else 64); RS rows staged per round with the next
-// round's loads in flight.
-template <typename T, int NT, int RS>
-__global__ void __launch_bounds__(256)
-k_utx(const T* __restrict__ U, int k, const T* __restrict__ X, int64_t n, int N, int64_t ldx,
-      int64_t chunk, T* __restrict__ part, const double* __restrict__ lam, T* __restrict__ M,
-      unsigned* __restrict__ counters, const int* run) {
-  constexpr int MC = NT / 16;        // micro tile columns
-  constexpr int LU = RS * 64 / 256;  // staged U values per thread
-  constexpr int LX = RS * NT / 256;  // staged X values per thread
-  const int lt = blockIdx.y, ct = blockIdx.z;  // 64 x NT tile of the k x N output
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int64_t i_begin = (int64_t)blockIdx.x * chunk, i_end = min(n, i_begin + chunk);
-  __shared__ T Us[RS][64 + 1];
-  __shared__ T Xs[RS][NT + 1];
-  __shared__ unsigned ticket;
-  T acc[4][MC];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int c = 0; c < MC; ++c) acc[a][c] = T(0);
-  const bool skip = run && *run == 0;
-  const int l0 = lt * 64, c0 = ct * NT;
-  if (!skip) {
-    T uv[LU], xv[LX];
-    auto fetch = [&](int64_t i0) {
-#pragma unroll
-      for (int m = 0; m < LU; ++m) {
-        const int e = threadIdx.x + 256 * m, rr = e >> 6, cc = e & 63;
-        const int64_t i = i0 + rr;
-        uv[m] = (i < i_end && l0 + cc < k) ? U[i * k + l0 + cc] : T(0);
-      }
-#pragma unroll
-      for (int m = 0; m < LX; ++m) {
-        const int e = threadIdx.x + 256 * m, rr = e / NT, cc = e % NT;
-        const int64_t i = i0 + rr;
-        xv[m] = (i < i_end && c0 + cc < N) ? X[i * ldx + c0 + cc] : T(0);
-      }
-    };
-    if (i_begin < i_end) fetch(i_begin);
-    for (int64_t i0 = i_begin; i0 < i_end; i0 += RS) {
-#pragma unroll
-      for (int m = 0; m < LU; ++m) {
-        const int e = threadIdx.x + 256 * m;
-        Us[e >> 6][e & 63] = uv[m];
-      }
-#pragma unroll
-      for (int m = 0; m < LX; ++m) {
-        const int e = threadIdx.x + 256 * m;
-        Xs[e / NT][e % NT] = xv[m];
-      }
-      __syncthreads();
-      if (i0 + RS < i_end) fetch(i0 + RS);  // the next round's loads fly during this one
-#pragma unroll 8
-      for (int rr = 0; rr < RS; ++rr) {
-        T ua[4], xb[MC];
-#pragma unroll
-        for (int a = 0; a < 4; ++a) ua[a] = Us[rr][ty + 16 * a];
-#pragma unroll
-        for (int c = 0; c < MC; ++c) xb[c] = Xs[rr][tx + 16 * c];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int c = 0; c < MC; ++c) acc[a][c] = fma(ua[a], xb[c], acc[a][c]);
-      }
-      __syncthreads();
-    }
-  }
-  const int64_t kn = (int64_t)k * N;
-  T* out = part + (int64_t)blockIdx.x * kn;
-#pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int l = l0 + ty + 16 * a;
-    if (l >= k) continue;
-#pragma unroll
-    for (int c = 0; c < MC; ++c) {
-      const int col = c0 + tx + 16 * c;
-      if (col < N) out[(int64_t)l * N + col] = acc[a][c];
-    }
-  }
-  __threadfence();
-  __syncthreads();
-  const int tile_id = lt * gridDim.z + ct;
-  if (threadIdx.x == 0) ticket = atomicAdd(&counters[tile_id], 1u);
-  __syncthreads();
-  if (ticket != gridDim.x - 1) return;
-  // last CTA of the tile: each thread sums its NE entries over the chunks in chunk order,
-  // several chunks' loads in flight
-  constexpr int NE = 64 * NT / 256;
-  constexpr int UF = NE >= 16 ? 2 : 4;
-  int64_t off[NE];
-  bool ok[NE];
-  T sacc[NE];
+// Bound by HBM (U and X read once): n = 2e6, k = 64, N = 32 took 757 us with two staged rounds and
+// scalar shared reads in 152 CTAs.
+template <typename T, int TQ, int VEC>
+__global__ void __launch_bounds__(256, 3)
+k_utx(const T* __restrict__ U, int k, const T* __restrict__ X, int64_t n, int N, int64_t ldx, int64_t chunk, int nch,
+      int ng, T* __restrict__ part, const double* __restrict__ lam, T* __restrict__ M, unsigned* __restrict__ counters,
+      const int* run) {
+  extern __shared__ __align__(16) unsigned char usm[];
+  if (run && *run == 0) return;
+  constexpr int TT = 64 * TQ, NE = tile_quads<64, TQ>();
+  const int l0 = blockIdx.y * 64, c0 = blockIdx.z * TQ, tile = blockIdx.y * gridDim.z + blockIdx.z;
+  const int64_t i0 = (int64_t)blockIdx.x * chunk;
+  Quad<T> s[NE];
+  gram_chunk<T, 64, TQ, VEC>(U + l0, X + c0, min(64, k - l0), min(TQ, N - c0), k, ldx, i0, min(n, i0 + chunk), false,
+                             reinterpret_cast<T*>(usm), s);
+  if (!sum_chunks<T, TT>(s, blockIdx.x, nch, ng, part + (int64_t)tile * (nch + ng) * TT, counters + tile * (1 + ng)))
+    return;
 #pragma unroll
   for (int u = 0; u < NE; ++u) {
-    const int e = threadIdx.x + 256 * u;
-    const int l = l0 + e / NT, col = c0 + e % NT;
-    ok[u] = l < k && col < N;
-    off[u] = ok[u] ? (int64_t)l * N + col : 0;
-    sacc[u] = T(0);
+    const int e = 4 * (threadIdx.x + 256 * u);
+    if (e >= TT) continue;
+    const int l = l0 + e / TQ;
+    if (l >= k) continue;
+    const T sc = (T)lam[l];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (c0 + e % TQ + q < N) M[(int64_t)l * N + c0 + e % TQ + q] = s[u].v[q] * sc;
   }
-#pragma unroll UF
-  for (int c = 0; c < (int)gridDim.x; ++c) {
-    T v[NE];
-#pragma unroll
-    for (int u = 0; u < NE; ++u) v[u] = ok[u] ? __ldcg(part + (int64_t)c * kn + off[u]) : T(0);
-#pragma unroll
-    for (int u = 0; u < NE; ++u) sacc[u] += v[u];
-  }
-#pragma unroll
-  for (int u = 0; u < NE; ++u)
-    if (ok[u]) M[off[u]] = sacc[u] * (T)lam[l0 + (threadIdx.x + 256 * u) / NT];
-  if (threadIdx.x == 0) counters[tile_id] = 0u;
 }
 
-// BR rows x NC columns per CTA (32 x 64, or 64 x 32 for m <= 32), K staged in chunks of 32.
-template <typename T, int BR, int NC>
-__global__ void __launch_bounds__(256)
-k_rowmul(const T* __restrict__ In, int64_t ldi, int K, const T* __restrict__ Mm, int m, int64_t n,
-         T* __restrict__ Out, int64_t ldo, const int* run) {
-  constexpr int PR = BR / 16, QC = NC / 16;  // rows and columns per thread
-  constexpr int LI = BR * 32 / 256, LM = 32 * NC / 256;
+template <typename T>
+constexpr size_t utx_smem(int tq) {
+  const size_t ring = (size_t)kGramStages * (kGramStageBytes + kGramStageBytes / 64 * tq);
+  return ring > 4096 * sizeof(T) ? ring : 4096 * sizeof(T);
+}
+
+// n = 2e6, K = 64, m = 32: 445 us in 64 x 32 tiles staged one round at a time, and a finish pass.
+template <typename C, int PER_SM>
+__global__ void __launch_bounds__(C::NT, PER_SM)
+k_rowmul(const typename C::T* __restrict__ In, int64_t ldi, int K, const typename C::T* __restrict__ Mm, int m, int64_t n,
+         typename C::T* __restrict__ Out, int64_t ldo, bool avec, bool xvec, bool yvec, typename C::T c,
+         const typename C::T* __restrict__ X2, const int* run) {
+  using T = typename C::T;
+  extern __shared__ __align__(16) unsigned char rsm[];
   if (run && *run == 0) return;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int64_t row0 = (int64_t)blockIdx.x * BR;
-  const int col0 = blockIdx.y * NC;
-  __shared__ T Is[BR][33];
-  __shared__ T Ms[32][NC + 1];
-  T acc[PR][QC];
+  const int64_t row0 = (int64_t)blockIdx.x * C::BM;
+  const int col0 = blockIdx.y * C::BN;
+  T acc[C::TM][C::TN];
+  gemm_tile<C>(In, ldi, Mm, m, n, m, row0, col0, 0, K, avec, xvec, GemmA8{}, reinterpret_cast<T*>(rsm), acc);
+  const int tx = threadIdx.x % C::TX, ty = threadIdx.x / C::TX;
 #pragma unroll
-  for (int p = 0; p < PR; ++p)
+  for (int i = 0; i < C::TM; ++i) {
+    const int64_t r = row0 + ty + C::TY * i;
+    if (r >= n) continue;
 #pragma unroll
-    for (int q = 0; q < QC; ++q) acc[p][q] = T(0);
-  for (int k0 = 0; k0 < K; k0 += 32) {
-    T iv[LI], mv[LM];
+    for (int j = 0; j < C::TN; j += C::VW) {
+      struct alignas(C::VW * sizeof(T)) Vec {
+        T v[C::VW];
+      };
+      const int col = col0 + C::col(tx, j);
+      const int64_t idx = r * ldo + col;
+      if (yvec) {
+        if (col >= m) continue;
+        Vec y, x2;
+        if (X2) x2 = *reinterpret_cast<const Vec*>(X2 + idx);
 #pragma unroll
-    for (int u = 0; u < LI; ++u) {
-      const int e = threadIdx.x + 256 * u, rr = e >> 5, kk = e & 31;
-      const int64_t i = row0 + rr;
-      iv[u] = (i < n && k0 + kk < K) ? In[i * ldi + k0 + kk] : T(0);
-    }
+        for (int u = 0; u < C::VW; ++u) y.v[u] = X2 ? acc[i][j + u] + c * x2.v[u] : acc[i][j + u];
+        *reinterpret_cast<Vec*>(Out + idx) = y;
+      } else {
 #pragma unroll
-    for (int u = 0; u < LM; ++u) {
-      const int e = threadIdx.x + 256 * u, kk = e / NC, cc = e % NC;
-      mv[u] = (k0 + kk < K && col0 + cc < m) ? Mm[(int64_t)(k0 + kk) * m + col0 + cc] : T(0);
-    }
-#pragma unroll
-    for (int u = 0; u < LI; ++u) {
-      const int e = threadIdx.x + 256 * u;
-      Is[e >> 5][e & 31] = iv[u];
-    }
-#pragma unroll
-    for (int u = 0; u < LM; ++u) {
-      const int e = threadIdx.x + 256 * u;
-      Ms[e / NC][e % NC] = mv[u];
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int kk = 0; kk < 32; ++kk) {
-      T a[PR];
-#pragma unroll
-      for (int p = 0; p < PR; ++p) a[p] = Is[ty + 16 * p][kk];
-#pragma unroll
-      for (int q = 0; q < QC; ++q) {
-        const T mq = Ms[kk][tx + 16 * q];
-#pragma unroll
-        for (int p = 0; p < PR; ++p) acc[p][q] = fma(a[p], mq, acc[p][q]);
+        for (int u = 0; u < C::VW; ++u)
+          if (col + u < m) Out[idx + u] = X2 ? acc[i][j + u] + c * X2[idx + u] : acc[i][j + u];
       }
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int p = 0; p < PR; ++p) {
-    const int64_t i = row0 + ty + 16 * p;
-    if (i >= n) continue;
-#pragma unroll
-    for (int q = 0; q < QC; ++q) {
-      const int c = col0 + tx + 16 * q;
-      if (c < m) Out[i * ldo + c] = acc[p][q];
     }
   }
 }
@@ -377,38 +272,77 @@ int ck(cudaError_t e, std::string& msg, const char* what) {
 
 }  // namespace
 
-void launch_rowmul(int tdtype, const void* In, int64_t ldi, int K, const void* M, int m, int64_t n, void* Out,
-                   int64_t ldo, const int* run, cudaStream_t s) {
-#define RM_ARGS(T) (const T*)In, ldi, K, (const T*)M, m, n, (T*)Out, ldo, run
-  if (m <= 32) {  // narrow output: 64 rows x 32 columns per CTA, no masked half
-    dim3 grid(cdivi(n, 64), 1);
-    if (tdtype == 0) k_rowmul<double, 64, 32><<<grid, 256, 0, s>>>(RM_ARGS(double));
-    else k_rowmul<float, 64, 32><<<grid, 256, 0, s>>>(RM_ARGS(float));
-  } else {
-    dim3 grid(cdivi(n, 32), cdivi(m, 64));
-    if (tdtype == 0) k_rowmul<double, 32, 64><<<grid, 256, 0, s>>>(RM_ARGS(double));
-    else k_rowmul<float, 32, 64><<<grid, 256, 0, s>>>(RM_ARGS(float));
-  }
-#undef RM_ARGS
+namespace {
+
+template <typename C, int PER_SM>
+void launch_rowmul_cfg(const void* In, int64_t ldi, int K, const void* M, int m, int64_t n, void* Out, int64_t ldo,
+                       const int* run, cudaStream_t s, double c, const void* X2) {
+  using T = typename C::T;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    cudaFuncSetAttribute(k_rowmul<C, PER_SM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+  });
+  constexpr int64_t KV = C::KV, VW = C::VW;
+  const bool avec = ldi % KV == 0 && K % KV == 0 && !((uintptr_t)In & 15);
+  const bool xvec = m % KV == 0 && !((uintptr_t)M & 15);
+  const bool yvec = ldo % VW == 0 && m % VW == 0 && !(((uintptr_t)Out | (uintptr_t)X2) & 15);
+  dim3 grid(cdivi(n, C::BM), cdivi(m, C::BN));
+  k_rowmul<C, PER_SM><<<grid, C::NT, C::SMEM, s>>>((const T*)In, ldi, K, (const T*)M, m, n, (T*)Out, ldo, avec, xvec,
+                                                   yvec, (T)c, (const T*)X2, run);
 }
+
+}  // namespace
+
+void launch_rowmul(int tdtype, const void* In, int64_t ldi, int K, const void* M, int m, int64_t n, void* Out,
+                   int64_t ldo, const int* run, cudaStream_t s, double c, const void* X2) {
+  // tiles as wide as the output needs (the product's rule, see launch_ax)
+#define ROWMUL(T, BM, BN, TM, TN, BK, OCC) \
+  return launch_rowmul_cfg<GemmCfg<T, GA_SAME, BM, BN, TM, TN, BK>, OCC>(In, ldi, K, M, m, n, Out, ldo, run, s, c, X2)
+  if (tdtype == 0) {
+    if (m <= 16) ROWMUL(double, 64, 16, 4, 4, 16, 6);
+    if (m <= 32) ROWMUL(double, 64, 32, 4, 4, 16, 4);
+    ROWMUL(double, 64, 64, 4, 4, 16, 2);
+  }
+  if (m <= 16) ROWMUL(float, 128, 16, 4, 4, 32, 3);
+  if (m <= 32) ROWMUL(float, 128, 32, 8, 4, 32, 3);
+  ROWMUL(float, 128, 64, 8, 8, 16, 4);
+#undef ROWMUL
+}
+
+namespace {
+
+// Columns per k_utx tile (its chunks of rows: one wave of three CTAs per SM, of at least 256 rows).
+int utx_tq(int N) { return N <= 16 ? 16 : (N <= 32 ? 32 : 64); }
+
+template <typename T, int TQ, int VEC>
+void launch_utx(const LaiOp& op, const void* X, int64_t n, int N, int64_t ldx, const int* run, cudaStream_t s) {
+  static std::once_flag once;
+  std::call_once(once, [] {
+    cudaFuncSetAttribute(k_utx<T, TQ, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)utx_smem<T>(TQ));
+  });
+  dim3 grid(op.nch, cdivi(op.k, 64), cdivi(N, TQ));
+  k_utx<T, TQ, VEC><<<grid, 256, utx_smem<T>(TQ), s>>>((const T*)op.U, op.k, (const T*)X, n, N, ldx, op.chunk, op.nch,
+                                                       op.ng, (T*)op.xpart, op.lam, (T*)op.M, op.counters, run);
+}
+
+}  // namespace
 
 int lai_apply(const LaiOp& op, int tdtype, const Dims& d, const void* X, void* Y, double c, const void* X2,
               const void* P1, const void* P2, double* part, const int* run, cudaStream_t s) {
-  const int N = d.N;
-  const int64_t chunk = (d.n + op.nchunks - 1) / op.nchunks;
-  const bool narrow = N <= 32;
-  dim3 g1(op.nchunks, cdivi(op.k, 64), narrow ? 1 : cdivi(N, 64));
-#define UTX_ARGS(T) (const T*)op.U, op.k, (const T*)X, d.n, N, d.ld, chunk, (T*)op.xpart, op.lam, (T*)op.M, \
-                    op.counters, run
-  if (tdtype == 0) {
-    if (narrow) k_utx<double, 32, 32><<<g1, 256, 0, s>>>(UTX_ARGS(double));
-    else k_utx<double, 64, 32><<<g1, 256, 0, s>>>(UTX_ARGS(double));
-  } else {
-    if (narrow) k_utx<float, 32, 64><<<g1, 256, 0, s>>>(UTX_ARGS(float));
-    else k_utx<float, 64, 32><<<g1, 256, 0, s>>>(UTX_ARGS(float));
-  }
-#undef UTX_ARGS
-  launch_rowmul(tdtype, op.U, op.k, op.k, op.M, N, d.n, Y, d.ld, run, s);
+  const int N = d.N, v = tdtype == 0 ? 2 : 4;
+  const bool vec = op.k % v == 0 && N % v == 0 && d.ld % v == 0 && !((uintptr_t)X & 15);
+#define UTX(T, TQ, V) launch_utx<T, TQ, V>(op, X, d.n, N, d.ld, run, s)
+#define UTX_T(T, V)                                           \
+  if (utx_tq(N) == 16) { if (vec) UTX(T, 16, V); else UTX(T, 16, 1); } \
+  else if (utx_tq(N) == 32) { if (vec) UTX(T, 32, V); else UTX(T, 32, 1); } \
+  else { if (vec) UTX(T, 64, V); else UTX(T, 64, 1); }
+  if (tdtype == 0) { UTX_T(double, 2) } else { UTX_T(float, 4) }
+#undef UTX_T
+#undef UTX
+  // the dots are of the product before c X2: with them the finish pass adds it
+  const bool dots = P1 || P2;
+  launch_rowmul(tdtype, op.U, op.k, op.k, op.M, N, d.n, Y, d.ld, run, s, c, dots ? nullptr : X2);
+  if (!dots) return cdivi(d.n, kRowTile);
   return launch_ax_finish_impl(tdtype, d, Y, nullptr, 1, c, X2, P1, P2, part, 0, run, s);
 }
 
@@ -537,11 +471,16 @@ int lai_build(LaiOp& op, const AxArgs& A, int td, int64_t n, int k, int ell, int
   op.n = n;
   op.normA2 = host_sums;
   op.maxN = maxN;
-  op.nchunks = (int)std::max<int64_t>(1, std::min<int64_t>(152 / ((maxN + 63) / 64), n / 1024));
-  LCK(cudaMalloc(&op.xpart, (size_t)op.nchunks * k * maxN * esz));
+  const int tq = utx_tq(maxN);
+  const int64_t tiles = (int64_t)cdivi(k, 64) * cdivi(maxN, tq);
+  int64_t nch = std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 3 * 152 / tiles));
+  op.chunk = ((n + nch - 1) / nch + 31) / 32 * 32;
+  op.nch = (int)((n + op.chunk - 1) / op.chunk);
+  op.ng = gram_groups(op.nch);
+  LCK(cudaMalloc(&op.xpart, (size_t)tiles * (op.nch + op.ng) * 64 * tq * esz));
   LCK(cudaMalloc(&op.M, (size_t)k * maxN * esz));
-  LCK(cudaMalloc(&op.counters, 4096 * sizeof(unsigned)));
-  LCK(cudaMemsetAsync(op.counters, 0, 4096 * sizeof(unsigned), s));
+  LCK(cudaMalloc(&op.counters, (size_t)tiles * (1 + op.ng) * sizeof(unsigned)));
+  LCK(cudaMemsetAsync(op.counters, 0, (size_t)tiles * (1 + op.ng) * sizeof(unsigned), s));
   LCK(cudaStreamSynchronize(s));
   cleanup();
   return 0;

@@ -11,11 +11,12 @@ namespace snmf {
 struct LaiOp {
   void* U = nullptr;        // n x k, factor type, row-major (ld = k)
   double* lam = nullptr;    // k eigenvalues (device FP64)
-  double* xpart = nullptr;  // split-K partials of U^T X [chunk][k][N] (FP64)
+  void* xpart = nullptr;    // chunk partials of U^T X (factor type)
   void* M = nullptr;        // E U^T X, k x N (factor type)
   unsigned* counters = nullptr;  // arrival counters of the U^T X reduction
   int k = 0;
-  int nchunks = 0;
+  int64_t chunk = 0;        // rows per chunk of U^T X, chunks and their groups (gram_dev.cuh)
+  int nch = 0, ng = 0;
   int maxN = 0;
   int64_t n = 0;
   double normA2 = 0.0;      // sum of kept eigenvalues squared
@@ -38,8 +39,8 @@ void lai_free(LaiOp& op);
 // the SVD start |U E^1/2| of Sec. 4.1 guideline (4) for symmetric A (H_0^T equals it).
 void launch_svd_start(int tdtype, const LaiOp& op, int64_t n, int r, int b, void* W, cudaStream_t s);
 
-// Out (n x m, ldo) = In (n x K, ldi) M (K x m row-major), K <= 128 (factor type).
+// Out (n x m, ldo) = In (n x K, ldi) M (K x m row-major) (+ c X2, ldo), K <= 128 (factor type).
 void launch_rowmul(int tdtype, const void* In, int64_t ldi, int K, const void* M, int m, int64_t n, void* Out,
-                   int64_t ldo, const int* run, cudaStream_t s);
+                   int64_t ldo, const int* run, cudaStream_t s, double c = 0.0, const void* X2 = nullptr);
 
 }  // namespace snmf

@@ -41,30 +41,75 @@ __global__ void k_zstep(int64_t n, int r, int b, int64_t ld, const T* __restrict
 
 // Relaxed update W' = Proj[Z + phi beta D] (Alg. 1 line 4), optional linear reuse
 // AW' = AZ + phi beta AD (valid when nothing is clipped), clip-count partials.
-template <typename T>
+// V values of a row per access (16 bytes where r and the pitch allow it).
+template <typename T, int V>
 __global__ void __launch_bounds__(256)
 k_xupd(int64_t n, int r, int b, int64_t ld, const T* __restrict__ Z, const T* __restrict__ D,
        T* __restrict__ Xn, const T* __restrict__ AZ, const T* __restrict__ AD,
        T* __restrict__ AXn, const Ctl* __restrict__ ctl, double* __restrict__ part) {
+  struct alignas(V * sizeof(T)) Vec {
+    T v[V];
+  };
   __shared__ double sh[32];
   const int j = blockIdx.y;
   const int64_t i0 = (int64_t)blockIdx.x * kRowTile;
-  double clip = 0.0;
+  int clip = 0;
   if (ctl[j].active) {
     const T pb = (T)ctl[j].phibeta;
-    const int tile = kRowTile * r;
+    const int rv = r / V, tile = (int)min((int64_t)kRowTile, n - i0) * rv;
+#pragma unroll 4
     for (int e = threadIdx.x; e < tile; e += blockDim.x) {
-      const int64_t i = i0 + e / r;
-      if (i >= n) break;
-      const int64_t idx = i * ld + (int64_t)j * r + (e % r);
-      const T v = Z[idx] + pb * D[idx];
-      if (v < T(0)) clip += 1.0;
-      Xn[idx] = v > T(0) ? v : T(0);
-      if (AXn) AXn[idx] = AZ[idx] + pb * AD[idx];
+      const int i = e / rv;
+      const int64_t idx = (i0 + i) * ld + (int64_t)j * r + (e - i * rv) * V;
+      const Vec z = *reinterpret_cast<const Vec*>(Z + idx), d = *reinterpret_cast<const Vec*>(D + idx);
+      Vec x;
+#pragma unroll
+      for (int k = 0; k < V; ++k) {
+        const T v = z.v[k] + pb * d.v[k];
+        clip += v < T(0);
+        x.v[k] = v > T(0) ? v : T(0);
+      }
+      *reinterpret_cast<Vec*>(Xn + idx) = x;
+      if (AXn) {
+        const Vec az = *reinterpret_cast<const Vec*>(AZ + idx), ad = *reinterpret_cast<const Vec*>(AD + idx);
+        Vec y;
+#pragma unroll
+        for (int k = 0; k < V; ++k) y.v[k] = az.v[k] + pb * ad.v[k];
+        *reinterpret_cast<Vec*>(AXn + idx) = y;
+      }
     }
   }
-  clip = block_sum(clip, sh);
-  if (threadIdx.x == 0) part[((int64_t)blockIdx.x * b + j) * kNQ + 0] = clip;
+  const double total = block_sum((double)clip, sh);
+  if (threadIdx.x == 0) part[((int64_t)blockIdx.x * b + j) * kNQ + 0] = total;
+}
+
+// The same without the clip count: blockIdx.y = 64 rows, a thread V columns of every fourth row.
+template <typename T, int V>
+__global__ void __launch_bounds__(256)
+k_xnext(int64_t n, int r, int N, int64_t ld, const T* __restrict__ Z, const T* __restrict__ D, T* __restrict__ Xn,
+        const Ctl* __restrict__ ctl) {
+  struct alignas(V * sizeof(T)) Vec {
+    T v[V];
+  };
+  const int col = (blockIdx.x * 64 + (threadIdx.x & 63)) * V;
+  if (col >= N) return;
+  const Ctl& c = ctl[col / r];  // V divides r: one restart
+  if (!c.active) return;
+  const T pb = (T)c.phibeta;
+  const int64_t i0 = (int64_t)blockIdx.y * 64 + (threadIdx.x >> 6);
+#pragma unroll 4
+  for (int k = 0; k < 16; ++k) {
+    const int64_t i = i0 + 4 * k;
+    if (i >= n) break;
+    const Vec z = *reinterpret_cast<const Vec*>(Z + i * ld + col), d = *reinterpret_cast<const Vec*>(D + i * ld + col);
+    Vec x;
+#pragma unroll
+    for (int q = 0; q < V; ++q) {
+      const T v = z.v[q] + pb * d.v[q];
+      x.v[q] = v > T(0) ? v : T(0);
+    }
+    *reinterpret_cast<Vec*>(Xn + i * ld + col) = x;
+  }
 }
 
 template <typename T>
@@ -460,15 +505,33 @@ void launch_zstep(int tdtype, const Dims& d, const void* X, const void* g, void*
 int launch_xupd(int tdtype, const Dims& d, const void* Z, const void* D, void* Xn, const void* AZ,
                 const void* AD, void* AXn, const Ctl* ctl, double* part, cudaStream_t s) {
   dim3 grid(cdiv(d.n, kRowTile), d.b);
-  if (tdtype == 0)
-    k_xupd<double><<<grid, 256, 0, s>>>(d.n, d.r, d.b, d.ld, (const double*)Z, (const double*)D,
-                                        (double*)Xn, (const double*)AZ, (const double*)AD,
-                                        (double*)AXn, ctl, part);
-  else
-    k_xupd<float><<<grid, 256, 0, s>>>(d.n, d.r, d.b, d.ld, (const float*)Z, (const float*)D,
-                                       (float*)Xn, (const float*)AZ, (const float*)AD, (float*)AXn,
-                                       ctl, part);
+  const int v = tdtype == 0 ? 2 : 4;
+  const uintptr_t all = (uintptr_t)Z | (uintptr_t)D | (uintptr_t)Xn | (uintptr_t)AZ | (uintptr_t)AD | (uintptr_t)AXn;
+  const bool vec = d.r % v == 0 && d.ld % v == 0 && !(all & 15);
+#define XUPD(T, V)                                                                                                  \
+  k_xupd<T, V><<<grid, 256, 0, s>>>(d.n, d.r, d.b, d.ld, (const T*)Z, (const T*)D, (T*)Xn, (const T*)AZ, (const T*)AD, \
+                                    (T*)AXn, ctl, part)
+  if (tdtype == 0) {
+    if (vec) XUPD(double, 2); else XUPD(double, 1);
+  } else {
+    if (vec) XUPD(float, 4); else XUPD(float, 1);
+  }
+#undef XUPD
   return grid.x;
+}
+
+void launch_xnext(int tdtype, const Dims& d, const void* Z, const void* D, void* Xn, const Ctl* ctl, cudaStream_t s) {
+  const int v = tdtype == 0 ? 2 : 4;
+  const bool vec = d.r % v == 0 && d.ld % v == 0 && !(((uintptr_t)Z | (uintptr_t)D | (uintptr_t)Xn) & 15);
+#define XNEXT(T, V)                                                                                            \
+  k_xnext<T, V><<<dim3(cdiv(d.N, 64 * V), cdiv(d.n, 64)), 256, 0, s>>>(d.n, d.r, d.N, d.ld, (const T*)Z, (const T*)D, \
+                                                                       (T*)Xn, ctl)
+  if (tdtype == 0) {
+    if (vec) XNEXT(double, 2); else XNEXT(double, 1);
+  } else {
+    if (vec) XNEXT(float, 4); else XNEXT(float, 1);
+  }
+#undef XNEXT
 }
 
 void launch_copy_live(int tdtype, const Dims& d, const void* src, void* dst, const Ctl* ctl,

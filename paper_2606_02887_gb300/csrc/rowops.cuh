@@ -47,7 +47,6 @@ struct RowArgs {
   double* part;
   int ctl_mode;        // CTL_*: control step run by the last CTA of each restart
   unsigned* counters;  // per-restart arrival counters (zero between launches)
-  unsigned* gcounters; // rowstep: arrival counters of a restart's groups of CTAs (NULL: no groups)
   const double* G64fix;
   Params P;
   int bm;              // general body, FP32: rows per CTA (32 or 64; 0 = built-in choice)
@@ -58,8 +57,8 @@ struct RowArgs {
 // given Z (graph term), and the relaxed update that recomputes Z and D.
 struct RowStepPlan {
   int threads, mr;  // threads per CTA, rows per thread
-  int rows, slots;  // rows per CTA, CTAs (partial slots) per restart
-  int groups;       // groups of CTAs per restart: their records follow the slots (0: none)
+  int rows, tiles;  // rows per tile, tiles per restart
+  int slots;        // CTAs (partial slots) per restart
 };
 RowStepPlan rowstep_plan(int tdtype, int64_t n, int r, int b);
 void launch_rowstep_grad(int tdtype, const RowArgs& a, const RowStepPlan& pl, cudaStream_t s);
@@ -91,7 +90,7 @@ struct GramPlan {
   int64_t chunk;
   size_t part_elems, counters;
 };
-GramPlan gram_plan(int64_t n, int r, int b);
+GramPlan gram_plan(int tdtype, int64_t n, int r, int b);
 // The split of the eigen-sketch's Grams (n x ell, one level of at most 152 chunks over the tiles).
 // Which eigenpairs a sketch keeps near its cut, where they are close, depends on the last bits
 // of these sums: their order is part of what a seed reproduces.
@@ -109,6 +108,8 @@ void launch_zstep(int tdtype, const Dims& d, const void* X, const void* g, void*
                   cudaStream_t s);
 int launch_xupd(int tdtype, const Dims& d, const void* Z, const void* D, void* Xn, const void* AZ,
                 const void* AD, void* AXn, const Ctl* ctl, double* part, cudaStream_t s);
+// Xn = Proj[Z + phi beta D] of the live restarts alone (the graph-regularised block)
+void launch_xnext(int tdtype, const Dims& d, const void* Z, const void* D, void* Xn, const Ctl* ctl, cudaStream_t s);
 void launch_copy_live(int tdtype, const Dims& d, const void* src, void* dst, const Ctl* ctl,
                       cudaStream_t s);
 // rho = scale ||G||_2 + shift per restart (shift: gamma ||L||_2 of a graph-regularised block)

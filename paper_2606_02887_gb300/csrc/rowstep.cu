@@ -11,17 +11,17 @@ namespace snmf {
 namespace {
 
 template <typename T, int STEP, int NC, int MR>
-__global__ void __launch_bounds__(256, 2) k_rowstep(RowArgs a, bool vec) {
+__global__ void __launch_bounds__(256, 2) k_rowstep(RowArgs a, int tiles, bool vec) {
   extern __shared__ __align__(16) unsigned char rsm[];
-  rowstep_body<T, STEP, NC, MR>(a, blockIdx.y, blockIdx.x, gridDim.x, vec, reinterpret_cast<T*>(rsm));
+  rowstep_body<T, STEP, NC, MR>(a, blockIdx.y, blockIdx.x, gridDim.x, tiles, vec, reinterpret_cast<T*>(rsm));
 }
 
 template <typename T, int STEP, int NC, int MR>
 void launch_t(const RowArgs& a, const RowStepPlan& pl, cudaStream_t s) {
   static std::once_flag once;
-  std::call_once(once, [] {  // the most over the ranks: r = 64 with 256 threads
+  std::call_once(once, [] {  // the most over the ranks: r = 64 with 256 threads and every input
     cudaFuncSetAttribute(k_rowstep<T, STEP, NC, MR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)rowstep_smem<T>(64, 256, MR) + 32 * 1024);
+                         (int)rowstep_smem<T>(64, 256, MR, 7));
   });
   uintptr_t all = 0;
   for (const void* p : {a.X, a.g_in, a.B, a.LX, (const void*)a.Xout, (const void*)a.gout, (const void*)a.Dout,
@@ -29,7 +29,8 @@ void launch_t(const RowArgs& a, const RowStepPlan& pl, cudaStream_t s) {
     all |= (uintptr_t)p;
   const bool vec = a.r % 4 == 0 && a.ld % 4 == 0 && !(all & 15);
   dim3 grid((unsigned)pl.slots, (unsigned)a.b);
-  k_rowstep<T, STEP, NC, MR><<<grid, pl.threads, rowstep_smem<T>(a.r, pl.threads, MR), s>>>(a, vec);
+  k_rowstep<T, STEP, NC, MR><<<grid, pl.threads, rowstep_smem<T>(a.r, pl.threads, MR, rowstep_inputs(STEP, a)), s>>>(a, pl.tiles,
+                                                                                                             vec);
 }
 
 }  // namespace
@@ -49,8 +50,11 @@ RowStepPlan rowstep_plan(int tdtype, int64_t n, int r, int b) {
     }
   }
   pl.rows = rowstep_rows(r, pl.threads, pl.mr);
-  pl.slots = (int)((n + pl.rows - 1) / pl.rows);
-  pl.groups = rowstep_groups(pl.slots);
+  pl.tiles = (int)((n + pl.rows - 1) / pl.rows);
+  // 512 threads per SM over the restarts, each CTA as many tiles as the next one
+  const int most = std::max(1, (152 * (512 / pl.threads) + b - 1) / b);
+  const int each = (pl.tiles + most - 1) / most;
+  pl.slots = (pl.tiles + each - 1) / each;
   return pl;
 }
 

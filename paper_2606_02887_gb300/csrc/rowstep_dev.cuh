@@ -14,12 +14,17 @@
 // Partial layout and control steps are those of the general row kernel (RowArgs).  A step moves
 // 4 + 6 arrays of n x r instead of the 6 + 8 of stored Z and D.
 //
-// CTA: TY MR rows of one restart, all r columns; thread (tx, ty), tx < ceil(r / 4), owns columns
-// 4 tx .. of rows ty + TY p, p < MR, in the loads, the row product and the epilogue alike, so inputs
-// stay in registers from the one to the other and nothing is transposed: the operand tile goes to
-// shared memory row-major (stride 4 more than the columns), a thread reads 16 bytes along k of its
-// rows and 16 bytes of each row of G.  Ranks between the powers of two pay for their next
-// multiple of 4 only.  Bound by HBM for long factors and by launch latency for short ones.
+// CTA: tiles of TY MR rows of one restart, all r columns; thread (tx, ty), tx < ceil(r / 4), owns
+// columns 4 tx .. of rows ty + TY p, p < MR, in the loads, the row product and the epilogue alike, so
+// inputs stay in registers from the one to the other and nothing is transposed: the operand tile
+// goes to shared memory row-major (stride 4 more than the columns), a thread reads 16 bytes along k
+// of its rows and 16 bytes of each row of G.  Ranks between the powers of two pay for their next
+// multiple of 4 only.  A CTA walks several tiles: each thread copies its own inputs of the next tile
+// to shared memory (asynchronously, no barrier) as soon as it has read the current one's there, the
+// operand's inputs first, B and what else the epilogue reads after it; G is read once, and one
+// record of partials, in FP64 over the tiles, leaves the CTA.  Bound by HBM for long factors (a
+// CTA per tile, without copies ahead: n = 2e6, r = 32 block-start gradient 407 us, D step 471, update
+// 501) and by launch latency for short ones.
 #pragma once
 
 #include "rowops_dev.cuh"
@@ -29,10 +34,6 @@ namespace snmf {
 namespace {
 
 enum { RS_GRAD = 0, RS_D, RS_DZ, RS_U };
-
-constexpr int kRowGroup = 128;  // CTAs of a restart whose partial records are summed together
-// groups of a restart of `per` CTAs (0: summed at once); their records follow the CTAs' in `part`
-__host__ __device__ inline int rowstep_groups(int per) { return per > 4 * kRowGroup ? (per + kRowGroup - 1) / kRowGroup : 0; }
 
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
@@ -51,25 +52,33 @@ __device__ __forceinline__ T upd(T z, T d, T pb) { return proj0(fma_rn(pb, d, z)
 template <typename T>
 __host__ __device__ constexpr int rowstep_mr() { return sizeof(T) == 4 ? 4 : 2; }
 
-// rows of a CTA and dynamic shared memory of rank r with `threads` threads and MR rows each
+// rows of a tile, the input arrays of a step, and the dynamic shared memory of rank r with
+// `threads` threads, mr rows each and `nin` inputs
 __host__ __device__ inline int rowstep_rows(int r, int threads, int mr) { return threads / ((r + 3) / 4) * mr; }
+inline int rowstep_inputs(int step, const RowArgs& a) {
+  if (step == RS_D) return 3;  // X, g, B
+  if (step == RS_U) return 4;  // X, g, g(Z), B
+  int k = 2 + (a.LX != nullptr);
+  if (step == RS_DZ) return k + 2;
+  return k + (a.Xold ? 2 : 0) + (a.Zold ? 2 : 0);
+}
 template <typename T>
-__host__ __device__ inline size_t rowstep_smem(int r, int threads, int mr) {
+__host__ __device__ inline size_t rowstep_smem(int r, int threads, int mr, int nin) {
   const int c = (r + 3) / 4 * 4;
-  return ((size_t)rowstep_rows(r, threads, mr) * (c + 4) + (size_t)c * c) * sizeof(T);
+  return ((size_t)rowstep_rows(r, threads, mr) * (c + 4) + (size_t)c * c + (size_t)nin * mr * threads * 4) * sizeof(T);
 }
 
-// Quad columns of one row of a global array: one or two 16-byte accesses, or single values
+// four columns of one row of a global array: 16-byte accesses, or single values of the w that exist
 template <typename T>
-__device__ __forceinline__ Quad<T> load_quad(const T* p, bool vec, int w) {
-  Quad<T> v;
+__device__ __forceinline__ void copy_quad(Quad<T>* dst, const T* base, int64_t off, bool on, bool vec, int w) {
   if (vec) {
-    v = *reinterpret_cast<const Quad<T>*>(p);
+    const char* p = reinterpret_cast<const char*>(on ? base + off : base);
+#pragma unroll
+    for (int q = 0; q < (int)sizeof(Quad<T>); q += 16) cp_async<16>(reinterpret_cast<char*>(dst) + q, p + q, on);
   } else {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) v.v[q] = q < w ? p[q] : T(0);
+    for (int q = 0; q < 4; ++q) cp_async<(int)sizeof(T)>(&dst->v[q], on && q < w ? base + off + q : base, on && q < w);
   }
-  return v;
 }
 template <typename T>
 __device__ __forceinline__ void store_quad(T* p, const Quad<T>& v, bool vec, int w) {
@@ -139,235 +148,267 @@ __device__ __forceinline__ T warp_sum8(const T (&v)[8]) {
   return c;
 }
 
-// CTA `tile` of `per` of restart j.  vec: every row of the restart starts on 16 bytes in all arrays
-// (r and the pitch multiples of 4).  sm: rowstep_smem bytes.
+// CTA `cta` of `per` of restart j: its tiles cta, cta + per, ... of `tiles`.  vec: every row of the
+// restart starts on 16 bytes in all arrays (r and the pitch multiples of 4).  sm: rowstep_smem bytes.
 template <typename T, int STEP, int NC, int MR>
-__device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int tile, unsigned per, bool vec, T* sm) {
-  __shared__ T shq[8][8];
+__device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, int per, int tiles, bool vec, T* sm) {
+  __shared__ double shq[8][8];
   __shared__ unsigned ticket;
   const Ctl& cj = a.ctl[j];
   const bool live = cj.active && !(a.run && *a.run == 0);
-  T dq[8];
-#pragma unroll
-  for (int m = 0; m < 8; ++m) dq[m] = T(0);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double total = 0.0;  // lane m < 8: the warp's sum of value m over the tiles
   if (live) {
-    const int r = a.r, TX = (r + 3) / 4, c4 = 4 * TX, ls = c4 + 4, TY = (int)blockDim.x / TX;
+    const int r = a.r, TX = (r + 3) / 4, c4 = 4 * TX, ls = c4 + 4, nt = blockDim.x, TY = nt / TX;
     const int t = threadIdx.x, ty = t / TX, tx = t - ty * TX;
     T* As = sm;
     T* Gs = sm + (size_t)TY * MR * ls;
+    Quad<T>* in = reinterpret_cast<Quad<T>*>(Gs + c4 * c4) + t;  // input i of row k at in[(i MR + k) nt]
     const bool on = ty < TY;  // the block may hold a few threads more than TX TY
     const int w = r - 4 * tx;
-    const int64_t row0 = (int64_t)tile * (TY * MR) + ty;
-    const int64_t off0 = row0 * a.ld + (int64_t)j * r + 4 * tx, step = (int64_t)TY * a.ld;
+    const int64_t colj = (int64_t)j * r + 4 * tx;
     const T inv_rho = (T)(1.0 / cj.rho);
     const T alpha0 = (T)(NC == 1 ? cj.alpha : cj.cand_alpha[STEP == RS_U ? (cj.dsel ? 1 : 0) : 0]);
     const T alpha1 = (T)(NC == 1 ? cj.alpha : cj.cand_alpha[1]);
     const T pb = (T)cj.phibeta;
     const T gam = (T)a.gamma;
-    bool rv[MR];
-    Quad<T> x[MR], g[MR], z[MR], b[MR];
-    auto get = [&](const void* p, int k) {
-      Quad<T> v = {{T(0), T(0), T(0), T(0)}};
-      if (rv[k]) v = load_quad((const T*)p + off0 + k * step, vec, w);
-      return v;
-    };
-    auto put = [&](void* p, int k, const Quad<T>& v) {
-      if (rv[k]) store_quad((T*)p + off0 + k * step, v, vec, w);
-    };
+    // inputs in the order of their slots
+    const bool lx = (STEP == RS_GRAD || STEP == RS_DZ) && a.LX, old = STEP == RS_GRAD && a.Xold,
+               zold = STEP == RS_GRAD && a.Zold;
+    const int iL = 2, iO = 2 + lx, iZ = iO + (old ? 2 : 0);
+    auto copy = [&](int tile, int i, const void* p) {
+      const int64_t row0 = (int64_t)tile * (TY * MR) + ty;
 #pragma unroll
-    for (int k = 0; k < MR; ++k) rv[k] = on && row0 + (int64_t)k * TY < a.n;
-    // every input of the tile in flight before the first use
-#pragma unroll
-    for (int k = 0; k < MR; ++k) {
-      x[k] = get(STEP == RS_U ? a.Xout : a.X, k);
-      if (STEP == RS_D) g[k] = get(a.g_in, k);
-      if (STEP == RS_U) {
-        g[k] = get(a.gout, k);
-        z[k] = get(a.gZold, k);
+      for (int k = 0; k < MR; ++k) {
+        const int64_t row = row0 + (int64_t)k * TY;
+        copy_quad(in + (i * MR + k) * nt, (const T*)p, row * a.ld + colj, on && row < a.n, vec, w);
       }
-      b[k] = get(a.B, k);
-    }
+    };
+    auto fetch_operand = [&](int tile) {  // one copy group each, empty past the last tile
+      if (tile < tiles) {
+        copy(tile, 0, STEP == RS_U ? a.Xout : a.X);
+        if (STEP == RS_D) copy(tile, 2, a.g_in);
+        if (STEP == RS_U) {
+          copy(tile, 2, a.gout);
+          copy(tile, 3, a.gZold);
+        }
+      }
+      cp_async_commit();
+    };
+    auto fetch_rest = [&](int tile) {
+      if (tile < tiles) {
+        copy(tile, 1, a.B);
+        if (lx) copy(tile, iL, a.LX);
+        if (STEP == RS_DZ) {
+          copy(tile, iO, a.Wcur);
+          copy(tile, iO + 1, a.gWcur);
+        }
+        if (old) {
+          copy(tile, iO, a.Xold);
+          copy(tile, iO + 1, a.gold);
+        }
+        if (zold) {
+          copy(tile, iZ, a.Zold);
+          copy(tile, iZ + 1, a.gZold);
+        }
+      }
+      cp_async_commit();
+    };
+    fetch_operand(cta);
+    fetch_rest(cta);
     {
       const T* G = (const T*)a.G + (int64_t)j * r * r;
-      for (int e = t; e < c4 * c4; e += blockDim.x) {
+      for (int e = t; e < c4 * c4; e += nt) {
         const int p = e / c4, q = e - p * c4;
         Gs[e] = p < r && q < r ? G[p * r + q] : T(0);
       }
     }
-    // the operand tile: X, Z or X' (z: g(Z) on entry of RS_U, then X')
+    for (int tile = cta; tile < tiles; tile += per) {
+      const int64_t row0 = (int64_t)tile * (TY * MR) + ty;
+      const int64_t off0 = row0 * a.ld + colj, step = (int64_t)TY * a.ld;
+      T dq[8];
 #pragma unroll
-    for (int k = 0; k < MR; ++k) {
-      Quad<T> op = x[k];
+      for (int m = 0; m < 8; ++m) dq[m] = T(0);
+      bool rv[MR];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (STEP == RS_D) op.v[q] = zstep(x[k].v[q], g[k].v[q], inv_rho);
-        if (STEP == RS_U) {
-          const T zz = zstep(x[k].v[q], g[k].v[q], inv_rho);
-          op.v[q] = upd(zz, dir(zz, z[k].v[q], alpha0), pb);
-        }
-      }
-      if (on) *reinterpret_cast<Quad<T>*>(As + (ty + k * TY) * ls + 4 * tx) = op;
-    }
-    __syncthreads();
-    Quad<T> acc[MR];
-    if (on) rowstep_product<T, MR>(As, ls, Gs, c4, tx, ty, TY, acc);
-    if (STEP == RS_GRAD) {
+      for (int k = 0; k < MR; ++k) rv[k] = on && row0 + (int64_t)k * TY < a.n;
+      auto get = [&](int i, int k) { return in[(i * MR + k) * nt]; };
+      auto put = [&](void* p, int k, const Quad<T>& v) {
+        if (rv[k]) store_quad((T*)p + off0 + k * step, v, vec, w);
+      };
+      cp_async_wait<1>();
+      Quad<T> x[MR], g[MR], z[MR];
 #pragma unroll
       for (int k = 0; k < MR; ++k) {
-        if (!rv[k]) continue;
-        Quad<T> gn, l, zn;
-        if (a.LX) l = get(a.LX, k);
+        x[k] = get(0, k);
+        if (STEP == RS_D || STEP == RS_U) g[k] = get(2, k);
+        if (STEP == RS_U) z[k] = get(3, k);
+      }
+      fetch_operand(tile + per);
+      // the operand tile: X, Z or X'
+#pragma unroll
+      for (int k = 0; k < MR; ++k) {
+        Quad<T> op = x[k];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          const T xv = x[k].v[q], bv = b[k].v[q];
-          T gv = acc[k].v[q] - bv;
-          if (a.LX) gv += gam * l.v[q];
-          gn.v[q] = gv;
-          zn.v[q] = zstep(xv, gv, inv_rho);
-          if (q >= w) continue;
-          const T pg = xv > T(0) ? gv : (gv < T(0) ? gv : T(0));
-          dq[0] += pg * pg;
-          dq[1] += T(0.5) * (gv - bv) * xv;
-          if (xv == T(0)) dq[6] += T(1);
+          if (STEP == RS_D) op.v[q] = zstep(x[k].v[q], g[k].v[q], inv_rho);
+          if (STEP == RS_U) {
+            const T zz = zstep(x[k].v[q], g[k].v[q], inv_rho);
+            op.v[q] = upd(zz, dir(zz, z[k].v[q], alpha0), pb);
+          }
         }
-        if (a.Xold) {
-          const Quad<T> xo = get(a.Xold, k), go = get(a.gold, k);
+        if (on) *reinterpret_cast<Quad<T>*>(As + (ty + k * TY) * ls + 4 * tx) = op;
+      }
+      __syncthreads();
+      Quad<T> acc[MR];
+      if (on) rowstep_product<T, MR>(As, ls, Gs, c4, tx, ty, TY, acc);
+      cp_async_wait<1>();
+      if (STEP == RS_GRAD) {
+#pragma unroll
+        for (int k = 0; k < MR; ++k) {
+          if (!rv[k]) continue;
+          Quad<T> gn, l, zn;
+          const Quad<T> b = get(1, k);
+          if (lx) l = get(iL, k);
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            const T s = x[k].v[q] - xo.v[q], y = gn.v[q] - go.v[q];
+            const T xv = x[k].v[q], bv = b.v[q];
+            T gv = acc[k].v[q] - bv;
+            if (lx) gv += gam * l.v[q];
+            gn.v[q] = gv;
+            zn.v[q] = zstep(xv, gv, inv_rho);
             if (q >= w) continue;
+            const T pg = xv > T(0) ? gv : (gv < T(0) ? gv : T(0));
+            dq[0] += pg * pg;
+            dq[1] += T(0.5) * (gv - bv) * xv;
+            if (xv == T(0)) dq[6] += T(1);
+          }
+          if (old) {
+            const Quad<T> xo = get(iO, k), go = get(iO + 1, k);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const T s = x[k].v[q] - xo.v[q], y = gn.v[q] - go.v[q];
+              if (q >= w) continue;
+              dq[2] += s * s;
+              dq[3] += s * y;
+              dq[4] += y * y;
+            }
+          }
+          if (zold) {
+            const Quad<T> zo = get(iZ, k), gz = get(iZ + 1, k);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              if (q < w) dq[5] += T(0.5) * (x[k].v[q] - zo.v[q]) * (gn.v[q] + gz.v[q]);
+          }
+          if (a.gout) put(a.gout, k, gn);
+          if (a.Xout) put(a.Xout, k, x[k]);
+          if (a.Znext) put(a.Znext, k, zn);
+        }
+      } else if (STEP == RS_U) {
+#pragma unroll
+        for (int k = 0; k < MR; ++k) {
+          if (!rv[k]) continue;
+          Quad<T> xn, gn;
+          const Quad<T> b = get(1, k);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const T xv = x[k].v[q], gv = g[k].v[q], gz = z[k].v[q], bv = b.v[q];
+            const T zz = zstep(xv, gv, inv_rho);
+            const T xw = upd(zz, dir(zz, gz, alpha0), pb);
+            const T gw = acc[k].v[q] - bv;
+            xn.v[q] = xw;
+            gn.v[q] = gw;
+            if (q >= w) continue;
+            const T pg = xw > T(0) ? gw : (gw < T(0) ? gw : T(0));
+            dq[0] += pg * pg;
+            dq[1] += T(0.5) * (gw - bv) * xw;
+            const T s = xw - xv, y = gw - gv;
             dq[2] += s * s;
             dq[3] += s * y;
             dq[4] += y * y;
+            dq[5] += T(0.5) * (xw - zz) * (gw + gz);
+            if (xw == T(0)) dq[6] += T(1);
           }
+          put(a.Xout, k, xn);
+          put(a.gout, k, gn);
         }
-        if (a.Zold) {
-          const Quad<T> zo = get(a.Zold, k), gz = get(a.gZold, k);
+      } else {
+        // RS_D / RS_DZ: g(Z), D, their inner products; then <D G, D> with D as the operand tile
+        Quad<T> d0[MR], d1[NC == 2 ? MR : 1];
 #pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (q < w) dq[5] += T(0.5) * (x[k].v[q] - zo.v[q]) * (gn.v[q] + gz.v[q]);
-        }
-        if (a.gout) put(a.gout, k, gn);
-        if (a.Xout) put(a.Xout, k, x[k]);
-        if (a.Znext) put(a.Znext, k, zn);
-      }
-    } else if (STEP == RS_U) {
-#pragma unroll
-      for (int k = 0; k < MR; ++k) {
-        if (!rv[k]) continue;
-        Quad<T> xn, gn;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const T xv = x[k].v[q], gv = g[k].v[q], gz = z[k].v[q], bv = b[k].v[q];
-          const T zz = zstep(xv, gv, inv_rho);
-          const T xw = upd(zz, dir(zz, gz, alpha0), pb);
-          const T gw = acc[k].v[q] - bv;
-          xn.v[q] = xw;
-          gn.v[q] = gw;
-          if (q >= w) continue;
-          const T pg = xw > T(0) ? gw : (gw < T(0) ? gw : T(0));
-          dq[0] += pg * pg;
-          dq[1] += T(0.5) * (gw - bv) * xw;
-          const T s = xw - xv, y = gw - gv;
-          dq[2] += s * s;
-          dq[3] += s * y;
-          dq[4] += y * y;
-          dq[5] += T(0.5) * (xw - zz) * (gw + gz);
-          if (xw == T(0)) dq[6] += T(1);
-        }
-        put(a.Xout, k, xn);
-        put(a.gout, k, gn);
-      }
-    } else {
-      // RS_D / RS_DZ: g(Z), D, their inner products; then <D G, D> with D as the operand tile
-      Quad<T> d0[MR], d1[NC == 2 ? MR : 1];
-#pragma unroll
-      for (int k = 0; k < MR; ++k) {
-        Quad<T> gz, l, wc, gw;
-        if (STEP == RS_DZ) {
-          if (a.LX) l = get(a.LX, k);
-          wc = get(a.Wcur, k);
-          gw = get(a.gWcur, k);
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const T zz = STEP == RS_D ? zstep(x[k].v[q], g[k].v[q], inv_rho) : x[k].v[q];
-          const T xv = STEP == RS_D ? x[k].v[q] : wc.v[q], gx = STEP == RS_D ? g[k].v[q] : gw.v[q];
-          T gv = acc[k].v[q] - b[k].v[q];
-          if (STEP == RS_DZ && a.LX) gv += gam * l.v[q];
-          gz.v[q] = gv;
-          const bool in = rv[k] && q < w;
-          const T d = in ? dir(zz, gv, alpha0) : T(0);
-          d0[k].v[q] = d;
-          if (NC == 2) d1[NC == 2 ? k : 0].v[q] = in ? dir(zz, gv, alpha1) : T(0);
-          if (!in) continue;
-          dq[0] += gv * d;
-          dq[1] += d * d;
-          dq[2] += T(0.5) * (zz - xv) * (gv + gx);
-          if (NC == 2) {
-            const T e = d1[NC == 2 ? k : 0].v[q];
-            dq[5] += gv * e;
-            dq[6] += e * e;
+        for (int k = 0; k < MR; ++k) {
+          Quad<T> gz, l, wc, gw;
+          const Quad<T> b = get(1, k);
+          if (STEP == RS_DZ) {
+            if (lx) l = get(iL, k);
+            wc = get(iO, k);
+            gw = get(iO + 1, k);
           }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const T zz = STEP == RS_D ? zstep(x[k].v[q], g[k].v[q], inv_rho) : x[k].v[q];
+            const T xv = STEP == RS_D ? x[k].v[q] : wc.v[q], gx = STEP == RS_D ? g[k].v[q] : gw.v[q];
+            T gv = acc[k].v[q] - b.v[q];
+            if (lx) gv += gam * l.v[q];
+            gz.v[q] = gv;
+            const bool ok = rv[k] && q < w;
+            const T d = ok ? dir(zz, gv, alpha0) : T(0);
+            d0[k].v[q] = d;
+            if (NC == 2) d1[NC == 2 ? k : 0].v[q] = ok ? dir(zz, gv, alpha1) : T(0);
+            if (!ok) continue;
+            dq[0] += gv * d;
+            dq[1] += d * d;
+            dq[2] += T(0.5) * (zz - xv) * (gv + gx);
+            if (NC == 2) {
+              const T e = d1[NC == 2 ? k : 0].v[q];
+              dq[5] += gv * e;
+              dq[6] += e * e;
+            }
+          }
+          put(a.gZout, k, gz);
+          if (STEP == RS_DZ) put(a.Dout, k, d0[k]);
         }
-        put(a.gZout, k, gz);
-        if (STEP == RS_DZ) put(a.Dout, k, d0[k]);
-      }
+        fetch_rest(tile + per);
 #pragma unroll
-      for (int m = 0; m < NC; ++m) {
-        __syncthreads();  // every thread is done with the operand tile
-#pragma unroll
-        for (int k = 0; k < MR; ++k)
-          if (on) *reinterpret_cast<Quad<T>*>(As + (ty + k * TY) * ls + 4 * tx) = m == 0 ? d0[k] : d1[NC == 2 ? k : 0];
-        __syncthreads();
-        if (on) {
-          rowstep_product<T, MR>(As, ls, Gs, c4, tx, ty, TY, acc);
-          T qq = T(0);
+        for (int m = 0; m < NC; ++m) {
+          __syncthreads();  // every thread is done with the operand tile
 #pragma unroll
           for (int k = 0; k < MR; ++k)
+            if (on) *reinterpret_cast<Quad<T>*>(As + (ty + k * TY) * ls + 4 * tx) = m == 0 ? d0[k] : d1[NC == 2 ? k : 0];
+          __syncthreads();
+          if (on) {
+            rowstep_product<T, MR>(As, ls, Gs, c4, tx, ty, TY, acc);
+            T qq = T(0);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) qq = fma(acc[k].v[q], m == 0 ? d0[k].v[q] : d1[NC == 2 ? k : 0].v[q], qq);
-          dq[m == 0 ? 4 : 7] = qq;
+            for (int k = 0; k < MR; ++k)
+#pragma unroll
+              for (int q = 0; q < 4; ++q) qq = fma(acc[k].v[q], m == 0 ? d0[k].v[q] : d1[NC == 2 ? k : 0].v[q], qq);
+            dq[m == 0 ? 4 : 7] = qq;
+          }
         }
       }
+      if (STEP == RS_GRAD || STEP == RS_U) fetch_rest(tile + per);
+      total += (double)warp_sum8(dq);
+      if (tile + per < tiles) __syncthreads();  // the operand tile is written again
     }
   }
   // fixed-order CTA sums, the partial record, and the control step in the restart's last CTA
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  {
-    const T v = warp_sum8(dq);
-    if (lane < 8) shq[lane][wid] = v;
-  }
+  if (lane < 8) shq[lane][wid] = total;
   __syncthreads();
   if (threadIdx.x < 8) {
-    T v = T(0);
+    double v = 0.0;
     for (int u = 0; u < (int)(blockDim.x >> 5); ++u) v += shq[threadIdx.x][u];
-    a.part[((int64_t)tile * a.b + j) * kNQ + threadIdx.x] = (double)v;
+    a.part[((int64_t)cta * a.b + j) * kNQ + threadIdx.x] = v;
   }
   if (!a.ctl_mode) return;
-  // the restart's last CTA runs its control step.  Where many CTAs make up a restart, the last of
-  // each kRowGroup of them sums the group's records first (n = 2e6, r = 32: 31250 CTAs)
-  auto arrive = [&](unsigned* counter, unsigned of) {
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      ticket = atomicAdd(counter, 1u);
-      if (ticket == of - 1) *counter = 0u;  // ready for the next launch
-    }
-    __syncthreads();
-    return ticket == of - 1;
-  };
-  const int ng = a.gcounters ? rowstep_groups((int)per) : 0;
-  if (!ng) {
-    if (arrive(&a.counters[j], per)) control_tail<8>(a, j, 0, (int)per, NC);
-    return;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    ticket = atomicAdd(&a.counters[j], 1u);
+    if (ticket == (unsigned)per - 1) a.counters[j] = 0u;  // ready for the next launch
   }
-  const int grp = tile / kRowGroup, first = grp * kRowGroup, size = min(kRowGroup, (int)per - first);
-  if (!arrive(&a.gcounters[(int64_t)j * ng + grp], size)) return;
-  __shared__ double rec[8][8], qs[8];
-  slot_sums<8>(a.part + (int64_t)first * a.b * kNQ, size, a.b, j, rec, qs);
-  if (threadIdx.x < 8) a.part[((int64_t)(per + grp) * a.b + j) * kNQ + threadIdx.x] = qs[threadIdx.x];
-  if (arrive(&a.counters[j], ng)) control_tail<8>(a, j, (int)per, ng, NC);
+  __syncthreads();
+  if (ticket == (unsigned)per - 1) control_tail<8>(a, j, 0, per, NC);
 }
 
 }  // namespace
