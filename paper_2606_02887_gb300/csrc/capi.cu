@@ -1833,6 +1833,7 @@ snmf_status snmf_controller_data(snmf_handle h, float* feat, float* targ, int ca
 
 snmf_status snmf_destroy(snmf_handle h) {
   if (!h) return SNMF_OK;
+  workspace_trim();
   if (h->bt) {
     batch_destroy(h->bt);
     delete h;

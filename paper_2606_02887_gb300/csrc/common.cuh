@@ -209,4 +209,9 @@ void launch_assign(int tdtype, const void* F, int64_t n, int64_t ld, int64_t col
 // on A's pattern), so that L X = X + out X.
 void launch_normalized_adjacency(const AxArgs& a, int tdtype, int64_t n, double* s, void* out, cudaStream_t st);
 
+// Workspaces of calls without a handle (pool.cu): stream-ordered, from the library's pool.
+cudaError_t workspace_alloc(void** p, size_t bytes, cudaStream_t s);
+void workspace_free(void* p, cudaStream_t s);
+void workspace_trim();  // gives back what the current device's pool holds unused
+
 }  // namespace snmf

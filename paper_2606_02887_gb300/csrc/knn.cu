@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "../../include/snmf.h"
+#include "ax_tc.cuh"
 #include "common.cuh"
 
 namespace snmf {
@@ -48,14 +49,22 @@ __device__ __forceinline__ void knn_insert(float& kd, int32_t& ki, float v, int3
   }
 }
 
+}  // namespace
+}  // namespace snmf
+
+#include "knn_tc.cuh"
+
+namespace snmf {
+namespace {
+
 // The k nearest of the candidates [z per, (z + 1) per) for the 64 queries of CTA (x, z): partial
 // lists at [z][n][k], sorted by distance and then index (empty slots are (inf, INT_MAX)).  Distances of a 128 x 64 tile, 8 candidates x 4 queries per thread, two
 // candidates per instruction: sum over t ascending of (q_t - c_t)^2 with one FMA each, candidates
 // staged negated.  A distance not above the query's k-th so far goes to the query's buffer in shared
 // memory; after the tile its warp (eight queries each) inserts the buffer, in any order with the
 // same result.  A non-finite distance counts as +inf and raises *bad.  Bound by the FP32 pipes (2 n^2 d
-// lane operations): n = 20000, d = 64, k = 10 took 23.1 ms with one thread per query and the list
-// updated for every candidate.
+// lane operations): n = 20000, d = 64, k = 10 2.94 ms (23.1 ms with one thread per query and the list
+// updated for every candidate).  For few or wide points, and where the filter (knn_tc.cuh) gave up.
 struct KnnSmem {
   float q[2][DT][QB];
   float c[2][DT][CB];
@@ -67,7 +76,8 @@ struct KnnSmem {
 
 __global__ void __launch_bounds__(256, 2)
 k_knn(const float* __restrict__ X, int64_t n, int d, int k, int64_t per, bool vec, int32_t* __restrict__ nbr,
-      float* __restrict__ nd2, int* __restrict__ bad) {
+      float* __restrict__ nd2, int* __restrict__ bad, const int* __restrict__ only_if) {
+  if (only_if && !*only_if) return;
   extern __shared__ __align__(16) unsigned char knn_raw[];
   KnnSmem& S = *reinterpret_cast<KnnSmem*>(knn_raw);
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
@@ -208,7 +218,9 @@ k_knn(const float* __restrict__ X, int64_t n, int d, int k, int64_t per, bool ve
 
 // one warp per query: the k best of its `parts` partial lists
 __global__ void __launch_bounds__(256) k_knn_merge(const int32_t* __restrict__ pi, const float* __restrict__ pd, int64_t n,
-                                                   int k, int parts, int32_t* __restrict__ nbr, float* __restrict__ nd2) {
+                                                   int k, int parts, int32_t* __restrict__ nbr, float* __restrict__ nd2,
+                                                   const int* __restrict__ only_if) {
+  if (only_if && !*only_if) return;
   const int lane = threadIdx.x & 31;
   const int64_t q = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   if (q >= n) return;
@@ -253,14 +265,22 @@ __global__ void __launch_bounds__(1024) k_scan(const int32_t* __restrict__ v, in
   for (int64_t i = b; i < e; ++i) s += v[i] + add;
   part[threadIdx.x] = s;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int64_t run = 0;
-    for (int t = 0; t < (int)blockDim.x; ++t) {
-      const int64_t x = part[t];
-      part[t] = run;
+  if (threadIdx.x < 32) {  // 32 sums a lane, then a scan over the lanes
+    int64_t* p = part + threadIdx.x * 32;
+    int64_t sum = 0;
+    for (int t = 0; t < 32; ++t) sum += p[t];
+    int64_t run = sum;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t x = __shfl_up_sync(0xffffffffu, run, o);
+      if ((int)threadIdx.x >= o) run += x;
+    }
+    if (threadIdx.x == 31) out[n] = (int32_t)run;
+    run -= sum;
+    for (int t = 0; t < 32; ++t) {
+      const int64_t x = p[t];
+      p[t] = run;
       run += x;
     }
-    out[n] = (int32_t)run;
   }
   __syncthreads();
   int64_t run = part[threadIdx.x];
@@ -384,17 +404,80 @@ int knn_parts(int64_t n) {
   return parts;
 }
 
-void launch_knn(const float* X, int64_t n, int d, int k, int parts, int32_t* pi, float* pd, int32_t* nbr, float* nd2,
-                int* bad, cudaStream_t s) {
+// The filter: for rows that two CTAs of an SM hold beside their rings, and where its launches are worth
+// it (whole call, d = 16, k = 10: n = 1024 256 us without it and 224 with it; n = 5001, d = 33, k = 12
+// 511 and 315; n = 20000, d = 64 3250 and 890).  The candidate's index is 26 bits.
+bool knn_tc_rule(int64_t n, int d) { return d <= KT_MAXD && n >= 1024 && n < (1 << 26); }
+
+// Candidate ranges of its passes: about four waves of CTAs (n = 20000, d = 64: 1401 us with one range,
+// 1171 with seven), none shorter than 256.
+int knn_tc_parts(int64_t n) {
+  const int64_t qt = (n + KT_Q - 1) / KT_Q;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(KT_PARTS, std::min<int64_t>(1216 / qt, n / 256)));
+}
+
+// Pass 0 over every second point halves it and doubles the candidates (n = 20000, d = 64, k = 10: pass 0
+// 439 to 325 us, exact distances 24 to 42); every fourth would save another 60 us, but a cluster of
+// fewer than 4 k points would then bring in all points.
+int knn_tc_stride(int64_t n) { return n >= 4096 ? 2 : 1; }
+
+struct KnnWork {
+  int parts, tc_parts;  // tc_parts: 0 without the filter
+  int32_t* pi;          // partial lists
+  float* pd;
+  float *Y, *nrm, *nrm0, *kth, *ctr, *lists;  // nrm, nrm0: room for a whole last tile
+  int32_t* cand;
+  int *ncand, *bad, *dense, *err;
+};
+
+template <int PASS, int KR>
+cudaError_t launch_knn_pass(const CUtensorMap& map, const CUtensorMap& cmap, const float* cnrm, int stride, int64_t n, int d,
+                            int k, const KnnWork& w, cudaStream_t s) {
+  static std::once_flag once;
+  static cudaError_t attr = cudaSuccess;
+  std::call_once(once, [] {
+    attr = cudaFuncSetAttribute(k_knn_tc<PASS, KR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)knn_tc_smem(KT_MAXD));
+  });
+  if (attr != cudaSuccess) return attr;
+  const int64_t nc = (n + stride - 1) / stride, per = ((nc + w.tc_parts - 1) / w.tc_parts + KT_C - 1) / KT_C * KT_C;
+  dim3 grid((unsigned)((n + KT_Q - 1) / KT_Q), w.tc_parts);
+  k_knn_tc<PASS, KR><<<grid, KT_THREADS, knn_tc_smem(d), s>>>(map, cmap, w.nrm, cnrm, nc, stride, w.kth, n, d, k, per,
+                                                              w.lists, w.cand, w.ncand, w.dense, w.err);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_knn(const float* X, int64_t n, int d, int k, const KnnWork& w, int32_t* nbr, float* nd2, cudaStream_t s) {
   static std::once_flag once;
   std::call_once(once, [] {
     cudaFuncSetAttribute(k_knn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(KnnSmem));
   });
-  const int64_t per = ((n + parts - 1) / parts + CB - 1) / CB * CB;
   const bool vec = d % 4 == 0 && !((uintptr_t)X & 15);
-  dim3 grid((unsigned)((n + QB - 1) / QB), parts);
-  k_knn<<<grid, 256, sizeof(KnnSmem), s>>>(X, n, d, k, per, vec, parts > 1 ? pi : nbr, parts > 1 ? pd : nd2, bad);
-  if (parts > 1) k_knn_merge<<<(unsigned)((n + 7) / 8), 256, 0, s>>>(pi, pd, n, k, parts, nbr, nd2);
+  const unsigned mb = (unsigned)((n + 7) / 8);
+  const int* only_if = nullptr;
+  CUtensorMap map, map0;
+  const int dp = (d + 31) / 32 * 32;
+  const int st = knn_tc_stride(n);
+  if (w.tc_parts && make_map_f32_tile(&map, w.Y, dp, n, dp, KT_C) &&
+      make_map_f32_tile(&map0, w.Y, dp, (n + st - 1) / st, (int64_t)st * dp, KT_C)) {
+    k_knn_center<<<1, 1024, 0, s>>>(X, n, d, w.ctr);
+    k_knn_prep<<<mb, 256, 0, s>>>(X, n, d, dp, w.ctr, w.Y, w.nrm, w.kth, w.ncand, st, w.nrm0, w.dense);
+    cudaError_t e = k <= 16 ? launch_knn_pass<0, 16>(map, map0, w.nrm0, st, n, d, k, w, s)
+                            : launch_knn_pass<0, 32>(map, map0, w.nrm0, st, n, d, k, w, s);
+    if (e != cudaSuccess) return e;
+    k_knn_bound<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(w.lists, w.nrm, n, k, 2 * w.tc_parts, w.kth);
+    e = launch_knn_pass<1, 1>(map, map, w.nrm, 1, n, d, k, w, s);
+    if (e != cudaSuccess) return e;
+    if (d % 8 == 0 && !((uintptr_t)X & 31)) k_knn_exact<8><<<mb, 256, 0, s>>>(X, n, d, k, w.cand, w.ncand, nbr, nd2, w.dense);
+    else if (vec) k_knn_exact<4><<<mb, 256, 0, s>>>(X, n, d, k, w.cand, w.ncand, nbr, nd2, w.dense);
+    else k_knn_exact<1><<<mb, 256, 0, s>>>(X, n, d, k, w.cand, w.ncand, nbr, nd2, w.dense);
+    only_if = w.dense;
+  }
+  const int64_t per = ((n + w.parts - 1) / w.parts + CB - 1) / CB * CB;
+  dim3 grid((unsigned)((n + QB - 1) / QB), w.parts);
+  k_knn<<<grid, 256, sizeof(KnnSmem), s>>>(X, n, d, k, per, vec, w.parts > 1 ? w.pi : nbr, w.parts > 1 ? w.pd : nd2, w.bad,
+                                           only_if);
+  if (w.parts > 1) k_knn_merge<<<mb, 256, 0, s>>>(w.pi, w.pd, n, k, w.parts, nbr, nd2, only_if);
+  return cudaGetLastError();
 }
 
 // Best one-to-one matching maximising the matched count: the Hungarian method with potentials
@@ -455,7 +538,10 @@ extern "C" snmf_status snmf_knn_graph(const float* X, int64_t n, int d, int k, i
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t nk = n * k;
   // the call's workspace in one piece
-  const int parts = knn_parts(n);
+  KnnWork w{};
+  w.parts = knn_parts(n);
+  w.tc_parts = knn_tc_rule(n, d) ? knn_tc_parts(n) : 0;
+  const int64_t dp = w.tc_parts ? (d + 31) / 32 * 32 : 0;
   unsigned char* ws = nullptr;
   size_t bytes = 0;
   auto take = [&](size_t b) {
@@ -466,29 +552,37 @@ extern "C" snmf_status snmf_knn_graph(const float* X, int64_t n, int d, int k, i
   const size_t o_nbr = take(nk * 4), o_nd2 = take(nk * 4), o_sval = take(nk * 4), o_cnt = take(n * 4), o_fill = take(n * 4),
                o_off = take((n + 1) * 4), o_cntu = take(n * 4), o_erow = take(2 * nk * 4), o_ecol = take(2 * nk * 4), o_eval = take(2 * nk * 4),
                o_sv = take(s_values ? 0 : 2 * nk * 4), o_dg = take(degree ? 0 : n * 4), o_erep = take(2 * nk),
-               o_bad = take(4), o_pi = take(parts > 1 ? parts * nk * 4 : 0), o_pd = take(parts > 1 ? parts * nk * 4 : 0);
-  auto cleanup = [&] { cudaFree(ws); };
+               o_bad = take(12), o_y = take(n * dp * 4),
+               o_nrm = take(dp ? (n + KT_C) * 4 : 0), o_nrm0 = take(dp ? (n + KT_C) * 4 : 0), o_kth = take(dp ? n * 4 : 0), o_ctr = take(dp * 4),
+               o_ncand = take(dp ? n * 4 : 0), o_lists = bytes, o_pi = bytes;
+  // k_knn's partial lists come after the filter's lists and candidates are done with
+  const size_t o_cand = o_lists + (2 * w.tc_parts * nk * 4 + 255) / 256 * 256, o_pd = o_pi + (w.parts * nk * 4 + 255) / 256 * 256;
+  take(std::max((o_cand - o_lists) + (dp ? n * KT_CAP * 4 : 0), (o_pd - o_pi) + w.parts * nk * 4));
+  auto cleanup = [&] { workspace_free(ws, s); };
   snmf_status st = SNMF_OK;
 #define KCK(call)                                                                                        \
   do {                                                                                                   \
     const cudaError_t e_ = (call);                                                                       \
     if (e_ != cudaSuccess) { st = e_ == cudaErrorMemoryAllocation ? SNMF_ERR_OOM : SNMF_ERR_CUDA; cleanup(); return st; } \
   } while (0)
-  KCK(cudaMalloc(&ws, bytes));
+  KCK(workspace_alloc((void**)&ws, bytes, s));
   auto i32 = [&](size_t o) { return reinterpret_cast<int32_t*>(ws + o); };
   auto f32 = [&](size_t o) { return reinterpret_cast<float*>(ws + o); };
   int32_t *nbr = i32(o_nbr), *cnt = i32(o_cnt), *off = i32(o_off), *fill = i32(o_fill), *erow = i32(o_erow), *ecol = i32(o_ecol),
-          *cntu = i32(o_cntu), *pi = i32(o_pi);
-  float *nd2 = f32(o_nd2), *sval = f32(o_sval), *eval = f32(o_eval), *pd = f32(o_pd);
+          *cntu = i32(o_cntu);
+  float *nd2 = f32(o_nd2), *sval = f32(o_sval), *eval = f32(o_eval);
   float* sv = s_values ? s_values : f32(o_sv);
   float* dg = degree ? degree : f32(o_dg);
   uint8_t* erep = ws + o_erep;
-  int* bad = i32(o_bad);
-  KCK(cudaMemsetAsync(bad, 0, sizeof(int), s));
+  int* bad = i32(o_bad);  // non-finite distances, the filter given up, a bounded wait ran out
+  w.pi = i32(o_pi); w.pd = f32(o_pd); w.Y = f32(o_y); w.nrm = f32(o_nrm); w.nrm0 = f32(o_nrm0); w.kth = f32(o_kth); w.ctr = f32(o_ctr);
+  w.lists = f32(o_lists); w.cand = i32(o_cand); w.ncand = i32(o_ncand);
+  w.bad = bad; w.dense = bad + 1; w.err = bad + 2;
+  KCK(cudaMemsetAsync(bad, 0, 3 * sizeof(int), s));
   KCK(cudaMemsetAsync(cnt, 0, n * sizeof(int32_t), s));
   KCK(cudaMemsetAsync(cntu, 0, n * sizeof(int32_t), s));
   KCK(cudaMemsetAsync(fill, 0, n * sizeof(int32_t), s));
-  launch_knn(X, n, d, k, parts, pi, pd, nbr, nd2, bad, s);
+  KCK(launch_knn(X, n, d, k, w, nbr, nd2, s));
   const int g = (int)std::min<int64_t>((nk + 255) / 256, 152 * 16);
   k_knn_sim<<<g, 256, 0, s>>>(nbr, nd2, n, k, sigma_rank, sval, cnt, bad);
   k_scan<<<1, 1024, 0, s>>>(cnt, n, k, off);  // row slots: k own + in-degree
@@ -498,12 +592,13 @@ extern "C" snmf_status snmf_knn_graph(const float* X, int64_t n, int d, int k, i
   k_knn_dedupe<<<eb, 256, 0, s>>>(off, erow, ecol, eval, 2 * nk, 0, erep, cntu, nullptr, nullptr, nullptr);
   k_scan<<<1, 1024, 0, s>>>(cntu, n, 0, rowptr);
   int32_t total = 0;
-  int hbad = 0;
+  int hbad[3] = {0, 0, 0};
   KCK(cudaMemcpyAsync(&total, rowptr + n, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  KCK(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
+  KCK(cudaMemcpyAsync(hbad, bad, sizeof(hbad), cudaMemcpyDeviceToHost, s));
   KCK(cudaStreamSynchronize(s));
   *nnz = total;
-  if (hbad) { cleanup(); return SNMF_ERR_NUMERIC; }
+  if (hbad[2]) { cleanup(); return SNMF_ERR_TIMEOUT; }
+  if (hbad[0]) { cleanup(); return SNMF_ERR_NUMERIC; }
   if (total > capacity) { cleanup(); return SNMF_ERR_ARG; }
   k_knn_dedupe<<<eb, 256, 0, s>>>(off, erow, ecol, eval, 2 * nk, 1, erep, cntu, rowptr, colidx, sv);
   k_knn_degree<<<rb, 256, 0, s>>>(rowptr, sv, n, dg);
