@@ -59,7 +59,7 @@ struct snmf_ctx {
   bool graph = false;
   double gamma = 0.0;
   double normL = 0.0;  // ||L||_2 (power method), enters rho of graph-regularised blocks
-  int use_row = 0;     // row kernels through rowstep.cu (penalty form, r <= 64, no record mode)
+  int use_row = 0;     // row kernels through rowstep.cu (penalty form, r <= 128, no record mode)
   RowStepPlan rplan{};
   int row_tc = 0;      // with use_row: row products on the tensor cores, 1 rowtc.cu, 2 rowtma.cu (r = 64; tuned)
   int row_bm = 0;      // general row kernel, FP32: rows per CTA (0: built-in choice; autotuned)
@@ -812,10 +812,10 @@ void dir_final(snmf_ctx* h, const Params& P) {
   launch_ctl_final_dir(h->ctl, h->G64fix, h->b, h->r, P, h->s);
 }
 
-// Row kernels through rowstep.cu: penalty (or naive) form, r <= 64, with or without a graph term;
+// Row kernels through rowstep.cu: penalty (or naive) form, r <= 128, with or without a graph term;
 // record mode's nine candidates, the direct form and larger ranks keep the general kernel.
 int row_rule(const snmf_ctx* h) {
-  return h->r <= 64 && h->opt.formulation != SNMF_DIRECT && h->opt.step_controller != 2;
+  return h->r <= 128 && h->opt.formulation != SNMF_DIRECT && h->opt.step_controller != 2;
 }
 
 snmf_status alloc_buffers(snmf_ctx* h) {
@@ -832,7 +832,7 @@ snmf_status alloc_buffers(snmf_ctx* h) {
   h->nax = (int)((h->n + kRowTile - 1) / kRowTile);
   // room for every row-kernel layout
   h->use_row = row_rule(h);
-  h->rplan = rowstep_plan(h->tdtype, h->n, std::min(h->r, 64), h->b);
+  h->rplan = rowstep_plan(h->tdtype, h->n, std::min(h->r, 128), h->b);
   const int nrow_max = std::max({h->nrow, rowgemm_slots(d, h->tdtype, 32), h->rplan.slots});
   const size_t prec_n = (size_t)std::max(nrow_max, h->nax) * h->b * kNQ;
   if (h->use_row) h->nrow = h->rplan.slots;

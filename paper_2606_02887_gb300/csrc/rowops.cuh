@@ -52,7 +52,7 @@ struct RowArgs {
   int bm;              // general body, FP32: rows per CTA (32 or 64; 0 = built-in choice)
 };
 
-// Row kernels of a step of the penalty form for r <= 64 (rowstep_dev.cuh): the block-start (or
+// Row kernels of a step of the penalty form for r <= 128 (rowstep_dev.cuh): the block-start (or
 // given-X') gradient, the D step from X and g (nc = 2: the learned step with fallback) or from a
 // given Z (graph term), and the relaxed update that recomputes Z and D.
 struct RowStepPlan {

@@ -19,9 +19,10 @@ __global__ void __launch_bounds__(256, 2) k_rowstep(RowArgs a, int tiles, bool v
 template <typename T, int STEP, int NC, int MR>
 void launch_t(const RowArgs& a, const RowStepPlan& pl, cudaStream_t s) {
   static std::once_flag once;
-  std::call_once(once, [] {  // the most over the ranks: r = 64 with 256 threads and every input
+  std::call_once(once, [] {  // the most over the ranks: r = 128 with 256 threads and every input
+    const int r = sizeof(T) == 8 && MR > 1 ? 64 : 128;
     cudaFuncSetAttribute(k_rowstep<T, STEP, NC, MR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)rowstep_smem<T>(64, 256, MR, 7));
+                         (int)rowstep_smem<T>(r, 256, MR, 7));
   });
   uintptr_t all = 0;
   for (const void* p : {a.X, a.g_in, a.B, a.LX, (const void*)a.Xout, (const void*)a.gout, (const void*)a.Dout,
@@ -39,10 +40,17 @@ RowStepPlan rowstep_plan(int tdtype, int64_t n, int r, int b) {
   // 4 (FP64: 2) rows per thread of 128 or (r > 32) 256 threads; one row, and half the threads, while that
   // still makes no more than two CTAs per SM (n = 1000, r = 20: 84 CTAs of 12 rows; the general
   // kernel had 32 of 32)
+  // Above r = 64 always 256 threads (G is copied by them) and one row each in FP64, whose G takes up
+  // to 128 KB of the shared memory.
   const int big = (r + 3) / 4 > 8 ? 256 : 128;
   RowStepPlan pl{big, tdtype == 0 ? rowstep_mr<double>() : rowstep_mr<float>(), 0, 0, 0};
   for (const auto& o : {std::pair<int, int>{big / 2, 1}, std::pair<int, int>{big, 1}}) {
     const int64_t rows = rowstep_rows(r, o.first, o.second);
+    if (r > 64 && o.first < big) continue;
+    if (r > 64 && tdtype == 0) {
+      pl.mr = 1;
+      break;
+    }
     if ((n + rows - 1) / rows * b <= 2 * 152) {
       pl.threads = o.first;
       pl.mr = o.second;
@@ -51,8 +59,9 @@ RowStepPlan rowstep_plan(int tdtype, int64_t n, int r, int b) {
   }
   pl.rows = rowstep_rows(r, pl.threads, pl.mr);
   pl.tiles = (int)((n + pl.rows - 1) / pl.rows);
-  // 512 threads per SM over the restarts, each CTA as many tiles as the next one
-  const int most = std::max(1, (152 * (512 / pl.threads) + b - 1) / b);
+  // 512 threads per SM (r > 64: 256, the shared memory holds one CTA) over the restarts, each CTA as
+  // many tiles as the next one
+  const int most = std::max(1, (152 * ((r > 64 ? 256 : 512) / pl.threads) + b - 1) / b);
   const int each = (pl.tiles + most - 1) / most;
   pl.slots = (pl.tiles + each - 1) / each;
   return pl;

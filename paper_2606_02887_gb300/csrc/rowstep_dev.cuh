@@ -1,4 +1,4 @@
-// Row kernels of an Algorithm-1 step for any rank r <= 64, FP64 or FP32, as a CTA body: block-start
+// Row kernels of an Algorithm-1 step for any rank r <= 128, FP64 or FP32, as a CTA body: block-start
 // gradient, D step and relaxed update, used per restart (rowstep.cu) and per problem of the uneven
 // batch (batch.cu).
 //
@@ -214,15 +214,21 @@ __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, i
       }
       cp_async_commit();
     };
-    fetch_operand(cta);
-    fetch_rest(cta);
     {
+      // G joins the first copy group where its rows start on 16 bytes
       const T* G = (const T*)a.G + (int64_t)j * r * r;
-      for (int e = t; e < c4 * c4; e += nt) {
-        const int p = e / c4, q = e - p * c4;
-        Gs[e] = p < r && q < r ? G[p * r + q] : T(0);
+      if (r == c4 && !((uintptr_t)G & 15)) {
+        constexpr int KV = 16 / (int)sizeof(T);
+        for (int e = t * KV; e < c4 * c4; e += nt * KV) cp_async<16>(Gs + e, G + e, true);
+      } else {
+        for (int e = t; e < c4 * c4; e += nt) {
+          const int p = e / c4, q = e - p * c4;
+          Gs[e] = p < r && q < r ? G[p * r + q] : T(0);
+        }
       }
     }
+    fetch_operand(cta);
+    fetch_rest(cta);
     for (int tile = cta; tile < tiles; tile += per) {
       const int64_t row0 = (int64_t)tile * (TY * MR) + ty;
       const int64_t off0 = row0 * a.ld + colj, step = (int64_t)TY * a.ld;
