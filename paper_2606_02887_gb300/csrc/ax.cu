@@ -11,6 +11,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cmath>
 #include <mutex>
 
 #include "common.cuh"
@@ -273,17 +274,31 @@ int launch_gemm_cfg(const AxArgs& a, int64_t n, int cols, int64_t ld, const void
     cudaFuncSetAttribute(k_gemm_dense<C, TA, PER_SM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
   });
   const int gx = cdiv64(cols, C::BN), gy = cdiv64(n, C::BM);
-  // split-K: the number of K chunks (of 64 columns and more, 32 in FP64, where a CTA is long) that
-  // fills whole waves of CTAs best; each further slice has to gain a per cent, for the finish
-  // pass (n = 8192, 64 columns: 8 slices leave a sixth of the SMs a CTA short)
+  // split-K.  FP32 (chunks of 64 columns and more): least time of an SM, its CTAs one after the other
+  // at their chunk's columns plus 64 for the start and the end of a CTA, slower by the root of the
+  // occupancy that its CTAs leave unused, plus a column's worth for each slice that the finish pass
+  // reads; a last short chunk fills gaps (over 99 sizes up to n = 8192 1.5 per cent from the best
+  // split, 20 at most; counting whole waves of CTAs 2.4 per cent, n = 3001, 300 columns 163 for 153 us).
+  // FP64 (chunks of 32, where a CTA is long): the number of chunks that fills whole waves best; each
+  // further slice has to gain a per cent, for the finish pass.
   constexpr int64_t kMin = sizeof(T) == 8 ? 32 : 64;
   const int64_t tiles = (int64_t)gx * gy, slots = (int64_t)152 * PER_SM;
   const int64_t most = std::min<int64_t>({(n + kMin - 1) / kMin, 32, (int64_t)(ws_elems / ((size_t)n * (size_t)ld))});
   int64_t splits = 1;
   double best = 0.0;
   for (int64_t sp = 1; sp <= std::max<int64_t>(1, most); ++sp) {
-    const int64_t ctas = tiles * sp, waves = (ctas + slots - 1) / slots;
-    const double gain = (double)ctas / (double)(waves * slots) * (1.0 - 0.01 * (double)sp);
+    double gain;
+    if (sizeof(T) == 8) {
+      const int64_t ctas = tiles * sp, waves = (ctas + slots - 1) / slots;
+      gain = (double)ctas / (double)(waves * slots) * (1.0 - 0.01 * (double)sp);
+    } else {
+      const int64_t kc = (cdiv64(n, (int)sp) + 31) / 32 * 32;
+      const double load = (double)tiles * std::max((double)(n / kc), (double)n / (double)kc);
+      const double m = std::max(1.0, std::ceil(load / 152.0));
+      const double slow = std::sqrt(std::max(1.0, (double)PER_SM / m));
+      const double slice = 8.0 * (double)n * cols / 6e12 * (96 * 1.9e9) / (C::BM * C::BN);
+      gain = 1.0 / (m * (double)(kc + 64) * slow + (sp > 1 ? (double)sp * slice : 0.0));
+    }
     if (gain > best) { best = gain; splits = sp; }
   }
   if (tune && tune->splits > 0) splits = tune->splits;  // autotuned
@@ -306,7 +321,9 @@ int launch_ax(const AxArgs& a, int tdtype, int64_t n, int cols, int64_t ld, cons
               size_t ws_elems, const int* run, cudaStream_t s, const ProdTune* tune, double c, const void* X2) {
   if (a.kind == AX_DENSE) {
     // The tile is as narrow as the columns allow: 128 columns where a tile of 64 would not save a
-    // padded half, else 64, 32, 16; FP64, whose pipes bound every size, down to 8 in steps that
+    // padded half (FP32 A: 8 x 16 values per thread, which reads a quarter less of the stages than
+    // 8 x 8: n = 8192, 512 columns 1281 -> 1174 us; the widened A need the registers: 1349 -> 1408), else 64 (three CTAs per SM, whose
+    // registers hold all operands, and for FP32 A stages of 32 columns: n = 8192, 64 columns 176 -> 161 us), 32, 16; FP64, whose pipes bound every size, down to 8 in steps that
     // waste at most a third (n = 2500, 10 columns: 910 us in a 64-wide tile).  Fewer than two CTAs
     // per SM at the most splits: half the rows per tile.
 #define GEMM(T, TA, KIND, BM, BN, TM, TN, BK, OCC) \
@@ -320,20 +337,20 @@ int launch_ax(const AxArgs& a, int tdtype, int64_t n, int cols, int64_t ld, cons
       GEMM(double, double, GA_SAME, 64, 64, 4, 4, 16, 2);
     }
     const bool wide = cols > 64 && (cols + 127) / 128 * 2 <= (cols + 63) / 64;
-#define GEMM_WIDTHS(TA, KIND)                                     \
-  if (wide) GEMM(float, TA, KIND, 128, 128, 8, 8, 16, 2);         \
-  if (cols > 32) GEMM(float, TA, KIND, 128, 64, 8, 8, 16, 4);     \
+#define GEMM_WIDTHS(TA, KIND, TNW, BK64)                          \
+  if (wide) GEMM(float, TA, KIND, 128, 128, 8, TNW, 16, 2);       \
+  if (cols > 32) GEMM(float, TA, KIND, 128, 64, 8, 8, BK64, 3);   \
   if (cols > 16) GEMM(float, TA, KIND, 128, 32, 8, 4, 32, 3);     \
   GEMM(float, TA, KIND, 128, 16, 4, 4, 32, 3)
-    if (a.a_dtype == 3) { GEMM_WIDTHS(__nv_fp8_storage_t, GA_FP8); }
-    if (a.a_dtype == 2 && a.sym) { GEMM_WIDTHS(__nv_bfloat16, GA_BF16_SYM); }
-    if (a.a_dtype == 2) { GEMM_WIDTHS(__nv_bfloat16, GA_BF16); }
+    if (a.a_dtype == 3) { GEMM_WIDTHS(__nv_fp8_storage_t, GA_FP8, 8, 16); }
+    if (a.a_dtype == 2 && a.sym) { GEMM_WIDTHS(__nv_bfloat16, GA_BF16_SYM, 8, 16); }
+    if (a.a_dtype == 2) { GEMM_WIDTHS(__nv_bfloat16, GA_BF16, 8, 16); }
     if ((int64_t)cdiv64(n, 128) * cdiv64(cols, 64) * std::min<int64_t>(n / 64, 32) < 2 * 152) {
       if (cols > 32) GEMM(float, float, GA_SAME, 64, 64, 4, 8, 16, 4);
       if (cols > 16) GEMM(float, float, GA_SAME, 64, 32, 4, 4, 32, 4);
       GEMM(float, float, GA_SAME, 64, 16, 4, 4, 32, 6);
     }
-    GEMM_WIDTHS(float, GA_SAME);
+    GEMM_WIDTHS(float, GA_SAME, 16, 32);
 #undef GEMM_WIDTHS
 #undef GEMM
   }
