@@ -56,7 +56,7 @@ struct RowArgs {
 // given-X') gradient, the D step from X and g (nc = 2: the learned step with fallback) or from a
 // given Z (graph term), and the relaxed update that recomputes Z and D.
 struct RowStepPlan {
-  int threads, mr;  // threads per CTA, rows per thread
+  int threads, mr, w;  // threads per CTA, rows and columns per thread
   int rows, tiles;  // rows per tile, tiles per restart
   int slots;        // CTAs (partial slots) per restart
 };

@@ -46,38 +46,43 @@ __device__ double reduce_slots(const double* part, int nslots, int b, int j, int
 
 // The first NV quantities of restart j, summed over the slots into qs[NV] (shared): NV / 2 threads
 // per slot read its record as 16-byte pairs.  sh: [8][NV] shared.  Ends with a barrier.
+// Four warps at most: an FP64 instruction occupies its SM partition for 64 cycles whatever the lanes
+// that are on, so more warps only add instructions to the shuffles and the last sum.
 template <int NV>
 __device__ __forceinline__ void slot_sums(const double* part, int nslots, int b, int j, double (*sh)[NV], double* qs) {
   constexpr int TPS = NV / 2;
-  const int t = threadIdx.x, lane = t & 31, wid = t >> 5, step = (int)blockDim.x / TPS, q = t % TPS;
-  double s0 = 0.0, s1 = 0.0;
-  auto ld = [&](int k) { return __ldcg(reinterpret_cast<const double2*>(part + ((int64_t)k * b + j) * kNQ) + q); };
-  int k = t / TPS;
-  for (; k + 3 * step < nslots; k += 4 * step) {
-    double2 v[4];
+  const int nt = min((int)blockDim.x, 128);
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5, step = nt / TPS, q = t % TPS;
+  if (t < nt) {
+    double s0 = 0.0, s1 = 0.0;
+    auto ld = [&](int k) { return __ldcg(reinterpret_cast<const double2*>(part + ((int64_t)k * b + j) * kNQ) + q); };
+    int k = t / TPS;
+    for (; k + 3 * step < nslots; k += 4 * step) {
+      double2 v[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) v[u] = ld(k + u * step);
+      for (int u = 0; u < 4; ++u) v[u] = ld(k + u * step);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) { s0 += v[u].x; s1 += v[u].y; }
-  }
-  for (; k < nslots; k += step) {
-    const double2 v = ld(k);
-    s0 += v.x;
-    s1 += v.y;
-  }
+      for (int u = 0; u < 4; ++u) { s0 += v[u].x; s1 += v[u].y; }
+    }
+    for (; k < nslots; k += step) {
+      const double2 v = ld(k);
+      s0 += v.x;
+      s1 += v.y;
+    }
 #pragma unroll
-  for (int o = TPS; o < 32; o <<= 1) {
-    s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-    s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-  }
-  if (lane < TPS) {
-    sh[wid][2 * lane] = s0;
-    sh[wid][2 * lane + 1] = s1;
+    for (int o = TPS; o < 32; o <<= 1) {
+      s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+    }
+    if (lane < TPS) {
+      sh[wid][2 * lane] = s0;
+      sh[wid][2 * lane + 1] = s1;
+    }
   }
   __syncthreads();
   if (t < NV) {
-    double v = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += sh[w][t];
+    double v = sh[0][t];
+    for (int w = 1; w < nt >> 5; ++w) v += sh[w][t];
     qs[t] = v;
   }
   __syncthreads();
@@ -137,6 +142,10 @@ __device__ double bb_step(const Ctl& c, const Params& P, double rho) {
   return fmin(P.alpha_max, fmax(P.alpha_min, a));
 }
 
+__device__ __forceinline__ bool finite_bits(double x) {
+  return (__double_as_longlong(x) & 0x7ff0000000000000ll) != 0x7ff0000000000000ll;
+}
+
 __device__ void hist_reset(Ctl& c, double f) {
   c.hlen = 1;
   c.hpos = 0;
@@ -154,9 +163,13 @@ __device__ void hist_push(Ctl& c, double f, int M) {
 // after f(X_k) has been pushed.
 __device__ double reference(const Ctl& c, const Params& P) {
   if (P.memory > 0) {
-    double m = -INFINITY;
-    for (int t = 0; t < c.hlen; ++t) m = fmax(m, c.fhist[t]);
-    return m;
+    // maximum by the ordered bits (NaN left out): an FP64 comparison takes 64 cycles
+    long long m = (long long)0xfff0000000000000ull ^ 0x7fffffffffffffffll;  // -inf
+    for (int t = 0; t < c.hlen; ++t) {
+      const long long v = __double_as_longlong(c.fhist[t]), a = v & 0x7fffffffffffffffll;
+      if (a <= 0x7ff0000000000000ll) m = max(m, v < 0 ? v ^ 0x7fffffffffffffffll : v);
+    }
+    return __longlong_as_double(m < 0 ? m ^ 0x7fffffffffffffffll : m);
   }
   return c.f + P.eta * (c.F - c.f);
 }
@@ -203,8 +216,10 @@ __device__ void pen_start_body(Ctl& c, const double* qs, int j, const Params& P,
 // backtracking from beta = 1 on f(Z + beta D) - f(Z) = beta gd + beta^2/2 q against the
 // reference (Alg. 1 line 4); returns beta (0 when no trial is accepted)
 __device__ double backtrack(double fZ, double F, double gd, double q, const Params& P, bool* ok) {
-  double beta = 1.0;
-  for (int t = 0; t < P.max_ls; ++t) {
+  // beta = 1 by itself: four FP64 instructions instead of ten, and the usual end (max_ls >= 1)
+  if (fZ + gd + 0.5 * q <= F + P.theta * gd) { *ok = true; return 1.0; }
+  double beta = P.beta_shrink;
+  for (int t = 1; t < P.max_ls; ++t) {
     const double fz = fZ + beta * gd + 0.5 * beta * beta * q;
     if (fz <= F + P.theta * beta * gd) { *ok = true; return beta; }
     beta *= P.beta_shrink;
@@ -278,7 +293,7 @@ __device__ void pen_ls_body(Ctl& c, const double* qs, double q, const Params& P,
     ok = ok4;
   }
   if (!ok) { beta = 0.0; c.ls_fail++; }
-  if (!isfinite(c.fZ) || !isfinite(q) || !isfinite(gd)) { c.nan_seen = 1; c.active = 0; }
+  if (!finite_bits(c.fZ) || !finite_bits(q) || !finite_bits(gd)) { c.nan_seen = 1; c.active = 0; }
   c.beta = beta;
   c.phibeta = P.phi * beta;
 }
@@ -361,7 +376,7 @@ __device__ void pen_upd_body(Ctl& c, const double* qs, int j, const Params& P, i
   } else if (last) {
     c.iters++;  // naive variant: the W block is the whole outer iteration
   }
-  if (!isfinite(c.f)) { c.nan_seen = 1; c.active = 0; }
+  if (!finite_bits(c.f)) { c.nan_seen = 1; c.active = 0; }
 }
 
 // Final per-restart statistics of the penalty form: pax q0 = <W, A Ht>, prow q0 = ||P grad_W||^2

@@ -38,9 +38,26 @@ enum { RS_GRAD = 0, RS_D, RS_DZ, RS_U };
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 
+// Comparisons with zero; FP64 by the bits, since an FP64 comparison takes the FP64 pipe for 64 cycles
+// of a warp (NaN is neither positive nor negative).
+__device__ __forceinline__ bool positive(float t) { return t > 0.f; }
+__device__ __forceinline__ bool positive(double t) {
+  return (unsigned long long)__double_as_longlong(t) - 1ull < 0x7ff0000000000000ull;
+}
+template <typename T>
+__device__ __forceinline__ bool negative(T t) { return positive(-t); }
+__device__ __forceinline__ bool is_zero(float t) { return t == 0.f; }
+__device__ __forceinline__ bool is_zero(double t) { return __double_as_longlong(t) << 1 == 0; }
+
+// W consecutive values of a row
+template <typename T, int W>
+struct alignas(W * sizeof(T) < 16 ? W * sizeof(T) : 16) Pack {
+  T v[W];
+};
+
 // explicit FMAs: the D step and the update compute the same bits
 template <typename T>
-__device__ __forceinline__ T proj0(T t) { return t > T(0) ? t : T(0); }
+__device__ __forceinline__ T proj0(T t) { return positive(t) ? t : T(0); }
 template <typename T>
 __device__ __forceinline__ T zstep(T x, T g, T inv_rho) { return proj0(fma_rn(-g, inv_rho, x)); }
 template <typename T>
@@ -54,7 +71,7 @@ __host__ __device__ constexpr int rowstep_mr() { return sizeof(T) == 4 ? 4 : 2; 
 
 // rows of a tile, the input arrays of a step, and the dynamic shared memory of rank r with
 // `threads` threads, mr rows each and `nin` inputs
-__host__ __device__ inline int rowstep_rows(int r, int threads, int mr) { return threads / ((r + 3) / 4) * mr; }
+__host__ __device__ inline int rowstep_rows(int r, int threads, int mr, int w = 4) { return threads / ((r + w - 1) / w) * mr; }
 inline int rowstep_inputs(int step, const RowArgs& a) {
   if (step == RS_D) return 3;  // X, g, B
   if (step == RS_U) return 4;  // X, g, g(Z), B
@@ -63,42 +80,46 @@ inline int rowstep_inputs(int step, const RowArgs& a) {
   return k + (a.Xold ? 2 : 0) + (a.Zold ? 2 : 0);
 }
 template <typename T>
-__host__ __device__ inline size_t rowstep_smem(int r, int threads, int mr, int nin) {
+__host__ __device__ inline size_t rowstep_smem(int r, int threads, int mr, int nin, int w = 4) {
   const int c = (r + 3) / 4 * 4;
-  return ((size_t)rowstep_rows(r, threads, mr) * (c + 4) + (size_t)c * c + (size_t)nin * mr * threads * 4) * sizeof(T);
+  return ((size_t)rowstep_rows(r, threads, mr, w) * (c + 4) + (size_t)c * c + (size_t)nin * mr * threads * w) * sizeof(T);
 }
 
-// four columns of one row of a global array: 16-byte accesses, or single values of the w that exist
-template <typename T>
-__device__ __forceinline__ void copy_quad(Quad<T>* dst, const T* base, int64_t off, bool on, bool vec, int w) {
+// W columns of one row of a global array: 16-byte (or W values') accesses, or single values of the w
+// that exist
+template <typename T, int W>
+__device__ __forceinline__ void copy_pack(Pack<T, W>* dst, const T* base, int64_t off, bool on, bool vec, int w) {
+  constexpr int B = W * (int)sizeof(T) < 16 ? W * (int)sizeof(T) : 16;
   if (vec) {
     const char* p = reinterpret_cast<const char*>(on ? base + off : base);
 #pragma unroll
-    for (int q = 0; q < (int)sizeof(Quad<T>); q += 16) cp_async<16>(reinterpret_cast<char*>(dst) + q, p + q, on);
+    for (int q = 0; q < (int)sizeof(Pack<T, W>); q += B) cp_async<B>(reinterpret_cast<char*>(dst) + q, p + q, on);
   } else {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) cp_async<(int)sizeof(T)>(&dst->v[q], on && q < w ? base + off + q : base, on && q < w);
+    for (int q = 0; q < W; ++q) cp_async<(int)sizeof(T)>(&dst->v[q], on && q < w ? base + off + q : base, on && q < w);
   }
 }
-template <typename T>
-__device__ __forceinline__ void store_quad(T* p, const Quad<T>& v, bool vec, int w) {
+template <typename T, int W>
+__device__ __forceinline__ void store_pack(T* p, const Pack<T, W>& v, bool vec, int w) {
   if (vec) {
-    *reinterpret_cast<Quad<T>*>(p) = v;
+    *reinterpret_cast<Pack<T, W>*>(p) = v;
   } else {
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
+    for (int q = 0; q < W; ++q)
       if (q < w) p[q] = v.v[q];
   }
 }
 
-// acc[p] = (row ty + TY p of As) G[:, 4 tx ..], k ascending in one chain per entry
-template <typename T, int MR>
+// acc[p] = (row ty + TY p of As) G[:, W tx ..], k ascending in one chain per entry
+template <typename T, int W, int MR>
 __device__ __forceinline__ void rowstep_product(const T* As, int ls, const T* Gs, int c4, int tx, int ty, int TY,
-                                                Quad<T> (&acc)[MR]) {
+                                                Pack<T, W> (&acc)[MR]) {
 #pragma unroll
-  for (int p = 0; p < MR; ++p) acc[p] = Quad<T>{{T(0), T(0), T(0), T(0)}};
+  for (int p = 0; p < MR; ++p)
+#pragma unroll
+    for (int q = 0; q < W; ++q) acc[p].v[q] = T(0);
   const T* ar = As + ty * ls;
-  const T* gr = Gs + 4 * tx;
+  const T* gr = Gs + W * tx;
 #pragma unroll 2
   for (int k = 0; k < c4; k += 4) {
     Quad<T> a[MR];
@@ -106,17 +127,20 @@ __device__ __forceinline__ void rowstep_product(const T* As, int ls, const T* Gs
     for (int p = 0; p < MR; ++p) a[p] = *reinterpret_cast<const Quad<T>*>(ar + p * TY * ls + k);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const Quad<T> g = *reinterpret_cast<const Quad<T>*>(gr + (k + u) * c4);
+      const Pack<T, W> g = *reinterpret_cast<const Pack<T, W>*>(gr + (k + u) * c4);
 #pragma unroll
       for (int p = 0; p < MR; ++p) {
-        if constexpr (sizeof(T) == 4) {
+        if constexpr (sizeof(T) == 4 && W == 4) {
           const float2 aa = make_float2(a[p].v[u], a[p].v[u]);
           const float2 lo = __ffma2_rn(aa, make_float2(g.v[0], g.v[1]), make_float2(acc[p].v[0], acc[p].v[1]));
           const float2 hi = __ffma2_rn(aa, make_float2(g.v[2], g.v[3]), make_float2(acc[p].v[2], acc[p].v[3]));
-          acc[p] = Quad<T>{{lo.x, lo.y, hi.x, hi.y}};
+          acc[p].v[0] = lo.x;
+          acc[p].v[1] = lo.y;
+          acc[p].v[2] = hi.x;
+          acc[p].v[3] = hi.y;
         } else {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) acc[p].v[q] = fma(a[p].v[u], g.v[q], acc[p].v[q]);
+          for (int q = 0; q < W; ++q) acc[p].v[q] = fma(a[p].v[u], g.v[q], acc[p].v[q]);
         }
       }
     }
@@ -150,7 +174,7 @@ __device__ __forceinline__ T warp_sum8(const T (&v)[8]) {
 
 // CTA `cta` of `per` of restart j: its tiles cta, cta + per, ... of `tiles`.  vec: every row of the
 // restart starts on 16 bytes in all arrays (r and the pitch multiples of 4).  sm: rowstep_smem bytes.
-template <typename T, int STEP, int NC, int MR>
+template <typename T, int STEP, int NC, int MR, int W = 4>
 __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, int per, int tiles, bool vec, T* sm) {
   __shared__ double shq[8][8];
   __shared__ unsigned ticket;
@@ -159,19 +183,14 @@ __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, i
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   double total = 0.0;  // lane m < 8: the warp's sum of value m over the tiles
   if (live) {
-    const int r = a.r, TX = (r + 3) / 4, c4 = 4 * TX, ls = c4 + 4, nt = blockDim.x, TY = nt / TX;
+    const int r = a.r, TX = (r + W - 1) / W, c4 = (r + 3) / 4 * 4, ls = c4 + 4, nt = blockDim.x, TY = nt / TX;
     const int t = threadIdx.x, ty = t / TX, tx = t - ty * TX;
     T* As = sm;
     T* Gs = sm + (size_t)TY * MR * ls;
-    Quad<T>* in = reinterpret_cast<Quad<T>*>(Gs + c4 * c4) + t;  // input i of row k at in[(i MR + k) nt]
+    Pack<T, W>* in = reinterpret_cast<Pack<T, W>*>(Gs + c4 * c4) + t;  // input i of row k at in[(i MR + k) nt]
     const bool on = ty < TY;  // the block may hold a few threads more than TX TY
-    const int w = r - 4 * tx;
-    const int64_t colj = (int64_t)j * r + 4 * tx;
-    const T inv_rho = (T)(1.0 / cj.rho);
-    const T alpha0 = (T)(NC == 1 ? cj.alpha : cj.cand_alpha[STEP == RS_U ? (cj.dsel ? 1 : 0) : 0]);
-    const T alpha1 = (T)(NC == 1 ? cj.alpha : cj.cand_alpha[1]);
-    const T pb = (T)cj.phibeta;
-    const T gam = (T)a.gamma;
+    const int w = r - W * tx;
+    const int64_t colj = (int64_t)j * r + W * tx;
     // inputs in the order of their slots
     const bool lx = (STEP == RS_GRAD || STEP == RS_DZ) && a.LX, old = STEP == RS_GRAD && a.Xold,
                zold = STEP == RS_GRAD && a.Zold;
@@ -181,7 +200,7 @@ __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, i
 #pragma unroll
       for (int k = 0; k < MR; ++k) {
         const int64_t row = row0 + (int64_t)k * TY;
-        copy_quad(in + (i * MR + k) * nt, (const T*)p, row * a.ld + colj, on && row < a.n, vec, w);
+        copy_pack<T, W>(in + (i * MR + k) * nt, (const T*)p, row * a.ld + colj, on && row < a.n, vec, w);
       }
     };
     auto fetch_operand = [&](int tile) {  // one copy group each, empty past the last tile
@@ -227,23 +246,32 @@ __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, i
         }
       }
     }
+    if (W < 4)  // the operand's columns past r, which no thread owns
+      for (int e = t; e < TY * MR * (c4 - r); e += nt) As[e / (c4 - r) * ls + r + e % (c4 - r)] = T(0);
     fetch_operand(cta);
     fetch_rest(cta);
+    // while the copies are on their way: the division is ten FP64 instructions
+    const T inv_rho = (T)(1.0 / cj.rho);
+    const T alpha0 = (T)(NC == 1 ? cj.alpha : cj.cand_alpha[STEP == RS_U ? (cj.dsel ? 1 : 0) : 0]);
+    const T alpha1 = (T)(NC == 1 ? cj.alpha : cj.cand_alpha[1]);
+    const T pb = (T)cj.phibeta;
+    const T gam = (T)a.gamma;
     for (int tile = cta; tile < tiles; tile += per) {
       const int64_t row0 = (int64_t)tile * (TY * MR) + ty;
       const int64_t off0 = row0 * a.ld + colj, step = (int64_t)TY * a.ld;
       T dq[8];
 #pragma unroll
       for (int m = 0; m < 8; ++m) dq[m] = T(0);
+      int zeros = 0;
       bool rv[MR];
 #pragma unroll
       for (int k = 0; k < MR; ++k) rv[k] = on && row0 + (int64_t)k * TY < a.n;
       auto get = [&](int i, int k) { return in[(i * MR + k) * nt]; };
-      auto put = [&](void* p, int k, const Quad<T>& v) {
-        if (rv[k]) store_quad((T*)p + off0 + k * step, v, vec, w);
+      auto put = [&](void* p, int k, const Pack<T, W>& v) {
+        if (rv[k]) store_pack<T, W>((T*)p + off0 + k * step, v, vec, w);
       };
       cp_async_wait<1>();
-      Quad<T> x[MR], g[MR], z[MR];
+      Pack<T, W> x[MR], g[MR], z[MR];
 #pragma unroll
       for (int k = 0; k < MR; ++k) {
         x[k] = get(0, k);
@@ -254,45 +282,45 @@ __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, i
       // the operand tile: X, Z or X'
 #pragma unroll
       for (int k = 0; k < MR; ++k) {
-        Quad<T> op = x[k];
+        Pack<T, W> op = x[k];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < W; ++q) {
           if (STEP == RS_D) op.v[q] = zstep(x[k].v[q], g[k].v[q], inv_rho);
           if (STEP == RS_U) {
             const T zz = zstep(x[k].v[q], g[k].v[q], inv_rho);
             op.v[q] = upd(zz, dir(zz, z[k].v[q], alpha0), pb);
           }
         }
-        if (on) *reinterpret_cast<Quad<T>*>(As + (ty + k * TY) * ls + 4 * tx) = op;
+        if (on) *reinterpret_cast<Pack<T, W>*>(As + (ty + k * TY) * ls + W * tx) = op;
       }
       __syncthreads();
-      Quad<T> acc[MR];
-      if (on) rowstep_product<T, MR>(As, ls, Gs, c4, tx, ty, TY, acc);
+      Pack<T, W> acc[MR];
+      if (on) rowstep_product<T, W, MR>(As, ls, Gs, c4, tx, ty, TY, acc);
       cp_async_wait<1>();
       if (STEP == RS_GRAD) {
 #pragma unroll
         for (int k = 0; k < MR; ++k) {
           if (!rv[k]) continue;
-          Quad<T> gn, l, zn;
-          const Quad<T> b = get(1, k);
+          Pack<T, W> gn, l, zn;
+          const Pack<T, W> b = get(1, k);
           if (lx) l = get(iL, k);
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
+          for (int q = 0; q < W; ++q) {
             const T xv = x[k].v[q], bv = b.v[q];
             T gv = acc[k].v[q] - bv;
             if (lx) gv += gam * l.v[q];
             gn.v[q] = gv;
             zn.v[q] = zstep(xv, gv, inv_rho);
             if (q >= w) continue;
-            const T pg = xv > T(0) ? gv : (gv < T(0) ? gv : T(0));
-            dq[0] += pg * pg;
-            dq[1] += T(0.5) * (gv - bv) * xv;
-            if (xv == T(0)) dq[6] += T(1);
+            const T pg = positive(xv) || negative(gv) ? gv : T(0);
+            dq[0] = fma_rn(pg, pg, dq[0]);
+            dq[1] = fma_rn(gv - bv, xv, dq[1]);
+            zeros += is_zero(xv);
           }
           if (old) {
-            const Quad<T> xo = get(iO, k), go = get(iO + 1, k);
+            const Pack<T, W> xo = get(iO, k), go = get(iO + 1, k);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
+            for (int q = 0; q < W; ++q) {
               const T s = x[k].v[q] - xo.v[q], y = gn.v[q] - go.v[q];
               if (q >= w) continue;
               dq[2] += s * s;
@@ -301,10 +329,10 @@ __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, i
             }
           }
           if (zold) {
-            const Quad<T> zo = get(iZ, k), gz = get(iZ + 1, k);
+            const Pack<T, W> zo = get(iZ, k), gz = get(iZ + 1, k);
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-              if (q < w) dq[5] += T(0.5) * (x[k].v[q] - zo.v[q]) * (gn.v[q] + gz.v[q]);
+            for (int q = 0; q < W; ++q)
+              if (q < w) dq[5] = fma_rn(x[k].v[q] - zo.v[q], gn.v[q] + gz.v[q], dq[5]);
           }
           if (a.gout) put(a.gout, k, gn);
           if (a.Xout) put(a.Xout, k, x[k]);
@@ -314,10 +342,10 @@ __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, i
 #pragma unroll
         for (int k = 0; k < MR; ++k) {
           if (!rv[k]) continue;
-          Quad<T> xn, gn;
-          const Quad<T> b = get(1, k);
+          Pack<T, W> xn, gn;
+          const Pack<T, W> b = get(1, k);
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
+          for (int q = 0; q < W; ++q) {
             const T xv = x[k].v[q], gv = g[k].v[q], gz = z[k].v[q], bv = b.v[q];
             const T zz = zstep(xv, gv, inv_rho);
             const T xw = upd(zz, dir(zz, gz, alpha0), pb);
@@ -325,33 +353,33 @@ __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, i
             xn.v[q] = xw;
             gn.v[q] = gw;
             if (q >= w) continue;
-            const T pg = xw > T(0) ? gw : (gw < T(0) ? gw : T(0));
-            dq[0] += pg * pg;
-            dq[1] += T(0.5) * (gw - bv) * xw;
+            const T pg = positive(xw) || negative(gw) ? gw : T(0);
+            dq[0] = fma_rn(pg, pg, dq[0]);
+            dq[1] = fma_rn(gw - bv, xw, dq[1]);
             const T s = xw - xv, y = gw - gv;
             dq[2] += s * s;
             dq[3] += s * y;
             dq[4] += y * y;
-            dq[5] += T(0.5) * (xw - zz) * (gw + gz);
-            if (xw == T(0)) dq[6] += T(1);
+            dq[5] = fma_rn(xw - zz, gw + gz, dq[5]);
+            zeros += is_zero(xw);
           }
           put(a.Xout, k, xn);
           put(a.gout, k, gn);
         }
       } else {
         // RS_D / RS_DZ: g(Z), D, their inner products; then <D G, D> with D as the operand tile
-        Quad<T> d0[MR], d1[NC == 2 ? MR : 1];
+        Pack<T, W> d0[MR], d1[NC == 2 ? MR : 1];
 #pragma unroll
         for (int k = 0; k < MR; ++k) {
-          Quad<T> gz, l, wc, gw;
-          const Quad<T> b = get(1, k);
+          Pack<T, W> gz, l, wc, gw;
+          const Pack<T, W> b = get(1, k);
           if (STEP == RS_DZ) {
             if (lx) l = get(iL, k);
             wc = get(iO, k);
             gw = get(iO + 1, k);
           }
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
+          for (int q = 0; q < W; ++q) {
             const T zz = STEP == RS_D ? zstep(x[k].v[q], g[k].v[q], inv_rho) : x[k].v[q];
             const T xv = STEP == RS_D ? x[k].v[q] : wc.v[q], gx = STEP == RS_D ? g[k].v[q] : gw.v[q];
             T gv = acc[k].v[q] - b.v[q];
@@ -364,7 +392,7 @@ __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, i
             if (!ok) continue;
             dq[0] += gv * d;
             dq[1] += d * d;
-            dq[2] += T(0.5) * (zz - xv) * (gv + gx);
+            dq[2] = fma_rn(zz - xv, gv + gx, dq[2]);
             if (NC == 2) {
               const T e = d1[NC == 2 ? k : 0].v[q];
               dq[5] += gv * e;
@@ -380,20 +408,27 @@ __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, i
           __syncthreads();  // every thread is done with the operand tile
 #pragma unroll
           for (int k = 0; k < MR; ++k)
-            if (on) *reinterpret_cast<Quad<T>*>(As + (ty + k * TY) * ls + 4 * tx) = m == 0 ? d0[k] : d1[NC == 2 ? k : 0];
+            if (on) *reinterpret_cast<Pack<T, W>*>(As + (ty + k * TY) * ls + W * tx) = m == 0 ? d0[k] : d1[NC == 2 ? k : 0];
           __syncthreads();
           if (on) {
-            rowstep_product<T, MR>(As, ls, Gs, c4, tx, ty, TY, acc);
+            rowstep_product<T, W, MR>(As, ls, Gs, c4, tx, ty, TY, acc);
             T qq = T(0);
 #pragma unroll
             for (int k = 0; k < MR; ++k)
 #pragma unroll
-              for (int q = 0; q < 4; ++q) qq = fma(acc[k].v[q], m == 0 ? d0[k].v[q] : d1[NC == 2 ? k : 0].v[q], qq);
+              for (int q = 0; q < W; ++q) qq = fma(acc[k].v[q], m == 0 ? d0[k].v[q] : d1[NC == 2 ? k : 0].v[q], qq);
             dq[m == 0 ? 4 : 7] = qq;
           }
         }
       }
-      if (STEP == RS_GRAD || STEP == RS_U) fetch_rest(tile + per);
+      if (STEP == RS_GRAD || STEP == RS_U) {
+        fetch_rest(tile + per);
+        dq[1] *= T(0.5);
+        dq[5] *= T(0.5);
+        dq[6] = (T)zeros;
+      } else {
+        dq[2] *= T(0.5);
+      }
       total += (double)warp_sum8(dq);
       if (tile + per < tiles) __syncthreads();  // the operand tile is written again
     }
