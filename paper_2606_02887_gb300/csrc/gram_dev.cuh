@@ -65,7 +65,7 @@ __device__ __forceinline__ void cp_async_wait() {
 // count of serial products bounds it, so an iteration is one shared read of v, the FMAs, the
 // lane butterfly and one barrier: v is double buffered and G scaled by a power of two to a
 // trace below one (exact; ||G|| <= trace for a Gram), so v only has to be rescaled every eighth
-// iteration (it shrinks by at most r each).  n = 64: 13 us with the norm taken in every
+// iteration (it shrinks by at most 2 r each).  n = 64: 13 us with the norm taken in every
 // iteration, 4 us so.
 // Threads t < nact = P2 TPR take part (a multiple of 32), on barrier 1.  vs: 2 (P2 + 4 TPR)
 // values, red: 2 nact / 32 values.  0 for a zero G.
@@ -107,10 +107,24 @@ __device__ __forceinline__ T power_norm(int r, int W, int nact, int iters, Dot d
   };
   for (int it = 0; it < iters; ++it) {
     T s = row();
-    if ((it & 7) == 7 || it == iters - 1) {
-      const T tot = total(fabs(s));
-      if (tot == T(0)) return T(0);
-      s /= tot;
+    // scaled by a power of two every eighth time (FP64 every 32nd: G's norm is between 1 / (2 r) and 1,
+    // and neither the vector nor its square leaves the range), by the largest exponent: integer steps,
+    // where a sum and a division are 17 FP64 instructions of 64 cycles
+    const bool scale = sizeof(T) == 8 ? (it & 31) == 31 : (it & 7) == 7 || it == iters - 1;
+    if (scale) {
+      const unsigned hi = sizeof(T) == 8 ? (unsigned)__double2hiint((double)s) & 0x7fffffffu
+                                         : __float_as_uint((float)s) & 0x7fffffffu;
+      const unsigned m = __reduce_max_sync(0xffffffffu, hi);
+      unsigned* ru = reinterpret_cast<unsigned*>(red);
+      if (lane == 0) ru[wid] = m;
+      bar_sync(1, nact);
+      unsigned top = 0u;
+      for (int w = 0; w < nw; ++w) top = max(top, ru[w]);
+      if (top == 0u) return T(0);
+      constexpr int MB = sizeof(T) == 8 ? 20 : 23, BIAS = sizeof(T) == 8 ? 1023 : 127;
+      const int ex = min(max((int)(top >> MB), 1), 2 * BIAS - 1);  // 2^(BIAS - ex) is a normal number
+      const unsigned sc = (unsigned)(2 * BIAS - ex) << MB;
+      s *= sizeof(T) == 8 ? (T)__hiloint2double((int)sc, 0) : (T)__uint_as_float(sc);
     }
     if (part == 0) nxt[at(p)] = s;
     bar_sync(1, nact);
@@ -122,7 +136,7 @@ __device__ __forceinline__ T power_norm(int r, int W, int nact, int iters, Dot d
   const T num = total(v * s);
   bar_sync(1, nact);  // red read by every thread before it is written again
   const T den = total(v * v);
-  return num / den;
+  return den == T(0) ? T(0) : num / den;
 }
 
 // power-of-two scale that brings a positive trace below one
@@ -153,6 +167,12 @@ __device__ __forceinline__ void rho_in_smem(const T* Gs, int r, int iters, doubl
   for (int u = 0; u < W; ++u) g[u] = (T)ldexp(Gs[(t >> 2) * TW + (t & 3) * W + u], -e);
   const T norm = power_norm<T, 4>(r, W, NACT, iters,
                                   [&](const T* v) {
+                                    if constexpr (sizeof(T) == 8) {  // one chain: no FP64 instruction hides another
+                                      T s = g[0] * v[0];
+#pragma unroll
+                                      for (int u = 1; u < W; ++u) s = fma(g[u], v[u], s);
+                                      return s;
+                                    }
                                     T s[4] = {T(0), T(0), T(0), T(0)};
 #pragma unroll
                                     for (int u = 0; u < W; u += 4) {
