@@ -104,7 +104,7 @@ struct snmf_ctx {
   int rec_cap = 0;
   int tc_fail = 0;               // status of a failed tensor-core launch (encoder / launch error)
   double* dsc = nullptr;   // device scratch doubles
-  int* h_flag = nullptr;   // pinned
+  int* h_flag = nullptr;   // pinned: the run flag, and from 8 bytes on two doubles of snmf_apply
   std::vector<Ctl> h_ctl;
   // captured solve phases: 0 init, 1 one iteration, 2 final evaluation
   cudaGraphExec_t exec[3] = {nullptr, nullptr, nullptr};
@@ -292,9 +292,20 @@ int ax_L(snmf_ctx* h, const void* X, void* Y, const void* P1, const void* P2, do
 // inside the iteration it follows ctl[j].active and the run flag, in the initial and
 // final evaluations (ctl == NULL) every restart is computed.
 void gram1(snmf_ctx* h, const void* X, const void* Y, int pair, const Ctl* ctl, double* G64, void* GT, int tpair,
-           double lam) {
+           double lam, cudaStream_t s = nullptr) {
   launch_gram(h->tdtype, X, Y, dims(h), h->gplan, pair, h->gpart, ctl, ctl ? h->run : nullptr, G64, GT, tpair, lam,
-              h->gcounters, h->s);
+              h->gcounters, s ? s : h->s);
+}
+
+// The side stream: work on it after fork() sees what the main stream did before it, and the main
+// stream sees that work after join() (a fork and a join of the captured graph).
+void fork(snmf_ctx* h) {
+  cudaEventRecord(h->evfork, h->s);
+  cudaStreamWaitEvent(h->s2, h->evfork, 0);
+}
+void join(snmf_ctx* h) {
+  cudaEventRecord(h->evjoin, h->s2);
+  cudaStreamWaitEvent(h->s, h->evjoin, 0);
 }
 
 RowArgs row_base(snmf_ctx* h, const Params* P = nullptr) {
@@ -560,8 +571,7 @@ void pen_block(snmf_ctx* h, int xv, int xf, bool is_w, const Params& P, bool nai
   // product (a fork and a join of the captured graph); they share no buffer with it.
   // G = Xfix^T Xfix (+ lambda I in the factor-type copy); rho_0 = ||Xfix^T Xfix||_2, computed
   // by the Gram's last CTA when the restart is one tile (r <= 64), else by k_rho_wide
-  cudaEventRecord(h->evfork, h->s);
-  cudaStreamWaitEvent(h->s2, h->evfork, 0);
+  fork(h);
   const bool rho_fused = h->gplan.ntile == 1;
   // graph-regularised H block: rho_0 = ||W^T W||_2 + gamma ||L||_2 (Lipschitz constant of its gradient)
   const double shift = gr ? h->gamma * h->normL : 0.0;
@@ -772,28 +782,35 @@ void dir_iteration(snmf_ctx* h, const Params& P) {
              h->graph ? h->gamma * h->normL : 0.0);
   launch_ctl_dir_alpha(h->ctl, h->b, P, h->s);
   launch_zstep(td, d, W, g, Z, h->ctl, h->s);
+  // each Gram on the side stream beside the product (they share no buffer)
+  fork(h);
+  gram1(h, Z, Z, 0, h->ctl, h->G64p, h->GT, 0, 0.0, h->s2);
   int nz = ax_A(h, Z, AZ, 0.0, nullptr, Z, nullptr, h->pax, h->run);
   if (h->graph) ax_L(h, Z, h->buf[B_LZ], Z, nullptr, h->pax3, h->run);
-  gram1(h, Z, Z, 0, h->ctl, h->G64p, h->GT, 0, 0.0);
+  join(h);
   {
     RowArgs a = row_base(h);
     a.X = Z; a.B = AZ; a.LX = h->graph ? h->buf[B_LZ] : nullptr;
     a.Dout = D;
     launch_rowgemm(td, OP_LOAD, EPI_DIR, a, h->s);
   }
+  fork(h);
+  gram1(h, Z, D, 0, h->ctl, h->G64p + rr, nullptr, -1, 0.0, h->s2);
+  gram1(h, D, D, 1, h->ctl, h->G64p + rr, nullptr, -1, 0.0, h->s2);
   int nd = ax_A(h, D, AD, 0.0, nullptr, Z, D, h->pax2, h->run);
   if (h->graph) ax_L(h, D, h->buf[B_LD], D, nullptr, h->pax4, h->run);
-  gram1(h, Z, D, 0, h->ctl, h->G64p + rr, nullptr, -1, 0.0);
-  gram1(h, D, D, 1, h->ctl, h->G64p + rr, nullptr, -1, 0.0);
+  join(h);
   launch_ctl_dir_ls(h->ctl, h->pax, nz, h->prow, h->nrow, h->pax2, nd, h->G64p, h->G64p + rr,
                     h->G64p + 2 * rr, h->graph ? h->pax3 : nullptr, h->graph ? h->pax4 : nullptr,
                     h->b, h->r, P, h->s);
   int ncl = launch_xupd(td, d, Z, D, Wn, AZ, AD, AWn, h->ctl, h->pclip, h->s);
+  fork(h);
+  gram1(h, Wn, Wn, 0, h->ctl, h->G64fix, h->GT, 0, 0.0, h->s2);
   launch_ctl_dir_clip(h->ctl, h->pclip, ncl, h->b, h->recompute, h->s);
   int nre = ax_A(h, Wn, AWn, 0.0, nullptr, Wn, nullptr, h->pax, h->recompute);
   int nlx = 0;
   if (h->graph) nlx = ax_L(h, Wn, h->buf[B_LX], Wn, nullptr, h->pax3, h->run);
-  gram1(h, Wn, Wn, 0, h->ctl, h->G64fix, h->GT, 0, 0.0);
+  join(h);
   {
     RowArgs a = row_base(h);
     a.X = Wn; a.B = AWn; a.LX = h->graph ? h->buf[B_LX] : nullptr;
@@ -802,9 +819,7 @@ void dir_iteration(snmf_ctx* h, const Params& P) {
   }
   launch_ctl_dir_upd(h->ctl, h->prow, h->nrow, h->pax, nre, h->graph ? h->pax3 : nullptr, nlx,
                      h->G64fix, h->recompute, h->b, h->r, P, h->s);
-  launch_copy_live(td, d, Wn, W, h->ctl, h->s);
-  launch_copy_live(td, d, AWn, AW, h->ctl, h->s);
-  launch_copy_live(td, d, gn, g, h->ctl, h->s);
+  launch_copy_live(td, d, {Wn, AWn, gn}, {W, AW, g}, h->ctl, h->s);
   launch_any_active(h->ctl, h->b, h->run, h->recompute, h->s);
 }
 
@@ -869,7 +884,7 @@ snmf_status alloc_buffers(snmf_ctx* h) {
   CK(cudaMalloc(&h->dsc, 4096 * sizeof(double)));
   CK(cudaMalloc(&h->ring, (size_t)h->b * h->ring_cap * kRingVals * sizeof(double)));
   CK(cudaMemsetAsync(h->ring, 0, (size_t)h->b * h->ring_cap * kRingVals * sizeof(double), h->s));
-  CK(cudaMallocHost(&h->h_flag, sizeof(int)));
+  CK(cudaMallocHost(&h->h_flag, 2 * sizeof(int) + 2 * sizeof(double)));
   return SNMF_OK;
 }
 
@@ -1580,19 +1595,27 @@ snmf_status snmf_apply(snmf_handle h, const void* X, void* Y, int cols, double* 
   if (h->bt) return fail(h, SNMF_ERR_STATE, "not available for a dense batch handle");
   if (!X || !Y || cols < 1 || cols > h->N) return fail(h, SNMF_ERR_ARG, "bad apply arguments");
   if (sync_user(h) != SNMF_OK) return SNMF_ERR_CUDA;
-  const size_t fe = (size_t)h->n * h->N;
-  // stage X into the (ld = N) layout, zero-padded columns
-  CK(cudaMemsetAsync(h->buf[B_Z], 0, fe * h->esz, h->s));
-  CK(cudaMemcpy2DAsync(h->buf[B_Z], h->N * h->esz, X, cols * h->esz, cols * h->esz, h->n,
-                       cudaMemcpyDeviceToDevice, h->s));
-  int nax = ax_A(h, h->buf[B_Z], h->buf[B_AZ], 0.0, nullptr, h->buf[B_Z], nullptr, h->pax, nullptr);
-  CK(cudaMemcpy2DAsync(Y, cols * h->esz, h->buf[B_AZ], h->N * h->esz, cols * h->esz, h->n,
-                       cudaMemcpyDeviceToDevice, h->s));
-  std::vector<double> part((size_t)nax * h->b * kNQ);
-  CK(cudaMemcpyAsync(part.data(), h->pax, part.size() * sizeof(double), cudaMemcpyDeviceToHost, h->s));
-  int derr = 0;
-  CK(cudaMemcpyAsync(&derr, h->dev_err, sizeof(int), cudaMemcpyDeviceToHost, h->s));
+  const size_t fbytes = (size_t)h->n * h->N * h->esz;
+  const uintptr_t px = (uintptr_t)X, py = (uintptr_t)Y;
+  // X and Y themselves when they have the handle's layout, 16-byte alignment and no byte in common;
+  // otherwise X is staged into the (ld = N) layout, zero-padded columns, and Y out of it
+  const bool direct = cols == h->N && !((px | py) & 15) && (px + fbytes <= py || py + fbytes <= px);
+  if (!direct) {
+    if (cols < h->N) CK(cudaMemsetAsync(h->buf[B_Z], 0, fbytes, h->s));
+    CK(cudaMemcpy2DAsync(h->buf[B_Z], h->N * h->esz, X, cols * h->esz, cols * h->esz, h->n,
+                         cudaMemcpyDeviceToDevice, h->s));
+  }
+  const void* Xs = direct ? X : h->buf[B_Z];
+  const int nax = ax_A(h, Xs, direct ? Y : h->buf[B_AZ], 0.0, nullptr, Xs, nullptr, h->pax, nullptr);
+  if (!direct)
+    CK(cudaMemcpy2DAsync(Y, cols * h->esz, h->buf[B_AZ], h->N * h->esz, cols * h->esz, h->n,
+                         cudaMemcpyDeviceToDevice, h->s));
+  // <X, A X> over the slots and restarts and the device error code, one copy to the host
+  launch_sum_slots(h->pax, nax * h->b, h->dev_err, h->dsc, h->s);
+  double* res = reinterpret_cast<double*>(h->h_flag + 2);
+  CK(cudaMemcpyAsync(res, h->dsc, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->s));
   CK(cudaStreamSynchronize(h->s));
+  const int derr = (int)res[1];
   if (h->tc_fail) {
     const int tf = h->tc_fail;
     h->tc_fail = 0;
@@ -1605,12 +1628,7 @@ snmf_status snmf_apply(snmf_handle h, const void* X, void* Y, int cols, double* 
     CK(cudaStreamSynchronize(h->s));
     return fail(h, SNMF_ERR_TIMEOUT, "a bounded device wait of the tensor-core product ran out");
   }
-  if (xax) {
-    double s = 0.0;
-    for (int t = 0; t < nax; ++t)
-      for (int j = 0; j < h->b; ++j) s += part[((size_t)t * h->b + j) * kNQ];
-    *xax = s;
-  }
+  if (xax) *xax = res[0];
   return SNMF_OK;
 }
 

@@ -112,15 +112,19 @@ k_xnext(int64_t n, int r, int N, int64_t ld, const T* __restrict__ Z, const T* _
   }
 }
 
+// dst[y] = src[y] of the restarts whose step is committed, three arrays (blockIdx.y)
 template <typename T>
-__global__ void k_copy_live(int64_t n, int r, int b, int64_t ld, const T* __restrict__ src,
-                            T* __restrict__ dst, const Ctl* __restrict__ ctl) {
+__global__ void k_copy_live(int64_t n, int r, int b, int64_t ld, const T* __restrict__ s0, const T* __restrict__ s1,
+                            const T* __restrict__ s2, T* __restrict__ d0, T* __restrict__ d1, T* __restrict__ d2,
+                            const Ctl* __restrict__ ctl) {
+  const T* src = blockIdx.y == 0 ? s0 : blockIdx.y == 1 ? s1 : s2;
+  T* dst = blockIdx.y == 0 ? d0 : blockIdx.y == 1 ? d1 : d2;
   const int64_t total = n * (int64_t)r * b;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = e / ((int64_t)r * b);
     const int col = (int)(e % ((int64_t)r * b));
-    if (ctl && !ctl[col / r].commit) continue;
+    if (!ctl[col / r].commit) continue;
     dst[i * ld + col] = src[i * ld + col];
   }
 }
@@ -158,25 +162,71 @@ __device__ double direct_f(double normA2, double xax, double gg, double gam, dou
   return 0.25 * (normA2 - 2.0 * xax + gg) + 0.5 * gam * xlx;
 }
 
+// Sums of sixteen values over a block of 128 threads into qs (shared, [16]); sh: [4][16].  Value m of
+// a warp ends in the lanes with lane & 15 == m: 16 FP64 additions for all of them (an FP64 instruction
+// takes 64 cycles of an SM partition; ten block sums one after the other made k_ctl_dir_ls 14.5 us).
+__device__ __forceinline__ void block_sums16(const double (&v)[16], double (*sh)[16], double* qs) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double a[8], b[4], c[2], d;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const double keep = lane & 8 ? v[8 + i] : v[i], give = lane & 8 ? v[i] : v[8 + i];
+    a[i] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const double keep = lane & 4 ? a[4 + i] : a[i], give = lane & 4 ? a[i] : a[4 + i];
+    b[i] = keep + __shfl_xor_sync(0xffffffffu, give, 4);
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const double keep = lane & 2 ? b[2 + i] : b[i], give = lane & 2 ? b[i] : b[2 + i];
+    c[i] = keep + __shfl_xor_sync(0xffffffffu, give, 2);
+  }
+  {
+    const double keep = lane & 1 ? c[1] : c[0], give = lane & 1 ? c[0] : c[1];
+    d = keep + __shfl_xor_sync(0xffffffffu, give, 1);
+  }
+  d += __shfl_xor_sync(0xffffffffu, d, 16);
+  if (lane < 16) sh[wid][lane] = d;
+  __syncthreads();
+  if (threadIdx.x < 16) qs[threadIdx.x] = (sh[0][threadIdx.x] + sh[1][threadIdx.x]) + (sh[2][threadIdx.x] + sh[3][threadIdx.x]);
+  __syncthreads();
+}
+
+// quantity q of restart j over this thread's slots
+__device__ __forceinline__ double thread_slots(const double* part, int nslots, int b, int j, int q) {
+  double s = 0.0;
+  if (part) {
+#pragma unroll 4
+    for (int t = threadIdx.x; t < nslots; t += 128) s += __ldcg(part + ((int64_t)t * b + j) * kNQ + q);
+  }
+  return s;
+}
+
 // init: pax q0 = <W, AW>; prow (EPI_GRAD) q0 = pg2; GW = W^T W; graph: plx q0 = <W,LW>
-__global__ void __launch_bounds__(256) k_ctl_dir_init(Ctl* __restrict__ ctl, const double* __restrict__ pax, int nax,
+__global__ void __launch_bounds__(128) k_ctl_dir_init(Ctl* __restrict__ ctl, const double* __restrict__ pax, int nax,
                                const double* __restrict__ prow, int nrow,
                                const double* __restrict__ plx, int nlx, const double* __restrict__ GW,
                                int b, int r, Params P) {
-  __shared__ double sh[32];
+  __shared__ double sh[4][16], qs[16];
   const int j = blockIdx.x;
   Ctl& c = ctl[j];
-  const double xax = reduce_slots(pax, nax, b, j, 0, sh);
-  const double pg2 = reduce_slots(prow, nrow, b, j, 0, sh);
-  const double gg = dot_rr(GW + (int64_t)j * r * r, GW + (int64_t)j * r * r, r, sh);
-  double xlx = 0.0;
-  if (plx) xlx = reduce_slots(plx, nlx, b, j, 0, sh);
+  double v[16] = {};
+  v[0] = thread_slots(pax, nax, b, j, 0);
+  v[1] = thread_slots(prow, nrow, b, j, 0);
+  v[2] = thread_slots(plx, nlx, b, j, 0);
+  for (int e = threadIdx.x; e < r * r; e += 128) {
+    const double g = GW[(int64_t)j * r * r + e];
+    v[3] += g * g;
+  }
+  block_sums16(v, sh, qs);
   if (threadIdx.x != 0) return;
-  c.xax = xax;
-  c.f = direct_f(P.normA2, xax, gg, P.gamma, xlx);
+  c.xax = qs[0];
+  c.f = direct_f(P.normA2, qs[0], qs[3], P.gamma, qs[2]);
   c.F = c.f;
   hist_reset(c, c.f);
-  c.pg0 = sqrt(pg2);
+  c.pg0 = sqrt(qs[1]);
   c.pg = c.pg0;
   c.k = 0;
   c.iters = 0;
@@ -198,34 +248,41 @@ __global__ void k_ctl_dir_alpha(Ctl* __restrict__ ctl, Params P) {
 // Quartic line search.  pz: q0 <Z,AZ>; prow (EPI_DIR): q0 gd, q1 dd; pd: q0 <Z,AD>, q1 <D,AD>;
 // Grams: P0 = Z^T Z (GZ), M = Z^T D (ZD), P2 = D^T D (DD).  Graph: pgl q0 <Z,LZ>, q1 <D,LZ>
 // (from the LZ finish) and pgd q0 <D,LD>.
-__global__ void __launch_bounds__(256) k_ctl_dir_ls(Ctl* __restrict__ ctl, const double* __restrict__ pz, int nz,
+__global__ void __launch_bounds__(128) k_ctl_dir_ls(Ctl* __restrict__ ctl, const double* __restrict__ pz, int nz,
                              const double* __restrict__ prow, int nrow,
                              const double* __restrict__ pd, int nd, const double* __restrict__ GZ,
                              const double* __restrict__ ZD, const double* __restrict__ DDm,
                              const double* __restrict__ pgl, const double* __restrict__ pgd,
                              int b, int r, Params P) {
-  __shared__ double sh[32];
+  __shared__ double sh[4][16], qs[16];
   const int j = blockIdx.x;
   Ctl& c = ctl[j];
   if (!c.active) return;
   const int64_t o = (int64_t)j * r * r;
-  const double xaz = reduce_slots(pz, nz, b, j, 0, sh);
-  const double gd = reduce_slots(prow, nrow, b, j, 0, sh);
-  const double zad = reduce_slots(pd, nd, b, j, 0, sh);
-  const double dad = reduce_slots(pd, nd, b, j, 1, sh);
-  const double p00 = dot_rr(GZ + o, GZ + o, r, sh);
-  const double p01 = dot_sym2(ZD + o, GZ + o, r, sh);
-  const double p02 = dot_rr(GZ + o, DDm + o, r, sh);
-  const double p11 = norm_sym2(ZD + o, r, sh);
-  const double p12 = dot_sym2(ZD + o, DDm + o, r, sh);
-  const double p22 = dot_rr(DDm + o, DDm + o, r, sh);
-  double zlz = 0.0, dlz = 0.0, dld = 0.0;
+  double v[16] = {};
+  v[0] = thread_slots(pz, nz, b, j, 0);
+  v[1] = thread_slots(prow, nrow, b, j, 0);
+  v[2] = thread_slots(pd, nd, b, j, 0);
+  v[3] = thread_slots(pd, nd, b, j, 1);
   if (pgl) {
-    zlz = reduce_slots(pgl, nz, b, j, 0, sh);
-    dlz = reduce_slots(prow, nrow, b, j, 3, sh);
-    dld = reduce_slots(pgd, nd, b, j, 0, sh);
+    v[4] = thread_slots(pgl, nz, b, j, 0);
+    v[5] = thread_slots(prow, nrow, b, j, 3);
+    v[6] = thread_slots(pgd, nd, b, j, 0);
   }
+#pragma unroll 2
+  for (int e = threadIdx.x; e < r * r; e += 128) {
+    const double gz = GZ[o + e], dd = DDm[o + e], m = ZD[o + e] + ZD[o + e % r * r + e / r];
+    v[7] += gz * gz;
+    v[8] += m * gz;
+    v[9] += gz * dd;
+    v[10] += m * m;
+    v[11] += m * dd;
+    v[12] += dd * dd;
+  }
+  block_sums16(v, sh, qs);
   if (threadIdx.x != 0) return;
+  const double xaz = qs[0], gd = qs[1], zad = qs[2], dad = qs[3], zlz = qs[4], dlz = qs[5], dld = qs[6], p00 = qs[7],
+               p01 = qs[8], p02 = qs[9], p11 = qs[10], p12 = qs[11], p22 = qs[12];
   c.xax_z = xaz; c.zad = zad; c.dad = dad; c.gd = gd;
   c.zlz = zlz; c.dlz = dlz; c.dld = dld;
   c.q = p22;  // kept for diagnostics
@@ -267,24 +324,29 @@ __global__ void __launch_bounds__(256) k_ctl_dir_clip(Ctl* __restrict__ ctl, con
 
 // after the gradient at W' (prow EPI_GRAD: q0 pg2, q2 ss, q3 sy, q4 yy), Gram GW of W',
 // optional recomputed <W', AW'> (pax q0), graph <W', LW'> (plx q0).
-__global__ void __launch_bounds__(256) k_ctl_dir_upd(Ctl* __restrict__ ctl, const double* __restrict__ prow, int nrow,
+__global__ void __launch_bounds__(128) k_ctl_dir_upd(Ctl* __restrict__ ctl, const double* __restrict__ prow, int nrow,
                               const double* __restrict__ pax, int nax,
                               const double* __restrict__ plx, int nlx,
                               const double* __restrict__ GW, const int* __restrict__ recompute,
                               int b, int r, Params P) {
-  __shared__ double sh[32];
+  __shared__ double sh[4][16], qs[16];
   const int j = blockIdx.x;
   Ctl& c = ctl[j];
   if (!c.active) return;
-  const double pg2 = reduce_slots(prow, nrow, b, j, 0, sh);
-  const double ss = reduce_slots(prow, nrow, b, j, 2, sh);
-  const double sy = reduce_slots(prow, nrow, b, j, 3, sh);
-  const double yy = reduce_slots(prow, nrow, b, j, 4, sh);
-  const double gg = dot_rr(GW + (int64_t)j * r * r, GW + (int64_t)j * r * r, r, sh);
-  double xax_re = 0.0, xlx = 0.0;
-  if (pax) xax_re = reduce_slots(pax, nax, b, j, 0, sh);
-  if (plx) xlx = reduce_slots(plx, nlx, b, j, 0, sh);
+  double v[16] = {};
+  v[0] = thread_slots(prow, nrow, b, j, 0);
+  v[1] = thread_slots(prow, nrow, b, j, 2);
+  v[2] = thread_slots(prow, nrow, b, j, 3);
+  v[3] = thread_slots(prow, nrow, b, j, 4);
+  v[4] = thread_slots(pax, nax, b, j, 0);
+  v[5] = thread_slots(plx, nlx, b, j, 0);
+  for (int e = threadIdx.x; e < r * r; e += 128) {
+    const double g = GW[(int64_t)j * r * r + e];
+    v[6] += g * g;
+  }
+  block_sums16(v, sh, qs);
   if (threadIdx.x != 0) return;
+  const double pg2 = qs[0], ss = qs[1], sy = qs[2], yy = qs[3], xax_re = qs[4], xlx = qs[5], gg = qs[6];
   if (*recompute) c.xax = xax_re;  // A W' was recomputed for every restart
   c.ss = ss; c.sy = sy; c.yy = yy;
   c.f = direct_f(P.normA2, c.xax, gg, P.gamma, xlx);
@@ -295,6 +357,17 @@ __global__ void __launch_bounds__(256) k_ctl_dir_upd(Ctl* __restrict__ ctl, cons
   c.commit = 1;
   if (!isfinite(c.f)) { c.nan_seen = 1; c.active = 0; c.commit = 0; return; }
   if (c.pg <= P.tol * c.pg0 || c.iters >= P.max_iter) c.active = 0;
+}
+
+// out[0] = quantity 0 of all `records` partial records, out[1] = *err; one block
+__global__ void __launch_bounds__(128) k_sum_slots(const double* __restrict__ part, int records, const int* __restrict__ err,
+                                                   double* __restrict__ out) {
+  __shared__ double sh[32];
+  const double s = block_sum(thread_slots(part, records, 1, 0, 0), sh);
+  if (threadIdx.x == 0) {
+    out[0] = s;
+    out[1] = (double)*err;
+  }
 }
 
 // *flag = OR over restarts of ctl[j].active
@@ -534,13 +607,14 @@ void launch_xnext(int tdtype, const Dims& d, const void* Z, const void* D, void*
 #undef XNEXT
 }
 
-void launch_copy_live(int tdtype, const Dims& d, const void* src, void* dst, const Ctl* ctl,
+void launch_copy_live(int tdtype, const Dims& d, const void* const (&src)[3], void* const (&dst)[3], const Ctl* ctl,
                       cudaStream_t s) {
-  const int blocks = grid1d(d.n * d.N);
-  if (tdtype == 0)
-    k_copy_live<double><<<blocks, 256, 0, s>>>(d.n, d.r, d.b, d.ld, (const double*)src, (double*)dst, ctl);
-  else
-    k_copy_live<float><<<blocks, 256, 0, s>>>(d.n, d.r, d.b, d.ld, (const float*)src, (float*)dst, ctl);
+  const dim3 grid(grid1d(d.n * d.N), 3);
+#define COPY(T)                                                                                                          \
+  k_copy_live<T><<<grid, 256, 0, s>>>(d.n, d.r, d.b, d.ld, (const T*)src[0], (const T*)src[1], (const T*)src[2], (T*)dst[0], \
+                                      (T*)dst[1], (T*)dst[2], ctl)
+  if (tdtype == 0) COPY(double); else COPY(float);
+#undef COPY
 }
 
 void launch_philox_uniform(int tdtype, void* out, int64_t rows, int cols, int64_t ld, uint64_t seed,
@@ -598,7 +672,7 @@ void launch_ctl_pen_ls(Ctl* ctl, const double* prow, int nrow, const double* pax
 void launch_ctl_dir_init(Ctl* ctl, const double* pax, int nax, const double* prow, int nrow,
                          const double* plx, int nlx, const double* GW, int b, int r, const Params& P,
                          cudaStream_t s) {
-  k_ctl_dir_init<<<b, 256, 0, s>>>(ctl, pax, nax, prow, nrow, plx, nlx, GW, b, r, P);
+  k_ctl_dir_init<<<b, 128, 0, s>>>(ctl, pax, nax, prow, nrow, plx, nlx, GW, b, r, P);
 }
 void launch_ctl_dir_alpha(Ctl* ctl, int b, const Params& P, cudaStream_t s) {
   k_ctl_dir_alpha<<<b, 32, 0, s>>>(ctl, P);
@@ -607,7 +681,7 @@ void launch_ctl_dir_ls(Ctl* ctl, const double* pz, int nz, const double* prow, i
                        const double* pd, int nd, const double* GZ, const double* ZD,
                        const double* DDm, const double* pgl, const double* pgd, int b, int r,
                        const Params& P, cudaStream_t s) {
-  k_ctl_dir_ls<<<b, 256, 0, s>>>(ctl, pz, nz, prow, nrow, pd, nd, GZ, ZD, DDm, pgl, pgd, b, r, P);
+  k_ctl_dir_ls<<<b, 128, 0, s>>>(ctl, pz, nz, prow, nrow, pd, nd, GZ, ZD, DDm, pgl, pgd, b, r, P);
 }
 void launch_ctl_dir_clip(Ctl* ctl, const double* pclip, int nslots, int b, int* recompute,
                          cudaStream_t s) {
@@ -616,7 +690,10 @@ void launch_ctl_dir_clip(Ctl* ctl, const double* pclip, int nslots, int b, int* 
 void launch_ctl_dir_upd(Ctl* ctl, const double* prow, int nrow, const double* pax, int nax,
                         const double* plx, int nlx, const double* GW, const int* recompute, int b,
                         int r, const Params& P, cudaStream_t s) {
-  k_ctl_dir_upd<<<b, 256, 0, s>>>(ctl, prow, nrow, pax, nax, plx, nlx, GW, recompute, b, r, P);
+  k_ctl_dir_upd<<<b, 128, 0, s>>>(ctl, prow, nrow, pax, nax, plx, nlx, GW, recompute, b, r, P);
+}
+void launch_sum_slots(const double* part, int records, const int* err, double* out, cudaStream_t s) {
+  k_sum_slots<<<1, 128, 0, s>>>(part, records, err, out);
 }
 void launch_any_active(const Ctl* ctl, int b, int* flag, int* recompute, cudaStream_t s) {
   k_any_active<<<1, 32, 0, s>>>(ctl, b, flag, recompute);

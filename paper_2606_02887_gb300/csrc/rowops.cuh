@@ -110,7 +110,7 @@ int launch_xupd(int tdtype, const Dims& d, const void* Z, const void* D, void* X
                 const void* AD, void* AXn, const Ctl* ctl, double* part, cudaStream_t s);
 // Xn = Proj[Z + phi beta D] of the live restarts alone (the graph-regularised block)
 void launch_xnext(int tdtype, const Dims& d, const void* Z, const void* D, void* Xn, const Ctl* ctl, cudaStream_t s);
-void launch_copy_live(int tdtype, const Dims& d, const void* src, void* dst, const Ctl* ctl,
+void launch_copy_live(int tdtype, const Dims& d, const void* const (&src)[3], void* const (&dst)[3], const Ctl* ctl,
                       cudaStream_t s);
 // rho = scale ||G||_2 + shift per restart (shift: gamma ||L||_2 of a graph-regularised block)
 void launch_rho(int tdtype, const double* G64, const Dims& d, int iters, double scale, Ctl* ctl, cudaStream_t s,
@@ -142,6 +142,7 @@ void launch_ctl_dir_upd(Ctl* ctl, const double* prow, int nrow, const double* pa
                         int r, const Params& P, cudaStream_t s);
 void init_kernel_attributes();
 void launch_sum_pairs(const double* part, int m, double* out, cudaStream_t s);
+void launch_sum_slots(const double* part, int records, const int* err, double* out, cudaStream_t s);
 void launch_any_active(const Ctl* ctl, int b, int* flag, int* recompute, cudaStream_t s);
 void launch_ctl_final_pen(Ctl* ctl, const double* pax, int nax, const double* prow, int nrow,
                           const double* GW, const double* GH, const double* WH, int b, int r,
