@@ -103,6 +103,111 @@ k_rowmul(const typename C::T* __restrict__ In, int64_t ldi, int K, const typenam
   }
 }
 
+// The same in FP32 for long inputs whose rows, M and Out allow 16-byte accesses, all m <= BN columns in
+// one tile: a CTA walks tiles of BM rows with M resident and a ring of three stages of BK columns of
+// In that runs on over the tiles, X2 on its way during the last stage.  FMAs in the order of k_rowmul.
+// Bound by HBM and, close behind, by the FMA pipes: n = 2e6, K = 64, m = 32 285 -> 217 us (1.0 GB).
+template <typename C, int PER_SM>
+__global__ void __launch_bounds__(C::NT, PER_SM)
+k_rowmul_walk(const float* __restrict__ In, int64_t ldi, int K, const float* __restrict__ Mm, int m, int64_t n, int tiles,
+              float* __restrict__ Out, int64_t ldo, float c, const float* __restrict__ X2, const int* run) {
+  extern __shared__ __align__(16) unsigned char rsm[];
+  if (run && *run == 0) return;
+  constexpr int BM = C::BM, BN = C::BN, BK = C::BK, AS = C::AS, ST = 3, STAGE = BM * AS;
+  const int t = threadIdx.x, tx = t % C::TX, ty = t / C::TX;
+  const int nk = (K + BK - 1) / BK;
+  float* ring = reinterpret_cast<float*>(rsm);
+  float* Ms = ring + ST * STAGE;
+  for (int e = t; e < nk * BK * BN; e += C::NT) {
+    const int k = e / BN, q = e % BN;
+    Ms[e] = k < K && q < m ? Mm[(int64_t)k * m + q] : 0.f;
+  }
+  const int mine = (tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x, steps = mine * nk;
+  auto fetch = [&](int s) {
+    if (s < steps) {
+      const int64_t row0 = ((int64_t)blockIdx.x + (int64_t)(s / nk) * gridDim.x) * BM;
+      const int k0 = s % nk * BK;
+      float* as = ring + s % ST * STAGE;
+      constexpr int NA = BM * BK / 4;
+#pragma unroll
+      for (int u = 0; u < NA / C::NT; ++u) {
+        const int e = t + C::NT * u, r = e / (BK / 4), k = k0 + e % (BK / 4) * 4;
+        const bool v = row0 + r < n && k < K;
+        cp_async<16>(as + r * AS + (k - k0), v ? In + (row0 + r) * ldi + k : In, v);
+      }
+    }
+    cp_async_commit();
+  };
+#pragma unroll
+  for (int s = 0; s < ST - 1; ++s) fetch(s);
+  float acc[C::TM][C::TN];
+  for (int s = 0; s < steps; ++s) {
+    const int kc = s % nk;
+    const int64_t row0 = ((int64_t)blockIdx.x + (int64_t)(s / nk) * gridDim.x) * BM;
+    cp_async_wait<ST - 2>();
+    __syncthreads();  // stage s is in (and M); every thread is done with the stage refilled below
+    fetch(s + ST - 1);
+    if (kc == 0) {
+#pragma unroll
+      for (int i = 0; i < C::TM; ++i)
+#pragma unroll
+        for (int j = 0; j < C::TN; ++j) acc[i][j] = 0.f;
+    }
+    float4 x2[C::TM][C::TN / 4];
+    if (X2 && kc == nk - 1) {
+#pragma unroll
+      for (int i = 0; i < C::TM; ++i)
+#pragma unroll
+        for (int j = 0; j < C::TN / 4; ++j) {
+          const int64_t r = row0 + ty + C::TY * i;
+          const int col = C::col(tx, 4 * j);
+          x2[i][j] = r < n && col < m ? *reinterpret_cast<const float4*>(X2 + r * ldo + col) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    }
+    const float* as = ring + s % ST * STAGE;
+    const float* xs = Ms + kc * BK * BN;
+#pragma unroll
+    for (int kk = 0; kk < BK; kk += 4) {
+      float a[C::TM][4];
+#pragma unroll
+      for (int i = 0; i < C::TM; ++i) {
+        const float4 v = *reinterpret_cast<const float4*>(as + (ty + C::TY * i) * AS + kk);
+        a[i][0] = v.x; a[i][1] = v.y; a[i][2] = v.z; a[i][3] = v.w;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        float x[C::TN];
+#pragma unroll
+        for (int j = 0; j < C::TN; j += 4) {
+          const float4 v = *reinterpret_cast<const float4*>(xs + (kk + u) * BN + C::col(tx, j));
+          x[j] = v.x; x[j + 1] = v.y; x[j + 2] = v.z; x[j + 3] = v.w;
+        }
+        fma_row<C>(a, u, x, acc);
+      }
+    }
+    if (kc != nk - 1) continue;
+#pragma unroll
+    for (int i = 0; i < C::TM; ++i) {
+      const int64_t r = row0 + ty + C::TY * i;
+      if (r >= n) continue;
+#pragma unroll
+      for (int j = 0; j < C::TN / 4; ++j) {
+        const int col = C::col(tx, 4 * j);
+        if (col >= m) continue;
+        float4 y = make_float4(acc[i][4 * j], acc[i][4 * j + 1], acc[i][4 * j + 2], acc[i][4 * j + 3]);
+        if (X2) {
+          y.x = y.x + c * x2[i][j].x;
+          y.y = y.y + c * x2[i][j].y;
+          y.z = y.z + c * x2[i][j].z;
+          y.w = y.w + c * x2[i][j].w;
+        }
+        *reinterpret_cast<float4*>(Out + r * ldo + col) = y;
+      }
+    }
+  }
+  cp_async_wait<0>();
+}
+
 // Cholesky of G + shift I (l x l FP64, row-major, overwritten by R, upper) and Rinv (FP64,
 // then copied to the working type).  *fail = 1 on a non-positive pivot.
 template <typename T>
@@ -286,6 +391,23 @@ void launch_rowmul_cfg(const void* In, int64_t ldi, int K, const void* M, int m,
   const bool avec = ldi % KV == 0 && K % KV == 0 && !((uintptr_t)In & 15);
   const bool xvec = m % KV == 0 && !((uintptr_t)M & 15);
   const bool yvec = ldo % VW == 0 && m % VW == 0 && !(((uintptr_t)Out | (uintptr_t)X2) & 15);
+  // long inputs walk: more than two tiles for each of three CTAs per SM (n = 2e6, K = 64, m = 32 285 us
+  // with a CTA per tile)
+  if constexpr (sizeof(T) == 4 && C::BK == 32) {
+    constexpr int kPerSm = 3;
+    const int64_t tiles = cdivi(n, C::BM);
+    if (avec && yvec && m <= C::BN && tiles > 2 * 152 * kPerSm) {
+      const size_t smem = (3 * C::BM * C::AS + (size_t)cdivi(K, C::BK) * C::BK * C::BN) * sizeof(float);
+      static std::once_flag walk;
+      std::call_once(walk, [] {
+        cudaFuncSetAttribute(k_rowmul_walk<C, kPerSm>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)((3 * C::BM * C::AS + 128 * C::BN) * sizeof(float)));
+      });
+      k_rowmul_walk<C, kPerSm><<<152 * kPerSm, C::NT, smem, s>>>((const float*)In, ldi, K, (const float*)M, m, n, (int)tiles,
+                                                                (float*)Out, ldo, (float)c, (const float*)X2, run);
+      return;
+    }
+  }
   dim3 grid(cdivi(n, C::BM), cdivi(m, C::BN));
   k_rowmul<C, PER_SM><<<grid, C::NT, C::SMEM, s>>>((const T*)In, ldi, K, (const T*)M, m, n, (T*)Out, ldo, avec, xvec,
                                                    yvec, (T)c, (const T*)X2, run);
@@ -305,7 +427,7 @@ void launch_rowmul(int tdtype, const void* In, int64_t ldi, int K, const void* M
   }
   if (m <= 16) ROWMUL(float, 128, 16, 4, 4, 32, 3);
   if (m <= 32) ROWMUL(float, 128, 32, 8, 4, 32, 3);
-  ROWMUL(float, 128, 64, 8, 8, 16, 4);
+  ROWMUL(float, 128, 64, 8, 8, 32, 3);
 #undef ROWMUL
 }
 
