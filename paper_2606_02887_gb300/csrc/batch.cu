@@ -578,18 +578,26 @@ void bany(BatchCtx* b) {
   k_bcompact<<<kLists, 1024, 0, b->s>>>(ca);
 }
 
+// The side stream: work on it between the two runs beside the main stream's (a fork and a join of
+// the captured graph); the Grams and the products share no buffer.
+void bfork(BatchCtx* b) {
+  cudaEventRecord(b->evfork, b->s);
+  cudaStreamWaitEvent(b->s2, b->evfork, 0);
+}
+void bjoin(BatchCtx* b) {
+  cudaEventRecord(b->evjoin, b->s2);
+  cudaStreamWaitEvent(b->s, b->evjoin, 0);
+}
+
 // one block of Algorithm 1 for all problems (penalty form; mirrors the single-problem path)
 void bpen_block(BatchCtx* b, int xv, int xf, bool is_w, const Params& P) {
   void* X = b->buf[xv];
   void* Xf = b->buf[xf];
-  // G = Xf^T Xf (+lam I) and rho depend on Xf alone: they run on the side stream beside the
-  // product (a fork and a join of the captured graph) and share no buffer with it
-  cudaEventRecord(b->evfork, b->s);
-  cudaStreamWaitEvent(b->s2, b->evfork, 0);
+  // G = Xf^T Xf (+lam I) and rho depend on Xf alone: beside the product
+  bfork(b);
   bgram(b, Xf, Xf, 0, b->ctl, b->run, b->G64fix, b->GT, b->ctl, b->s2);
-  cudaEventRecord(b->evjoin, b->s2);
   bprod(b, Xf, b->buf[XB_B], nullptr, nullptr, b->ctl, b->run);             // B = A Xf + lam Xf
-  cudaStreamWaitEvent(b->s, b->evjoin, 0);
+  bjoin(b);
   {
     RowArgs a = brow_base(b, P);
     a.X = X; a.B = b->buf[XB_B]; a.gout = b->buf[XB_G];
@@ -613,8 +621,10 @@ void bpen_block(BatchCtx* b, int xv, int xf, bool is_w, const Params& P) {
 
 void bpen_init(BatchCtx* b, const Params& P) {
   bany(b);
+  bfork(b);
+  bgram(b, b->buf[XB_W], b->buf[XB_W], 0, b->ctl, b->run, b->G64fix, b->GT, nullptr, b->s2);
   bprod(b, b->buf[XB_W], b->buf[XB_B], nullptr, nullptr, b->ctl, b->run);
-  bgram(b, b->buf[XB_W], b->buf[XB_W], 0, b->ctl, b->run, b->G64fix, b->GT, nullptr);
+  bjoin(b);
   RowArgs a = brow_base(b, P);
   a.X = b->buf[XB_HT]; a.B = b->buf[XB_B]; a.gout = b->buf[XB_G];
   a.ctl_mode = CTL_START_INIT;
@@ -633,10 +643,12 @@ void bpen_final(BatchCtx* b, const Params& P) {
   // accumulation bias would be amplified by the cancellation in the residual).
   b->use_full = true;
   b->accurate = true;
+  bfork(b);
+  bgram(b, b->buf[XB_W], b->buf[XB_W], 0, nullptr, nullptr, b->G64p, nullptr, nullptr, b->s2);
+  bgram(b, b->buf[XB_HT], b->buf[XB_HT], 1, nullptr, nullptr, b->G64p, b->GT, nullptr, b->s2);
+  bgram(b, b->buf[XB_W], b->buf[XB_HT], 2, nullptr, nullptr, b->G64p, nullptr, nullptr, b->s2);
   bprod(b, b->buf[XB_HT], b->buf[XB_B], b->buf[XB_W], b->pax, nullptr, nullptr);
-  bgram(b, b->buf[XB_W], b->buf[XB_W], 0, nullptr, nullptr, b->G64p, nullptr, nullptr);
-  bgram(b, b->buf[XB_HT], b->buf[XB_HT], 1, nullptr, nullptr, b->G64p, b->GT, nullptr);
-  bgram(b, b->buf[XB_W], b->buf[XB_HT], 2, nullptr, nullptr, b->G64p, nullptr, nullptr);
+  bjoin(b);
   RowArgs a = brow_base(b, P);
   a.X = b->buf[XB_W]; a.B = b->buf[XB_B]; a.gout = b->buf[XB_G];
   a.run = nullptr;
@@ -1015,9 +1027,13 @@ snmf_status batch_solve(BatchCtx* b, bool host, void* W, void* Ht, snmf_stats* o
     const int m = std::min(chunk, maxit - launched);
     for (int t = 0; t < m; ++t) BCK(cudaGraphLaunch(b->exec[1], b->s));
     launched += m;
+    if (launched == maxit) break;
     BCK(cudaMemcpyAsync(b->h_flag, b->run, sizeof(int), cudaMemcpyDeviceToHost, b->s));
-    BCK(cudaStreamSynchronize(b->s));
+    BCK(cudaEventRecord(b->evsync, b->s));
+    BCK(cudaGraphLaunch(b->exec[1], b->s));  // before the flag is read, as in solve_impl
+    BCK(cudaEventSynchronize(b->evsync));
     if (*b->h_flag == 0) break;
+    ++launched;
     chunk = std::min(chunk * 2, 8);
   }
   launches += (int64_t)b->nodes[1] * launched;

@@ -695,9 +695,11 @@ void pen_block(snmf_ctx* h, int xv, int xf, bool is_w, const Params& P, bool nai
 // H gradient at the start point (enters the first joint projected gradient).
 void pen_init(snmf_ctx* h, const Params& P) {
   launch_any_active(h->ctl, h->b, h->run, nullptr, h->s);
+  fork(h);
+  gram1(h, h->buf[B_W], h->buf[B_W], 0, h->ctl, h->G64fix, h->GT, 0, h->lam, h->s2);
   ax_A(h, h->buf[B_W], h->buf[B_B], h->lam, h->buf[B_W], nullptr, nullptr, h->pax, h->run);
-  gram1(h, h->buf[B_W], h->buf[B_W], 0, h->ctl, h->G64fix, h->GT, 0, h->lam);
   if (h->graph) ax_L(h, h->buf[B_HT], h->buf[B_LX], nullptr, nullptr, h->pax2, h->run);
+  join(h);
   RowArgs a = row_base(h, &P);
   a.X = h->buf[B_HT]; a.B = h->buf[B_B]; a.LX = h->graph ? h->buf[B_LX] : nullptr;
   a.gout = h->buf[B_G];
@@ -729,11 +731,14 @@ void pen_final(snmf_ctx* h, const Params& P) {
   // a relative bias of about 1e-5 over K = 8192, which that cancellation would amplify.
   AxArgs fin = h->A;
   fin.accurate = 1;
+  // The three Grams run on the side stream beside it (10 to 45 us each one after the other).
+  fork(h);
+  gram1(h, h->buf[B_W], h->buf[B_W], 0, nullptr, h->G64p, h->GT, 1, h->lam, h->s2);
+  gram1(h, h->buf[B_HT], h->buf[B_HT], 1, nullptr, h->G64p, h->GT, 1, h->lam, h->s2);
+  gram1(h, h->buf[B_W], h->buf[B_HT], 2, nullptr, h->G64p, h->GT, 1, h->lam, h->s2);
   int nax = ax_apply(h, fin, h->lai, h->buf[B_HT], h->buf[B_B], h->lam, h->buf[B_HT],
                      h->buf[B_W], nullptr, h->pax, nullptr);
-  gram1(h, h->buf[B_W], h->buf[B_W], 0, nullptr, h->G64p, h->GT, 1, h->lam);
-  gram1(h, h->buf[B_HT], h->buf[B_HT], 1, nullptr, h->G64p, h->GT, 1, h->lam);
-  gram1(h, h->buf[B_W], h->buf[B_HT], 2, nullptr, h->G64p, h->GT, 1, h->lam);
+  join(h);
   // W gradient at the final point (projected-gradient statistic); uses a temporary
   // "all active" view: the row kernel is run with ctl entries forced live by the host.
   RowArgs a = row_base(h);
@@ -1471,7 +1476,7 @@ static snmf_status solve_impl(snmf_ctx* h, bool host, void* W, void* Ht, snmf_st
   }
   nvtxRangePop();
   nvtxRangePushA("snmf_solve: iterations");
-  int done = 0, launched = 0, chunk = 1;
+  int launched = 0, chunk = 1;
   int done_before = 0;  // outer iterations of an imported state
   for (int j = 0; j < h->b; ++j) done_before = std::max(done_before, resume ? h->h_ctl[j].iters : 0);
   const int maxit = std::max(0, h->opt.max_iter - (h->opt.formulation == SNMF_DIRECT ? 0 : done_before));
@@ -1479,12 +1484,17 @@ static snmf_status solve_impl(snmf_ctx* h, bool host, void* W, void* Ht, snmf_st
     const int m = std::min(chunk, maxit - launched);
     for (int t = 0; t < m; ++t) CK(cudaGraphLaunch(h->exec[1], h->s));
     launched += m;
+    if (launched == maxit) break;
+    // the next iteration is launched before the flag is read (its kernels return at once when nothing is
+    // active), so the GPU has work while the host waits
     CK(cudaMemcpyAsync(h->h_flag, h->run, sizeof(int), cudaMemcpyDeviceToHost, h->s));
-    CK(cudaStreamSynchronize(h->s));
-    if (*h->h_flag == 0) { done = 1; break; }
+    CK(cudaEventRecord(h->evsync, h->s));
+    CK(cudaGraphLaunch(h->exec[1], h->s));
+    CK(cudaEventSynchronize(h->evsync));
+    if (*h->h_flag == 0) break;
+    ++launched;
     chunk = std::min(chunk * 2, 8);
   }
-  (void)done;
   nvtxRangePop();
   launches += (int64_t)h->nodes[1] * launched;
   nvtxRangePushA("snmf_solve: final evaluation");
