@@ -22,9 +22,11 @@
 // multiple of 4 only.  A CTA walks several tiles: each thread copies its own inputs of the next tile
 // to shared memory (asynchronously, no barrier) as soon as it has read the current one's there, the
 // operand's inputs first, B and what else the epilogue reads after it; G is read once, and one
-// record of partials, in FP64 over the tiles, leaves the CTA.  Bound by HBM for long factors (a
-// CTA per tile, without copies ahead: n = 2e6, r = 32 block-start gradient 407 us, D step 471, update
-// 501) and by launch latency for short ones.
+// record of partials, in FP64 over the tiles, leaves the CTA.  For long factors HBM, the shared
+// loads and the instructions around the product are within a factor of two of one another (n = 2e6, r =
+// 32: block-start gradient 209 us, D step 300, update 293; a CTA per tile, without copies ahead 407, 471,
+// 501; with Z and X' recomputed after the product instead of read from the operand tile and every row and
+// column tested 227, 320, 316); short ones are bound by launch latency.
 #pragma once
 
 #include "rowops_dev.cuh"
@@ -56,8 +58,8 @@ struct alignas(W * sizeof(T) < 16 ? W * sizeof(T) : 16) Pack {
 };
 
 // explicit FMAs: the D step and the update compute the same bits
-template <typename T>
-__device__ __forceinline__ T proj0(T t) { return positive(t) ? t : T(0); }
+__device__ __forceinline__ float proj0(float t) { return fmaxf(t, 0.f); }  // NaN: 0, in both
+__device__ __forceinline__ double proj0(double t) { return positive(t) ? t : 0.0; }
 template <typename T>
 __device__ __forceinline__ T zstep(T x, T g, T inv_rho) { return proj0(fma_rn(-g, inv_rho, x)); }
 template <typename T>
@@ -110,14 +112,15 @@ __device__ __forceinline__ void store_pack(T* p, const Pack<T, W>& v, bool vec, 
   }
 }
 
-// acc[p] = (row ty + TY p of As) G[:, W tx ..], k ascending in one chain per entry
+// acc[p] = (row ty + TY p of As) G[:, W tx ..], k ascending in one chain per entry; zeros when not on
 template <typename T, int W, int MR>
 __device__ __forceinline__ void rowstep_product(const T* As, int ls, const T* Gs, int c4, int tx, int ty, int TY,
-                                                Pack<T, W> (&acc)[MR]) {
+                                                Pack<T, W> (&acc)[MR], bool on) {
 #pragma unroll
   for (int p = 0; p < MR; ++p)
 #pragma unroll
     for (int q = 0; q < W; ++q) acc[p].v[q] = T(0);
+  if (!on) return;
   const T* ar = As + ty * ls;
   const T* gr = Gs + W * tx;
 #pragma unroll 2
@@ -267,6 +270,15 @@ __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, i
 #pragma unroll
       for (int k = 0; k < MR; ++k) rv[k] = on && row0 + (int64_t)k * TY < a.n;
       auto get = [&](int i, int k) { return in[(i * MR + k) * nt]; };
+      // this thread's values of the operand tile; rows, columns and threads beyond the tile hold zeros in
+      // every array, which add nothing to the sums
+      auto operand = [&](int k) {
+        Pack<T, W> v;
+#pragma unroll
+        for (int q = 0; q < W; ++q) v.v[q] = T(0);
+        if (on) v = *reinterpret_cast<const Pack<T, W>*>(As + (ty + k * TY) * ls + W * tx);
+        return v;
+      };
       auto put = [&](void* p, int k, const Pack<T, W>& v) {
         if (rv[k]) store_pack<T, W>((T*)p + off0 + k * step, v, vec, w);
       };
@@ -295,12 +307,11 @@ __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, i
       }
       __syncthreads();
       Pack<T, W> acc[MR];
-      if (on) rowstep_product<T, W, MR>(As, ls, Gs, c4, tx, ty, TY, acc);
+      rowstep_product<T, W, MR>(As, ls, Gs, c4, tx, ty, TY, acc, on);
       cp_async_wait<1>();
       if (STEP == RS_GRAD) {
 #pragma unroll
         for (int k = 0; k < MR; ++k) {
-          if (!rv[k]) continue;
           Pack<T, W> gn, l, zn;
           const Pack<T, W> b = get(1, k);
           if (lx) l = get(iL, k);
@@ -311,7 +322,6 @@ __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, i
             if (lx) gv += gam * l.v[q];
             gn.v[q] = gv;
             zn.v[q] = zstep(xv, gv, inv_rho);
-            if (q >= w) continue;
             const T pg = positive(xv) || negative(gv) ? gv : T(0);
             dq[0] = fma_rn(pg, pg, dq[0]);
             dq[1] = fma_rn(gv - bv, xv, dq[1]);
@@ -322,7 +332,6 @@ __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, i
 #pragma unroll
             for (int q = 0; q < W; ++q) {
               const T s = x[k].v[q] - xo.v[q], y = gn.v[q] - go.v[q];
-              if (q >= w) continue;
               dq[2] += s * s;
               dq[3] += s * y;
               dq[4] += y * y;
@@ -332,7 +341,7 @@ __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, i
             const Pack<T, W> zo = get(iZ, k), gz = get(iZ + 1, k);
 #pragma unroll
             for (int q = 0; q < W; ++q)
-              if (q < w) dq[5] = fma_rn(x[k].v[q] - zo.v[q], gn.v[q] + gz.v[q], dq[5]);
+              dq[5] = fma_rn(x[k].v[q] - zo.v[q], gn.v[q] + gz.v[q], dq[5]);
           }
           if (a.gout) put(a.gout, k, gn);
           if (a.Xout) put(a.Xout, k, x[k]);
@@ -341,18 +350,16 @@ __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, i
       } else if (STEP == RS_U) {
 #pragma unroll
         for (int k = 0; k < MR; ++k) {
-          if (!rv[k]) continue;
-          Pack<T, W> xn, gn;
+          Pack<T, W> gn;
           const Pack<T, W> b = get(1, k);
+          const Pack<T, W> xn = operand(k);
 #pragma unroll
           for (int q = 0; q < W; ++q) {
             const T xv = x[k].v[q], gv = g[k].v[q], gz = z[k].v[q], bv = b.v[q];
             const T zz = zstep(xv, gv, inv_rho);
-            const T xw = upd(zz, dir(zz, gz, alpha0), pb);
+            const T xw = xn.v[q];
             const T gw = acc[k].v[q] - bv;
-            xn.v[q] = xw;
             gn.v[q] = gw;
-            if (q >= w) continue;
             const T pg = positive(xw) || negative(gw) ? gw : T(0);
             dq[0] = fma_rn(pg, pg, dq[0]);
             dq[1] = fma_rn(gw - bv, xw, dq[1]);
@@ -373,6 +380,8 @@ __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, i
         for (int k = 0; k < MR; ++k) {
           Pack<T, W> gz, l, wc, gw;
           const Pack<T, W> b = get(1, k);
+          Pack<T, W> op;
+          if (STEP == RS_D) op = operand(k);
           if (STEP == RS_DZ) {
             if (lx) l = get(iL, k);
             wc = get(iO, k);
@@ -380,16 +389,14 @@ __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, i
           }
 #pragma unroll
           for (int q = 0; q < W; ++q) {
-            const T zz = STEP == RS_D ? zstep(x[k].v[q], g[k].v[q], inv_rho) : x[k].v[q];
+            const T zz = STEP == RS_D ? op.v[q] : x[k].v[q];
             const T xv = STEP == RS_D ? x[k].v[q] : wc.v[q], gx = STEP == RS_D ? g[k].v[q] : gw.v[q];
             T gv = acc[k].v[q] - b.v[q];
             if (lx) gv += gam * l.v[q];
             gz.v[q] = gv;
-            const bool ok = rv[k] && q < w;
-            const T d = ok ? dir(zz, gv, alpha0) : T(0);
+            const T d = dir(zz, gv, alpha0);
             d0[k].v[q] = d;
-            if (NC == 2) d1[NC == 2 ? k : 0].v[q] = ok ? dir(zz, gv, alpha1) : T(0);
-            if (!ok) continue;
+            if (NC == 2) d1[NC == 2 ? k : 0].v[q] = dir(zz, gv, alpha1);
             dq[0] += gv * d;
             dq[1] += d * d;
             dq[2] = fma_rn(zz - xv, gv + gx, dq[2]);
@@ -411,7 +418,7 @@ __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, i
             if (on) *reinterpret_cast<Pack<T, W>*>(As + (ty + k * TY) * ls + W * tx) = m == 0 ? d0[k] : d1[NC == 2 ? k : 0];
           __syncthreads();
           if (on) {
-            rowstep_product<T, W, MR>(As, ls, Gs, c4, tx, ty, TY, acc);
+            rowstep_product<T, W, MR>(As, ls, Gs, c4, tx, ty, TY, acc, true);
             T qq = T(0);
 #pragma unroll
             for (int k = 0; k < MR; ++k)
@@ -425,6 +432,9 @@ __device__ __forceinline__ void rowstep_body(const RowArgs& a, int j, int cta, i
         fetch_rest(tile + per);
         dq[1] *= T(0.5);
         dq[5] *= T(0.5);
+        // the rows and columns that do not exist: all zeros, which only the count sees
+#pragma unroll
+        for (int k = 0; k < MR; ++k) zeros -= rv[k] ? max(0, W - w) : W;
         dq[6] = (T)zeros;
       } else {
         dq[2] *= T(0.5);
