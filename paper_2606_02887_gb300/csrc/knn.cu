@@ -406,8 +406,8 @@ int knn_parts(int64_t n) {
 
 // The filter: for rows that two CTAs of an SM hold beside their rings, and where its launches are worth
 // it (whole call, d = 16, k = 10: n = 1024 256 us without it and 224 with it; n = 5001, d = 33, k = 12
-// 511 and 315; n = 20000, d = 64 3250 and 890).  The candidate's index is 26 bits.
-bool knn_tc_rule(int64_t n, int d) { return d <= KT_MAXD && n >= 1024 && n < (1 << 26); }
+// 511 and 315; n = 20000, d = 64 3250 and 890); up to 4 million points, whose candidate lists are 4 GB.
+bool knn_tc_rule(int64_t n, int d) { return d <= KT_MAXD && n >= 1024 && n < (1 << 22); }
 
 // Candidate ranges of its passes: about four waves of CTAs (n = 20000, d = 64: 1401 us with one range,
 // 1171 with seven), none shorter than 256.
