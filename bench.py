@@ -215,14 +215,13 @@ def run_reference(args):
 
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch, from the ncu captures summarised
-# in profiles/ (k_gemm_tc_dense8192_N512.md, k_rowfuse_dstep_dense8192_N512.md,
-# k_rowtc_dense8192_N512.md, k_rowtma_dense8192_N512.md, k_bgemm_tc_uneven256.md); keys:
+# in profiles/ (k_gemm_tc_dense8192_N512.md, k_rowtc_dense8192_N512.md,
+# k_rowtma_dense8192_N512.md, k_bgemm_tc_uneven256.md); keys:
 # (workload, precision, r, batch, kernel, row-kernel body or X parts; "dense8192-sym": A held
 # as its upper tiles), values: (bytes, the tuned tile shapes of the capture, which the run must
 # share).  Other configurations, and runs tuned to other tiles, report null.
 PROFILED_TRAFFIC = {
     ("uneven", "bf16", None, None, "product"): (875.5e6, {}),
-    ("dense8192", "bf16", 64, 8, "dstep", 2): (51.4e6, {"row_bm": 128}),
     ("dense8192", "bf16", 64, 8, "product", 2): (274.31e6, {"splits": 4, "bn": 128}),
     ("dense8192-sym", "bf16", 64, 8, "product", 2): (213.78e6, {"splits": 4, "bn": 128}),
     ("dense8192", "bf16", 64, 8, "dstep", 3): (51.03e6, {}),
@@ -755,10 +754,10 @@ def main():
         # the library reports which row-kernel body runs and the arrays each launch moves
         sc = S.snmf_step_config(h)
         body = {0: "k_rowgemm (general)", 1: "k_rowtile (shared-memory tile body)",
-                2: "k_rowfuse (Z and D recomputed, not stored; row products on CUDA cores)",
+                2: "k_rowstep (Z and D recomputed, not stored; row products on CUDA cores)",
                 3: "k_rowtc (Z and D recomputed, not stored; row products on tcgen05, TF32 hi + lo)",
                 4: "k_rowtma (as k_rowtc, persistent: one CTA per SM, inputs streamed by TMA)"}[sc["body"]]
-        prefix = {2: "k_rowfuse", 3: "k_rowtc"}.get(sc["body"])
+        prefix = {2: "k_rowstep", 3: "k_rowtc"}.get(sc["body"])
         names = {"dstep": (prefix + "_dstep" if prefix else "k_rowgemm<OP_ZSTEP, EPI_DIR>"),
                  "update": (prefix + "_update" if prefix else "k_rowgemm<OP_UPD, EPI_GRAD>")}
         if sc["body"] == 4:

@@ -372,7 +372,7 @@ SNMF_API snmf_status snmf_profile_steps(snmf_handle h, int iters, double* ms_dst
  * the update of this handle's penalty blocks, and their algorithmic bytes per launch (every
  * n x (r batch) array a launch reads or writes, once).  *body: 0 the general row kernel
  * (Z and D stored; D step 6 arrays, 7 with the learned step's second direction, update 8),
- * 1 the shared-memory tile body (same traffic), 2 the recomputing kernels (Z and D not stored:
+ * 1 not used, 2 the recomputing kernels (r <= 128; Z and D not stored:
  * D step 4 arrays, update 6), 3 the recomputing kernels with their row products on the tensor
  * cores (tcgen05 TF32 with hi / lo operand parts; r = 64, chosen by the autotuner when faster),
  * 4 the same arithmetic as persistent kernels (one CTA per SM over 128-row tiles, inputs streamed
@@ -393,11 +393,9 @@ SNMF_API snmf_status snmf_tuned_config(snmf_handle h, int32_t* splits, int32_t* 
 
 /*
  * The tile shapes chosen by the same autotuner: *bn = columns of X per tensor-core product
- * tile (0 where the product kernel has no such choice) and *row_bm = rows per CTA of the row
- * kernels of a step (FP32 penalty form: the recomputing kernels' 64 / 128 (r = 16: 128 / 256)
- * where snmf_step_config reports body 2, else the general kernel's 32 / 64; 0 where the
- * shared-memory tile body with its fixed height runs).  SNMF_ERR_STATE when the handle was not
- * tuned.
+ * tile (0 where the product kernel has no such choice) and *row_bm = rows per CTA of the
+ * general row kernel (32 / 64) where it was tuned; 0 for the other row kernels, whose tiles follow from
+ * the size.  SNMF_ERR_STATE when the handle was not tuned.
  */
 SNMF_API snmf_status snmf_tuned_tiles(snmf_handle h, int32_t* bn, int32_t* row_bm);
 
@@ -498,9 +496,12 @@ SNMF_API snmf_status snmf_set_timeout(snmf_handle h, int64_t cycles);
  *   degree       device, n FP32, out (may be NULL): d_i
  *   capacity     entries available; 2 n k always suffices.  *nnz (host) receives the count;
  *                a count above capacity returns SNMF_ERR_ARG with *nnz set.
- * Work runs on `stream`; the call returns when it is done.  Allocates device scratch.
+ * Work runs on `stream`; the call returns when it is done.  Device scratch is allocated in stream order
+ * from a pool of the library's own, which keeps up to 128 MB per device between calls; snmf_destroy of
+ * any handle gives it back.
  * Errors: SNMF_ERR_ARG, SNMF_ERR_OOM, SNMF_ERR_CUDA; SNMF_ERR_NUMERIC when a distance is not
- * finite or a scale s_i is zero (more than sigma_rank - 1 copies of a point), with no output.
+ * finite or a scale s_i is zero (more than sigma_rank - 1 copies of a point), SNMF_ERR_TIMEOUT when a
+ * bounded device wait ran out, both with no output.
  */
 SNMF_API snmf_status snmf_knn_graph(const float* X, int64_t n, int d, int k, int sigma_rank, int32_t* rowptr,
                                     int32_t* colidx, float* a_hat, float* s_values, float* degree,
