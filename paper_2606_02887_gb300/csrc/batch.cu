@@ -604,7 +604,7 @@ void bpen_block(BatchCtx* b, int xv, int xf, bool is_w, const Params& P) {
     a.ctl_mode = is_w ? CTL_START_W : CTL_START_H;
     brow(b, RS_GRAD, a);
   }
-  bany(b);
+  if (is_w) bany(b);  // the step that ends a problem
   const int K = b->opt.inner_iters;
   const int nc = b->opt.step_controller == 1 ? 2 : 1;  // record mode is not offered on batch handles
   for (int k = 0; k < K; ++k) {
@@ -634,7 +634,6 @@ void bpen_init(BatchCtx* b, const Params& P) {
 void bpen_iteration(BatchCtx* b, const Params& P) {
   bpen_block(b, XB_W, XB_HT, true, P);
   bpen_block(b, XB_HT, XB_W, false, P);
-  bany(b);
 }
 
 void bpen_final(BatchCtx* b, const Params& P) {
