@@ -83,7 +83,8 @@ k_xupd(int64_t n, int r, int b, int64_t ld, const T* __restrict__ Z, const T* __
   if (threadIdx.x == 0) part[((int64_t)blockIdx.x * b + j) * kNQ + 0] = total;
 }
 
-// The same without the clip count: blockIdx.y = 64 rows, a thread V columns of every fourth row.
+// The same without the clip count: blockIdx.x = 64 rows (their tiles may be more than grid.y holds),
+// blockIdx.y = 64 V columns, a thread V columns of every fourth row.
 template <typename T, int V>
 __global__ void __launch_bounds__(256)
 k_xnext(int64_t n, int r, int N, int64_t ld, const T* __restrict__ Z, const T* __restrict__ D, T* __restrict__ Xn,
@@ -91,12 +92,12 @@ k_xnext(int64_t n, int r, int N, int64_t ld, const T* __restrict__ Z, const T* _
   struct alignas(V * sizeof(T)) Vec {
     T v[V];
   };
-  const int col = (blockIdx.x * 64 + (threadIdx.x & 63)) * V;
+  const int col = (blockIdx.y * 64 + (threadIdx.x & 63)) * V;
   if (col >= N) return;
   const Ctl& c = ctl[col / r];  // V divides r: one restart
   if (!c.active) return;
   const T pb = (T)c.phibeta;
-  const int64_t i0 = (int64_t)blockIdx.y * 64 + (threadIdx.x >> 6);
+  const int64_t i0 = (int64_t)blockIdx.x * 64 + (threadIdx.x >> 6);
 #pragma unroll 4
   for (int k = 0; k < 16; ++k) {
     const int64_t i = i0 + 4 * k;
@@ -597,7 +598,7 @@ void launch_xnext(int tdtype, const Dims& d, const void* Z, const void* D, void*
   const int v = tdtype == 0 ? 2 : 4;
   const bool vec = d.r % v == 0 && d.ld % v == 0 && !(((uintptr_t)Z | (uintptr_t)D | (uintptr_t)Xn) & 15);
 #define XNEXT(T, V)                                                                                            \
-  k_xnext<T, V><<<dim3(cdiv(d.N, 64 * V), cdiv(d.n, 64)), 256, 0, s>>>(d.n, d.r, d.N, d.ld, (const T*)Z, (const T*)D, \
+  k_xnext<T, V><<<dim3(cdiv(d.n, 64), cdiv(d.N, 64 * V)), 256, 0, s>>>(d.n, d.r, d.N, d.ld, (const T*)Z, (const T*)D, \
                                                                        (T*)Xn, ctl)
   if (tdtype == 0) {
     if (vec) XNEXT(double, 2); else XNEXT(double, 1);
