@@ -1003,20 +1003,30 @@ snmf_status batch_solve(BatchCtx* b, bool host, void* W, void* Ht, snmf_stats* o
   static const int one = 1;
   BCK(cudaMemcpyAsync(b->run, &one, sizeof(int), cudaMemcpyHostToDevice, b->s));
   const Params P = bparams(b);
-  if (!b->exec[0]) {
-    for (int g = 0; g < 3; ++g) {
-      cudaGraph_t gr;
-      BCK(cudaStreamBeginCapture(b->s, cudaStreamCaptureModeThreadLocal));
-      if (g == 0) bpen_init(b, P);
-      else if (g == 1) bpen_iteration(b, P);
-      else bpen_final(b, P);
-      BCK(cudaStreamEndCapture(b->s, &gr));
-      size_t nn = 0;
-      BCK(cudaGraphGetNodes(gr, nullptr, &nn));
-      b->nodes[g] = (int)nn;
-      BCK(cudaGraphInstantiate(&b->exec[g], gr, 0));
-      cudaGraphDestroy(gr);
+  for (int g = 0; g < 3; ++g) {
+    if (b->exec[g]) continue;
+    cudaGraph_t gr = nullptr;
+    BCK(cudaStreamBeginCapture(b->s, cudaStreamCaptureModeThreadLocal));
+    if (g == 0) bpen_init(b, P);
+    else if (g == 1) bpen_iteration(b, P);
+    else bpen_final(b, P);
+    // a graph in which a refused launch is missing is not kept: the next solve would replay it
+    const cudaError_t refused_launch = cudaGetLastError();
+    cudaError_t ended = cudaStreamEndCapture(b->s, &gr);
+    size_t nn = 0;
+    if (refused_launch == cudaSuccess && !b->tc_fail && ended == cudaSuccess) {
+      ended = cudaGraphGetNodes(gr, nullptr, &nn);
+      if (ended == cudaSuccess) ended = cudaGraphInstantiate(&b->exec[g], gr, 0);
     }
+    if (gr) cudaGraphDestroy(gr);
+    if (b->tc_fail) {
+      *err = "tensor-core product not launched (status " + std::to_string(b->tc_fail) + ")";
+      b->tc_fail = 0;
+      return SNMF_ERR_CUDA;
+    }
+    BCK(refused_launch);
+    BCK(ended);
+    b->nodes[g] = (int)nn;
   }
   BCK(cudaGraphLaunch(b->exec[0], b->s));
   launches += b->nodes[0];

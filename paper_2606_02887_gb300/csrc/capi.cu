@@ -1450,21 +1450,33 @@ static snmf_status solve_impl(snmf_ctx* h, bool host, void* W, void* Ht, snmf_st
   // capture init / iteration / final once per configuration (buffers are fixed)
   const int form = naive ? 2 : (pen ? 0 : 1);
   if (h->exec_form != form) {
+    h->exec_form = -1;
     for (int g = 0; g < 3; ++g) {
       if (h->exec[g]) { cudaGraphExecDestroy(h->exec[g]); h->exec[g] = nullptr; }
-      cudaGraph_t gr;
+      cudaGraph_t gr = nullptr;
       CK(cudaStreamBeginCapture(h->s, cudaStreamCaptureModeThreadLocal));
       h->ax_count = 0;
       if (g == 0) { if (naive) naive_init(h); else if (pen) pen_init(h, P); else dir_init(h, P); }
       else if (g == 1) { if (naive) naive_iteration(h, P); else if (pen) pen_iteration(h, P); else dir_iteration(h, P); }
       else { if (pen) pen_final(h, P); else dir_final(h, P); }
-      CK(cudaStreamEndCapture(h->s, &gr));
+      // a graph in which a refused launch is missing is not kept: the next solve would replay it
+      const cudaError_t refused_launch = cudaGetLastError();
+      cudaError_t ended = cudaStreamEndCapture(h->s, &gr);
       size_t nn = 0;
-      CK(cudaGraphGetNodes(gr, nullptr, &nn));
+      if (refused_launch == cudaSuccess && !h->tc_fail && ended == cudaSuccess) {
+        ended = cudaGraphGetNodes(gr, nullptr, &nn);
+        if (ended == cudaSuccess) ended = cudaGraphInstantiate(&h->exec[g], gr, 0);
+      }
+      if (gr) cudaGraphDestroy(gr);
+      if (h->tc_fail) {
+        const int tf = h->tc_fail;
+        h->tc_fail = 0;
+        return fail(h, SNMF_ERR_CUDA, "tensor-core product not launched (status " + std::to_string(tf) + ")");
+      }
+      CK(refused_launch);
+      CK(ended);
       h->nodes[g] = (int)nn;
       h->axn[g] = h->ax_count - ((!pen && g == 1) ? 1 : 0);  // direct: clipped recompute is conditional
-      CK(cudaGraphInstantiate(&h->exec[g], gr, 0));
-      cudaGraphDestroy(gr);
     }
     h->exec_form = form;
   }

@@ -76,3 +76,38 @@ except S.SnmfError as e:
 print(json.dumps([st, [l for l in log() if l[0]], sum("k_xnext" in l[2] for l in log())]))
 """)
     assert got[1] == [] and got[2] > 0 and got[0] == S.SNMF_OK
+
+
+@pytest.mark.parametrize("kind,kernel", [("csr", "k_rowstep"), ("csr", "k_ctl_final_pen"), ("direct", "k_xupd"),
+                                         ("bf16", "k_gemm_tc"), ("batch", "k_bfinal"), ("batch", "k_brow")])
+def test_refused_launch_is_not_recorded(fake, kind, kernel):
+    """A solve whose launch is refused while its iteration is recorded fails, and the next one on the handle
+    launches that kernel again instead of replaying the rest."""
+    first, again, state = fake(f"""
+kind, kernel = {kind!r}, {kernel!r}
+n, r = 320, 4
+o = dict(max_iter=1, inner_iters=2)
+if kind == "csr":
+    h = S.snmf_create(S.csr_matrix(n, *ring(n)), r, S.snmf_default_options(**o))
+elif kind == "batch":
+    h = S.snmf_create(S.dense_batch_matrix(np.ones(2 * n * n, np.float32), [n, n], [r, r]), 0, S.snmf_default_options(**o))
+else:
+    if kind == "direct":
+        o["formulation"] = S.SNMF_DIRECT
+    else:
+        o["precision"] = S.SNMF_BF16
+    h = S.snmf_create(S.dense_matrix(np.ones((n, n), np.float32)), r, S.snmf_default_options(**o))
+W = np.ones(2 * n * r if kind == "batch" else (n, r), np.float32)
+out = []
+for refuse in (kernel, "none"):
+    fake.fake_refuse(refuse.encode())
+    fake.fake_clear()
+    try:
+        S.snmf_solve_host(h, W, None if kind == "direct" else W.copy())
+        out.append("solved")
+    except S.SnmfError as e:
+        out.append("failed")
+out.append([l[0] for l in log() if kernel in l[2]])
+print(json.dumps(out))
+""")
+    assert first == "failed" and again == "solved" and state and not any(state)
