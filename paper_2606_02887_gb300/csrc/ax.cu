@@ -12,7 +12,6 @@
 
 #include <algorithm>
 #include <cmath>
-#include <mutex>
 
 #include "common.cuh"
 #include "gemm_dev.cuh"
@@ -269,10 +268,8 @@ template <typename C, typename TA, int PER_SM>
 int launch_gemm_cfg(const AxArgs& a, int64_t n, int cols, int64_t ld, const void* X, void* Y, void* ws, size_t ws_elems,
                     const int* run, cudaStream_t s, const ProdTune* tune) {
   using T = typename C::T;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    cudaFuncSetAttribute(k_gemm_dense<C, TA, PER_SM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-  });
+  static SmemLimit limit;
+  raise_smem_limit(limit, (const void*)k_gemm_dense<C, TA, PER_SM>, C::SMEM);
   const int gx = cdiv64(cols, C::BN), gy = cdiv64(n, C::BM);
   // split-K.  FP32 (chunks of 64 columns and more): least time of an SM, its CTAs one after the other
   // at their chunk's columns plus 64 for the start and the end of a CTA, slower by the root of the

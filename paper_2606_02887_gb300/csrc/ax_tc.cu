@@ -1096,18 +1096,11 @@ int launch_tc_impl(const void* A16, int64_t n, const float* X, int N, int64_t ld
   if (!make_map(&mh, xh, ldk, N, ldk, pl.BN) || !make_map(&ml, xparts == 2 ? xl : xh, ldk, N, ldk, pl.BN))
     return -1;
   if (!sym) mt = ma;
-  static bool attr_done[2] = {false, false};
-  if (!attr_done[a8]) {
-    // the plan never asks for more than ~206 KB; static shared memory comes on top
-    const cudaError_t ae = a8 ? cudaFuncSetAttribute(k_gemm_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     210 * 1024)
-                              : cudaFuncSetAttribute(k_gemm_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     210 * 1024);
-    if (ae != cudaSuccess) {
-      g_last_cu = 10000 + (int)cudaGetLastError();
-      return -3;
-    }
-    attr_done[a8] = true;
+  static SmemLimit limit[2];
+  // the plan never asks for more than ~206 KB; static shared memory comes on top
+  if (raise_smem_limit(limit[a8], a8 ? (const void*)k_gemm_tc<true> : (const void*)k_gemm_tc<false>, 210 * 1024) != cudaSuccess) {
+    g_last_cu = 10000 + (int)cudaGetLastError();
+    return -3;
   }
   TcParams p;
   p.n = n;
@@ -1187,13 +1180,10 @@ int launch_bgemm_tc(const void* A16, int64_t lda, int64_t rows_total, const void
       !make_map(&ml, xl, lda, xt_rows, lda, 16))
     return -1;
   const size_t smem = (size_t)kBStages * kBStageBytes + 1024 + 8 * (2 * kBStages + 2) + 64;
-  static bool attr_done = false;
-  if (!attr_done) {
-    if (cudaFuncSetAttribute(k_bgemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-      g_last_cu = 10000 + (int)cudaGetLastError();
-      return -3;
-    }
-    attr_done = true;
+  static SmemLimit limit;
+  if (raise_smem_limit(limit, (const void*)k_bgemm_tc, smem) != cudaSuccess) {
+    g_last_cu = 10000 + (int)cudaGetLastError();
+    return -3;
   }
   k_bgemm_tc<<<nitems, 128, smem, s>>>(ma, mh, ml, items, cnt, X, Y, add_lam, P1, part, nq,
                                        (const unsigned char*)ctl, ctl_stride, active_off, run, err, budget);

@@ -25,7 +25,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstddef>
-#include <mutex>
 #include <numeric>
 #include <string>
 #include <vector>
@@ -496,10 +495,8 @@ void bprod(BatchCtx* b, const void* X, void* Y, const void* P1, double* part, co
 #define BGEMM(T, TA, KIND)                                                                                            \
   do {                                                                                                                \
     constexpr size_t smem = bgemm_smem<BGemm<T, KIND>>();                                                             \
-    static std::once_flag once;                                                                                       \
-    std::call_once(once, [] {                                                                                         \
-      cudaFuncSetAttribute(k_bgemm<T, TA, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);             \
-    });                                                                                                               \
+    static SmemLimit limit;                                                                                           \
+    raise_smem_limit(limit, (const void*)k_bgemm<T, TA, KIND>, smem);                                                 \
     k_bgemm<T, TA, KIND><<<g, BGemm<T, KIND>::NT, smem, b->s>>>((const TA*)b->A, b->lda, b->dp, il, c, (const T*)X,   \
                                                                 (T*)Y, 1, (const T*)P1, part, ctl, run);              \
   } while (0)
@@ -538,11 +535,8 @@ RowArgs brow_base(BatchCtx* b, const Params& P) {
 
 template <typename T, int STEP, int NC>
 void launch_brow(BatchCtx* b, const RowArgs& a) {
-  static std::once_flag once;
-  std::call_once(once, [] {
-    cudaFuncSetAttribute(k_brow<T, STEP, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)rowstep_smem<T>(64, kRowThreads, rowstep_mr<T>(), 4));
-  });
+  static SmemLimit limit;
+  raise_smem_limit(limit, (const void*)k_brow<T, STEP, NC>, rowstep_smem<T>(64, kRowThreads, rowstep_mr<T>(), 4));
   k_brow<T, STEP, NC><<<(unsigned)b->h_row.size(), kRowThreads, b->row_smem, b->s>>>(a, b->dp, blist(b, 0), bcnt(b, 0));
 }
 

@@ -989,7 +989,6 @@ snmf_status snmf_create(snmf_handle* out, const snmf_matrix* Am, int r, const sn
     int dev_count = 0;
     if (cudaGetDeviceCount(&dev_count) != cudaSuccess || dev_count == 0)
       return fail(nullptr, SNMF_ERR_CUDA, "no CUDA device");
-    init_kernel_attributes();
     h = new snmf_ctx();
     h->opt = o;
     h->prec = o.precision;
@@ -1053,7 +1052,6 @@ snmf_status snmf_create(snmf_handle* out, const snmf_matrix* Am, int r, const sn
       return bail(e_ == cudaErrorMemoryAllocation ? SNMF_ERR_OOM : SNMF_ERR_CUDA);         \
     }                                                                                      \
   } while (0)
-  init_kernel_attributes();
   CKC(cudaStreamCreateWithFlags(&h->s, cudaStreamNonBlocking));
   CKC(cudaStreamCreateWithFlags(&h->s2, cudaStreamNonBlocking));
   CKC(cudaEventCreateWithFlags(&h->evfork, cudaEventDisableTiming));

@@ -12,6 +12,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "tune.cuh"
 
 namespace snmf {
@@ -208,6 +210,15 @@ void launch_assign(int tdtype, const void* F, int64_t n, int64_t ld, int64_t col
 // -D^-1/2 A D^-1/2 in the factor type (dense: n x n with leading dimension n; CSR: the values
 // on A's pattern), so that L X = X + out X.
 void launch_normalized_adjacency(const AxArgs& a, int tdtype, int64_t n, double* s, void* out, cudaStream_t st);
+
+// Dynamic shared memory above 48 KB (pool.cu): the limit of a kernel belongs to the kernel in one context,
+// so it is raised on the kernel's first launch there, and again after a device reset or on another device.
+// One SmemLimit per kernel (of static storage).  An error is also the runtime's last one, and the launch
+// without the limit is refused.
+struct SmemLimit {
+  std::atomic<unsigned long long> ctx[64] = {};  // id of the context per device
+};
+cudaError_t raise_smem_limit(SmemLimit& l, const void* kernel, size_t bytes);
 
 // Workspaces of calls without a handle (pool.cu): stream-ordered, from the library's pool.
 cudaError_t workspace_alloc(void** p, size_t bytes, cudaStream_t s);

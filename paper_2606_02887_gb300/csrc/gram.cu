@@ -1,7 +1,6 @@
 // r x r Gram X_j^T Y_j of each restart j (Eq. (2.1): H H^T, and the Z^T D, D^T D products of the
 // line-search polynomial) and rho = ||G||_2 by the power method (Alg. 1 line 2, Eq. (2.11)).
 #include <algorithm>
-#include <mutex>
 
 #include "common.cuh"
 #include "gram_dev.cuh"
@@ -142,10 +141,8 @@ template <typename T, int TW, int VEC>
 static void launch_gram_t(const void* X, const void* Y, const Dims& d, const GramPlan& pl, void* gpart, const Ctl* ctl,
                           const int* run, double* G64, void* GT, double lam, unsigned* counters, Ctl* rho_ctl,
                           int rho_iters, double rho_scale, double rho_shift, cudaStream_t s) {
-  static std::once_flag once;
-  std::call_once(once, [] {
-    cudaFuncSetAttribute(k_gram<T, TW, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gram_smem<T>(false));
-  });
+  static SmemLimit limit;
+  raise_smem_limit(limit, (const void*)k_gram<T, TW, VEC>, gram_smem<T>(false));
   const size_t smem = gram_smem<T>(X == Y && pl.ntile == 1);
   dim3 grid(pl.nch, d.b * pl.ntile * pl.ntile);
   k_gram<T, TW, VEC><<<grid, 256, smem, s>>>((const T*)X, (const T*)Y, d.n, d.r, d.ld, pl, (T*)gpart, ctl, run, G64,
@@ -177,13 +174,6 @@ void launch_gram(int tdtype, const void* X, const void* Y, const Dims& d, const 
 #undef GRAM
 }
 
-void init_kernel_attributes() {
-  static std::once_flag once;
-  std::call_once(once, [] {
-    cudaFuncSetAttribute(k_rho_wide<float, 4, 64, 32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
-  });
-}
-
 void launch_rho(int tdtype, const double* G64, const Dims& d, int iters, double scale, Ctl* ctl, cudaStream_t s,
                 double shift) {
 #define RHO_ARGS G64, d.r, iters, scale, shift, ctl
@@ -195,7 +185,11 @@ void launch_rho(int tdtype, const double* G64, const Dims& d, int iters, double 
   if (tdtype == 0) {
     RHO(double) else k_rho_wide<double, 4, 64, 0, false><<<d.b, 1024, 0, s>>>(RHO_ARGS);
   } else {
-    RHO(float) else k_rho_wide<float, 4, 64, 32, true><<<d.b, 1024, 128 * 1024, s>>>(RHO_ARGS);
+    RHO(float) else {
+      static SmemLimit limit;
+      raise_smem_limit(limit, (const void*)k_rho_wide<float, 4, 64, 32, true>, 128 * 1024);
+      k_rho_wide<float, 4, 64, 32, true><<<d.b, 1024, 128 * 1024, s>>>(RHO_ARGS);
+    }
   }
 #undef RHO
 #undef RHO_ARGS

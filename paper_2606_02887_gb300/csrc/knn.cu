@@ -16,7 +16,6 @@
 #include <climits>
 #include <cmath>
 #include <limits>
-#include <mutex>
 #include <vector>
 
 #include "../../include/snmf.h"
@@ -433,12 +432,8 @@ struct KnnWork {
 template <int PASS, int KR>
 cudaError_t launch_knn_pass(const CUtensorMap& map, const CUtensorMap& cmap, const float* cnrm, int stride, int64_t n, int d,
                             int k, const KnnWork& w, cudaStream_t s) {
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(k_knn_tc<PASS, KR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)knn_tc_smem(KT_MAXD));
-  });
-  if (attr != cudaSuccess) return attr;
+  static SmemLimit limit;
+  if (const cudaError_t e = raise_smem_limit(limit, (const void*)k_knn_tc<PASS, KR>, knn_tc_smem(KT_MAXD))) return e;
   const int64_t nc = (n + stride - 1) / stride, per = ((nc + w.tc_parts - 1) / w.tc_parts + KT_C - 1) / KT_C * KT_C;
   dim3 grid((unsigned)((n + KT_Q - 1) / KT_Q), w.tc_parts);
   k_knn_tc<PASS, KR><<<grid, KT_THREADS, knn_tc_smem(d), s>>>(map, cmap, w.nrm, cnrm, nc, stride, w.kth, n, d, k, per,
@@ -447,10 +442,8 @@ cudaError_t launch_knn_pass(const CUtensorMap& map, const CUtensorMap& cmap, con
 }
 
 cudaError_t launch_knn(const float* X, int64_t n, int d, int k, const KnnWork& w, int32_t* nbr, float* nd2, cudaStream_t s) {
-  static std::once_flag once;
-  std::call_once(once, [] {
-    cudaFuncSetAttribute(k_knn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(KnnSmem));
-  });
+  static SmemLimit limit;
+  if (const cudaError_t e = raise_smem_limit(limit, (const void*)k_knn, sizeof(KnnSmem))) return e;
   const bool vec = d % 4 == 0 && !((uintptr_t)X & 15);
   const unsigned mb = (unsigned)((n + 7) / 8);
   const int* only_if = nullptr;

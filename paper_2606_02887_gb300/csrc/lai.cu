@@ -12,7 +12,6 @@
 #include <math.h>
 
 #include <algorithm>
-#include <mutex>
 #include <string>
 
 #include "ax_tc.cuh"
@@ -383,10 +382,6 @@ template <typename C, int PER_SM>
 void launch_rowmul_cfg(const void* In, int64_t ldi, int K, const void* M, int m, int64_t n, void* Out, int64_t ldo,
                        const int* run, cudaStream_t s, double c, const void* X2) {
   using T = typename C::T;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    cudaFuncSetAttribute(k_rowmul<C, PER_SM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-  });
   constexpr int64_t KV = C::KV, VW = C::VW;
   const bool avec = ldi % KV == 0 && K % KV == 0 && !((uintptr_t)In & 15);
   const bool xvec = m % KV == 0 && !((uintptr_t)M & 15);
@@ -398,16 +393,15 @@ void launch_rowmul_cfg(const void* In, int64_t ldi, int K, const void* M, int m,
     const int64_t tiles = cdivi(n, C::BM);
     if (avec && yvec && m <= C::BN && tiles > 2 * 152 * kPerSm) {
       const size_t smem = (3 * C::BM * C::AS + (size_t)cdivi(K, C::BK) * C::BK * C::BN) * sizeof(float);
-      static std::once_flag walk;
-      std::call_once(walk, [] {
-        cudaFuncSetAttribute(k_rowmul_walk<C, kPerSm>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)((3 * C::BM * C::AS + 128 * C::BN) * sizeof(float)));
-      });
+      static SmemLimit walk;
+      raise_smem_limit(walk, (const void*)k_rowmul_walk<C, kPerSm>, (3 * C::BM * C::AS + 128 * C::BN) * sizeof(float));
       k_rowmul_walk<C, kPerSm><<<152 * kPerSm, C::NT, smem, s>>>((const float*)In, ldi, K, (const float*)M, m, n, (int)tiles,
                                                                 (float*)Out, ldo, (float)c, (const float*)X2, run);
       return;
     }
   }
+  static SmemLimit limit;
+  raise_smem_limit(limit, (const void*)k_rowmul<C, PER_SM>, C::SMEM);
   dim3 grid(cdivi(n, C::BM), cdivi(m, C::BN));
   k_rowmul<C, PER_SM><<<grid, C::NT, C::SMEM, s>>>((const T*)In, ldi, K, (const T*)M, m, n, (T*)Out, ldo, avec, xvec,
                                                    yvec, (T)c, (const T*)X2, run);
@@ -438,10 +432,8 @@ int utx_tq(int N) { return N <= 16 ? 16 : (N <= 32 ? 32 : 64); }
 
 template <typename T, int TQ, int VEC>
 void launch_utx(const LaiOp& op, const void* X, int64_t n, int N, int64_t ldx, const int* run, cudaStream_t s) {
-  static std::once_flag once;
-  std::call_once(once, [] {
-    cudaFuncSetAttribute(k_utx<T, TQ, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)utx_smem<T>(TQ));
-  });
+  static SmemLimit limit;
+  raise_smem_limit(limit, (const void*)k_utx<T, TQ, VEC>, utx_smem<T>(TQ));
   dim3 grid(op.nch, cdivi(op.k, 64), cdivi(N, TQ));
   k_utx<T, TQ, VEC><<<grid, 256, utx_smem<T>(TQ), s>>>((const T*)op.U, op.k, (const T*)X, n, N, ldx, op.chunk, op.nch,
                                                        op.ng, (T*)op.xpart, op.lam, (T*)op.M, op.counters, run);

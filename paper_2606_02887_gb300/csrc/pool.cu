@@ -1,4 +1,5 @@
-// Device memory for the workspaces of calls that have no handle: stream-ordered allocations from a
+// What the library keeps per device and context: the shared-memory limits of its kernels (SmemLimit), and
+// device memory for the workspaces of calls that have no handle: stream-ordered allocations from a
 // pool of the library's own on each device, which keeps up to kPoolKeep bytes between calls (a
 // cudaMalloc and cudaFree of the kNN workspace took about a third of the call).  snmf_destroy gives back
 // what the pool holds unused.  The runtime orders reuse over streams and threads.
@@ -68,6 +69,16 @@ cudaMemPool_t device_pool(bool make) {
 }
 
 }  // namespace
+
+cudaError_t raise_smem_limit(SmemLimit& l, const void* kernel, size_t bytes) {
+  int dev = 0;
+  unsigned long long id = 0;
+  const bool known = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices && context_id(&id) && id;
+  if (known && l.ctx[dev].load(std::memory_order_relaxed) == id) return cudaSuccess;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess && known) l.ctx[dev].store(id, std::memory_order_relaxed);
+  return e;
+}
 
 cudaError_t workspace_alloc(void** p, size_t bytes, cudaStream_t s) {
   cudaMemPool_t pool = device_pool(true);

@@ -140,7 +140,6 @@ void launch_ctl_dir_clip(Ctl* ctl, const double* pclip, int nslots, int b, int* 
 void launch_ctl_dir_upd(Ctl* ctl, const double* prow, int nrow, const double* pax, int nax,
                         const double* plx, int nlx, const double* GW, const int* recompute, int b,
                         int r, const Params& P, cudaStream_t s);
-void init_kernel_attributes();
 void launch_sum_pairs(const double* part, int m, double* out, cudaStream_t s);
 void launch_sum_slots(const double* part, int records, const int* err, double* out, cudaStream_t s);
 void launch_any_active(const Ctl* ctl, int b, int* flag, int* recompute, cudaStream_t s);

@@ -1,6 +1,5 @@
 // Launchers of the row kernels of rowstep_dev.cuh over the restarts of a handle.
 #include <algorithm>
-#include <mutex>
 
 #include "common.cuh"
 #include "rowops.cuh"
@@ -18,12 +17,9 @@ __global__ void __launch_bounds__(256, 2) k_rowstep(RowArgs a, int tiles, bool v
 
 template <typename T, int STEP, int NC, int MR, int W>
 void launch_t(const RowArgs& a, const RowStepPlan& pl, cudaStream_t s) {
-  static std::once_flag once;
-  std::call_once(once, [] {  // the most over the ranks: r = 128 with 256 threads and every input
-    const int r = sizeof(T) == 8 && MR > 1 ? 64 : 128;
-    cudaFuncSetAttribute(k_rowstep<T, STEP, NC, MR, W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)rowstep_smem<T>(r, 256, MR, 7, W));
-  });
+  static SmemLimit limit;  // the most over the ranks: r = 128 with 256 threads and every input
+  raise_smem_limit(limit, (const void*)k_rowstep<T, STEP, NC, MR, W>,
+                   rowstep_smem<T>(sizeof(T) == 8 && MR > 1 ? 64 : 128, 256, MR, 7, W));
   uintptr_t all = 0;
   for (const void* p : {a.X, a.g_in, a.B, a.LX, (const void*)a.Xout, (const void*)a.gout, (const void*)a.Dout,
                         (const void*)a.gZout, a.Xold, a.gold, a.Zold, a.gZold, a.Wcur, a.gWcur, (const void*)a.Znext})

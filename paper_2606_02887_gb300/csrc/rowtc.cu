@@ -588,31 +588,22 @@ __global__ void __launch_bounds__(256, 2) k_rowtc_grad(RowArgs a, int* err) {
 bool rowtc_supported(int tdtype, int r, int nc) { return tdtype == 1 && r == RC && nc == 1; }
 
 void launch_rowtc_dstep(const RowArgs& a, int* err, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_rowtc_dstep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
-    attr = true;
-  }
+  static SmemLimit limit;
+  raise_smem_limit(limit, (const void*)k_rowtc_dstep, SMEM_BYTES);
   dim3 grid((unsigned)((a.n + TR - 1) / TR), (unsigned)a.b);
   k_rowtc_dstep<<<grid, 256, SMEM_BYTES, s>>>(a, err);
 }
 
 void launch_rowtc_grad(const RowArgs& a, int* err, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_rowtc_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
-    attr = true;
-  }
+  static SmemLimit limit;
+  raise_smem_limit(limit, (const void*)k_rowtc_grad, SMEM_BYTES);
   dim3 grid((unsigned)((a.n + TR - 1) / TR), (unsigned)a.b);
   k_rowtc_grad<<<grid, 256, SMEM_BYTES, s>>>(a, err);
 }
 
 void launch_rowtc_update(const RowArgs& a, int* err, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_rowtc_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
-    attr = true;
-  }
+  static SmemLimit limit;
+  raise_smem_limit(limit, (const void*)k_rowtc_update, SMEM_BYTES);
   dim3 grid((unsigned)((a.n + TR - 1) / TR), (unsigned)a.b);
   k_rowtc_update<<<grid, 256, SMEM_BYTES, s>>>(a, err);
 }

@@ -604,13 +604,8 @@ bool launch_kind(const RowArgs& a, const void* const* arrays, int* err, cudaStre
   RowMaps maps;
   for (int q = 0; q < 4; ++q)
     if (!make_map_f32_tile(&maps.m[q], arrays[q], a.ld, a.n, a.ld)) return false;
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(k_rowtma<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DYN_BYTES) !=
-        cudaSuccess)
-      return false;
-    attr = true;
-  }
+  static SmemLimit limit;
+  if (raise_smem_limit(limit, (const void*)k_rowtma<KIND>, DYN_BYTES) != cudaSuccess) return false;
   const int64_t T = ((a.n + TR - 1) / TR) * a.b;
   const int grid = (int)(T < sm_count() ? T : sm_count());
   if ((T + grid - 1) / grid > kMaxTodo) return false;  // a range could hold more runs than the list

@@ -111,3 +111,66 @@ out.append([l[0] for l in log() if kernel in l[2]])
 print(json.dumps(out))
 """)
     assert first == "failed" and again == "solved" and state and not any(state)
+
+
+@pytest.mark.parametrize("kind", ["noalloc_f32", "noalloc_f64", "knn", "f32_r200", "f64", "direct", "bf16", "fp8", "lai",
+                                  "batch"])
+def test_shared_memory_limit_of_each_context(fake, kind):
+    """The dynamic shared memory above 48 KB that a kernel is launched with has been allowed in the context of
+    the launch: on the first device, on another one, and after a device reset."""
+    codes, most = fake(f"""
+kind = {kind!r}
+def call():
+    if kind.startswith("noalloc"):
+        t = np.float64 if kind.endswith("64") else np.float32
+        A, X, Y, x = np.ones((2048, 2048), t), np.ones((2048, 64), t), np.ones((2048, 64), t), C.c_double()
+        p = lambda a: a.ctypes.data_as(C.c_void_p)
+        return S.load_library().snmf_apply_dense_noalloc(p(A), S.SNMF_F64 if t is np.float64 else S.SNMF_F32, 2048, 2048,
+                                                         p(X), p(Y), 64, C.byref(x), None)
+    if kind == "knn":
+        n, k = 1500, 8
+        X, i, f, nnz = np.ones((n, 100), np.float32), np.zeros(2 * n * k, np.int32), np.zeros(2 * n * k, np.float32), C.c_int64()
+        p = lambda a: a.ctypes.data_as(C.c_void_p)
+        rp = np.zeros(n + 1, np.int32)
+        return S.load_library().snmf_knn_graph(p(X), C.c_int64(n), 100, k, 7, p(rp), p(i), p(f), None, None,
+                                               C.c_int64(2 * n * k), C.byref(nnz), None)
+    n, r, o = 1024, 40, dict(max_iter=1, inner_iters=1, batch=2)
+    if kind == "f32_r200":
+        r = 200
+    elif kind == "f64":
+        r, o["precision"] = 100, S.SNMF_F64
+    elif kind == "direct":
+        n, r, o["formulation"] = 4096, 64, S.SNMF_DIRECT
+    elif kind in ("bf16", "fp8"):
+        r, o["precision"] = 64, S.SNMF_BF16 if kind == "bf16" else S.SNMF_FP8
+    if kind == "batch":
+        A = S.dense_batch_matrix(np.ones(2 * n * n, np.float32), [n, n], [10, 60])
+        r, o["batch"] = 0, 1
+    elif kind == "lai":
+        A = S.csr_matrix(n, *ring(n))
+    else:
+        A = S.dense_matrix(np.ones((n, n), np.float64 if kind == "f64" else np.float32))
+    h = S.snmf_create(A, r, S.snmf_default_options(**o))
+    if kind == "lai":
+        S.snmf_lai_sketch(h, 64, 10, 1, 1)
+    W = np.ones(n * 70 if kind == "batch" else (n, r * 2), np.float64 if kind == "f64" else np.float32)
+    st = S.snmf_solve_host(h, W, None if kind == "direct" else W.copy())[0]
+    S.snmf_destroy(h)
+    return st
+def tried():
+    try:
+        return call()
+    except S.SnmfError as e:
+        return str(e)
+codes = [tried()]
+fake.fake_device(1)
+codes.append(tried())
+fake.fake_device(0)
+codes.append(tried())
+fake.fake_reset(0)
+codes.append(tried())
+print(json.dumps([codes + sorted(set((l[0], l[2][:80]) for l in log() if l[0])), max(l[5] for l in log())]))
+""")
+    assert all(c == codes[0] and not isinstance(c, str) for c in codes), codes
+    assert codes[0] >= 0 or kind == "knn"  # no kernel runs, so the graph of the points holds what it may
+    assert most > 48 * 1024
