@@ -220,6 +220,10 @@ struct SmemLimit {
 };
 cudaError_t raise_smem_limit(SmemLimit& l, const void* kernel, size_t bytes);
 
+// The id of the current context, which no other context of the process gets (a context made after a device
+// reset may have the address of the one before); false without a current context.
+bool context_id(unsigned long long* id);
+
 // Workspaces of calls without a handle (pool.cu): stream-ordered, from the library's pool.
 cudaError_t workspace_alloc(void** p, size_t bytes, cudaStream_t s);
 void workspace_free(void* p, cudaStream_t s);

@@ -4,7 +4,6 @@
 // slices and the FP64 partial sums live in one file-scope __device__ array of fixed
 // size instead of memory obtained from cudaMalloc.  Nothing here allocates: no
 // cudaMalloc / cudaFree, no host heap.
-#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -30,26 +29,10 @@ static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 // own driver-API context) resolves it again.
 struct ScratchAddr {
   void* ptr = nullptr;
-  CUcontext ctx = nullptr;
+  unsigned long long ctx = 0;  // the context's id
 };
 ScratchAddr g_scratch_addr[kMaxDevices];
 std::mutex g_scratch_mu;
-
-using CtxGetCurrentFn = CUresult (*)(CUcontext*);
-
-// cuCtxGetCurrent through the runtime's driver entry point (no link against libcuda).
-CtxGetCurrentFn ctx_get_current() {
-  static CtxGetCurrentFn fn = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<CtxGetCurrentFn>(p);
-  });
-  return fn;
-}
 
 // Sum part[slot][0][q] over slots in a fixed order (one block).
 __global__ void k_sum_slots(const double* __restrict__ part, int nslots, int q, double* __restrict__ out) {
@@ -73,10 +56,9 @@ extern "C" snmf_status snmf_apply_dense_noalloc(const void* A, int dtype, int64_
   if (n > SNMF_NOALLOC_MAX_ROWS || 2 * slice > SNMF_NOALLOC_MAX_SLICE_PAIR_BYTES) return SNMF_ERR_ARG;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return SNMF_ERR_CUDA;
-  // the current context (NULL before the first runtime call of the thread initialises one)
-  CUcontext ctx = nullptr;
-  const CtxGetCurrentFn get_ctx = ctx_get_current();
-  if (!get_ctx || get_ctx(&ctx) != CUDA_SUCCESS) ctx = nullptr;
+  // the current context (none before the first runtime call of the thread initialises one)
+  unsigned long long ctx = 0;
+  if (!snmf::context_id(&ctx)) ctx = 0;
   void* base = nullptr;
   {
     std::lock_guard<std::mutex> lock(g_scratch_mu);

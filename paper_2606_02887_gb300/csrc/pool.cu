@@ -34,13 +34,6 @@ F entry(const char* name) {
   return reinterpret_cast<F>(p);
 }
 
-bool context_id(unsigned long long* id) {
-  static auto get_ctx = entry<CUresult (*)(CUcontext*)>("cuCtxGetCurrent");
-  static auto get_id = entry<CUresult (*)(CUcontext, unsigned long long*)>("cuCtxGetId");
-  CUcontext ctx = nullptr;
-  return get_ctx && get_id && get_ctx(&ctx) == CUDA_SUCCESS && ctx && get_id(ctx, id) == CUDA_SUCCESS;
-}
-
 // the current device's pool; nullptr without one (`make`: created when missing)
 cudaMemPool_t device_pool(bool make) {
   int dev = 0;
@@ -70,10 +63,17 @@ cudaMemPool_t device_pool(bool make) {
 
 }  // namespace
 
+bool context_id(unsigned long long* id) {
+  static auto get_ctx = entry<CUresult (*)(CUcontext*)>("cuCtxGetCurrent");
+  static auto get_id = entry<CUresult (*)(CUcontext, unsigned long long*)>("cuCtxGetId");
+  CUcontext ctx = nullptr;
+  return get_ctx && get_id && get_ctx(&ctx) == CUDA_SUCCESS && ctx && get_id(ctx, id) == CUDA_SUCCESS && *id;
+}
+
 cudaError_t raise_smem_limit(SmemLimit& l, const void* kernel, size_t bytes) {
   int dev = 0;
   unsigned long long id = 0;
-  const bool known = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices && context_id(&id) && id;
+  const bool known = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices && context_id(&id);
   if (known && l.ctx[dev].load(std::memory_order_relaxed) == id) return cudaSuccess;
   const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e == cudaSuccess && known) l.ctx[dev].store(id, std::memory_order_relaxed);

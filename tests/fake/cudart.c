@@ -20,7 +20,7 @@ static int g_fns = 0;
 static char g_log[1 << 20];
 static size_t g_logged = 0, g_most_bytes = 0;
 static char g_refuse[128];
-static int g_nodes = 0;
+static int g_nodes = 0, g_symbols = 0;
 static float g_event_ms = 1.0f;
 
 static cudaError_t err(cudaError_t e) { if (e) t_last = e; return e; }
@@ -85,8 +85,8 @@ OUT cudaError_t cudaFuncSetAttribute(const void* fn, enum cudaFuncAttribute a, i
 }
 
 // ---- devices and the driver's entry points
-static int ctx_current(void** c) { *c = (void*)(size_t)g_ctx[t_dev]; return 0; }
-static int ctx_id(void* c, unsigned long long* id) { *id = (unsigned long long)(size_t)c; return 0; }
+static int ctx_current(void** c) { *c = &g_ctx[t_dev]; return 0; }  // a reset gives the same address
+static int ctx_id(void* c, unsigned long long* id) { *id = *(unsigned long long*)c; return 0; }
 static int encode(void) { return 0; }
 OUT cudaError_t cudaGetDriverEntryPointByVersion(const char* n, void** p, unsigned v, unsigned long long f,
                                                  enum cudaDriverEntryPointQueryResult* q) {
@@ -112,9 +112,11 @@ OUT cudaError_t cudaGetDeviceProperties(struct cudaDeviceProp* p, int d) {
 }
 OUT cudaError_t cudaGetLastError(void) { cudaError_t e = t_last; t_last = cudaSuccess; return e; }
 OUT cudaError_t cudaPeekAtLastError(void) { return t_last; }
+OUT int fake_symbols(void) { return g_symbols; }  // addresses asked for
 OUT cudaError_t cudaGetSymbolAddress(void** p, const void* s) {
   static void* mem;
   (void)s;
+  ++g_symbols;
   if (!mem) mem = mmap(NULL, 128u << 20, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
   *p = mem;
   return cudaSuccess;

@@ -174,3 +174,20 @@ print(json.dumps([codes + sorted(set((l[0], l[2][:80]) for l in log() if l[0])),
     assert all(c == codes[0] and not isinstance(c, str) for c in codes), codes
     assert codes[0] >= 0 or kind == "knn"  # no kernel runs, so the graph of the points holds what it may
     assert most > 48 * 1024
+
+
+def test_noalloc_scratch_of_each_context(fake):
+    """The address of the allocation-free product's scratch is resolved once in a context, and again in the
+    one after a device reset, whose handle may have the address of the old one."""
+    assert fake("""
+def call():
+    A, X, Y, x = np.ones((512, 512)), np.ones((512, 8)), np.ones((512, 8)), C.c_double()
+    p = lambda a: a.ctypes.data_as(C.c_void_p)
+    assert S.load_library().snmf_apply_dense_noalloc(p(A), S.SNMF_F64, 512, 512, p(X), p(Y), 8, C.byref(x), None) == 0
+    return fake.fake_symbols()
+out = [call(), call()]
+fake.fake_reset(0)
+out += [call(), call()]
+fake.fake_device(1)
+print(json.dumps(out + [call(), call()]))
+""") == [1, 1, 2, 2, 3, 3]
