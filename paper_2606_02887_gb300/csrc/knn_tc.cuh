@@ -4,14 +4,18 @@
 // k_knn, bit for bit.
 //
 // The bounds.  y = fl(x - c) for any centre c, rounded to TF32 (relative error 2^-11), n = |x - c|^2:
-//   | |x_q - x_j|^2 - (n_q + n_j - 2 <y_q, y_j>) | <= e (n_q + n_j),
+//   | |x_q - x_j|^2 - (n_q + n_j - 2 <y_q, y_j>) | <= e (n_q + n_j) + a,
 // where e covers 2 (2^-11 + 2^-11) |y_q| |y_j| <= 2^-10 (n_q + n_j) of the operands' rounding, 16 steps
 // of truncating accumulation, the rounding of the centring, of the norms and of the comparison, and
-// that of the FP32 sum which is bounded (1.13e-3 together for d <= 128; e = 1.25e-3).
+// that of the FP32 sum which is bounded (1.13e-3 together for d <= 128; e = 1.25e-3).  a covers what
+// underflows: a coordinate or a product below 2^-126 may count as zero, and a square rounds to a multiple of
+// 2^-149.  Lost products and squares are at most 4 d 2^-126 = 6e-36 together, and lost coordinates at most
+// 2 d 2^-126 |y|, which is below the 1.2e-4 n left in e for |y| > 3e-32 and below 1e-67 otherwise; a = 1e-34.
 //
 //   pass 0  the k smallest upper bounds of every query over every second point, values only, kept sorted
 //           in registers (a lane per query and half a tile); k_knn_bound takes the k-th of all lists
-//           of a query, T_q
+//           of a query, T_q (with 2 a: a neighbour's lower bound is at most its distance plus a, and that at
+//           most the k-th upper bound plus a)
 //   pass 1  over all points the pairs whose lower bound is not above T_q, appended to the query's
 //           candidates (about four times k of them for clustered data)
 //   k_knn_exact  their distances and the k nearest, a warp per query
@@ -43,6 +47,7 @@ constexpr int KT_PARTS = 8;            // at most, of the candidates (two lists 
 constexpr int KT_CAP = 256;            // candidates of a query
 constexpr float KT_E = 1.25e-3f;
 constexpr float KT_UP = 2.f * KT_E / (1.f - KT_E);
+constexpr float KT_ABS = 2e-34f;       // 2 a
 constexpr float KT_MAXNORM = 1e36f;    // n below it: no distance or product overflows
 constexpr long long KT_BUDGET = 2000000000LL;
 
@@ -289,7 +294,7 @@ k_knn_tc(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtens
           thr = fminf(thr, kd[KR - 1]);
         }
         if ((i & 7) == 7 && qv) {  // the bound of the query's other lists
-          const float mine = fmaxf(0.f, 2.f * kd[KR - 1] + nq * (1.f + KT_UP));
+          const float mine = fmaxf(0.f, 2.f * kd[KR - 1] + nq * (1.f + KT_UP)) + KT_ABS;
           if (mine < told) {
             atomicMin(reinterpret_cast<int*>(kth) + q, __float_as_int(mine));
             told = mine;
@@ -325,7 +330,7 @@ k_knn_tc(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtens
   }
 }
 
-// kth[q]: the k-th smallest upper bound of the query's sorted lists (or what a list gave already).
+// kth[q]: T_q, from the k-th smallest upper bound of the query's sorted lists (or what a list gave already).
 __global__ void __launch_bounds__(128) k_knn_bound(const float* __restrict__ lists, const float* __restrict__ nrm, int64_t n,
                                                    int k, int count, float* __restrict__ kth) {
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -351,7 +356,7 @@ __global__ void __launch_bounds__(128) k_knn_bound(const float* __restrict__ lis
     for (int l = 0; l < 2 * KT_PARTS; ++l)
       if (l == from && l < count) head[l] = ++at[l] < k ? lists[((int64_t)l * k + at[l]) * n + q] : INFINITY;
   }
-  kth[q] = fminf(kth[q], 2.f * v + nrm[q] * (1.f + KT_UP));
+  kth[q] = fminf(kth[q], fmaxf(0.f, 2.f * v + nrm[q] * (1.f + KT_UP)) + KT_ABS);
 }
 
 // One warp per query: the distances of its candidates and the k nearest.
