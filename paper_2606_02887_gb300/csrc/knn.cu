@@ -534,7 +534,6 @@ extern "C" snmf_status snmf_knn_graph(const float* X, int64_t n, int d, int k, i
   KnnWork w{};
   w.parts = knn_parts(n);
   w.tc_parts = knn_tc_rule(n, d) ? knn_tc_parts(n) : 0;
-  const int64_t dp = w.tc_parts ? (d + 31) / 32 * 32 : 0;
   unsigned char* ws = nullptr;
   size_t bytes = 0;
   auto take = [&](size_t b) {
@@ -545,12 +544,24 @@ extern "C" snmf_status snmf_knn_graph(const float* X, int64_t n, int d, int k, i
   const size_t o_nbr = take(nk * 4), o_nd2 = take(nk * 4), o_sval = take(nk * 4), o_cnt = take(n * 4), o_fill = take(n * 4),
                o_off = take((n + 1) * 4), o_cntu = take(n * 4), o_erow = take(2 * nk * 4), o_ecol = take(2 * nk * 4), o_eval = take(2 * nk * 4),
                o_sv = take(s_values ? 0 : 2 * nk * 4), o_dg = take(degree ? 0 : n * 4), o_erep = take(2 * nk),
-               o_bad = take(12), o_y = take(n * dp * 4),
-               o_nrm = take(dp ? (n + KT_C) * 4 : 0), o_nrm0 = take(dp ? (n + KT_C) * 4 : 0), o_kth = take(dp ? n * 4 : 0), o_ctr = take(dp * 4),
-               o_ncand = take(dp ? n * 4 : 0), o_lists = bytes, o_pi = bytes;
-  // k_knn's partial lists come after the filter's lists and candidates are done with
-  const size_t o_cand = o_lists + (2 * w.tc_parts * nk * 4 + 255) / 256 * 256, o_pd = o_pi + (w.parts * nk * 4 + 255) / 256 * 256;
-  take(std::max((o_cand - o_lists) + (dp ? n * KT_CAP * 4 : 0), (o_pd - o_pi) + w.parts * nk * 4));
+               o_bad = take(12), always = bytes;
+  size_t o_y, o_nrm, o_nrm0, o_kth, o_ctr, o_ncand, o_lists, o_cand, o_pi, o_pd;
+  auto plan = [&] {  // the rest with or without the filter
+    bytes = always;
+    const int64_t dp = w.tc_parts ? (d + 31) / 32 * 32 : 0;
+    o_y = take(n * dp * 4);
+    o_nrm = take(dp ? (n + KT_C) * 4 : 0);
+    o_nrm0 = take(dp ? (n + KT_C) * 4 : 0);
+    o_kth = take(dp ? n * 4 : 0);
+    o_ctr = take(dp * 4);
+    o_ncand = take(dp ? n * 4 : 0);
+    // k_knn's partial lists come after the filter's lists and candidates are done with
+    o_lists = o_pi = bytes;
+    o_cand = o_lists + (2 * w.tc_parts * nk * 4 + 255) / 256 * 256;
+    const size_t part = w.parts > 1 ? (w.parts * nk * 4 + 255) / 256 * 256 : 0;
+    o_pd = o_pi + part;
+    take(std::max((o_cand - o_lists) + (dp ? n * KT_CAP * 4 : 0), 2 * part));
+  };
   auto cleanup = [&] { workspace_free(ws, s); };
   snmf_status st = SNMF_OK;
 #define KCK(call)                                                                                        \
@@ -558,7 +569,18 @@ extern "C" snmf_status snmf_knn_graph(const float* X, int64_t n, int d, int k, i
     const cudaError_t e_ = (call);                                                                       \
     if (e_ != cudaSuccess) { st = e_ == cudaErrorMemoryAllocation ? SNMF_ERR_OOM : SNMF_ERR_CUDA; cleanup(); return st; } \
   } while (0)
-  KCK(workspace_alloc((void**)&ws, bytes, s));
+  plan();
+  cudaError_t got = workspace_alloc((void**)&ws, bytes, s);
+  while (got == cudaErrorMemoryAllocation && (w.tc_parts || w.parts > 1)) {
+    // without the filter's 1 KB of candidates and its copy of each point, then without partial lists: k_knn
+    // gives the same lists alone
+    cudaGetLastError();
+    if (w.tc_parts) w.tc_parts = 0;
+    else w.parts = 1;
+    plan();
+    got = workspace_alloc((void**)&ws, bytes, s);
+  }
+  KCK(got);
   auto i32 = [&](size_t o) { return reinterpret_cast<int32_t*>(ws + o); };
   auto f32 = [&](size_t o) { return reinterpret_cast<float*>(ws + o); };
   int32_t *nbr = i32(o_nbr), *cnt = i32(o_cnt), *off = i32(o_off), *fill = i32(o_fill), *erow = i32(o_erow), *ecol = i32(o_ecol),

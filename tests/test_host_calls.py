@@ -191,3 +191,24 @@ out += [call(), call()]
 fake.fake_device(1)
 print(json.dumps(out + [call(), call()]))
 """) == [1, 1, 2, 2, 3, 3]
+
+
+def test_knn_graph_without_room_for_the_filter(fake):
+    """Where the filter's workspace cannot be had, the call runs without the filter instead of failing, and where
+    the partial lists cannot be had without those; where nothing can be had, it fails."""
+    got = fake("""
+n, d, k = 20000, 64, 10
+X, i, f = np.ones((n, d), np.float32), np.zeros(2 * n * k, np.int32), np.zeros(2 * n * k, np.float32)
+rp, nnz = np.zeros(n + 1, np.int32), C.c_int64()
+p = lambda a: a.ctypes.data_as(C.c_void_p)
+out = []
+for most in (0, 40 << 20, 12 << 20, 1 << 20):
+    fake.fake_memory(most)
+    fake.fake_clear()
+    st = S.load_library().snmf_knn_graph(p(X), n, d, k, 7, p(rp), p(i), p(f), None, None, 2 * n * k, C.byref(nnz), None)
+    out.append([st, sum("k_knn_tc" in l[2] for l in log()), sum("5k_knnE" in l[2] for l in log()),
+                sum("k_knn_merge" in l[2] for l in log())])
+print(json.dumps(out))
+""")
+    assert [g[0] for g in got] == [S.SNMF_OK] * 3 + [S.SNMF_ERR_OOM]
+    assert got[0][1] == 2 and got[1][1:] == [0, 1, 1] and got[2][1:] == [0, 1, 0] and got[3][1:] == [0, 0, 0]
