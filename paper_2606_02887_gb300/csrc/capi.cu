@@ -323,23 +323,30 @@ RowArgs row_base(snmf_ctx* h, const Params* P = nullptr) {
   return a;
 }
 
-// The D step and the update of a block without graph term: on the tensor cores where the autotuner
-// chose them, else rowstep.cu.
+// The tensor-core row bodies (TF32 parts) that run: the autotuner's choice on a handle without graph term,
+// whose steps are all theirs.
+int row_tc_body(const snmf_ctx* h) { return h->use_row && !h->graph ? h->row_tc : 0; }
+
+// The D step and the update of a block without graph term: on the tensor cores where they run, else
+// rowstep.cu.
 void row_dstep(snmf_ctx* h, const RowArgs& a, int nc) {
-  if (h->row_tc == 2 && launch_rowtma_dstep(a, h->dev_err, h->s)) return;
-  if (h->row_tc) launch_rowtc_dstep(a, h->dev_err, h->s);
+  const int tc = row_tc_body(h);
+  if (tc == 2 && launch_rowtma_dstep(a, h->dev_err, h->s)) return;
+  if (tc) launch_rowtc_dstep(a, h->dev_err, h->s);
   else launch_rowstep_d(h->tdtype, a, h->rplan, nc, h->s);
 }
 
 void row_update(snmf_ctx* h, const RowArgs& a, int nc) {
-  if (h->row_tc == 2 && launch_rowtma_update(a, h->dev_err, h->s)) return;
-  if (h->row_tc) launch_rowtc_update(a, h->dev_err, h->s);
+  const int tc = row_tc_body(h);
+  if (tc == 2 && launch_rowtma_update(a, h->dev_err, h->s)) return;
+  if (tc) launch_rowtc_update(a, h->dev_err, h->s);
   else launch_rowstep_update(h->tdtype, a, h->rplan, nc, h->s);
 }
 
-// Gradient of a given X (block start; an update of a graph-regularised block; the final point).
+// Gradient of a given X (block start; an update of a graph-regularised block; the start and the final point
+// of a solve, which are in FP32 whatever the steps run on).
 void row_grad(snmf_ctx* h, const RowArgs& a) {
-  if (h->use_row && h->row_tc && !a.LX && !a.Xold && a.ctl_mode) launch_rowtc_grad(a, h->dev_err, h->s);
+  if (row_tc_body(h) && (a.ctl_mode == CTL_START_W || a.ctl_mode == CTL_START_H)) launch_rowtc_grad(a, h->dev_err, h->s);
   else if (h->use_row) launch_rowstep_grad(h->tdtype, a, h->rplan, h->s);
   else launch_rowgemm(h->tdtype, OP_LOAD, EPI_GRAD, a, h->s);
 }

@@ -212,3 +212,23 @@ print(json.dumps(out))
 """)
     assert [g[0] for g in got] == [S.SNMF_OK] * 3 + [S.SNMF_ERR_OOM]
     assert got[0][1] == 2 and got[1][1:] == [0, 1, 1] and got[2][1:] == [0, 1, 0] and got[3][1:] == [0, 0, 0]
+
+
+def test_tensor_core_row_kernels_run_block_steps_alone(fake):
+    """A tuned handle's TF32 row kernels run the steps of its two blocks and no other: not the gradient of the
+    start, and no step of a handle with a graph term, which run in FP32."""
+    tuned, with_graph, without = fake("""
+n, r = 1024, 64
+h = S.snmf_create(S.dense_matrix(np.ones((n, n), np.float32)), r, S.snmf_default_options(max_iter=1, inner_iters=2, autotune=1))
+out = []
+for gamma in (None, 0.1, 0.0):
+    if gamma is not None:
+        S.snmf_set_graph_reg(h, S.csr_matrix(n, *ring(n)) if gamma else None, gamma)
+    W = np.ones((n, r), np.float32)
+    fake.fake_clear()
+    S.snmf_solve_host(h, W, W.copy())
+    names = [l[2] for l in log()]
+    out.append([sum(k in m for m in names) for k in ("k_rowtc_grad", "k_rowtma", "k_rowtc_dstep")])
+print(json.dumps(out))
+""")
+    assert tuned == without and tuned[0] == 2 and tuned[1] + 2 * tuned[2] == 8 and with_graph == [0, 0, 0]
