@@ -753,7 +753,7 @@ def main():
         K = opts.inner_iters
         # the library reports which row-kernel body runs and the arrays each launch moves
         sc = S.snmf_step_config(h)
-        body = {0: "k_rowgemm (general)", 1: "k_rowtile (shared-memory tile body)",
+        body = {0: "k_rowgemm (general)",
                 2: "k_rowstep (Z and D recomputed, not stored; row products on CUDA cores)",
                 3: "k_rowtc (Z and D recomputed, not stored; row products on tcgen05, TF32 hi + lo)",
                 4: "k_rowtma (as k_rowtc, persistent: one CTA per SM, inputs streamed by TMA)"}[sc["body"]]

@@ -369,12 +369,13 @@ SNMF_API snmf_status snmf_profile_steps(snmf_handle h, int iters, double* ms_dst
 
 /*
  * Measurement utility (no counterpart in the paper): which row-kernel body runs the D step and
- * the update of this handle's penalty blocks, and their algorithmic bytes per launch (every
- * n x (r batch) array a launch reads or writes, once).  *body: 0 the general row kernel
- * (Z and D stored; D step 6 arrays, 7 with the learned step's second direction, update 8),
- * 1 not used, 2 the recomputing kernels (r <= 128; Z and D not stored:
- * D step 4 arrays, update 6), 3 the recomputing kernels with their row products on the tensor
- * cores (tcgen05 TF32 with hi / lo operand parts; r = 64, chosen by the autotuner when faster),
+ * the update of this handle's W block (a graph term, which is part of the H block, does not change
+ * the body unless it is 3 or 4), and their algorithmic bytes per launch (every n x (r batch) array a
+ * launch reads or writes, once).  *body: 0 the general row kernel
+ * (Z and D stored; D step 6 arrays, update 8), 1 not used, 2 the recomputing kernels (r <= 128;
+ * Z and D not stored: D step 4 arrays, update 6), 3 the recomputing kernels with their row products
+ * on the tensor cores (tcgen05 TF32 with hi / lo operand parts; r = 64 without graph term, chosen by
+ * the autotuner when faster),
  * 4 the same arithmetic as persistent kernels (one CTA per SM over 128-row tiles, inputs streamed
  * by TMA into shared slots while the previous tile computes; same traffic as 2 and 3).
  * *rows_per_cta: rows of one tile.  Any pointer may be NULL.

@@ -1734,18 +1734,18 @@ snmf_status snmf_step_config(snmf_handle h, int32_t* body, int32_t* rows_per_cta
   if (!h) return SNMF_ERR_STATE;
   if (h->bt) return fail(h, SNMF_ERR_STATE, "not available for a dense batch handle");
   const int64_t fb = h->n * (int64_t)h->N * (int64_t)h->esz;  // one n x (r b) factor array
-  const int nc = h->opt.step_controller == 1 ? 2 : (h->opt.step_controller == 2 ? kNCand : 1);
   int kind = 0, rows = 0;
   int64_t bd = 0, bu = 0;
-  if (h->use_row && !h->graph) {
-    kind = h->row_tc == 2 ? 4 : (h->row_tc ? 3 : 2);
-    rows = h->row_tc ? 128 : h->rplan.rows;
+  if (h->use_row) {  // the W block's kernels, with or without a graph term on the H block
+    const int tc = row_tc_body(h);
+    kind = 2 + tc;
+    rows = tc ? 128 : h->rplan.rows;
     bd = 4 * fb;  // X, g, B in; g(Z) out
     bu = 6 * fb;  // X, g, g(Z), B in; X', g(X') out
   } else {
     rows = (int)((h->n + h->nrow / ((h->r + 63) / 64) - 1) / (h->nrow / ((h->r + 63) / 64)));
-    bd = (6 + (nc == 2 ? 1 : 0)) * fb;  // X, g, B in; Z, g(Z), D (+ the second direction) out
-    bu = 8 * fb;                        // Z, D, B, X, g, g(Z) in; X', g(X') out
+    bd = 6 * fb;  // X, g, B in; Z, g(Z), D out
+    bu = 8 * fb;  // Z, D, B, X, g, g(Z) in; X', g(X') out
   }
   if (body) *body = kind;
   if (rows_per_cta) *rows_per_cta = rows;

@@ -232,3 +232,23 @@ for gamma in (None, 0.1, 0.0):
 print(json.dumps(out))
 """)
     assert tuned == without and tuned[0] == 2 and tuned[1] + 2 * tuned[2] == 8 and with_graph == [0, 0, 0]
+
+
+@pytest.mark.parametrize("controller", [0, 1])
+def test_step_config_with_a_graph_term(fake, controller):
+    """snmf_step_config reports the W block's kernels, which a graph term on the H block does not change: the
+    recomputing body, 4 and 6 arrays, rows of its own tiles."""
+    got = fake(f"""
+n, r = 1000, 20
+o = S.snmf_default_options(max_iter=1, step_controller={controller}, mlp_weights=True)
+w = np.zeros(S.SNMF_MLP_NPARAMS, np.float32)
+h = S.snmf_create(S.csr_matrix(n, *ring(n)), r, o, mlp_weights=w if {controller} else None)
+out = []
+for gamma in (0.0, 0.1):
+    S.snmf_set_graph_reg(h, S.csr_matrix(n, *ring(n)) if gamma else None, gamma)
+    out.append(S.snmf_step_config(h))
+print(json.dumps(out))
+""")
+    n_bytes = 1000 * 20 * 4
+    assert got[0] == got[1] and got[0]["body"] == 2
+    assert got[0]["dstep_bytes"] == 4 * n_bytes and got[0]["update_bytes"] == 6 * n_bytes and got[0]["rows_per_cta"] == 12
