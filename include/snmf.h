@@ -226,6 +226,9 @@ SNMF_API void snmf_default_options(snmf_options* opt);
  * Errors: SNMF_ERR_ARG for r out of range, batch < 1, r*batch > 4096, non-square or
  * negative sizes, ld < n, CSR with nnz mismatch, unknown enum values; SNMF_ERR_OOM,
  * SNMF_ERR_CUDA.  ||A||_F^2 of the stored (possibly quantized) A is computed here.
+ * Beside A the handle takes device memory for about 16 factors (n x (r batch) values each) and, with
+ * a dense A, for ten more as slices of split products (32 where that is below 2M values; eight where
+ * ten cannot be had).
  */
 SNMF_API snmf_status snmf_create(snmf_handle* h, const snmf_matrix* A, int r,
                         const snmf_options* opt, void* stream);

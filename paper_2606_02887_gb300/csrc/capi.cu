@@ -853,9 +853,6 @@ snmf_status alloc_buffers(snmf_ctx* h) {
     CK(cudaMalloc(&h->buf[i], fe * h->esz));
     CK(cudaMemsetAsync(h->buf[i], 0, fe * h->esz, h->s));
   }
-  // split-K slices: ten, and more of a small factor, whose K has to be split further to fill the GPU
-  h->ws_elems = (h->kind == AX_DENSE) ? std::max<size_t>(10 * fe, std::min<size_t>(32 * fe, 2 << 20)) : 0;
-  if (h->ws_elems) CK(cudaMalloc(&h->ws, h->ws_elems * h->esz));
   const Dims d = dims(h);
   h->nrow = rowgemm_slots(d, h->tdtype);
   h->nax = (int)((h->n + kRowTile - 1) / kRowTile);
@@ -899,6 +896,18 @@ snmf_status alloc_buffers(snmf_ctx* h) {
   CK(cudaMalloc(&h->ring, (size_t)h->b * h->ring_cap * kRingVals * sizeof(double)));
   CK(cudaMemsetAsync(h->ring, 0, (size_t)h->b * h->ring_cap * kRingVals * sizeof(double), h->s));
   CK(cudaMallocHost(&h->h_flag, 2 * sizeof(int) + 2 * sizeof(double)));
+  if (h->kind == AX_DENSE) {
+    // split-K slices: ten, and more of a small factor, whose K has to be split further to fill the GPU.  Last of
+    // all, so that a handle that fits with eight slices is not refused for the others (splits follow the room).
+    h->ws_elems = std::max<size_t>(10 * fe, std::min<size_t>(32 * fe, 2 << 20));
+    cudaError_t e = cudaMalloc(&h->ws, h->ws_elems * h->esz);
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      h->ws_elems = 8 * fe;
+      e = cudaMalloc(&h->ws, h->ws_elems * h->esz);
+    }
+    CK(e);
+  }
   return SNMF_OK;
 }
 

@@ -282,3 +282,23 @@ print(json.dumps(out))
     n_bytes = 1000 * 20 * 4
     assert got[0] == got[1] and got[0]["body"] == 2
     assert got[0]["dstep_bytes"] == 4 * n_bytes and got[0]["update_bytes"] == 6 * n_bytes and got[0]["rows_per_cta"] == 12
+
+
+def test_handle_with_room_for_eight_slices(fake):
+    """A dense handle whose device has no room for ten split-K slices takes eight, and is not refused."""
+    most, codes = fake("""
+n, r = 1024, 256
+A, codes = np.ones((n, n), np.float32), []
+for most in (0, 9 << 20, 7 << 20):  # a factor is 1 MB
+    fake.fake_memory(most)
+    try:
+        h = S.snmf_create(S.dense_matrix(A), r, S.snmf_default_options(max_iter=1, inner_iters=1))
+        W = np.ones((n, r), np.float32)
+        fake.fake_clear()
+        codes.append(S.snmf_solve_host(h, W, W.copy())[0])
+        slices = max(l[3][2] for l in log() if "k_gemm_dense" in l[2])
+    except S.SnmfError as e:
+        codes.append(e.status)
+print(json.dumps([slices, codes]))
+""")
+    assert codes == [S.SNMF_OK, S.SNMF_OK, S.SNMF_ERR_OOM] and most <= 8
