@@ -388,7 +388,8 @@ SNMF_API snmf_status snmf_step_config(snmf_handle h, int32_t* body, int32_t* row
 
 /*
  * The product configuration chosen by the autotuner (no counterpart in the paper):
- * split-K slices, tcgen05 ring stages and CTAs per SM (0 where the kernel has none), the
+ * split-K slices (0: the built-in rule's, where a cache of other tiles gave the rest),
+ * tcgen05 ring stages and CTAs per SM (0 where the kernel has none), the
  * measured mean time in ms, and *from_cache = 1 when it came from the cache file or an
  * earlier handle of this process.  SNMF_ERR_STATE when the handle was not tuned.
  */

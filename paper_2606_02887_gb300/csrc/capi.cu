@@ -432,7 +432,6 @@ snmf_status autotune_product(snmf_ctx* h) {
   std::vector<int> bms;
   if (!h->use_row) bms = {64, 32};
   if (tune_lookup(h->opt.tune_cache, dev, key, &e)) {
-    if (h->A.a_dtype <= 1 && e.cfg.tiles != kProdTiles) e.cfg.splits = 0;
     h->tune = e;
     h->tuned = 2;
     if (tune_rows && std::find(bms.begin(), bms.end(), e.cfg.row_bm) != bms.end()) {
@@ -562,7 +561,6 @@ snmf_status autotune_product(snmf_ctx* h) {
     }
     h->tune.cfg.row_tc = h->row_tc;
   }
-  h->tune.cfg.tiles = kProdTiles;
   tune_store(h->opt.tune_cache, dev, key, h->tune);
   return SNMF_OK;
 }

@@ -1,6 +1,6 @@
 // JSON cache of the product autotuner (the search itself runs in capi.cu, where the
 // handle's buffers are).  File layout:
-//   {"format": "...", "devices": {"<name>/<SMs>": {"dense/bf16/n8192/N64":
+//   {"format": "...", "devices": {"<name>/<SMs>": {"dense/bf16/n8192/r64/N64":
 //       {"splits": 2, "stages": 3, "per_sm": 2, "bn": 64, "ms": 0.0441}, ...}, ...}}
 // The reader accepts any JSON of that shape (objects, strings, numbers, true/false/null);
 // unknown keys are ignored.  Entries of other devices are kept when the file is rewritten.
@@ -23,6 +23,9 @@ namespace {
 
 using Table = std::map<std::string, std::map<std::string, TuneEntry>>;
 
+const char* const kFormat = "snmf_gb300 product tuning cache, v2";
+const char* const kFormat1 = "snmf_gb300 product tuning cache, v1";  // other tiles of the CUDA-core product
+
 std::mutex g_mu;
 Table g_mem;  // in-process cache (also holds what was read from files)
 
@@ -30,6 +33,7 @@ struct Parser {
   const std::string& t;
   size_t i = 0;
   bool ok = true;
+  std::string format;
   explicit Parser(const std::string& s) : t(s) {}
   void ws() {
     while (i < t.size() && std::isspace((unsigned char)t[i])) ++i;
@@ -99,7 +103,6 @@ struct Parser {
       else if (k == "bn") e.cfg.bn = (int)num();
       else if (k == "row_bm") e.cfg.row_bm = (int)num();
       else if (k == "row_tc") e.cfg.row_tc = (int)num();
-      else if (k == "tiles") e.cfg.tiles = (int)num();
       else if (k == "ms") e.ms = num();
       else skip();
     } while (ok && eat(','));
@@ -112,6 +115,7 @@ struct Parser {
     do {
       const std::string k = str();
       if (!eat(':')) { ok = false; return; }
+      if (k == "format" && (ws(), i < t.size() && t[i] == '"')) { format = str(); continue; }
       if (k != "devices") { skip(); continue; }
       if (!eat('{')) { ok = false; return; }
       if (eat('}')) continue;
@@ -143,7 +147,11 @@ bool read_file(const char* path, Table* out) {
   p.file(&t);
   if (!p.ok) return false;
   for (auto& d : t)
-    for (auto& e : d.second) (*out)[d.first][e.first] = e.second;
+    for (auto& e : d.second) {
+      if (p.format == kFormat1 && (e.first.compare(0, 10, "dense/f32/") == 0 || e.first.compare(0, 10, "dense/f64/") == 0))
+        e.second.cfg.splits = 0;
+      (*out)[d.first][e.first] = e.second;
+    }
   return true;
 }
 
@@ -160,7 +168,7 @@ bool write_file(const char* path, const Table& t) {
   const std::string tmp = std::string(path) + ".tmp";
   FILE* f = std::fopen(tmp.c_str(), "w");
   if (!f) return false;
-  std::fprintf(f, "{\n  \"format\": \"snmf_gb300 product tuning cache, v1\",\n  \"devices\": {");
+  std::fprintf(f, "{\n  \"format\": \"%s\",\n  \"devices\": {", kFormat);
   bool first_dev = true;
   for (const auto& d : t) {
     std::fprintf(f, "%s\n    %s: {", first_dev ? "" : ",", quoted(d.first).c_str());
@@ -169,10 +177,9 @@ bool write_file(const char* path, const Table& t) {
     for (const auto& e : d.second) {
       std::fprintf(f,
                    "%s\n      %s: {\"splits\": %d, \"stages\": %d, \"per_sm\": %d, \"bn\": %d, \"row_bm\": %d, "
-                   "\"row_tc\": %d, \"tiles\": %d, \"ms\": %.6g}",
+                   "\"row_tc\": %d, \"ms\": %.6g}",
                    first ? "" : ",", quoted(e.first).c_str(), e.second.cfg.splits, e.second.cfg.stages,
-                   e.second.cfg.per_sm, e.second.cfg.bn, e.second.cfg.row_bm, e.second.cfg.row_tc, e.second.cfg.tiles,
-                   e.second.ms);
+                   e.second.cfg.per_sm, e.second.cfg.bn, e.second.cfg.row_bm, e.second.cfg.row_tc, e.second.ms);
       first = false;
     }
     std::fprintf(f, "\n    }");

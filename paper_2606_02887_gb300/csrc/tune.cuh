@@ -14,13 +14,7 @@ struct ProdTune {
   int bn = 0;       // tcgen05 product: output columns per CTA tile (multiple of 16, <= 256)
   int row_bm = 0;   // row kernels of a step (FP32): rows per CTA
   int row_tc = 0;   // the step's row products on the tensor cores (r = 64): 1 rowtc.cu, 2 rowtma.cu
-  int tiles = 0;    // kProdTiles of the library that timed it
 };
-
-// The tiles of the CUDA-core product (ax.cu).  An entry of other tiles says nothing about how to split K
-// for these: its `splits` of an FP64 or FP32 A is left to the built-in rule.  (Entries of the first tiles, 64 x
-// 64 for every size, have no such field.)
-constexpr int kProdTiles = 2;
 
 struct TuneEntry {
   ProdTune cfg;
@@ -30,7 +24,10 @@ struct TuneEntry {
 // "<device name>/<SM count>" of the current device ("" when it cannot be queried).
 std::string tune_device_key();
 // Cache lookup / store in the JSON file at `path` (NULL or empty: an in-process cache
-// only).  The file maps device keys to shape keys ("dense/<dtype>/n<n>/r<r>/N<N>") to entries.
+// only).  The file maps device keys to shape keys ("dense/<dtype>/n<n>/r<r>/N<N>") to entries.  A file
+// of the format's first version was timed with other tiles of the CUDA-core product (64 x 64 for every
+// size), which says nothing about how to split K for the present ones: the `splits` of its FP64 and
+// FP32 entries are left to the built-in rule (0).
 bool tune_lookup(const char* path, const std::string& dev, const std::string& key, TuneEntry* out);
 bool tune_store(const char* path, const std::string& dev, const std::string& key, const TuneEntry& e);
 

@@ -235,33 +235,32 @@ print(json.dumps(out))
 
 
 def test_cached_splits_of_other_tiles(fake, tmp_path):
-    """A tuning cache's K split of an FP32 product counts for the tiles that it was timed with alone; an entry
-    that does not name them (a cache of the 64 x 64 tiles) leaves the split to the built-in rule, and keeps the
-    rest.  A cache that the library writes names them."""
-    plain, old, new, kept, written = fake(f"""
+    """A tuning cache's K split of an FP32 product counts for the tiles that it was timed with alone: a cache
+    in the first format leaves the split to the built-in rule and keeps the rest, one in the present
+    format, or in none that the library writes, counts as it is."""
+    plain, got, written = fake(f"""
 r = 64
-def solve(entry, n=4096):
+def solve(fmt, n=4096):
     o = dict(max_iter=1, inner_iters=1)
-    if entry is not None:
-        path = {str(tmp_path)!r} + f"/{{len(entry)}}.json"
-        if entry:
-            json.dump({{"devices": {{"fake/152": {{f"dense/f32/n{{n}}/r{{r}}/N{{r}}": dict(entry, ms=1.0)}}}}}}, open(path, "w"))
+    if fmt is not None:
+        path = {str(tmp_path)!r} + f"/{{len(fmt)}}.json"
+        if fmt:
+            entry = dict(splits=3, row_tc=1, ms=1.0)
+            json.dump({{"format": fmt, "devices": {{"fake/152": {{f"dense/f32/n{{n}}/r{{r}}/N{{r}}": entry}}}}}}, open(path, "w"))
         o.update(autotune=1, tune_cache=path)
     h = S.snmf_create(S.dense_matrix(np.ones((n, n), np.float32)), r, S.snmf_default_options(**o))
     W = np.ones((n, r), np.float32)
     fake.fake_clear()
     S.snmf_solve_host(h, W, W.copy())
     # the final evaluation is not tuned
-    return sorted(set(l[3][2] for l in log() if "k_gemm_dense" in l[2])), S.snmf_step_config(h)["body"]
-out = [solve(None)[0]]
-out.append(solve(dict(splits=3, row_tc=1)))
-out.append(solve(dict(splits=3, row_tc=1, tiles=2)))
-out[1], out[2], kept = out[1][0], out[2][0], [out[1][1], out[2][1]]
-solve(dict(), 2048)  # not in the cache that this process has read
-d = json.load(open({str(tmp_path)!r} + "/0.json"))["devices"]["fake/152"]
-print(json.dumps(out + [kept, [e["tiles"] for e in d.values()]]))
+    return [sorted(set(l[3][2] for l in log() if "k_gemm_dense" in l[2])), S.snmf_step_config(h)["body"]]
+v = "snmf_gb300 product tuning cache, v"
+out = [solve(None)[0], [solve(v + "1"), solve(v + "2"), solve("another")]]
+solve("", 2048)  # not in the cache that this process has read
+print(json.dumps(out + [json.load(open({str(tmp_path)!r} + "/0.json"))["format"]]))
 """)
-    assert plain == old and 3 not in plain and new == [3] + plain and kept == [3, 3] and set(written) == {2}
+    assert 3 not in plain and got == [[plain, 3], [[3] + plain, 3], [[3] + plain, 3]]
+    assert written == "snmf_gb300 product tuning cache, v2"
 
 
 @pytest.mark.parametrize("controller", [0, 1])
