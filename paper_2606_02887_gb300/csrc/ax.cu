@@ -82,18 +82,21 @@ k_spmm_csr(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colid
   Vec acc;
 #pragma unroll
   for (int k = 0; k < V; ++k) acc.v[k] = T(0);
-  const int beg = rowptr[row], end = rowptr[row + 1];
+  // counted from the row's first entry and unsigned: an index past the end may be above 2^31 - 1
+  const int32_t* cols_i = colidx + rowptr[row];
+  const TV* vals_i = vals + rowptr[row];
+  const unsigned len = (unsigned)(rowptr[row + 1] - rowptr[row]);
   int32_t ci[U];
   T va[U];
-  auto load = [&](int e) {
+  auto load = [&](unsigned e) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      ci[u] = e + u < end ? __ldg(colidx + e + u) : -1;
-      va[u] = e + u < end ? (T)__ldg(vals + e + u) : T(0);
+      ci[u] = e + u < len ? __ldg(cols_i + e + u) : -1;
+      va[u] = e + u < len ? (T)__ldg(vals_i + e + u) : T(0);
     }
   };
-  load(beg);
-  for (int e = beg; e < end; e += U) {
+  load(0u);
+  for (unsigned e = 0u; e < len; e += U) {
     Vec x[U];
     T w[U];
     bool on[U];
