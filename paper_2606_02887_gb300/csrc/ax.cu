@@ -65,7 +65,11 @@ k_gemm_dense(const TA* __restrict__ A, int64_t lda, const typename C::T* __restr
 // the next indices already in flight, and added in their order.  Bound by the gather from L2 (n =
 // 20000, 15 entries per row, 640 columns: 353 us with single columns and one entry at a time, and a
 // finish pass of its own).
-template <typename TV, typename T, int V, int LPR>
+// What is read ahead is tested with an index up to 2 U - 2 beyond the row's end, which has to fit into 32 bits:
+// kCsrAhead (the test by the entries that are left instead: n = 20000, 640 columns 12 per cent slower).
+constexpr int64_t kCsrAhead = INT32_MAX - 16;
+
+template <typename TV, typename T, int V, int LPR, int U = V * sizeof(T) == 16 ? 4 : 8>
 __global__ void __launch_bounds__(256)
 k_spmm_csr(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colidx,
            const TV* __restrict__ vals, const T* __restrict__ X, int64_t ld,
@@ -73,7 +77,6 @@ k_spmm_csr(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colid
   struct alignas(V * sizeof(T)) Vec {
     T v[V];
   };
-  constexpr int U = V * sizeof(T) == 16 ? 4 : 8;
   if (run && *run == 0) return;
   const int lane = threadIdx.x & 31;
   const int64_t row = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * (32 / LPR) + lane / LPR;
@@ -82,21 +85,18 @@ k_spmm_csr(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colid
   Vec acc;
 #pragma unroll
   for (int k = 0; k < V; ++k) acc.v[k] = T(0);
-  // counted from the row's first entry and unsigned: an index past the end may be above 2^31 - 1
-  const int32_t* cols_i = colidx + rowptr[row];
-  const TV* vals_i = vals + rowptr[row];
-  const unsigned len = (unsigned)(rowptr[row + 1] - rowptr[row]);
+  const int beg = rowptr[row], end = rowptr[row + 1];
   int32_t ci[U];
   T va[U];
-  auto load = [&](unsigned e) {
+  auto load = [&](int e) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      ci[u] = e + u < len ? __ldg(cols_i + e + u) : -1;
-      va[u] = e + u < len ? (T)__ldg(vals_i + e + u) : T(0);
+      ci[u] = e + u < end ? __ldg(colidx + e + u) : -1;
+      va[u] = e + u < end ? (T)__ldg(vals + e + u) : T(0);
     }
   };
-  load(0u);
-  for (unsigned e = 0u; e < len; e += U) {
+  load(beg);
+  for (int e = beg; e < end; e += U) {
     Vec x[U];
     T w[U];
     bool on[U];
@@ -368,6 +368,18 @@ int launch_ax(const AxArgs& a, int tdtype, int64_t n, int cols, int64_t ld, cons
   if (sizeof(T) == 4 && cols % 4 == 0 && ld % 4 == 0 && !(all & 15)) { SPMM_L(TV, T, (16 / (int)sizeof(T))); } \
   else if (cols % 2 == 0 && ld % 2 == 0 && !(all & (2 * sizeof(T) - 1))) { SPMM_L(TV, T, 2); }          \
   else { SPMM_L(TV, T, 1); }
+  if (a.lda > kCsrAhead) {  // entries one at a time, the next index at most the row's end
+#define SPMM_ONE(TV, T)                                                                                              \
+  k_spmm_csr<TV, T, 1, 32, 1><<<dim3(cdiv64(n, 8), cdiv64(cols, 32)), 256, 0, s>>>(                                  \
+      a.rowptr, a.colidx, (const TV*)a.vals, (const T*)X, ld, (T*)Y, n, cols, (T)c, (const T*)X2, run)
+    if (tdtype == 0) {
+      if (a.v_dtype == 0) SPMM_ONE(double, double); else SPMM_ONE(float, double);
+    } else {
+      if (a.v_dtype == 0) SPMM_ONE(double, float); else SPMM_ONE(float, float);
+    }
+#undef SPMM_ONE
+    return 1;
+  }
   if (tdtype == 0) {
     if (a.v_dtype == 0) { SPMM_V(double, double) } else { SPMM_V(float, double) }
   } else {

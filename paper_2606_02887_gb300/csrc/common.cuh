@@ -174,7 +174,7 @@ struct AxArgs {
   const void* A; int64_t lda; int a_dtype;  // a_dtype: 0 f64, 1 f32, 2 bf16, 3 fp8(e4m3) + scales
   const float* a_scale;                     // fp8: per 128x128 tile scale (power of two)
   // csr
-  const int32_t* rowptr; const int32_t* colidx; const void* vals; int v_dtype;
+  const int32_t* rowptr; const int32_t* colidx; const void* vals; int v_dtype;  // lda: entries
   int kind;
   int accurate;  // BF16 dense: FP32 CUDA-core accumulation instead of the tensor-core product
   int sym;       // BF16 dense: A holds the upper tiles of the symmetric matrix (sym_tile)
