@@ -303,7 +303,8 @@ int launch_gemm_cfg(const AxArgs& a, int64_t n, int cols, int64_t ld, const void
   }
   if (tune && tune->splits > 0) splits = tune->splits;  // autotuned
   splits = std::max<int64_t>(1, std::min<int64_t>(splits, ws_elems / ((size_t)n * (size_t)ld)));
-  const int64_t kchunk = (cdiv64(n, (int)splits) + 31) / 32 * 32;
+  int64_t kchunk = (cdiv64(n, (int)splits) + 31) / 32 * 32;
+  if (C::KIND == GA_SAME && tune && tune->kchunk > 0) kchunk = tune->kchunk;
   splits = cdiv64(n, kchunk);
   constexpr int64_t KV = C::KV;
   const bool avec = C::KIND == GA_SAME && a.lda % KV == 0 && n % KV == 0 && !((uintptr_t)a.A & 15);

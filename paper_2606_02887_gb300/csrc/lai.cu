@@ -471,10 +471,17 @@ static int sketch_product(const AxArgs& A, int td, int64_t n, int cols, const vo
                           2000000000LL, s, nullptr, 2, A.sym);
     if (splits < 1) return -1;
   } else {
-    splits = launch_ax(A, td, n, cols, cols, X, Y, ws, ws_elems, nullptr, s);
+    // A dense product's sums in one order whatever its tiles are (as gram_plan_sketch): K in powers of two
+    // until 64 x 64 tiles would be two CTAs per SM, at least 256 columns each, or in one piece without the room.
+    ProdTune order;
+    const int64_t tiles = (int64_t)cdivi(cols, 64) * cdivi(n, 64);
+    int64_t sp = 1;
+    while (tiles * sp < 2 * 152 && n / (2 * sp) >= 256) sp *= 2;
+    if ((size_t)sp * (size_t)n * (size_t)cols > ws_elems) sp = 1;
+    order.splits = (int)sp;
+    order.kchunk = ((n + sp - 1) / sp + 15) / 16 * 16;
+    splits = launch_ax(A, td, n, cols, cols, X, Y, ws, ws_elems, nullptr, s, A.kind == AX_DENSE ? &order : nullptr);
   }
-  double* dummy = nullptr;
-  (void)dummy;
   return splits;
 }
 

@@ -93,7 +93,8 @@ struct GramPlan {
 GramPlan gram_plan(int tdtype, int64_t n, int r, int b);
 // The split of the eigen-sketch's Grams (n x ell, one level of at most 152 chunks over the tiles).
 // Which eigenpairs a sketch keeps near its cut, where they are close, depends on the last bits
-// of these sums: their order is part of what a seed reproduces.
+// of these sums and of the products (sketch_product in lai.cu): their order is part of what a seed
+// reproduces.
 GramPlan gram_plan_sketch(int64_t n, int ell);
 // G64[pair][b][r x r] = X_j^T Y_j per restart, GT the factor-type copy with lam_shift I when pair ==
 // tpair; rho_ctl: also rho = rho_scale ||G||_2 + rho_shift where the Gram is one tile (r <= 64).

@@ -2,6 +2,8 @@
 // its JSON cache keyed by device.
 #pragma once
 
+#include <stdint.h>
+
 #include <string>
 
 namespace snmf {
@@ -14,6 +16,7 @@ struct ProdTune {
   int bn = 0;       // tcgen05 product: output columns per CTA tile (multiple of 16, <= 256)
   int row_bm = 0;   // row kernels of a step (FP32): rows per CTA
   int row_tc = 0;   // the step's row products on the tensor cores (r = 64): 1 rowtc.cu, 2 rowtma.cu
+  int64_t kchunk = 0;  // CUDA-core product: columns of A per split, a multiple of 16 (not in the cache)
 };
 
 struct TuneEntry {

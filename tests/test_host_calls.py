@@ -301,3 +301,27 @@ for most in (0, 9 << 20, 7 << 20):  # a factor is 1 MB
 print(json.dumps([slices, codes]))
 """)
     assert codes == [S.SNMF_OK, S.SNMF_OK, S.SNMF_ERR_OOM] and most <= 8
+
+
+@pytest.mark.parametrize("n,k,precision", [(500, 10, S.SNMF_F32), (700, 64, S.SNMF_F64), (2048, 64, S.SNMF_F32),
+                                           (4100, 20, S.SNMF_F64), (12000, 64, S.SNMF_F32)])
+def test_sketch_product_keeps_its_order(fake, n, k, precision):
+    """K of a dense sketch's products is split by the rule that a seed's eigenpairs go with, whatever the
+    product's tiles: powers of two up to 304 CTAs of 64 x 64, 256 columns and four slices of workspace."""
+    got = fake(f"""
+n, k, precision = {n}, {k}, {precision}
+t = np.float64 if precision == S.SNMF_F64 else np.float32
+h = S.snmf_create(S.dense_matrix(np.ones((n, n), t)), 4, S.snmf_default_options(precision=precision))
+fake.fake_clear()
+try:
+    S.snmf_lai_sketch(h, k, 10, 2, 1)
+except S.SnmfError:
+    pass  # nothing runs, so the factorizations see zeros
+print(json.dumps([l[3][2] for l in log() if "k_gemm_dense" in l[2]]))
+""")
+    tiles, sp = -(-(k + 10) // 64) * -(-n // 64), 1
+    while tiles * sp < 304 and n // (2 * sp) >= 256:
+        sp *= 2
+    if sp > 4:
+        sp = 1
+    assert got == 4 * [-(-n // (-(-(-(-n // sp)) // 16) * 16))]
