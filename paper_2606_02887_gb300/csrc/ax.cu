@@ -152,9 +152,12 @@ k_ax_sum(int64_t total, T* __restrict__ Y, const T* __restrict__ ws, int splits,
 
 // Epilogue with inner products over a row tile x one restart.  splits > 1: Y = sum_s ws[s] (fixed
 // order).  V values of a row per access (16 bytes where r and the pitch allow it), two accesses of a
-// thread and their slices in flight.
+// thread and their slices in flight.  Single values are four times as many, for four times the threads.
+template <int V>
+constexpr int kFinishThreads = V > 1 ? 128 : 512;
+
 template <typename T, int V>
-__global__ void __launch_bounds__(128, 8)
+__global__ void __launch_bounds__(kFinishThreads<V>, 1024 / kFinishThreads<V>)
 k_ax_finish(int64_t n, int r, int64_t ld, T* __restrict__ Y, const T* __restrict__ ws,
             int splits, double c, const T* __restrict__ X2, const T* __restrict__ P1,
             const T* __restrict__ P2, double* __restrict__ part, int q0, int b,
@@ -162,7 +165,8 @@ k_ax_finish(int64_t n, int r, int64_t ld, T* __restrict__ Y, const T* __restrict
   struct alignas(V * sizeof(T)) Vec {
     T v[V];
   };
-  __shared__ T sh[2][4];
+  constexpr int NT = kFinishThreads<V>;
+  __shared__ T sh[2][NT / 32];
   const int j = blockIdx.y;
   const int64_t i0 = (int64_t)blockIdx.x * kRowTile;
   T d1 = T(0), d2 = T(0);  // per-CTA partials in the working type (FP64 across CTAs)
@@ -171,13 +175,13 @@ k_ax_finish(int64_t n, int r, int64_t ld, T* __restrict__ Y, const T* __restrict
     const int tile = rows * rv;
     const int64_t slice = n * ld;
     constexpr int U = 2;
-    for (int e0 = threadIdx.x; e0 < tile; e0 += 128 * U) {
+    for (int e0 = threadIdx.x; e0 < tile; e0 += NT * U) {
       Vec y[U];
       int64_t idx[U];
       bool ok[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int e = e0 + 128 * u;
+        const int e = e0 + NT * u;
         ok[u] = e < tile;
         const int i = ok[u] ? e / rv : 0;
         idx[u] = (i0 + i) * ld + (int64_t)j * r + (ok[u] ? e - i * rv : 0) * V;
@@ -230,8 +234,10 @@ k_ax_finish(int64_t n, int r, int64_t ld, T* __restrict__ Y, const T* __restrict
   }
   __syncthreads();
   if (threadIdx.x < 2) {
-    const T* v = sh[threadIdx.x];
-    part[((int64_t)blockIdx.x * b + j) * kNQ + q0 + threadIdx.x] = (double)(((v[0] + v[1]) + v[2]) + v[3]);
+    T v = sh[threadIdx.x][0];
+#pragma unroll
+    for (int w = 1; w < NT / 32; ++w) v += sh[threadIdx.x][w];
+    part[((int64_t)blockIdx.x * b + j) * kNQ + q0 + threadIdx.x] = (double)v;
   }
 }
 
@@ -413,7 +419,7 @@ int launch_ax_finish_impl(int tdtype, const Dims& d, void* Y, const void* ws, in
   }
   const bool vec = d.r % v == 0 && d.ld % v == 0 && !(all & 15);
 #define FIN(T, V)                                                                                                    \
-  k_ax_finish<T, V><<<grid, 128, 0, s>>>(d.n, d.r, d.ld, (T*)Y, (const T*)ws, splits, c, (const T*)X2, (const T*)P1, \
+  k_ax_finish<T, V><<<grid, kFinishThreads<V>, 0, s>>>(d.n, d.r, d.ld, (T*)Y, (const T*)ws, splits, c, (const T*)X2, (const T*)P1, \
                                          (const T*)P2, part, q0, d.b, run, dots_after)
   if (tdtype == 0) {
     if (vec) FIN(double, 2); else FIN(double, 1);

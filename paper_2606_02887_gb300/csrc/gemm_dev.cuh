@@ -100,6 +100,16 @@ __device__ __forceinline__ void gemm_tile(const TA* __restrict__ A, int64_t lda,
         const bool v = k + kk < k1 && col0 + c < cols;
         cp_async<16>(xs + kk * BN + c, v ? X + (k + kk) * ldx + col0 + c : X, v);
       }
+    } else if constexpr (NT % BN == 0) {  // one column of X per thread: no index arithmetic per value
+      const int c = t % BN, left = (int)min((int64_t)BK, k1 - k) - t / BN;
+      const bool on = col0 + c < cols;
+      const T* p = X + (k + t / BN) * ldx + col0 + c;
+#pragma unroll
+      for (int u = 0; u < BK * BN / NT; ++u) {
+        const bool v = on && u * (NT / BN) < left;
+        cp_async<(int)sizeof(T)>(xs + t + NT * u, v ? p : X, v);
+        p += NT / BN * ldx;
+      }
     } else {
       for (int e = t; e < BK * BN; e += NT) {
         const int kk = e / BN, c = e % BN;
@@ -163,11 +173,17 @@ __device__ __forceinline__ void gemm_tile(const TA* __restrict__ A, int64_t lda,
           const bool v = row0 + m < na && k + kk < k1;
           cp_async<16>(as + m * AS + kk, v ? A + (row0 + m) * lda + k + kk : A, v);
         }
-      } else {
-        for (int e = t; e < BM * BK; e += NT) {
-          const int m = e / BK, kk = e % BK;
-          const bool v = row0 + m < na && k + kk < k1;
-          cp_async<(int)sizeof(T)>(as + m * AS + kk, v ? A + (row0 + m) * lda + k + kk : A, v);
+      } else {  // one column of the stage per thread
+        static_assert(NT % BK == 0 && BM * BK % NT == 0, "whole rows of the stage");
+        const int kk = t % BK, m0 = t / BK, rows = (int)min((int64_t)BM, na - row0);
+        const bool on = k + kk < k1;
+        const T* p = A + (row0 + m0) * lda + k + kk;
+#pragma unroll
+        for (int u = 0; u < BM * BK / NT; ++u) {
+          const int m = m0 + u * (NT / BK);
+          const bool v = on && m < rows;
+          cp_async<(int)sizeof(T)>(as + m * AS + kk, v ? p : A, v);
+          p += NT / BK * lda;
         }
       }
       copy_x(k, as + C::A_ELEMS);
