@@ -294,7 +294,7 @@ k_knn_tc(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtens
           thr = fminf(thr, kd[KR - 1]);
         }
         if ((i & 7) == 7 && qv) {  // the bound of the query's other lists
-          const float mine = fmaxf(0.f, 2.f * kd[KR - 1] + nq * (1.f + KT_UP)) + KT_ABS;
+          const float mine = fmaxf(0.f, 2.f * kd[KR - 1] + nq * (1.f + KT_UP));
           if (mine < told) {
             atomicMin(reinterpret_cast<int*>(kth) + q, __float_as_int(mine));
             told = mine;
@@ -330,7 +330,8 @@ k_knn_tc(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtens
   }
 }
 
-// kth[q]: T_q, from the k-th smallest upper bound of the query's sorted lists (or what a list gave already).
+// kth[q]: T_q, from the k-th smallest upper bound of the query's sorted lists (or what a list gave already,
+// which pass 0 takes without the 2 a: its lists then miss none of the k smallest bounds).
 __global__ void __launch_bounds__(128) k_knn_bound(const float* __restrict__ lists, const float* __restrict__ nrm, int64_t n,
                                                    int k, int count, float* __restrict__ kth) {
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -356,7 +357,7 @@ __global__ void __launch_bounds__(128) k_knn_bound(const float* __restrict__ lis
     for (int l = 0; l < 2 * KT_PARTS; ++l)
       if (l == from && l < count) head[l] = ++at[l] < k ? lists[((int64_t)l * k + at[l]) * n + q] : INFINITY;
   }
-  kth[q] = fminf(kth[q], fmaxf(0.f, 2.f * v + nrm[q] * (1.f + KT_UP)) + KT_ABS);
+  kth[q] = fminf(kth[q], 2.f * v + nrm[q] * (1.f + KT_UP)) + KT_ABS;
 }
 
 // One warp per query: the distances of its candidates and the k nearest.
