@@ -329,8 +329,9 @@ int launch_ax(const AxArgs& a, int tdtype, int64_t n, int cols, int64_t ld, cons
   if (a.kind == AX_DENSE) {
     // The tile is as narrow as the columns allow: 128 columns where a tile of 64 would not save a
     // padded half (FP32 A: 8 x 16 values per thread, which reads a quarter less of the stages than
-    // 8 x 8: n = 8192, 512 columns 1281 -> 1174 us; the widened A need the registers: 1349 -> 1408), else 64 (three CTAs per SM, whose
-    // registers hold all operands, and for FP32 A stages of 32 columns: n = 8192, 64 columns 176 -> 161 us), 32, 16; FP64, whose pipes bound every size, down to 8 in steps that
+    // 8 x 8: n = 8192, 512 columns 1281 -> 1174 us; the widened A need the registers: 1349 -> 1408), else
+    // 64 (three CTAs per SM, whose registers hold all operands, and for FP32 A stages of 32 columns: n =
+    // 8192, 64 columns 176 -> 161 us), 32, 16; FP64, whose pipes bound every size, down to 8 in steps that
     // waste at most a third (n = 2500, 10 columns: 910 us in a 64-wide tile).  Fewer than two CTAs
     // per SM at the most splits: half the rows per tile.
 #define GEMM(T, TA, KIND, BM, BN, TM, TN, BK, OCC) \

@@ -528,7 +528,6 @@ RowArgs brow_base(BatchCtx* b, const Params& P) {
   a.run = b->run;
   a.part = b->prow;
   a.counters = b->counters;
-  a.G64fix = b->G64fix;
   a.P = P;
   return a;
 }

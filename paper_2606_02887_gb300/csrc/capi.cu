@@ -317,7 +317,6 @@ RowArgs row_base(snmf_ctx* h, const Params* P = nullptr) {
   a.gamma = h->graph ? h->gamma : 0.0;
   a.part = h->prow;
   a.counters = h->counters;
-  a.G64fix = h->G64fix;
   a.bm = h->row_bm;
   if (P) a.P = *P;
   return a;
@@ -377,7 +376,6 @@ snmf_status time_steps(snmf_ctx* h, int iters, double* ms_dstep, double* ms_upda
   ad.want_q = 1;
   ad.ctl_mode = CTL_LS;
   ad.dstore = nc == kNCand ? 4 : 0;
-  ad.D2out = h->buf[B_AD];
   RowArgs au = row_base(h, &P);  // the update of a W block
   au.B = h->buf[B_B];
   au.gout = h->buf[B_G];
@@ -385,7 +383,7 @@ snmf_status time_steps(snmf_ctx* h, int iters, double* ms_dstep, double* ms_upda
   au.Zold = h->buf[B_Z]; au.gZold = h->buf[B_GZ];
   au.Xout = X;
   au.ctl_mode = CTL_UPD_W;
-  au.Zin = h->buf[B_Z]; au.Din = h->buf[B_D]; au.Din2 = h->buf[B_AD];
+  au.Zin = h->buf[B_Z]; au.Din = h->buf[B_D];
   auto dstep = [&] {
     if (h->use_row) row_dstep(h, ad, nc);
     else launch_rowgemm(td, OP_ZSTEP, EPI_DIR, ad, h->s, nc);
@@ -664,7 +662,6 @@ void pen_block(snmf_ctx* h, int xv, int xf, bool is_w, const Params& P, bool nai
         a.ctl_mode = fused_q ? CTL_LS : CTL_NONE;  // line search in the last CTA of each restart
         const int nc = h->opt.step_controller == 2 ? kNCand : 1;  // record mode: 9 candidates
         a.dstore = nc == kNCand ? 4 : 0;
-        a.D2out = h->buf[B_AD];
         launch_rowgemm(td, OP_ZSTEP, EPI_DIR, a, h->s, nc);
       }
     }
@@ -692,7 +689,7 @@ void pen_block(snmf_ctx* h, int xv, int xf, bool is_w, const Params& P, bool nai
         a.X = h->buf[B_XN]; a.LX = h->buf[B_LX];
         launch_rowgemm(td, OP_LOAD, EPI_GRAD, a, h->s);
       } else {
-        a.Zin = h->buf[B_Z]; a.Din = h->buf[B_D]; a.Din2 = h->buf[B_AD];
+        a.Zin = h->buf[B_Z]; a.Din = h->buf[B_D];
         launch_rowgemm(td, OP_UPD, EPI_GRAD, a, h->s);
       }
     }

@@ -5,7 +5,7 @@
 //   columns [j r, (j+1) r).  Element type T = double (FP64 precision) or float.
 //   partial sums: part[slot][restart][NQ] (double), one slot per CTA of a row kernel,
 //   reduced in a fixed order by the control kernels (deterministic, no atomics).
-//   Gram partials: gpart[chunk][pair][restart][r*r] (double), reduced in fixed order.
+//   Gram partials: gpart[restart tile][chunk, then group][tile] in the factor type, reduced in a fixed order.
 #pragma once
 
 #include <cuda_bf16.h>

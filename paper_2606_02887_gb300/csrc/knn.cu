@@ -57,11 +57,11 @@ namespace snmf {
 namespace {
 
 // The k nearest of the candidates [z per, (z + 1) per) for the 64 queries of CTA (x, z): partial
-// lists at [z][n][k], sorted by distance and then index (empty slots are (inf, INT_MAX)).  Distances of a 128 x 64 tile, 8 candidates x 4 queries per thread, two
-// candidates per instruction: sum over t ascending of (q_t - c_t)^2 with one FMA each, candidates
-// staged negated.  A distance not above the query's k-th so far goes to the query's buffer in shared
-// memory; after the tile its warp (eight queries each) inserts the buffer, in any order with the
-// same result.  A non-finite distance counts as +inf and raises *bad.  Bound by the FP32 pipes (2 n^2 d
+// lists at [z][n][k], sorted by distance and then index (empty slots are (inf, INT_MAX)).  Distances of
+// a 128 x 64 tile, 8 candidates x 4 queries per thread, two candidates per instruction: sum over t
+// ascending of (q_t - c_t)^2 with one FMA each, candidates staged negated.  A distance not above the
+// query's k-th so far goes to the query's buffer in shared memory; after the tile its warp (eight queries
+// each) inserts the buffer, in any order with the same result.  A non-finite distance counts as +inf and raises *bad.  Bound by the FP32 pipes (2 n^2 d
 // lane operations): n = 20000, d = 64, k = 10 2.94 ms (23.1 ms with one thread per query and the list
 // updated for every candidate).  For few or wide points, and where the filter (knn_tc.cuh) gave up.
 struct KnnSmem {

@@ -526,9 +526,6 @@ __global__ void __launch_bounds__(256) k_ctl_final_dir(Ctl* __restrict__ ctl, co
 // ---------------------------------------------------------------------------
 // host launchers
 // ---------------------------------------------------------------------------
-// ---------------------------------------------------------------------------
-// host launchers
-// ---------------------------------------------------------------------------
 static int rowgemm_bm(const Dims& d, int tdtype) {
   if (tdtype == 0) return 32;  // FP64: keeps the operand/D tile and the G tile within 48 KB
   return (d.n + 63) / 64 * ((d.r + 63) / 64) * d.b >= 2 * 152 ? 64 : 32;

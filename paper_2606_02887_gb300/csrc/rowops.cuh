@@ -35,8 +35,6 @@ struct RowArgs {
   void* Xout;          // operand value written (Z for OP_ZSTEP, X' for OP_UPD/OP_LOAD copy)
   void* gout;          // EPI_GRAD: gradient
   void* Dout;          // EPI_DIR: direction (candidate `dstore`)
-  void* D2out;         // EPI_DIR with two candidates: the plain BB direction
-  const void* Din2;    // OP_UPD: second direction, used where ctl[j].dsel == 1
   int dstore;          // EPI_DIR: candidate written to Dout
   void* gZout;         // EPI_DIR: gradient at Z
   const void* Xold; const void* gold;    // EPI_GRAD: S = X - Xold, Y = g - gold
@@ -47,7 +45,6 @@ struct RowArgs {
   double* part;
   int ctl_mode;        // CTL_*: control step run by the last CTA of each restart
   unsigned* counters;  // per-restart arrival counters (zero between launches)
-  const double* G64fix;
   Params P;
   int bm;              // general body, FP32: rows per CTA (32 or 64; 0 = built-in choice)
 };

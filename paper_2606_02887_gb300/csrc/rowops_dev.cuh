@@ -113,27 +113,6 @@ __device__ double dot_rr(const double* A, const double* B, int r, double* sh) {
   return block_sum(s, sh);
 }
 
-// sum_{p,q} (M + M^T)_{pq} X_{pq} for a general r x r M and symmetric X
-__device__ double dot_sym2(const double* M, const double* X, int r, double* sh) {
-  double s = 0.0;
-  for (int e = threadIdx.x; e < r * r; e += blockDim.x) {
-    const int p = e / r, q = e % r;
-    s += (M[e] + M[q * r + p]) * X[e];
-  }
-  return block_sum(s, sh);
-}
-
-// <M+M^T, M+M^T> for general M
-__device__ double norm_sym2(const double* M, int r, double* sh) {
-  double s = 0.0;
-  for (int e = threadIdx.x; e < r * r; e += blockDim.x) {
-    const int p = e / r, q = e % r;
-    const double v = M[e] + M[q * r + p];
-    s += v * v;
-  }
-  return block_sum(s, sh);
-}
-
 __device__ double bb_step(const Ctl& c, const Params& P, double rho) {
   // Alg. 1 line 3 / Eq. (2.10), with the fallback 1/rho when <S,Y> <= 0
   double a;
@@ -451,8 +430,8 @@ __device__ __forceinline__ void rowgemm_body(const RowArgs& a, int j, int bx, in
   constexpr int XS_ELEMS = BM * (KC + 1);
   constexpr int DS_ELEMS = (EPI == EPI_DIR) ? BM * 65 : 1;
   constexpr int U_ELEMS = XS_ELEMS > DS_ELEMS ? XS_ELEMS : DS_ELEMS;
-  constexpr int NV = NC > 2 ? 32 : 8;  // partial values written per CTA (NC = 2 uses 8)
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  constexpr int NV = NC > 1 ? 32 : 8;  // partial values written per CTA
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const int64_t row0 = (int64_t)bx * BM;
   const int col0 = by * 64;  // within restart
   const int r = a.r;
@@ -475,7 +454,7 @@ __device__ __forceinline__ void rowgemm_body(const RowArgs& a, int j, int bx, in
     const T* X = (const T*)a.X;
     const T* gin = (const T*)a.g_in;
     const T* Zin = (const T*)a.Zin;
-    const T* Din = (const T*)((OP == OP_UPD && cj.dsel) ? a.Din2 : a.Din);
+    const T* Din = (const T*)a.Din;
     T alph[NC];
 #pragma unroll
     for (int m = 0; m < NC; ++m) alph[m] = (T)(NC == 1 ? cj.alpha : cj.cand_alpha[m]);
@@ -605,7 +584,6 @@ __device__ __forceinline__ void rowgemm_body(const RowArgs& a, int j, int bx, in
             T d = xv - alph[m] * g;
             d = (d > T(0) ? d : T(0)) - xv;
             if (m == a.dstore) ((T*)a.Dout)[idx] = d;
-            if (NC == 2 && m == 1) ((T*)a.D2out)[idx] = d;
             const int base = m == 0 ? 0 : 5 + 3 * (m - 1);
             dq[base] += g * d;                              // <grad f(Z), D_m>
             dq[base + 1] += d * d;                          // ||D_m||^2
@@ -701,7 +679,7 @@ __device__ __forceinline__ void rowgemm_body(const RowArgs& a, int j, int bx, in
     __syncthreads();
     if (ticket == per - 1) {
       if (threadIdx.x == 0) a.counters[j] = 0u;
-      control_tail<(NC > 2 ? kNQ : 8)>(a, j, 0, (int)per, NC);
+      control_tail<NV>(a, j, 0, (int)per, NC);
     }
   }
 }
