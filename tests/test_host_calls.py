@@ -287,11 +287,13 @@ def test_handle_with_room_for_eight_slices(fake):
     """A dense handle whose device has no room for ten split-K slices takes eight, and is not refused."""
     most, codes = fake("""
 n, r = 1024, 256
-A, codes = np.ones((n, n), np.float32), []
-for most in (0, 9 << 20, 7 << 20):  # a factor is 1 MB
-    fake.fake_memory(most)
+A, codes, whole = np.ones((n, n), np.float32), [], 0
+for less in (0, 1, 3 << 20):  # a factor is 1 MB, and eight slices take 2 MB less than ten
+    fake.fake_memory(max(0, whole - less))
     try:
+        fake.fake_clear()
         h = S.snmf_create(S.dense_matrix(A), r, S.snmf_default_options(max_iter=1, inner_iters=1))
+        whole = whole or max(int(l.split()[1]) for l in fake.fake_log().decode().splitlines() if l.startswith("alloc"))
         W = np.ones((n, r), np.float32)
         fake.fake_clear()
         codes.append(S.snmf_solve_host(h, W, W.copy())[0])
