@@ -11,7 +11,7 @@ namespace snmf {
 namespace {
 
 // Gram of one restart's columns: CTA (chunk, restart x tile), see gram_body.
-template <typename T, int TW, int VEC>
+template <typename T, int TW, int VEC, int M = 4>
 __global__ void __launch_bounds__(256, 3)
 k_gram(const T* __restrict__ X, const T* __restrict__ Y, int64_t n, int r, int64_t ld, GramPlan pl,
        T* __restrict__ gpart, const Ctl* __restrict__ ctl, const int* run, double* __restrict__ G64,
@@ -31,7 +31,7 @@ k_gram(const T* __restrict__ X, const T* __restrict__ Y, int64_t n, int r, int64
   o.rho_iters = rho_iters;
   o.rho_scale = rho_scale;
   o.rho_shift = rho_shift;
-  gram_body<T, TW, VEC>(X + (int64_t)j * r + o.p0, Y + (int64_t)j * r + o.q0, min(TW, r - o.p0), min(TW, r - o.q0), ld,
+  gram_body<T, TW, VEC, M>(X + (int64_t)j * r + o.p0, Y + (int64_t)j * r + o.q0, min(TW, r - o.p0), min(TW, r - o.q0), ld,
                         n, pl.chunk, blockIdx.x, pl.nch, pl.ng, X == Y && o.p0 == o.q0,
                         gpart + (int64_t)blockIdx.y * (pl.nch + pl.ng) * (TW * TW), counters + (int64_t)blockIdx.y * (1 + pl.ng),
                         o, reinterpret_cast<T*>(gsm));
@@ -127,8 +127,11 @@ GramPlan gram_plan(int tdtype, int64_t n, int r, int b) {
 }
 
 GramPlan gram_plan_sketch(int64_t n, int ell) {
+  // one chain per entry: 2 x 2 micro tiles in a 32-wide tile (a sketch of 18 columns, FP64 n = 500: 5.60 ms with
+  // the 64-wide tile for every width, 2.94 so)
   GramPlan pl;
-  pl.tw = 64;
+  pl.micro = ell <= 32 ? 2 : 4;
+  pl.tw = 16 * pl.micro;
   pl.ntile = (ell + 63) / 64;
   const int64_t tiles = (int64_t)pl.ntile * pl.ntile;
   const int64_t nch = std::max<int64_t>(1, std::min<int64_t>(152 / tiles, n / 512));
@@ -140,15 +143,15 @@ GramPlan gram_plan_sketch(int64_t n, int ell) {
   return pl;
 }
 
-template <typename T, int TW, int VEC>
+template <typename T, int TW, int VEC, int M = 4>
 static void launch_gram_t(const void* X, const void* Y, const Dims& d, const GramPlan& pl, void* gpart, const Ctl* ctl,
                           const int* run, double* G64, void* GT, double lam, unsigned* counters, Ctl* rho_ctl,
                           int rho_iters, double rho_scale, double rho_shift, cudaStream_t s) {
   static SmemLimit limit;
-  raise_smem_limit(limit, (const void*)k_gram<T, TW, VEC>, gram_smem<T>(false));
+  raise_smem_limit(limit, (const void*)k_gram<T, TW, VEC, M>, gram_smem<T>(false));
   const size_t smem = gram_smem<T>(X == Y && pl.ntile == 1);
   dim3 grid(pl.nch, d.b * pl.ntile * pl.ntile);
-  k_gram<T, TW, VEC><<<grid, 256, smem, s>>>((const T*)X, (const T*)Y, d.n, d.r, d.ld, pl, (T*)gpart, ctl, run, G64,
+  k_gram<T, TW, VEC, M><<<grid, 256, smem, s>>>((const T*)X, (const T*)Y, d.n, d.r, d.ld, pl, (T*)gpart, ctl, run, G64,
                                              (T*)GT, (T)lam, counters, rho_ctl, rho_iters, rho_scale, rho_shift);
 }
 
@@ -161,11 +164,13 @@ void launch_gram(int tdtype, const void* X, const void* Y, const Dims& d, const 
   // 16-byte copies when every restart's rows start on 16 bytes
   const int v = tdtype == 0 ? 2 : 4;
   const bool vec = d.r % v == 0 && d.ld % v == 0 && !((uintptr_t)X & 15) && !((uintptr_t)Y & 15);
-#define GRAM(T, TW, V)                                                                                             \
-  launch_gram_t<T, TW, V>(X, Y, d, pl, gpart, ctl, run, G64, GT, lam_shift, counters, rho_ctl, rho_iters, rho_scale, \
+#define GRAM(T, ...)                                                                                               \
+  launch_gram_t<T, __VA_ARGS__>(X, Y, d, pl, gpart, ctl, run, G64, GT, lam_shift, counters, rho_ctl, rho_iters, rho_scale, \
                           rho_shift, s)
 #define GRAM_T(T, V)                            \
-  if (pl.tw == 16) {                            \
+  if (pl.micro == 2) {                          \
+    if (vec) GRAM(T, 32, V, 2); else GRAM(T, 32, 1, 2); \
+  } else if (pl.tw == 16) {                     \
     if (vec) GRAM(T, 16, V); else GRAM(T, 16, 1); \
   } else if (pl.tw == 32) {                     \
     if (vec) GRAM(T, 32, V); else GRAM(T, 32, 1); \

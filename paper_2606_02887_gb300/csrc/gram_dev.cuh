@@ -189,22 +189,23 @@ __device__ __forceinline__ void rho_in_smem(const T* Gs, int r, int iters, doubl
 // ------------------------------------------------------------------------------
 // One chunk of rows [i_begin, i_end) of a TP x TQ tile of X^T Y: X, Y at the tile's first columns
 // (wx, wy of them exist), row pitches ldx, ldy, VEC elements per copy (16 bytes when the columns and
-// the pitches allow it, else single elements).  256 threads: NG = 4096 / (TP TQ) row groups, each a
-// (TP / 4) x (TQ / 4) grid of 4 x 4 micro tiles read as two 16-byte shared loads per row.  The
+// the pitches allow it, else single elements).  256 threads: NG = 256 M M / (TP TQ) row groups, each a
+// (TP / M) x (TQ / M) grid of M x M micro tiles, M = 4 read as two 16-byte shared loads per row.  The
 // groups' sums leave the row loop in shared memory; the thread returns its entries e = 4 (t + 256 u).
+// NG = 1: every entry is one chain over the chunk's rows in order.
 // Bound by HBM for long factors (n = 2e6, r = 32: 797 us with 152 chunks of two staged rounds
 // and scalar shared reads, 177 us so) and by latency for short ones.
 // ------------------------------------------------------------------------------
 template <int TP, int TQ>
 __host__ __device__ constexpr int tile_quads() { return TP * TQ >= 1024 ? TP * TQ / 1024 : 1; }  // 16-byte entries per thread
 
-template <typename T, int TP, int TQ, int VEC>
+template <typename T, int TP, int TQ, int VEC, int M = 4>
 __device__ __forceinline__ void gram_chunk(const T* __restrict__ X, const T* __restrict__ Y, int wx, int wy, int64_t ldx,
                                            int64_t ldy, int64_t i_begin, int64_t i_end, bool same, T* sm,
                                            Quad<T> (&out)[tile_quads<TP, TQ>()]) {
   constexpr int TM = TP > TQ ? TP : TQ;
   constexpr int RS = kGramStageBytes / (TM * (int)sizeof(T));  // rows per stage
-  constexpr int NG = 4096 / (TP * TQ), GT = 256 / NG, TX = TQ / 4;
+  constexpr int NG = 256 * M * M / (TP * TQ), GT = 256 / NG, TX = TQ / M;
   constexpr int SX = RS * TP, SY = RS * TQ;
   const int t = threadIdx.x;
   T* Xs = sm;
@@ -230,11 +231,14 @@ __device__ __forceinline__ void gram_chunk(const T* __restrict__ X, const T* __r
     if (s < rounds) fetch(i_begin + (int64_t)s * RS, s);
     cp_async_commit();
   }
-  T acc[4][4];
+  struct alignas(M * sizeof(T) < 16 ? M * sizeof(T) : 16) Few {
+    T v[M];
+  };
+  T acc[M][M];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < M; ++a)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) acc[a][c] = T(0);
+    for (int c = 0; c < M; ++c) acc[a][c] = T(0);
   const int grp = t / GT, tx = (t % GT) % TX, ty = (t % GT) / TX;
   for (int k = 0; k < rounds; ++k) {
     cp_async_wait<kGramStages - 2>();
@@ -242,24 +246,27 @@ __device__ __forceinline__ void gram_chunk(const T* __restrict__ X, const T* __r
     if (k + kGramStages - 1 < rounds)
       fetch(i_begin + (int64_t)(k + kGramStages - 1) * RS, (k + kGramStages - 1) % kGramStages);
     cp_async_commit();
-    const T* xs = Xs + (k % kGramStages) * SX + 4 * ty;
-    const T* ys = Ys + (k % kGramStages) * SY + 4 * tx;
+    const T* xs = Xs + (k % kGramStages) * SX + M * ty;
+    const T* ys = Ys + (k % kGramStages) * SY + M * tx;
 #pragma unroll 4
     for (int rr = grp; rr < RS; rr += NG) {
-      const Quad<T> xa = *reinterpret_cast<const Quad<T>*>(xs + rr * TP);
-      const Quad<T> yb = *reinterpret_cast<const Quad<T>*>(ys + rr * TQ);
+      const Few xa = *reinterpret_cast<const Few*>(xs + rr * TP);
+      const Few yb = *reinterpret_cast<const Few*>(ys + rr * TQ);
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
+      for (int a = 0; a < M; ++a)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[a][c] = fma(xa.v[a], yb.v[c], acc[a][c]);
+        for (int c = 0; c < M; ++c) acc[a][c] = fma(xa.v[a], yb.v[c], acc[a][c]);
     }
   }
   cp_async_wait<0>();
   __syncthreads();  // the ring is free: it takes the groups' tiles
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
-    *reinterpret_cast<Quad<T>*>(sm + grp * TP * TQ + (4 * ty + a) * TQ + 4 * tx) =
-        Quad<T>{{acc[a][0], acc[a][1], acc[a][2], acc[a][3]}};
+  for (int a = 0; a < M; ++a) {
+    Few f;
+#pragma unroll
+    for (int c = 0; c < M; ++c) f.v[c] = acc[a][c];
+    *reinterpret_cast<Few*>(sm + grp * TP * TQ + (M * ty + a) * TQ + M * tx) = f;
+  }
   __syncthreads();
 #pragma unroll
   for (int u = 0; u < tile_quads<TP, TQ>(); ++u) {
@@ -353,7 +360,7 @@ struct GramOut {
 };
 
 // CTA `c` of the nch chunks of one Gram tile (see sum_chunks).
-template <typename T, int TW, int VEC>
+template <typename T, int TW, int VEC, int M = 4>
 __device__ __forceinline__ void gram_body(const T* X, const T* Y, int wx, int wy, int64_t ld, int64_t n, int64_t chunk,
                                           int c, int nch, int ng, bool same, T* gp, unsigned* cnt, const GramOut<T>& o,
                                           T* sm) {
@@ -362,7 +369,7 @@ __device__ __forceinline__ void gram_body(const T* X, const T* Y, int wx, int wy
   const bool owns = 4 * t < TW * TW;
   Quad<T> s[NE];
   const int64_t i0 = (int64_t)c * chunk;
-  gram_chunk<T, TW, TW, VEC>(X, Y, wx, wy, ld, ld, i0, min(n, i0 + chunk), same, sm, s);
+  gram_chunk<T, TW, TW, VEC, M>(X, Y, wx, wy, ld, ld, i0, min(n, i0 + chunk), same, sm, s);
   if (!sum_chunks<T, TW * TW>(s, c, nch, ng, gp, cnt)) return;
 #pragma unroll
   for (int u = 0; u < NE; ++u) {

@@ -84,6 +84,7 @@ bool launch_rowtma_update(const RowArgs& a, int* err, cudaStream_t s);
 // part_elems factor-type elements of partials and `counters` zeroed arrival counters.
 struct GramPlan {
   int tw, ntile, nch, ng;
+  int micro = 4;  // edge of a thread's micro tile
   int64_t chunk;
   size_t part_elems, counters;
 };
